@@ -11,6 +11,7 @@
 #include "cv_mlp.cuh"
 #include "dd_df64.cuh"
 #include "kernels.cuh"
+#include "mo.cuh"
 #include "oz_gemm.cuh"
 #include "tc_gemm.cuh"
 #include "tc_group.cuh"
@@ -132,6 +133,11 @@ struct rssri_handle {
   DevBuf facHl, xgHl, cHl, bHl;
   bool d_df64_ready = false;
   bool kp_hl_ready = false;  // K_P as pairs (KPhl) made for this setup
+  // orbital-basis chain (mo.cuh): diagonals of G per tau, C as pairs, the transformed
+  // factors, M of a chunk of tau points, its traces, Sigma in the orbital basis
+  DevBuf moTab, moChl, moZ, moM, moTr, moAcc, moWork;
+  bool mo_tab_ready = false;  // moTab, moChl made for this setup
+  bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
   // bf16 chain buffers
   DevBuf hxsl, hy3, hg, hgb, hP, hdc32, hcl32, hdcl16, hxy32, ha6, hct, hdct, hpart, hfold;
   DevBuf hclt, hfl;  // learned control variate on the tensor-core chain: (C^L)^T, F^L per pair
@@ -414,6 +420,12 @@ int metric_inv_sqrt(rssri_handle *h, int *rc, bool df64) {
 }
 
 
+// Largest |C^T C - I| for which the orbital-basis chain replaces the general
+// one: its result is (C C^T) Sigma (C C^T), so a deviation d costs about 2 d
+// relative, which stays at the rounding error of the products themselves
+// (orbitals from QR or a symmetric eigensolver are at 1e-15 to 1e-14).
+constexpr double MO_ORTH_TOL = 5e-14;
+
 // S6 and S7 for every tau (defined below).
 int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double *gb_in);
 
@@ -486,7 +498,8 @@ void rssri_destroy(rssri_handle *h) {
                     &h->hdcl16, &h->hxy32, &h->ha6, &h->hct, &h->hdct, &h->hpart, &h->hfold, &h->hclt, &h->hfl, &h->Dhl,
                     &h->Ahl, &h->KPhl, &h->PGhl, &h->APhl, &h->Gamhl, &h->GGhl, &h->litMP, &h->litT, &h->litMhl, &h->eri_hl, &h->ut_hl, &h->nsA2, &h->nsB2, &h->elHl, &h->facHl, &h->xgHl, &h->cHl, &h->bHl, &h->cv_params, &h->cv_m, &h->cv_v, &h->cv_grad, &h->cv_ptmp,
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
-                    &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp};
+                    &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
+                    &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork};
   for (DevBuf *b : bufs) release(*b);
   release(h->oz_pidx);
   release(h->oz_tmp);
@@ -525,6 +538,7 @@ int rssri_setup(rssri_handle *h, const rssri_problem *p, const rssri_options *o)
   h->block_ok = false;
   h->gg_valid = false;
   h->oz_ready = false;
+  h->mo_tab_ready = false;
   const int n = p->n, na = p->n_aux, nt = p->n_tau;
   const long long nn = (long long)n * n;
   cudaError_t e;
@@ -575,8 +589,22 @@ int rssri_setup(rssri_handle *h, const rssri_problem *p, const rssri_options *o)
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(nonfinite_check(h->metric, (long long)na * na, flags + 1, s)); }
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(nonfinite_check(h->orb_e, n, flags + 1, s)); }
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(nonfinite_check(h->orb_c, nn, flags + 1, s)); }
-  int hflags[2];
-  RS_CK(fetch(hflags, flags, s, 2));
+  // C^T C = I to rounding, as the interface asks for: where it does not hold
+  // that closely, every product keeps the general form that needs no C^T C = I
+  {
+    RS_CK(ensure(h->moAcc, nn * sizeof(double)));
+    GemmArgs g;
+    g.M = g.N = g.K = n;
+    g.A = h->orb_c; g.lda = n; g.transA = 1;
+    g.B = h->orb_c; g.ldb = n;
+    g.C = h->moAcc.as<double>(); g.ldc = n;
+    RS_CK(gemm_p(h, RSSRI_PROF_OTHER, g));
+    SPAN(RSSRI_PROF_OTHER, 0.0);
+    RS_CK(mo_orth_check(h->moAcc.as<double>(), n, MO_ORTH_TOL, flags + 2, s));
+  }
+  int hflags[3];
+  RS_CK(fetch(hflags, flags, s, 3));
+  h->orth_ok = hflags[2] == 0;
   if (hflags[1]) return RSSRI_ERR_NONFINITE;
   if (hflags[0]) return RSSRI_ERR_NONSYMMETRIC_ERI;
 
@@ -1542,6 +1570,161 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
   return cudaSuccess;
 }
 
+// ------------------------------------------- the chain on the orbitals (S8) --
+// Layout of moTab: gv [nt][nv] and go [nt][no] in fp64, the same as scaled
+// pairs, and the two exponents per tau (see mo_tables).
+struct MoTab {
+  double *gv, *go;
+  float2 *gvhl, *gohl;
+  int *texp, *eexp;
+};
+MoTab mo_tab(rssri_handle *h) {
+  const size_t nt = h->n_tau, no = h->n_occ, nv = h->n - h->n_occ;
+  MoTab t;
+  t.gv = h->moTab.as<double>();
+  t.go = t.gv + nt * nv;
+  t.gvhl = reinterpret_cast<float2 *>(t.go + nt * no);
+  t.gohl = t.gvhl + nt * nv;
+  t.texp = reinterpret_cast<int *>(t.gohl + nt * no);
+  t.eexp = t.texp + nt;
+  return t;
+}
+cudaError_t ensure_mo_tab(rssri_handle *h) {
+  if (h->mo_tab_ready) return cudaSuccess;
+  const size_t nt = h->n_tau, n = h->n;
+  RS_TRY(ensure(h->moTab, nt * n * 16 + nt * 2 * sizeof(int)));
+  RS_TRY(ensure(h->moChl, n * n * sizeof(float2)));
+  const MoTab t = mo_tab(h);
+  SPAN(RSSRI_PROF_GREEN, 0.0);
+  RS_TRY(mo_tables(h->orb_e, h->n, h->n_occ, h->mu, h->tau, h->n_tau, 1, t.gv, t.go, t.gvhl,
+                   t.gohl, t.texp, t.eexp, h->stream));
+  RS_TRY(to_df64(h->orb_c, (long long)n * n, h->moChl.as<float2>(), h->stream));
+  h->mo_tab_ready = true;
+  return cudaSuccess;
+}
+
+// Whether S8 runs on the orbitals: G is the orbitals' (not a caller's), and
+// its flops per pair and kind, 8 n^2 n_v for the transforms and 2 n^3 per tau
+// point, are fewer than the general form's 8 n^3 per tau point.
+bool use_mo_chain(const rssri_handle *h) {
+  return h->orth_ok && 4LL * (h->n - h->n_occ) < 3LL * h->n_tau * h->n;
+}
+
+// S8 and the orbital-basis sum of S10 for all pairs, in batches of nb pairs and
+// chunks of tau points: sig[t] = sdd[t] + (C (sum over pairs of F) C^T) / ns, and
+// the pair energies are added to e_st.
+cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const double *sdd,
+                     double *sig) {
+  cudaStream_t s = h->stream;
+  const int n = h->n, no = h->n_occ, nv = n - no, nt = h->n_tau;
+  const long long nn = (long long)n * n, nz = (long long)n * nv;
+  RS_TRY(ensure_mo_tab(h));
+  const MoTab tab = mo_tab(h);
+  // M of a chunk of tau points: 256 MB at most (small problems: all tau points
+  // in one launch), one tau point at least
+  const size_t per_tau = (size_t)nkind * nb * nn * 8;
+  const int tc = (int)std::max<size_t>(1, std::min<size_t>(nt, ((size_t)256 << 20) / per_tau));
+  RS_TRY(ensure(h->moZ, (size_t)2 * nkind * nb * nz * 8));
+  RS_TRY(ensure(h->moM, std::max({per_tau * tc, (size_t)(2LL * nkind * nb * nz * 8),
+                                 (size_t)(nt * nn * 8)})));
+  RS_TRY(ensure(h->moTr, (size_t)2 * tc * nkind * nb * sizeof(double)));
+  RS_TRY(ensure(h->moAcc, (size_t)nt * nn * sizeof(double)));
+  MoSum q;
+  q.df = df; q.n = n; q.no = no; q.nkind = nkind;
+  size_t work = 0;
+  for (int c : {std::min(nb, ns), ns % nb ? ns % nb : nb})
+    for (int t : {tc, nt % tc ? nt % tc : tc}) {
+      q.cnt = c;
+      q.nt = t;
+      work = std::max(work, mo_sum_work(q));
+    }
+  RS_TRY(ensure(h->moWork, work * sizeof(double)));
+  // Z = C^T F C_v of `batch` consecutive factors F, T = F C_v in the buffer of M
+  auto transform = [&](long long f0, long long z0, int batch) -> cudaError_t {
+    if (df) {
+      float2 *T = h->moM.as<float2>();
+      DfGemm g;
+      g.M = n; g.N = nv; g.K = n; g.batch = batch;
+      g.A = h->facHl.as<float2>() + f0; g.lda = n; g.sA = nn;
+      g.B = h->moChl.as<float2>() + no; g.ldb = n;
+      g.C2 = T; g.ldc = nv; g.sC = nz;
+      RS_TRY(df_gemm_c(h, RSSRI_PROF_CHAIN_GEMM, g));
+      g.A = h->moChl.as<float2>(); g.sA = 0; g.transA = 1;
+      g.B = T; g.ldb = nv; g.sB = nz;
+      g.C2 = h->moZ.as<float2>() + z0;
+      return df_gemm_c(h, RSSRI_PROF_CHAIN_GEMM, g);
+    }
+    double *T = h->moM.as<double>();
+    GemmArgs g;
+    g.M = n; g.N = nv; g.K = n; g.batch = batch;
+    g.A = h->fac.as<double>() + f0; g.lda = n; g.sA = nn;
+    g.B = h->orb_c + no; g.ldb = n;
+    g.C = T; g.ldc = nv; g.sC = nz;
+    RS_TRY(gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g));
+    g.A = h->orb_c; g.sA = 0; g.transA = 1;
+    g.B = T; g.ldb = nv; g.sB = nz;
+    g.C = h->moZ.as<double>() + z0;
+    return gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g);
+  };
+  for (int x0 = 0; x0 < ns; x0 += nb) {
+    const int cnt = std::min(nb, ns - x0);
+    // Z [set][kind][x]; fac is [set][2 kinds][ns]
+    if (cnt == ns && nkind == 2 && 4LL * ns <= 65535) {
+      RS_TRY(transform(0, 0, 4 * ns));
+    } else {
+      for (int set = 0; set < 2; ++set)
+        for (int k = 0; k < nkind; ++k)
+          RS_TRY(transform(((2LL * set + k) * ns + x0) * nn, ((long long)set * nkind + k) * cnt * nz,
+                           cnt));
+    }
+    for (int t0 = 0; t0 < nt; t0 += tc) {
+      const int c = std::min(tc, nt - t0);
+      const void *gv = df ? (const void *)(tab.gvhl + (long long)t0 * nv)
+                          : (const void *)(tab.gv + (long long)t0 * nv);
+      const void *go = df ? (const void *)(tab.gohl + (long long)t0 * no)
+                          : (const void *)(tab.go + (long long)t0 * no);
+      double *tr = h->moTr.as<double>(), *s2 = tr + (long long)c * nkind * cnt;
+      MoNt g;
+      g.df = df;
+      g.M = g.N = n; g.K = nv; g.nb = nkind * cnt; g.nt = c;
+      g.A = h->moZ.p;
+      g.B = static_cast<const char *>(h->moZ.p) + (size_t)nkind * cnt * nz * 8;
+      g.lda = g.ldb = nv; g.sA = g.sB = nz;
+      g.ks = gv; g.sks = nv;
+      g.out = h->moM.p;
+      {
+        SPAN(RSSRI_PROF_CHAIN_GEMM, 2.0 * nn * nv * nkind * (double)cnt * c * 1e-9);
+        RS_TRY(mo_nt(g, s));
+      }
+      {
+        SPAN(RSSRI_PROF_OTHER, 0.0);
+        RS_TRY(mo_traces(df, h->moM.p, c, nkind * cnt, n, no, go, no, tr, s2, s));
+        RS_TRY(mo_energy(tr, s2, c, nkind, cnt, h->tau_w + t0, df ? tab.eexp + t0 : nullptr,
+                         2.0 * no, h->e_st.as<double>() + x0, s));
+      }
+      q.cnt = cnt; q.nt = c;
+      q.M = h->moM.p; q.go = go; q.sgo = no; q.tr = tr;
+      q.texp = df ? tab.texp + t0 : nullptr;
+      q.acc = h->moAcc.as<double>() + t0 * nn;
+      q.accumulate = x0 > 0;
+      SPAN(RSSRI_PROF_CHAIN_GEMM, 2.0 * nn * no * nkind * (double)cnt * c * 1e-9);
+      RS_TRY(mo_sum(q, h->moWork.as<double>(), s));
+    }
+  }
+  // sig = sdd + C acc C^T / ns
+  RS_TRY(cudaMemcpyAsync(sig, sdd, nt * nn * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  GemmArgs g;
+  g.M = g.N = g.K = n; g.batch = nt;
+  g.lda = g.ldb = g.ldc = n;
+  g.A = h->orb_c; g.B = h->moAcc.as<double>(); g.sB = nn;
+  g.C = h->moM.as<double>(); g.sC = nn;
+  RS_TRY(gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g));
+  g.A = h->moM.as<double>(); g.sA = nn;
+  g.B = h->orb_c; g.sB = 0; g.transB = 1;
+  g.C = sig; g.alpha = 1.0 / ns; g.beta = 1.0;
+  return gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g);
+}
+
 // Coefficients c(tau, i, j) of the trained network for the current G and Sigma_DD.
 constexpr int CV_CHUNK = 65536;
 
@@ -1714,6 +1897,8 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
   if (bf16 && (n < 16 || !tc_available())) return RSSRI_ERR_INVALID_ARG;
   // the chain in double-float (fp64-accurate) instead of IEEE fp64
   const bool chain_df64 = o->precision == RSSRI_PREC_DF64;
+  // the chain on the orbitals (fp64 and double-float, G of the orbitals)
+  const bool mo = !bf16 && !literal && !use_cv && !collect_stats && !g_in && use_mo_chain(h);
   cudaError_t e;
 #define RS_CK(x)                                       \
   do {                                                 \
@@ -1743,9 +1928,9 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
   RS_CK(ensure(h->Ut, (size_t)2 * ns * na * sizeof(double)));
   RS_CK(ensure(h->fac, (size_t)4 * ns * nn * sizeof(double)));  // [set][kind][xi][n][n]
   RS_CK(ensure(h->RLp, (size_t)2 * ns * std::max(h->P, 1) * sizeof(double)));
-  if (!bf16) {
+  if (chain_df64) RS_CK(ensure(h->facHl, (size_t)4 * ns * nn * sizeof(float2)));
+  if (!bf16 && !mo) {
     if (chain_df64) {
-      RS_CK(ensure(h->facHl, (size_t)4 * ns * nn * sizeof(float2)));
       RS_CK(ensure(h->xgHl, (size_t)nbat2 * nn * sizeof(float2)));
       RS_CK(ensure(h->cHl, (size_t)nbat2 * nn * sizeof(float2)));
       RS_CK(ensure(h->bHl, (size_t)nbat2 * nn * sizeof(float2)));
@@ -1786,7 +1971,14 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
     RS_CK(cudaMemsetAsync(h->sdd0.p, 0, (size_t)nt * nn * sizeof(double), s));
     sdd = h->sdd0.as<double>();
   }
-  if (chain_df64) RS_CK(ensure_gg(h));
+  if (chain_df64 && mo && !h->gg_valid) {
+    // the range rule of the pairs' conversion, without the conversion
+    SPAN(RSSRI_PROF_OTHER, 0.0);
+    RS_CK(mo_range_check(G, nt, nn, range_flag(h), s));
+    RS_CK(mo_range_check(Gb, nt, nn, range_flag(h), s));
+  } else if (chain_df64) {
+    RS_CK(ensure_gg(h));
+  }
   RS_CK(cudaEventRecord(h->ev[3], s));
 
   // ---- S4: theta, theta' and U^T = theta W (W symmetric)
@@ -1924,7 +2116,8 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
     RS_CK(chain_tc(h, tc_kind, ns, G, Gb, sdd, h->sig_raw.as<double>(), tc_err,
                    use_cv ? h->cv_c.as<double>() : nullptr));
   }
-  for (int t = 0; t < nt && !bf16; ++t) {
+  if (mo) RS_CK(chain_mo(h, ns, nb, nkind, chain_df64, sdd, h->sig_raw.as<double>()));
+  for (int t = 0; t < nt && !bf16 && !mo; ++t) {
     const double *Gt = G + t * nn, *Gbt = Gb + t * nn;
     double *sig = h->sig_raw.as<double>() + t * nn;
     for (int x0 = 0; x0 < ns; x0 += nb) {

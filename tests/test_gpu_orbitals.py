@@ -1,0 +1,88 @@
+"""The orbital-basis chain against the general one.
+
+rssri_sigma evaluates S8 on the orbitals of the setup's G; rssri_sigma_from_g
+given that same G evaluates it with the general products.  Both sum the same
+terms in fp64 (or in double-float, ~1e-13 per product), in other orders, so
+they agree to rounding: 1e-12 relative per tau point in fp64 (contractions of
+at most a few hundred terms, three in a row, ~1e-15 each), 1e-11 in
+double-float.  Sizes sit at the edges of the kernels' tiles (24, 32, 40, 48,
+64, 100) and at extreme numbers of occupied orbitals.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2005_12338_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def B():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2005_12338_gb300 import binding, build
+    build.build()
+    return binding
+
+
+def both(B, s, opts):
+    """(Sigma, pair energies, E_corr) from the orbitals and from the same G given explicitly."""
+    dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda()
+           for a in (s.eri3, s.metric, s.orb_e, s.orb_c, s.tau, s.tau_w)]
+    gs, gbs = zip(*(O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t) for t in s.tau))
+    h = B.Handle(0)
+    h.setup(*dev, n_occ=s.n_occ, mu=s.mu, beta=s.beta, opts=opts)
+    out = []
+    for g in ((None, None), (torch.from_numpy(np.array(gs)).cuda(),
+                             torch.from_numpy(np.array(gbs)).cuda())):
+        sig = torch.empty((s.n_tau, s.n, s.n), dtype=torch.float64, device="cuda")
+        ep = torch.empty(opts.n_s, dtype=torch.float64, device="cuda")
+        e, _, _ = h.sigma(opts, sig, ep, g=g[0], gb=g[1])
+        torch.cuda.synchronize()
+        out.append((sig.cpu().numpy(), ep.cpu().numpy(), e))
+    h.close()
+    return out
+
+
+def close(a, b, tol):
+    for x, y in zip(a[0], b[0]):
+        assert np.linalg.norm(x - y) <= tol * np.linalg.norm(y)
+    assert np.abs(a[1] - b[1]).max() <= tol * np.abs(b[1]).max()
+    assert abs(a[2] - b[2]) <= tol * abs(b[2])
+
+
+SIZES = [(2, 1, 3, 2), (24, 12, 30, 5), (25, 24, 31, 4), (33, 1, 40, 3), (40, 13, 50, 4),
+         (49, 30, 60, 3), (65, 32, 70, 2), (101, 47, 110, 2)]
+
+
+@pytest.mark.parametrize("n,n_occ,n_aux,n_tau", SIZES)
+@pytest.mark.parametrize("prec", [0, 3], ids=["fp64", "df64"])
+def test_orbital_and_general_form_agree(B, n, n_occ, n_aux, n_tau, prec):
+    s = synth.make_system(n, n_occ, n_aux, n_tau, input_seed=n)
+    gmax = [max(np.abs(m).max() for m in O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t))
+            for t in s.tau]
+    gmin = [min(np.abs(m).max() for m in O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t))
+            for t in s.tau]
+    refused = prec and (min(gmin) < 2.0 ** -40 or max(gmax) > 2.0 ** 40)
+    for kw in (dict(), dict(estimator=B.RSSRI_EST_SRI), dict(pair_batch=3)):
+        o = B.Handle.options(0.02, 1e-2, 7, 5, precision=prec, dd_arith=1 if prec else 0, **kw)
+        if refused:  # a lone occupied orbital far below mu: G(beta - tau) leaves the pairs' range
+            with pytest.raises(B.RssriError) as err:
+                both(B, s, o)
+            assert err.value.code == -9
+            continue
+        a, b = both(B, s, o)
+        close(a, b, 1e-11 if prec else 1e-12)
+
+
+def test_orbitals_that_are_not_orthonormal_keep_the_general_form(B):
+    """G = -C_v g C_v^T is formed from whatever C is given; an estimate that
+    used C^T C = I would be off by the deviation, 1e-6 here."""
+    s = synth.make_system(40, 13, 50, 4, input_seed=3)
+    rng = np.random.default_rng(4)
+    s.orb_c = s.orb_c + 1e-6 * rng.standard_normal(s.orb_c.shape)
+    o = B.Handle.options(0.02, 1e-2, 7, 5)
+    a, b = both(B, s, o)
+    close(a, b, 1e-12)
