@@ -131,11 +131,15 @@ struct rssri_handle {
   DevBuf elHl;  // (ij|A)^L rows as pairs (double-float [K]^L)
   // double-float chain: factor pairs, X G and C pairs, (2tI - B) pairs
   DevBuf facHl, xgHl, cHl, bHl;
+  bool d_ready = false;  // D (v^L on the kept pairs) formed for this setup
   bool d_df64_ready = false;
   bool kp_hl_ready = false;  // K_P as pairs (KPhl) made for this setup
   // orbital-basis chain (mo.cuh): diagonals of G per tau, C as pairs, the transformed
   // factors, M of a chunk of tau points, its traces, Sigma in the orbital basis
   DevBuf moTab, moChl, moZ, moM, moTr, moAcc, moWork;
+  // orbital-basis block: K^Q_ia and K^Q_bc, V and U of a chunk of occupied orbitals, the
+  // weights of a chunk of tau points, row norms of K_P
+  DevBuf moB1, moB2, moV, moU, moW, moRow;
   bool mo_tab_ready = false;  // moTab, moChl made for this setup
   bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
   // bf16 chain buffers
@@ -426,6 +430,12 @@ int metric_inv_sqrt(rssri_handle *h, int *rc, bool df64) {
 // (orbitals from QR or a symmetric eigensolver are at 1e-15 to 1e-14).
 constexpr double MO_ORTH_TOL = 5e-14;
 
+// Setup pieces defined below.
+bool use_mo_block(const rssri_handle *h, int dd_arith);
+cudaError_t ensure_d(rssri_handle *h);
+cudaError_t ensure_d_df64(rssri_handle *h);
+cudaError_t ensure_kp_df64(rssri_handle *h);
+
 // S6 and S7 for every tau (defined below).
 int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double *gb_in);
 
@@ -499,7 +509,8 @@ void rssri_destroy(rssri_handle *h) {
                     &h->Ahl, &h->KPhl, &h->PGhl, &h->APhl, &h->Gamhl, &h->GGhl, &h->litMP, &h->litT, &h->litMhl, &h->eri_hl, &h->ut_hl, &h->nsA2, &h->nsB2, &h->elHl, &h->facHl, &h->xgHl, &h->cHl, &h->bHl, &h->cv_params, &h->cv_m, &h->cv_v, &h->cv_grad, &h->cv_ptmp,
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
                     &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
-                    &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork};
+                    &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork,
+                    &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow};
   for (DevBuf *b : bufs) release(*b);
   release(h->oz_pidx);
   release(h->oz_tmp);
@@ -532,6 +543,7 @@ int rssri_setup(rssri_handle *h, const rssri_problem *p, const rssri_options *o)
   cudaStream_t s = h->stream;
   h->ready = false;
   h->have_sigma = false;
+  h->d_ready = false;
   h->d_df64_ready = false;
   h->kp_hl_ready = false;
   h->cv_c_ready = false;
@@ -687,50 +699,28 @@ int rssri_setup(rssri_handle *h, const rssri_problem *p, const rssri_options *o)
   RS_CK(ensure(h->pcol, (size_t)std::max(P, 1) * sizeof(int)));
   RS_CK(ensure(h->rowptr, (size_t)(n + 1) * sizeof(int)));
   RS_CK(ensure(h->KP, (size_t)std::max(P, 1) * na * sizeof(double)));
-  RS_CK(ensure(h->D, (size_t)std::max(P, 1) * std::max(P, 1) * sizeof(double)));
+  h->setup_arith = o->dd_arith;
   if (P > 0) {
     { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(gather_int(h->spairs.as<int>(), h->lidx.as<int>(), P, h->pij.as<int>(), s)); }
     { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(gather_rows(h->KLs.as<double>(), h->lidx.as<int>(), P, na, h->KP.as<double>(), s)); }
-    // D[a][b] = sum_Q K_P[a][Q] K_P[b][Q] = v^L for the pair of pairs (Eq. 8 on [K]^L),
-    // in the arithmetic the deterministic block is asked to use
-    if (o->dd_arith == RSSRI_DD_OZ) {
-      RS_CK(oz_product(h, RSSRI_PROF_SETUP_GEMM,
-                       oz_rows(h->KP.as<double>(), na, na, (long long)P * na), 1, P, nullptr, P,
-                       na, h->D.as<double>(), P, 0, h->flags.as<int>() + 5));
-      // K_P as pairs for the block's one double-float product (K^Q G)
-      RS_CK(ensure(h->KPhl, (size_t)P * na * sizeof(float2)));
-      { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(to_df64(h->KP.as<double>(), (long long)P * na, h->KPhl.as<float2>(), s, range_flag(h))); }
-      h->kp_hl_ready = true;
-    } else if (o->dd_arith != RSSRI_DD_FP64) {
-      RS_CK(ensure(h->Dhl, (size_t)P * P * sizeof(float2)));
-      RS_CK(ensure(h->KPhl, (size_t)P * na * sizeof(float2)));
-      { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(to_df64(h->KP.as<double>(), (long long)P * na, h->KPhl.as<float2>(), s, range_flag(h))); }
-      {
-        SPAN(RSSRI_PROF_SETUP_GEMM, 2.0 * P * (double)P * na * 1e-9);
-        DfGemm g;
-        g.M = P; g.N = P; g.K = na;
-        g.A = h->KPhl.as<float2>(); g.lda = na;
-        g.B = h->KPhl.as<float2>(); g.ldb = na; g.transB = 1;
-        g.C64 = h->D.as<double>(); g.ldc = P;
-        RS_CK(df_gemm_w(h, g));
-      }
-      { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(to_df64(h->D.as<double>(), (long long)P * P, h->Dhl.as<float2>(), s, range_flag(h))); }
-      h->d_df64_ready = true;
-      h->kp_hl_ready = true;
-    } else {
-      GemmArgs g;
-      g.M = P; g.N = P; g.K = na;
-      g.A = h->KP.as<double>(); g.lda = na;
-      g.B = h->KP.as<double>(); g.ldb = na; g.transB = 1;
-      g.C = h->D.as<double>(); g.ldc = P;
-      RS_CK(gemm_p(h, RSSRI_PROF_SETUP_GEMM, g));
+    // K_P as pairs (the double-float products of the block and of R^L)
+    if (o->dd_arith != RSSRI_DD_FP64) RS_CK(ensure_kp_df64(h));
+    // D: only where the block contracts it; the double-float setup refuses the
+    // same magnitudes of v^L either way
+    if (!use_mo_block(h, o->dd_arith)) {
+      RS_CK(ensure_d(h));
+      if (o->dd_arith == RSSRI_DD_DF64) RS_CK(ensure_d_df64(h));
+    } else if (o->dd_arith == RSSRI_DD_DF64) {
+      SPAN(RSSRI_PROF_OTHER, 0.0);
+      RS_CK(ensure(h->moRow, (size_t)P * sizeof(double)));
+      RS_CK(mo_row_norm2(h->KP.as<double>(), P, na, h->moRow.as<double>(), s));
+      RS_CK(mo_range_check(h->moRow.as<double>(), 1, P, range_flag(h), s));
     }
   }
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(pair_csr(h->pij.as<int>(), P, n, h->rowptr.as<int>(), h->prow.as<int>(),
                  h->pcol.as<int>(), s)); }
   // S6, S7: G(tau), G(beta - tau) and the deterministic block for every tau,
   // cached for every sampling call on this setup (they do not depend on the draws)
-  h->setup_arith = o->dd_arith;
   rc = build_block(h, o->dd_arith, nullptr, nullptr);
   if (rc) { if (rc == RSSRI_ERR_CUDA) h->broken = true; return rc; }
   RS_CK(cudaEventRecord(h->ev[1], s));
@@ -1008,6 +998,7 @@ int oz_setup(rssri_handle *h) {
     e = (x);                         \
     if (e != cudaSuccess) { note_error_site(__FILE__, __LINE__); return map_err(e); } \
   } while (0)
+  RS_CK(ensure_d(h));
   RS_CK(ensure(h->oz_pidx, (size_t)n * n * sizeof(int)));
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(oz_pair_index(h->pij.as<int>(), P, n, h->oz_pidx.as<int>(), s)); }
   // band half-width of the kept pairs
@@ -1182,21 +1173,63 @@ size_t dd_work_need(rssri_handle *h) {
   return w;
 }
 
-// The pair copies of D and K_P used by the double-float block (made once per setup).
-cudaError_t ensure_d_df64(rssri_handle *h) {
-  if (h->d_df64_ready || h->P == 0) return cudaSuccess;
+// D[a][b] = sum_Q K_P[a][Q] K_P[b][Q] = v^L for the pair of pairs (Eq. 8 on
+// [K]^L), in the arithmetic the setup asked for; formed when a contraction over
+// the kept pairs first needs it.  (A bounded wait of the sliced product that
+// expires sets flag 5, which build_block checks.)
+cudaError_t ensure_d(rssri_handle *h) {
+  if (h->d_ready || h->P == 0) return cudaSuccess;
   const int P = h->P, na = h->n_aux;
-  RS_TRY(ensure(h->Dhl, (size_t)P * P * sizeof(float2)));
-  RS_TRY(ensure(h->KPhl, (size_t)P * na * sizeof(float2)));
-  SPAN(RSSRI_PROF_OTHER, 0.0);
-  RS_TRY(to_df64(h->D.as<double>(), (long long)P * P, h->Dhl.as<float2>(), h->stream, range_flag(h)));
-  RS_TRY(to_df64(h->KP.as<double>(), (long long)P * na, h->KPhl.as<float2>(), h->stream, range_flag(h)));
-  h->d_df64_ready = true;
-  h->kp_hl_ready = true;
+  RS_TRY(ensure(h->D, (size_t)P * P * sizeof(double)));
+  if (h->setup_arith == RSSRI_DD_OZ) {
+    RS_TRY(oz_product(h, RSSRI_PROF_SETUP_GEMM, oz_rows(h->KP.as<double>(), na, na, (long long)P * na),
+                      1, P, nullptr, P, na, h->D.as<double>(), P, 0, h->flags.as<int>() + 5));
+  } else if (h->setup_arith != RSSRI_DD_FP64) {
+    RS_TRY(ensure_kp_df64(h));
+    SPAN(RSSRI_PROF_SETUP_GEMM, 2.0 * P * (double)P * na * 1e-9);
+    DfGemm g;
+    g.M = P; g.N = P; g.K = na;
+    g.A = h->KPhl.as<float2>(); g.lda = na;
+    g.B = h->KPhl.as<float2>(); g.ldb = na; g.transB = 1;
+    g.C64 = h->D.as<double>(); g.ldc = P;
+    RS_TRY(df_gemm_w(h, g));
+  } else {
+    GemmArgs g;
+    g.M = P; g.N = P; g.K = na;
+    g.A = h->KP.as<double>(); g.lda = na;
+    g.B = h->KP.as<double>(); g.ldb = na; g.transB = 1;
+    g.C = h->D.as<double>(); g.ldc = P;
+    RS_TRY(gemm_p(h, RSSRI_PROF_SETUP_GEMM, g));
+  }
+  h->d_ready = true;
   return cudaSuccess;
 }
 
-// K_P as pairs only (the sliced block's K^Q G product).
+// D and K_P as pairs (the double-float contractions over the kept pairs; once per setup).
+cudaError_t ensure_d_df64(rssri_handle *h) {
+  if (h->d_df64_ready || h->P == 0) return cudaSuccess;
+  const int P = h->P;
+  RS_TRY(ensure_d(h));
+  RS_TRY(ensure_kp_df64(h));
+  RS_TRY(ensure(h->Dhl, (size_t)P * P * sizeof(float2)));
+  SPAN(RSSRI_PROF_OTHER, 0.0);
+  RS_TRY(to_df64(h->D.as<double>(), (long long)P * P, h->Dhl.as<float2>(), h->stream, range_flag(h)));
+  h->d_df64_ready = true;
+  return cudaSuccess;
+}
+
+// Whether a bounded wait of the block's tensor-core products gave up since the
+// flag was cleared; if so, what they formed for the setup is formed anew.
+int oz_waits(rssri_handle *h) {
+  int fl = 0;
+  const cudaError_t e = fetch(&fl, h->flags.as<int>() + 5, h->stream);
+  if (e != cudaSuccess) { note_error_site(__FILE__, __LINE__); return map_err(e); }
+  if (!fl) return RSSRI_OK;
+  h->d_ready = h->d_df64_ready = h->oz_ready = false;
+  return RSSRI_ERR_TIMEOUT;
+}
+
+// K_P as pairs.
 cudaError_t ensure_kp_df64(rssri_handle *h) {
   if (h->kp_hl_ready || h->P == 0) return cudaSuccess;
   RS_TRY(ensure(h->KPhl, (size_t)h->P * h->n_aux * sizeof(float2)));
@@ -1224,6 +1257,149 @@ cudaError_t ensure_gg(rssri_handle *h) {
   return cudaSuccess;
 }
 
+// ----------------------------------------- the block on the orbitals (S7) --
+// Layout of moTab: gv [nt][nv] and go [nt][no] in fp64, the same as scaled
+// pairs, and the two exponents per tau (see mo_tables).
+struct MoTab {
+  double *gv, *go;
+  float2 *gvhl, *gohl;
+  int *texp, *eexp;
+};
+MoTab mo_tab(rssri_handle *h) {
+  const size_t nt = h->n_tau, no = h->n_occ, nv = h->n - h->n_occ;
+  MoTab t;
+  t.gv = h->moTab.as<double>();
+  t.go = t.gv + nt * nv;
+  t.gvhl = reinterpret_cast<float2 *>(t.go + nt * no);
+  t.gohl = t.gvhl + nt * nv;
+  t.texp = reinterpret_cast<int *>(t.gohl + nt * no);
+  t.eexp = t.texp + nt;
+  return t;
+}
+cudaError_t ensure_mo_tab(rssri_handle *h) {
+  if (h->mo_tab_ready) return cudaSuccess;
+  const size_t nt = h->n_tau, n = h->n;
+  RS_TRY(ensure(h->moTab, nt * n * 16 + nt * 2 * sizeof(int)));
+  RS_TRY(ensure(h->moChl, n * n * sizeof(float2)));
+  const MoTab t = mo_tab(h);
+  SPAN(RSSRI_PROF_GREEN, 0.0);
+  RS_TRY(mo_tables(h->orb_e, h->n, h->n_occ, h->mu, h->tau, h->n_tau, 1, t.gv, t.go, t.gvhl,
+                   t.gohl, t.texp, t.eexp, h->stream));
+  RS_TRY(to_df64(h->orb_c, (long long)n * n, h->moChl.as<float2>(), h->stream));
+  h->mo_tab_ready = true;
+  return cudaSuccess;
+}
+
+
+// Whether S7 for the orbitals' G is the Gram matrix of U (mo.cuh) or the
+// contraction over the P kept pairs: by flops, n^2 n_v^2 n_o (and a fifth for
+// the tiles on the diagonal) per tau point plus U once, against D once plus
+// 2 N_aux P^2 and the dense products per tau point.  Both run at the same
+// rate of the fp64 (or fp32) pipe.  At N = 100, N_aux = 300, eps = 1e-3 (P =
+// 3,560) a tau point is 1.5 against 9.5 GFLOP; the lines cross near N = 270.
+bool use_mo_block(const rssri_handle *h, int dd_arith) {
+  if (h->P == 0 || dd_arith == RSSRI_DD_OZ) return false;
+  const double n = h->n, no = h->n_occ, nv = n - no, na = h->n_aux, P = h->P, nt = h->n_tau;
+  const double pairs = 2.0 * P * P * na +
+                       nt * (2.0 * na * P * P + 2.0 * P * n * na + 4.0 * na * n * n * n +
+                             4.0 * P * na * na);
+  const double orbitals = 2.0 * P * nv * na + 2.0 * no * n * nv * na + 2.0 * n * nv * nv * no * na +
+                          nt * 1.2 * n * n * nv * nv * no;
+  return orbitals < pairs;
+}
+
+// S7 for all tau points on the orbitals: out[t] = -U diag(w_t) U^T, in chunks of
+// occupied orbitals c (U and V of a chunk, 256 MB each at most) and of tau
+// points (their weights).
+cudaError_t block_mo(rssri_handle *h, bool df, double *out) {
+  cudaStream_t s = h->stream;
+  const int n = h->n, no = h->n_occ, nv = n - no, nt = h->n_tau, na = h->n_aux;
+  const long long nva = (long long)nv * na, row = (long long)n * nv;
+  RS_TRY(ensure_mo_tab(h));
+  const MoTab tab = mo_tab(h);
+  const size_t budget = (size_t)256 << 20;
+  const long long per_c = row * nv;
+  const int cc = (int)std::max<long long>(1, std::min<long long>(no, (long long)(budget / 8) / per_c));
+  const long long kc = (long long)cc * nv * nv;
+  const int tcw = (int)std::max<long long>(1, std::min<long long>(nt, (long long)(budget / 8) / kc));
+  RS_TRY(ensure(h->moB1, (size_t)n * nva * 8));
+  RS_TRY(ensure(h->moB2, (size_t)no * nva * 8));
+  RS_TRY(ensure(h->moV, (size_t)cc * per_c * 8));
+  RS_TRY(ensure(h->moU, (size_t)cc * per_c * 8));
+  RS_TRY(ensure(h->moW, (size_t)tcw * kc * 8));
+  MoGram q;
+  q.df = df; q.n = n;
+  size_t work = 0;
+  for (long long c : {cc, no % cc ? no % cc : cc})
+    for (int t : {tcw, nt % tcw ? nt % tcw : tcw}) {
+      q.K = c * nv * nv;
+      q.nt = t;
+      work = std::max(work, mo_gram_work(q));
+    }
+  RS_TRY(ensure(h->moWork, work * sizeof(double)));
+  // K^Q_ia = sum_k K^Q_ik C_ka over the kept pairs, K^Q_bc = sum_i C_ic K^Q_ib
+  if (df) {
+    RS_TRY(ensure_kp_df64(h));
+    SPAN(RSSRI_PROF_DD_GEMM, (2.0 * h->P + 2.0 * no * n) * nva * 1e-9);
+    RS_TRY(df_gemm_segmented(n, nv, na, h->rowptr.as<int>(), h->pcol.as<int>(),
+                             h->moChl.as<float2>() + no, n, h->KPhl.as<float2>(), na,
+                             h->moB1.as<float2>(), na, nva, s));
+    DfGemm g;
+    g.M = no; g.N = (int)nva; g.K = n;
+    g.A = h->moChl.as<float2>(); g.lda = n; g.transA = 1;
+    g.B = h->moB1.as<float2>(); g.ldb = nva;
+    g.C2 = h->moB2.as<float2>(); g.ldc = nva;
+    RS_TRY(df_gemm_w(h, g));
+  } else {
+    { SPAN(RSSRI_PROF_DD_GEMM, 2.0 * h->P * nva * 1e-9);
+      RS_TRY(dgemm_segmented(n, nv, na, h->rowptr.as<int>(), h->pcol.as<int>(), h->orb_c + no, n,
+                             h->KP.as<double>(), na, h->moB1.as<double>(), na, nva, s)); }
+    GemmArgs g;
+    g.M = no; g.N = (int)nva; g.K = n;
+    g.A = h->orb_c; g.lda = n; g.transA = 1;
+    g.B = h->moB1.as<double>(); g.ldb = nva;
+    g.C = h->moB2.as<double>(); g.ldc = nva;
+    RS_TRY(gemm_p(h, RSSRI_PROF_DD_GEMM, g));
+  }
+  for (int c0 = 0; c0 < no; c0 += cc) {
+    const int c = std::min(cc, no - c0);
+    // V[c][b][i][a] = sum_Q K^Q_bc K^Q_ia
+    if (df) {
+      SPAN(RSSRI_PROF_DD_GEMM, 2.0 * c * (double)per_c * na * 1e-9);
+      DfGemm g;
+      g.M = nv; g.N = (int)row; g.K = na; g.batch = c;
+      g.A = h->moB2.as<float2>() + c0 * nva; g.lda = na; g.sA = nva;
+      g.B = h->moB1.as<float2>(); g.ldb = na; g.transB = 1;
+      g.C64 = h->moV.as<double>(); g.ldc = row; g.sC = per_c;
+      RS_TRY(df_gemm_w(h, g));
+    } else {
+      GemmArgs g;
+      g.M = nv; g.N = (int)row; g.K = na; g.batch = c;
+      g.A = h->moB2.as<double>() + c0 * nva; g.lda = na; g.sA = nva;
+      g.B = h->moB1.as<double>(); g.ldb = na; g.transB = 1;
+      g.C = h->moV.as<double>(); g.ldc = row; g.sC = per_c;
+      RS_TRY(gemm_p(h, RSSRI_PROF_DD_GEMM, g));
+    }
+    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_TRY(mo_pack(df, h->moV.as<double>(), n, nv, c, h->moU.p, s)); }
+    for (int t0 = 0; t0 < nt; t0 += tcw) {
+      const int t = std::min(tcw, nt - t0);
+      q.K = (long long)c * nv * nv;
+      q.nt = t;
+      { SPAN(RSSRI_PROF_OTHER, 0.0);
+        RS_TRY(mo_weights(df, tab.gv + (long long)t0 * nv, tab.go + (long long)t0 * no, nv, no, c0, c,
+                          t, tab.texp + t0, h->moW.p, s)); }
+      q.U = h->moU.p; q.ldu = q.K;
+      q.w = h->moW.p;
+      q.wexp = df ? tab.texp + t0 : nullptr;
+      q.out = out + (long long)t0 * n * n;
+      q.accumulate = c0 > 0;
+      SPAN(RSSRI_PROF_DD_GEMM, mo_gram_flops(q) * 1e-9);
+      RS_TRY(mo_gram(q, h->moWork.as<double>(), s));
+    }
+  }
+  return cudaSuccess;
+}
+
 // S6 and S7 for every tau point: G(tau) and G(beta - tau) from the orbitals
 // (Eq. 17) or copied from the caller (g_in, gb_in: [n_tau][n][n] of the
 // problem's pointer kind), then Sigma_DD(tau) (Eq. 20 on v^L = sum_Q
@@ -1244,9 +1420,11 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   RS_CK(ensure(h->G, (size_t)nt * nn * sizeof(double)));
   RS_CK(ensure(h->Gb, (size_t)nt * nn * sizeof(double)));
   RS_CK(ensure(h->sdd, (size_t)nt * nn * sizeof(double)));
-  const bool dd_df64 = P > 0 && dd_arith == RSSRI_DD_DF64;
-  const bool dd_oz = P > 0 && dd_arith == RSSRI_DD_OZ;
-  if (P > 0) {
+  const bool mo = P > 0 && !g_in && use_mo_block(h, dd_arith);
+  const bool dd_df64 = P > 0 && !mo && dd_arith == RSSRI_DD_DF64;
+  const bool dd_oz = P > 0 && !mo && dd_arith == RSSRI_DD_OZ;
+  if (P > 0 && !mo) RS_CK(ensure_d(h));
+  if (P > 0 && !mo) {
     if (dd_oz) {
       // the exchange operand first (its fp64 gather is freed before the
       // per-tau buffers are made), then the per-tau buffers; T shares At's
@@ -1300,9 +1478,16 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   } else {
     RS_CK(build_green(h));
   }
-  // S7 per tau
+  // S7: all tau points on the orbitals, or tau by tau
   if (dd_df64) RS_CK(ensure_gg(h));
-  for (int t = 0; t < nt; ++t) {
+  if (mo && dd_arith != RSSRI_DD_FP64) {
+    // the range rule of the pairs' conversion, without the conversion
+    SPAN(RSSRI_PROF_OTHER, 0.0);
+    RS_CK(mo_range_check(G, nt, nn, range_flag(h), s));
+    RS_CK(mo_range_check(Gb, nt, nn, range_flag(h), s));
+  }
+  if (mo) RS_CK(block_mo(h, dd_arith != RSSRI_DD_FP64, h->sdd.as<double>()));
+  for (int t = 0; t < nt && !mo; ++t) {
     double *out = h->sdd.as<double>() + t * nn;
     if (dd_oz) {
       RS_CK(sigma_dd_tau_oz(h, G + t * nn, Gb + t * nn, out));
@@ -1312,11 +1497,9 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
     else
       RS_CK(sigma_dd_tau(h, G + t * nn, Gb + t * nn, out));
   }
-  if (dd_oz) {
-    // a bounded wait of the tensor-core kernels that gave up
-    int fl = 0;
-    RS_CK(fetch(&fl, h->flags.as<int>() + 5, s));
-    if (fl) return RSSRI_ERR_TIMEOUT;
+  if (dd_arith == RSSRI_DD_OZ || h->setup_arith == RSSRI_DD_OZ) {
+    const int rc = oz_waits(h);
+    if (rc) return rc;
 #ifdef RSSRI_CHECKS
     int chk[4];
     RS_CK(oz_check_fetch(chk));
@@ -1571,38 +1754,6 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
 }
 
 // ------------------------------------------- the chain on the orbitals (S8) --
-// Layout of moTab: gv [nt][nv] and go [nt][no] in fp64, the same as scaled
-// pairs, and the two exponents per tau (see mo_tables).
-struct MoTab {
-  double *gv, *go;
-  float2 *gvhl, *gohl;
-  int *texp, *eexp;
-};
-MoTab mo_tab(rssri_handle *h) {
-  const size_t nt = h->n_tau, no = h->n_occ, nv = h->n - h->n_occ;
-  MoTab t;
-  t.gv = h->moTab.as<double>();
-  t.go = t.gv + nt * nv;
-  t.gvhl = reinterpret_cast<float2 *>(t.go + nt * no);
-  t.gohl = t.gvhl + nt * nv;
-  t.texp = reinterpret_cast<int *>(t.gohl + nt * no);
-  t.eexp = t.texp + nt;
-  return t;
-}
-cudaError_t ensure_mo_tab(rssri_handle *h) {
-  if (h->mo_tab_ready) return cudaSuccess;
-  const size_t nt = h->n_tau, n = h->n;
-  RS_TRY(ensure(h->moTab, nt * n * 16 + nt * 2 * sizeof(int)));
-  RS_TRY(ensure(h->moChl, n * n * sizeof(float2)));
-  const MoTab t = mo_tab(h);
-  SPAN(RSSRI_PROF_GREEN, 0.0);
-  RS_TRY(mo_tables(h->orb_e, h->n, h->n_occ, h->mu, h->tau, h->n_tau, 1, t.gv, t.go, t.gvhl,
-                   t.gohl, t.texp, t.eexp, h->stream));
-  RS_TRY(to_df64(h->orb_c, (long long)n * n, h->moChl.as<float2>(), h->stream));
-  h->mo_tab_ready = true;
-  return cudaSuccess;
-}
-
 // Whether S8 runs on the orbitals: G is the orbitals' (not a caller's), and
 // its flops per pair and kind, 8 n^2 n_v for the transforms and 2 n^3 per tau
 // point, are fewer than the general form's 8 n^3 per tau point.
@@ -1948,9 +2099,16 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
   if (literal && P > 0) {
     RS_CK(ensure(h->litMP, (size_t)P * nbat2 * sizeof(double)));
     RS_CK(ensure(h->litT, (size_t)na * nbat2 * sizeof(double)));
+    const bool had_d = h->d_ready;
     if (o->dd_arith != RSSRI_DD_FP64) {
       RS_CK(ensure(h->litMhl, (size_t)nbat2 * nn * sizeof(float2)));
       RS_CK(ensure_d_df64(h));
+    } else {
+      RS_CK(ensure_d(h));
+    }
+    if (!had_d && h->setup_arith == RSSRI_DD_OZ) {
+      rc = oz_waits(h);
+      if (rc) return rc;
     }
   }
 

@@ -9,6 +9,16 @@
 //   F = 2 t C - C Gb C = M_(:,o) go M_(o,:) - 2 t M
 // in the orbital basis: 2 n^3 flops per factor pair and tau point against
 // 8 n^3 for the four products X G, (X G) Y, C Gb, (2 t I - B) C.
+//
+// Deterministic block (S7).  Eq. 20 on v^L = sum_Q K^Q K^Q is
+//   Sigma_DD,ij = -sum_abc gv_a gv_b go_c V_i,abc (2 V_j,abc - V_j,bac),
+//   V_i,abc = sum_Q K^Q_ia K^Q_bc  (a, b virtual, c occupied, i an AO),
+// and with U = the symmetric (a <= b, weight sqrt(2 - delta_ab)) and
+// antisymmetric (sqrt(6)) parts of V in (a, b) it is minus a Gram matrix,
+//   Sigma_DD,ij = -sum_k w_k(tau) U_ik U_jk,  w_k = gv_a gv_b go_c > 0,
+// whose U does not depend on tau.  n^2 n_v^2 n_o flops per tau point
+// (half of the symmetric product), against 2 N_aux P^2 + ~4 N_aux n^3 for the
+// contraction over the P kept pairs.
 #pragma once
 
 #include "common.cuh"
@@ -29,6 +39,25 @@ struct MoNt {
   void *out = nullptr;  // [nt][nb][M][N], of the operands' type
 };
 cudaError_t mo_nt(const MoNt &g, cudaStream_t s);
+
+// Gram matrices out[t] (+)= -2^e_t U diag(w_t) U^T for t < nt, U [n x K] row
+// stride ldu, w [nt][K], e_t = wexp[t] (null: 0); symmetric, fp64 results.  K is
+// split over CTAs; the partial sums go to `work` (mo_gram_work() doubles) and
+// are added in a fixed order.
+struct MoGram {
+  int df = 0;
+  int n = 0, nt = 1;
+  long long K = 0;
+  const void *U = nullptr, *w = nullptr;
+  long long ldu = 0;
+  const int *wexp = nullptr;
+  double *out = nullptr;  // [nt][n][n]
+  int accumulate = 0;
+};
+size_t mo_gram_work(const MoGram &g);
+cudaError_t mo_gram(const MoGram &g, double *work, cudaStream_t s);
+// Flops of the tiles mo_gram computes.
+double mo_gram_flops(const MoGram &g);
 
 // Sum over sample pairs x < cnt and kinds k < nkind (k = 0: sign +, else -) of
 // sgn (M_(:,o) go M_(o,:) - 2 t M) per tau: M [nt][nkind][cnt][n][n], go
@@ -66,6 +95,17 @@ cudaError_t mo_energy(const double *tr, const double *s2, int nt, int nkind, int
 cudaError_t mo_tables(const double *orb_e, int n, int no, double mu, const double *tau, int nt,
                       int df, double *gv, double *go, float2 *gvhl, float2 *gohl, int *texp,
                       int *eexp, cudaStream_t s);
+// w[t][((c - c0) nv + a) nv + b] = go[t][c] gv[t][a] gv[t][b], c0 <= c < c0 + nc, for nt tau
+// points; df: pairs of the same times 2^-texp[t].
+cudaError_t mo_weights(int df, const double *gv, const double *go, int nv, int no, int c0, int nc,
+                       int nt, const int *texp, void *w, cudaStream_t s);
+// U[i][((c nv) + a) nv + b] from V[c][b][i][a] (fp64, nc x nv x n x nv): slot a < b holds
+// (V_ab + V_ba) / sqrt 2, a = b holds V_aa, a > b holds (V_ba - V_ab) sqrt(3/2); df: pairs.
+cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, void *U, cudaStream_t s);
+
+// out[a] = sum_q x[a][q]^2 (the diagonal of v^L on the kept pairs, where its largest magnitude is).
+cudaError_t mo_row_norm2(const double *x, int rows, int cols, double *out, cudaStream_t s);
+
 // flag |= 1 when some |CtC - I| element exceeds tol.
 cudaError_t mo_orth_check(const double *CtC, int n, double tol, int *flag, cudaStream_t s);
 // The range rule of to_df64 (dd_df64.cuh) on each of `segments` matrices of len values, without

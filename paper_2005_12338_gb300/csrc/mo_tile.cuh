@@ -1,6 +1,6 @@
 // Register-tiled products of the orbital-basis path (mo.cuh): the two kinds of
 // arithmetic, the tile shapes and their choice, and the kernel
-// out = A diag(ks) B^T.
+// out = A diag(ks) B^T that the chain and the deterministic block share.
 //
 // The products run on the fp64 pipe (IEEE form) or on
 // the fp32 pipes (double-float form: each value a pair of floats, about a

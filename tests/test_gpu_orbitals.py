@@ -53,6 +53,13 @@ def close(a, b, tol):
     assert abs(a[2] - b[2]) <= tol * abs(b[2])
 
 
+def out_of_range(s):
+    """Whether some G(tau) or G(beta - tau) leaves the range the double-float forms take (a lone
+    occupied orbital far below mu does)."""
+    m = [np.abs(x).max() for t in s.tau for x in O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t)]
+    return min(m) < 2.0 ** -40 or max(m) > 2.0 ** 40
+
+
 SIZES = [(2, 1, 3, 2), (24, 12, 30, 5), (25, 24, 31, 4), (33, 1, 40, 3), (40, 13, 50, 4),
          (49, 30, 60, 3), (65, 32, 70, 2), (101, 47, 110, 2)]
 
@@ -61,20 +68,37 @@ SIZES = [(2, 1, 3, 2), (24, 12, 30, 5), (25, 24, 31, 4), (33, 1, 40, 3), (40, 13
 @pytest.mark.parametrize("prec", [0, 3], ids=["fp64", "df64"])
 def test_orbital_and_general_form_agree(B, n, n_occ, n_aux, n_tau, prec):
     s = synth.make_system(n, n_occ, n_aux, n_tau, input_seed=n)
-    gmax = [max(np.abs(m).max() for m in O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t))
-            for t in s.tau]
-    gmin = [min(np.abs(m).max() for m in O.green(s.orb_e, s.orb_c, s.n_occ, s.mu, t))
-            for t in s.tau]
-    refused = prec and (min(gmin) < 2.0 ** -40 or max(gmax) > 2.0 ** 40)
+    refused = prec and out_of_range(s)
     for kw in (dict(), dict(estimator=B.RSSRI_EST_SRI), dict(pair_batch=3)):
         o = B.Handle.options(0.02, 1e-2, 7, 5, precision=prec, dd_arith=1 if prec else 0, **kw)
-        if refused:  # a lone occupied orbital far below mu: G(beta - tau) leaves the pairs' range
+        if refused:
             with pytest.raises(B.RssriError) as err:
                 both(B, s, o)
             assert err.value.code == -9
             continue
         a, b = both(B, s, o)
         close(a, b, 1e-11 if prec else 1e-12)
+
+
+# The deterministic block as a Gram matrix over (virtual, virtual, occupied)
+# triples against the contraction over the kept pairs: nothing cut (eps = eps' =
+# 0, P = n^2) and n_tau = 8, so that the orbital form is the cheaper one; numbers of
+# virtual orbitals around the packing tiles' 32, one occupied orbital, one virtual.
+BLOCKS = [(20, 4, 24), (21, 20, 24), (40, 7, 42), (70, 38, 40), (66, 1, 40), (45, 13, 60)]
+
+
+@pytest.mark.parametrize("n,n_occ,n_aux", BLOCKS)
+@pytest.mark.parametrize("dd", [0, 1], ids=["fp64", "df64"])
+def test_gram_block_equals_the_pair_contraction(B, n, n_occ, n_aux, dd):
+    s = synth.make_system(n, n_occ, n_aux, 8, input_seed=n + 1)
+    o = B.Handle.options(0.0, 0.0, 4, 6, dd_arith=dd)
+    if dd and out_of_range(s):
+        with pytest.raises(B.RssriError) as err:
+            both(B, s, o)
+        assert err.value.code == -9
+        return
+    a, b = both(B, s, o)
+    close(a, b, 1e-11 if dd else 1e-12)
 
 
 def test_orbitals_that_are_not_orthonormal_keep_the_general_form(B):
