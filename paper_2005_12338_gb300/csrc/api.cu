@@ -134,12 +134,18 @@ struct rssri_handle {
   bool d_ready = false;  // D (v^L on the kept pairs) formed for this setup
   bool d_df64_ready = false;
   bool kp_hl_ready = false;  // K_P as pairs (KPhl) made for this setup
+  struct OzBuf {
+    DevBuf d, e;
+    OzDigits v;
+  };
   // orbital-basis chain (mo.cuh): diagonals of G per tau, C as pairs, the transformed
   // factors, M of a chunk of tau points, its traces, Sigma in the orbital basis
   DevBuf moTab, moChl, moZ, moM, moTr, moAcc, moWork;
   // orbital-basis block: K^Q_ia and K^Q_bc, V and U of a chunk of occupied orbitals, the
   // weights of a chunk of tau points, row norms of K_P
   DevBuf moB1, moB2, moV, moU, moW, moRow;
+  OzBuf ozY;    // its digits on the tensor cores (RSSRI_DD_OZ)
+  DevBuf ozYm, ozY6;  // row maxima per tau point, the slicer's level-6 sums
   bool mo_tab_ready = false;  // moTab, moChl made for this setup
   bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
   // bf16 chain buffers
@@ -165,10 +171,6 @@ struct rssri_handle {
   DevBuf sdd0;            // zeros: the block of the plain stochastic-RI estimator
   // the sliced (RSSRI_DD_OZ) block: pair index map, the exchange contraction's
   // left operand and the digits of K_P (setup); per-tau digit buffers
-  struct OzBuf {
-    DevBuf d, e;
-    OzDigits v;
-  };
   bool oz_ready = false;
   OzExch oz_geo;
   DevBuf oz_gs, oz_gexp;  // G(tau) 2^-e(tau) as pairs, and e(tau), for K^Q G
@@ -510,13 +512,13 @@ void rssri_destroy(rssri_handle *h) {
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
                     &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
                     &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork,
-                    &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow};
+                    &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow, &h->ozYm, &h->ozY6};
   for (DevBuf *b : bufs) release(*b);
   release(h->oz_pidx);
   release(h->oz_tmp);
   release(h->oz_gr);
   for (rssri_handle::OzBuf *o : {&h->ozX, &h->ozKP, &h->ozKPt, &h->ozGb, &h->ozBig0, &h->ozBig1,
-                                 &h->ozAtP, &h->ozGam, &h->ozPA, &h->ozPB, &h->ozKPr,
+                                 &h->ozAtP, &h->ozGam, &h->ozPA, &h->ozPB, &h->ozKPr, &h->ozY,
                                  &h->ozGr}) {
     release(o->d);
     release(o->e);
@@ -1258,38 +1260,32 @@ cudaError_t ensure_gg(rssri_handle *h) {
 }
 
 // ----------------------------------------- the block on the orbitals (S7) --
-// Layout of moTab: gv [nt][nv] and go [nt][no] in fp64, the same as scaled
-// pairs, and the two exponents per tau (see mo_tables).
-struct MoTab {
-  double *gv, *go;
-  float2 *gvhl, *gohl;
-  int *texp, *eexp;
-};
+// The arrays of moTab.
 MoTab mo_tab(rssri_handle *h) {
   const size_t nt = h->n_tau, no = h->n_occ, nv = h->n - h->n_occ;
   MoTab t;
   t.gv = h->moTab.as<double>();
   t.go = t.gv + nt * nv;
-  t.gvhl = reinterpret_cast<float2 *>(t.go + nt * no);
+  t.hv = t.go + nt * no;
+  t.ho = t.hv + nt * nv;
+  t.gvhl = reinterpret_cast<float2 *>(t.ho + nt * no);
   t.gohl = t.gvhl + nt * nv;
   t.texp = reinterpret_cast<int *>(t.gohl + nt * no);
   t.eexp = t.texp + nt;
+  t.hexp = t.eexp + nt;
   return t;
 }
 cudaError_t ensure_mo_tab(rssri_handle *h) {
   if (h->mo_tab_ready) return cudaSuccess;
   const size_t nt = h->n_tau, n = h->n;
-  RS_TRY(ensure(h->moTab, nt * n * 16 + nt * 2 * sizeof(int)));
+  RS_TRY(ensure(h->moTab, nt * n * 24 + nt * 3 * sizeof(int)));
   RS_TRY(ensure(h->moChl, n * n * sizeof(float2)));
-  const MoTab t = mo_tab(h);
   SPAN(RSSRI_PROF_GREEN, 0.0);
-  RS_TRY(mo_tables(h->orb_e, h->n, h->n_occ, h->mu, h->tau, h->n_tau, 1, t.gv, t.go, t.gvhl,
-                   t.gohl, t.texp, t.eexp, h->stream));
+  RS_TRY(mo_tables(h->orb_e, h->n, h->n_occ, h->mu, h->tau, h->n_tau, mo_tab(h), h->stream));
   RS_TRY(to_df64(h->orb_c, (long long)n * n, h->moChl.as<float2>(), h->stream));
   h->mo_tab_ready = true;
   return cudaSuccess;
 }
-
 
 // Whether S7 for the orbitals' G is the Gram matrix of U (mo.cuh) or the
 // contraction over the P kept pairs: by flops, n^2 n_v^2 n_o (and a fifth for
@@ -1297,9 +1293,26 @@ cudaError_t ensure_mo_tab(rssri_handle *h) {
 // 2 N_aux P^2 and the dense products per tau point.  Both run at the same
 // rate of the fp64 (or fp32) pipe.  At N = 100, N_aux = 300, eps = 1e-3 (P =
 // 3,560) a tau point is 1.5 against 9.5 GFLOP; the lines cross near N = 270.
+// The sliced block by time: the products of the kept pairs run at ~26e12 of
+// those flops per second (45% of the exchange's tile rows are outside the band,
+// and its digits are written for every tau point); the Gram tiles at ~78e12
+// with 20 bytes of HBM traffic per value and tau point, V at ~60e12.
 bool use_mo_block(const rssri_handle *h, int dd_arith) {
-  if (h->P == 0 || dd_arith == RSSRI_DD_OZ) return false;
+  if (h->P == 0) return false;
   const double n = h->n, no = h->n_occ, nv = n - no, na = h->n_aux, P = h->P, nt = h->n_tau;
+  if (dd_arith == RSSRI_DD_OZ) {
+    if (h->n > 1024) return false;
+    const double K = nv * nv * no, tiles = std::ceil(n / 128.0);
+    const double width = std::ceil((n - 128.0 * (tiles - 1)) / 16.0) * 16.0;  // last column tile
+    const double area = 128.0 * (128.0 * tiles * (tiles - 1) / 2 + tiles * width);
+    const double pairs = 2.0 * P * P * na / 60e12 +
+                         nt * ((2.0 * na * P * P + 4.0 * na * n * n * n + 4.0 * P * na * na) / 26e12 +
+                               60e-6);
+    const double orbitals = (2.0 * P * nv * na + 2.0 * no * n * nv * na) / 4e12 +
+                            2.0 * n * nv * no * std::ceil(nv / 128.0) * 128.0 * na / 60e12 +
+                            40.0 * n * K / 5e12 + nt * (2.0 * area * K / 78e12 + 20.0 * n * K / 5e12);
+    return orbitals < pairs;
+  }
   const double pairs = 2.0 * P * P * na +
                        nt * (2.0 * na * P * P + 2.0 * P * n * na + 4.0 * na * n * n * n +
                              4.0 * P * na * na);
@@ -1309,34 +1322,57 @@ bool use_mo_block(const rssri_handle *h, int dd_arith) {
 }
 
 // S7 for all tau points on the orbitals: out[t] = -U diag(w_t) U^T, in chunks of
-// occupied orbitals c (U and V of a chunk, 256 MB each at most) and of tau
-// points (their weights).
-cudaError_t block_mo(rssri_handle *h, bool df, double *out) {
+// occupied orbitals c (U and V of a chunk, 256 MB each at most; 1 GB of U for
+// the sliced form, whose launches per tau point want a long contraction) and of
+// tau points (their weights; the sliced form's digits, 1.6 GB).
+cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
+  const bool df = dd_arith != RSSRI_DD_FP64, oz = dd_arith == RSSRI_DD_OZ;
   cudaStream_t s = h->stream;
   const int n = h->n, no = h->n_occ, nv = n - no, nt = h->n_tau, na = h->n_aux;
   const long long nva = (long long)nv * na, row = (long long)n * nv;
   RS_TRY(ensure_mo_tab(h));
   const MoTab tab = mo_tab(h);
-  const size_t budget = (size_t)256 << 20;
+  const size_t budget = (size_t)(oz ? 1024 : 256) << 20;
   const long long per_c = row * nv;
   const int cc = (int)std::max<long long>(1, std::min<long long>(no, (long long)(budget / 8) / per_c));
-  const long long kc = (long long)cc * nv * nv;
-  const int tcw = (int)std::max<long long>(1, std::min<long long>(nt, (long long)(budget / 8) / kc));
+  // V of as many c at a time as fit 256 MB
+  const int vc = (int)std::max<long long>(1, std::min<long long>(cc, (32LL << 20) / per_c));
+  const long long kc = (long long)cc * nv * nv, ldc = oz ? (kc + 15) / 16 * 16 : kc;
+  const int tcw = (int)std::max<long long>(
+      1, std::min<long long>(nt, oz ? (1600LL << 20) / (12 * n * ldc) : (long long)(budget / 8) / kc));
   RS_TRY(ensure(h->moB1, (size_t)n * nva * 8));
   RS_TRY(ensure(h->moB2, (size_t)no * nva * 8));
-  RS_TRY(ensure(h->moV, (size_t)cc * per_c * 8));
-  RS_TRY(ensure(h->moU, (size_t)cc * per_c * 8));
-  RS_TRY(ensure(h->moW, (size_t)tcw * kc * 8));
+  RS_TRY(ensure(h->moV, (size_t)vc * per_c * 8));
+  RS_TRY(ensure(h->moU, (size_t)n * ldc * 8));
+  RS_TRY(ensure(h->moW, (size_t)(oz ? nt : tcw) * ldc * 8));
   MoGram q;
   q.df = df; q.n = n;
+  OzGram z;
+  z.n = n;
   size_t work = 0;
   for (long long c : {cc, no % cc ? no % cc : cc})
     for (int t : {tcw, nt % tcw ? nt % tcw : tcw}) {
-      q.K = c * nv * nv;
-      q.nt = t;
-      work = std::max(work, mo_gram_work(q));
+      q.K = z.K = c * nv * nv;
+      z.ldy = (z.K + 15) / 16 * 16;
+      q.nt = z.nt = t;
+      work = std::max(work, oz ? oz_gram_work(z) : mo_gram_work(q));
     }
   RS_TRY(ensure(h->moWork, work * sizeof(double)));
+  int *err = h->flags.as<int>() + 5;
+  if (oz) {
+    RS_TRY(ensure(h->ozY.d, (size_t)tcw * n * ldc * OZ_S * sizeof(__nv_bfloat16)));
+    RS_TRY(ensure(h->ozY.e, (size_t)tcw * n * sizeof(int)));
+    RS_TRY(ensure(h->ozYm, (size_t)nt * n * sizeof(int)));
+    z.ldy = ldc;
+    z.nt = tcw;
+    RS_TRY(ensure(h->ozY6, (size_t)tcw * n * sizeof(double) + oz_gram_lev6_floats(z) * sizeof(float)));
+    z.diag = h->ozY6.as<double>();
+    z.lev6 = reinterpret_cast<float *>(z.diag + (long long)tcw * n);
+  }
+  // U's pairs are scaled into the middle of fp32's range by [K]^L's largest
+  // magnitude, 2^-2e each, an exact power of two (the sliced form takes [K]^L up
+  // to 2^+-40, beyond what a product of two of it keeps as a pair)
+  const int e2 = oz && h->k_l_max > 0 ? 2 * std::ilogb(h->k_l_max) : 0;
   // K^Q_ia = sum_k K^Q_ik C_ka over the kept pairs, K^Q_bc = sum_i C_ic K^Q_ib
   if (df) {
     RS_TRY(ensure_kp_df64(h));
@@ -1361,9 +1397,27 @@ cudaError_t block_mo(rssri_handle *h, bool df, double *out) {
     g.C = h->moB2.as<double>(); g.ldc = nva;
     RS_TRY(gemm_p(h, RSSRI_PROF_DD_GEMM, g));
   }
-  for (int c0 = 0; c0 < no; c0 += cc) {
-    const int c = std::min(cc, no - c0);
-    // V[c][b][i][a] = sum_Q K^Q_bc K^Q_ia
+  if (oz) {  // the right operand of every V, K^Q_ia
+    OzView v;
+    v.x2 = h->moB1.as<float2>();
+    v.rs = na; v.cs2 = 1; v.k2pad = v.k2n = na; v.xlen = row * na;
+    RS_TRY(oz_make(h->ozPB, 1, (int)row, na));
+    RS_TRY(oz_slice_p(h, v, h->ozPB.v));
+  }
+  // V[c][b][i][a] = sum_Q K^Q_bc K^Q_ia for c occupied orbitals from c0
+  auto form_v = [&](int c0, int c) -> cudaError_t {
+    if (oz) {
+      OzView v;
+      v.x2 = h->moB2.as<float2>() + c0 * nva;
+      v.bs = nva; v.rs = na; v.cs2 = 1; v.k2pad = v.k2n = na; v.xlen = c * nva;
+      RS_TRY(oz_make(h->ozPA, c, nv, na));
+      RS_TRY(oz_slice_p(h, v, h->ozPA.v));
+      OzGemm g;
+      g.A = h->ozPA.v; g.B = h->ozPB.v;
+      g.M = nv; g.N = (int)row; g.batch = c;
+      g.C = h->moV.as<double>(); g.ldc = row; g.sC = per_c; g.ccap = c * per_c; g.err = err;
+      return oz_gemm_p(h, RSSRI_PROF_DD_GEMM, g);
+    }
     if (df) {
       SPAN(RSSRI_PROF_DD_GEMM, 2.0 * c * (double)per_c * na * 1e-9);
       DfGemm g;
@@ -1371,23 +1425,53 @@ cudaError_t block_mo(rssri_handle *h, bool df, double *out) {
       g.A = h->moB2.as<float2>() + c0 * nva; g.lda = na; g.sA = nva;
       g.B = h->moB1.as<float2>(); g.ldb = na; g.transB = 1;
       g.C64 = h->moV.as<double>(); g.ldc = row; g.sC = per_c;
-      RS_TRY(df_gemm_w(h, g));
-    } else {
-      GemmArgs g;
-      g.M = nv; g.N = (int)row; g.K = na; g.batch = c;
-      g.A = h->moB2.as<double>() + c0 * nva; g.lda = na; g.sA = nva;
-      g.B = h->moB1.as<double>(); g.ldb = na; g.transB = 1;
-      g.C = h->moV.as<double>(); g.ldc = row; g.sC = per_c;
-      RS_TRY(gemm_p(h, RSSRI_PROF_DD_GEMM, g));
+      return df_gemm_w(h, g);
     }
-    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_TRY(mo_pack(df, h->moV.as<double>(), n, nv, c, h->moU.p, s)); }
+    GemmArgs g;
+    g.M = nv; g.N = (int)row; g.K = na; g.batch = c;
+    g.A = h->moB2.as<double>() + c0 * nva; g.lda = na; g.sA = nva;
+    g.B = h->moB1.as<double>(); g.ldb = na; g.transB = 1;
+    g.C = h->moV.as<double>(); g.ldc = row; g.sC = per_c;
+    return gemm_p(h, RSSRI_PROF_DD_GEMM, g);
+  };
+  for (int c0 = 0; c0 < no; c0 += cc) {
+    const int c = std::min(cc, no - c0);
+    q.K = z.K = (long long)c * nv * nv;
+    z.ldy = (z.K + 15) / 16 * 16;
+    for (int v0 = 0; v0 < c; v0 += vc) {
+      const int cv = std::min(vc, c - v0);
+      RS_TRY(form_v(c0 + v0, cv));
+      SPAN(RSSRI_PROF_OTHER, 0.0);
+      RS_TRY(mo_pack(df, h->moV.as<double>(), n, nv, cv, std::ldexp(1.0, -e2), oz ? 0 : q.K,
+                     (long long)v0 * nv * nv, h->moU.p, s));
+    }
+    if (oz) {
+      {
+        SPAN(RSSRI_PROF_SLICE, 0.0);
+        RS_TRY(mo_weights(1, tab.hv, tab.ho, nv, no, c0, c, nt, tab.hexp, z.ldy, h->moW.p, s));
+        RS_TRY(oz_gram_max(h->moU.as<float2>(), h->moW.as<float2>(), n, z.K, z.ldy, nt,
+                           h->ozYm.as<int>(), s));
+      }
+      for (int t0 = 0; t0 < nt; t0 += tcw) {
+        z.nt = std::min(tcw, nt - t0);
+        z.U = h->moU.as<float2>(); z.y = h->moW.as<float2>() + t0 * z.ldy;
+        z.m = h->ozYm.as<int>() + (long long)t0 * n;
+        z.d = h->ozY.d.as<__nv_bfloat16>(); z.ef = h->ozY.e.as<int>();
+        z.scale = std::ldexp(1.0, 2 * e2); z.yexp = tab.hexp + t0;
+        z.out = out + (long long)t0 * n * n; z.accumulate = c0 > 0;
+        z.err = err; z.wait_polls = h->test_wait_polls;
+        { SPAN(RSSRI_PROF_SLICE, 0.0); RS_TRY(oz_gram_slice(z, s)); }
+        SPAN_T(RSSRI_PROF_DD_SPMM, (double)n * n * z.K * z.nt * 1e-9, oz_gram_flops(z) * 1e-9);
+        RS_TRY(oz_gram(z, h->moWork.as<double>(), s));
+      }
+      continue;
+    }
     for (int t0 = 0; t0 < nt; t0 += tcw) {
       const int t = std::min(tcw, nt - t0);
-      q.K = (long long)c * nv * nv;
       q.nt = t;
       { SPAN(RSSRI_PROF_OTHER, 0.0);
         RS_TRY(mo_weights(df, tab.gv + (long long)t0 * nv, tab.go + (long long)t0 * no, nv, no, c0, c,
-                          t, tab.texp + t0, h->moW.p, s)); }
+                          t, tab.texp + t0, q.K, h->moW.p, s)); }
       q.U = h->moU.p; q.ldu = q.K;
       q.w = h->moW.p;
       q.wexp = df ? tab.texp + t0 : nullptr;
@@ -1480,13 +1564,13 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   }
   // S7: all tau points on the orbitals, or tau by tau
   if (dd_df64) RS_CK(ensure_gg(h));
-  if (mo && dd_arith != RSSRI_DD_FP64) {
+  if (mo && dd_arith == RSSRI_DD_DF64) {
     // the range rule of the pairs' conversion, without the conversion
     SPAN(RSSRI_PROF_OTHER, 0.0);
     RS_CK(mo_range_check(G, nt, nn, range_flag(h), s));
     RS_CK(mo_range_check(Gb, nt, nn, range_flag(h), s));
   }
-  if (mo) RS_CK(block_mo(h, dd_arith != RSSRI_DD_FP64, h->sdd.as<double>()));
+  if (mo) RS_CK(block_mo(h, dd_arith, h->sdd.as<double>()));
   for (int t = 0; t < nt && !mo; ++t) {
     double *out = h->sdd.as<double>() + t * nn;
     if (dd_oz) {

@@ -91,17 +91,24 @@ cudaError_t mo_energy(const double *tr, const double *s2, int nt, int nkind, int
 // and, with df, as pairs of gv 2^-ev_t and go 2^-eo_t, the largest entry of each tau point
 // in [1, 2): pairs keep their precision only well inside fp32's exponent range.  texp[t] =
 // 2 ev_t + eo_t (the power of two that a term quadratic in gv and linear in go carries),
-// eexp[t] = ev_t + eo_t.
+// eexp[t] = ev_t + eo_t.  hv, ho: the square roots of gv and go; hexp[t] = the exponent of the
+// largest hv hv ho.
+struct MoTab {
+  double *gv, *go, *hv, *ho;
+  float2 *gvhl, *gohl;
+  int *texp, *eexp, *hexp;
+};
 cudaError_t mo_tables(const double *orb_e, int n, int no, double mu, const double *tau, int nt,
-                      int df, double *gv, double *go, float2 *gvhl, float2 *gohl, int *texp,
-                      int *eexp, cudaStream_t s);
+                      const MoTab &t, cudaStream_t s);
 // w[t][((c - c0) nv + a) nv + b] = go[t][c] gv[t][a] gv[t][b], c0 <= c < c0 + nc, for nt tau
-// points; df: pairs of the same times 2^-texp[t].
+// points, rows at stride ldw; df: pairs of the same times 2^-exps[t].
 cudaError_t mo_weights(int df, const double *gv, const double *go, int nv, int no, int c0, int nc,
-                       int nt, const int *texp, void *w, cudaStream_t s);
-// U[i][((c nv) + a) nv + b] from V[c][b][i][a] (fp64, nc x nv x n x nv): slot a < b holds
-// (V_ab + V_ba) / sqrt 2, a = b holds V_aa, a > b holds (V_ba - V_ab) sqrt(3/2); df: pairs.
-cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, void *U, cudaStream_t s);
+                       int nt, const int *exps, long long ldw, void *w, cudaStream_t s);
+// U_ik, k = k0 + (c nv + a) nv + b, from V[c][b][i][a] (fp64, nc x nv x n x nv): slot a < b holds
+// (V_ab + V_ba) / sqrt 2, a = b holds V_aa, a > b holds (V_ba - V_ab) sqrt(3/2), all times
+// scale; df: pairs.  U_ik is at U[i ldu + k], or with ldu = 0 at U[((k / 16) n + i) 16 + k % 16].
+cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, double scale, long long ldu,
+                    long long k0, void *U, cudaStream_t s);
 
 // out[a] = sum_q x[a][q]^2 (the diagonal of v^L on the kept pairs, where its largest magnitude is).
 cudaError_t mo_row_norm2(const double *x, int rows, int cols, double *out, cudaStream_t s);

@@ -14,7 +14,8 @@ namespace {
 template <class P>
 __global__ void mo_weights_kernel(const double *__restrict__ gv, const double *__restrict__ go,
                                   int nv, int no, int c0, int nc, int nt,
-                                  const int *__restrict__ texp, typename P::V *__restrict__ w) {
+                                  const int *__restrict__ texp, long long ldw,
+                                  typename P::V *__restrict__ w) {
   const long long kk = (long long)nc * nv * nv, total = kk * nt;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
@@ -23,7 +24,7 @@ __global__ void mo_weights_kernel(const double *__restrict__ gv, const double *_
     const int a = ab / nv, b = ab - a * nv;
     double v = go[t * no + c0 + c] * gv[t * nv + a] * gv[t * nv + b];
     if (texp) v = scalbn(v, -texp[t]);
-    w[e] = P::from_double(v);
+    w[t * ldw + k] = P::from_double(v);
   }
 }
 
@@ -31,7 +32,8 @@ __global__ void mo_weights_kernel(const double *__restrict__ gv, const double *_
 // so that reads (contiguous in a) and writes (contiguous in b) are coalesced.
 template <class P>
 __global__ void __launch_bounds__(256) mo_pack_kernel(const double *__restrict__ V, int n, int nv,
-                                                      int nc, int T, typename P::V *__restrict__ U) {
+                                                      int nc, int T, double scale, long long ldu,
+                                                      long long koff, typename P::V *__restrict__ U) {
   __shared__ double x[32][33], y[32][33];
   int ta, tb;
   tri_tile(blockIdx.x, T, ta, tb);
@@ -46,22 +48,26 @@ __global__ void __launch_bounds__(256) mo_pack_kernel(const double *__restrict__
     y[r][tx] = a2 < nv && b2 < nv ? Vc[((long long)b2 * n + i) * nv + a2] : 0.0;
   }
   __syncthreads();
-  typename P::V *Ui = U + ((long long)i * nc + c) * nv * nv;
-  const double rs = 0.70710678118654752440, ra = 1.2247448713915890491;  // 1/sqrt 2, sqrt(3/2)
+  const long long kc = koff + (long long)c * nv * nv;
+  auto at = [&](int a, int b) {
+    const long long k = kc + (long long)a * nv + b;
+    return ldu ? i * ldu + k : ((k >> 4) * n + i) * 16 + (k & 15);
+  };
+  const double rs = scale * 0.70710678118654752440, ra = scale * 1.2247448713915890491;  // 1/sqrt 2, sqrt(3/2)
   for (int r = ty; r < 32; r += 8) {
     // row a of slot (a, b), a in block ta, b in block tb
     int a = ta * 32 + r, b = tb * 32 + tx;
     if (a < nv && b < nv) {
       const double ab = x[tx][r], ba = y[r][tx];
-      const double v = a == b ? ab : (a < b ? (ab + ba) * rs : (ba - ab) * ra);
-      Ui[(long long)a * nv + b] = P::from_double(v);
+      const double v = a == b ? scale * ab : (a < b ? (ab + ba) * rs : (ba - ab) * ra);
+      U[at(a, b)] = P::from_double(v);
     }
     if (ta != tb) {  // the mirrored slot (a in block tb, b in block ta): a > b
       a = tb * 32 + r;
       b = ta * 32 + tx;
       if (a < nv && b < nv) {
         const double ab = y[tx][r], ba = x[r][tx];
-        Ui[(long long)a * nv + b] = P::from_double((ba - ab) * ra);
+        U[at(a, b)] = P::from_double((ba - ab) * ra);
       }
     }
   }
@@ -129,24 +135,26 @@ cudaError_t mo_gram(const MoGram &g, double *work, cudaStream_t s) {
 }
 
 cudaError_t mo_weights(int df, const double *gv, const double *go, int nv, int no, int c0, int nc,
-                       int nt, const int *texp, void *w, cudaStream_t s) {
+                       int nt, const int *exps, long long ldw, void *w, cudaStream_t s) {
   const long long total = (long long)nt * nc * nv * nv;
   if (df)
-    mo_weights_kernel<DF><<<grid_cap(total, 256), 256, 0, s>>>(gv, go, nv, no, c0, nc, nt, texp,
+    mo_weights_kernel<DF><<<grid_cap(total, 256), 256, 0, s>>>(gv, go, nv, no, c0, nc, nt, exps, ldw,
                                                               static_cast<float2 *>(w));
   else
     mo_weights_kernel<F64><<<grid_cap(total, 256), 256, 0, s>>>(gv, go, nv, no, c0, nc, nt, nullptr,
-                                                               static_cast<double *>(w));
+                                                               ldw, static_cast<double *>(w));
   ++launch_counter();
   return cudaGetLastError();
 }
 
-cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, void *U, cudaStream_t s) {
+cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, double scale, long long ldu,
+                    long long k0, void *U, cudaStream_t s) {
   const int T = ceil_div(nv, 32);
   dim3 grid(T * (T + 1) / 2, n, nc);
-  if (nc > 65535) return cudaErrorInvalidValue;
-  if (df) mo_pack_kernel<DF><<<grid, 256, 0, s>>>(V, n, nv, nc, T, static_cast<float2 *>(U));
-  else mo_pack_kernel<F64><<<grid, 256, 0, s>>>(V, n, nv, nc, T, static_cast<double *>(U));
+  if (df)
+    mo_pack_kernel<DF><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, k0, static_cast<float2 *>(U));
+  else
+    mo_pack_kernel<F64><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, k0, static_cast<double *>(U));
   ++launch_counter();
   return cudaGetLastError();
 }

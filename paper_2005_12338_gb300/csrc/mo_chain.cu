@@ -236,36 +236,34 @@ __global__ void mo_energy_kernel(const double *__restrict__ tr, const double *__
 // One block per tau point.
 __global__ void __launch_bounds__(256) mo_tables_kernel(const double *__restrict__ e, int n, int no,
                                                         double mu, const double *__restrict__ tau,
-                                                        int df, double *__restrict__ gv,
-                                                        double *__restrict__ go,
-                                                        float2 *__restrict__ gvhl,
-                                                        float2 *__restrict__ gohl,
-                                                        int *__restrict__ texp,
-                                                        int *__restrict__ eexp) {
-  __shared__ int mx[2];
+                                                        const MoTab tab) {
+  __shared__ int mx[4];
   const int t = blockIdx.x, nv = n - no;
-  if (threadIdx.x < 2) mx[threadIdx.x] = -100000;
+  if (threadIdx.x < 4) mx[threadIdx.x] = -100000;
   __syncthreads();
   const double tt = tau[t];
+  double *gv = tab.gv + (long long)t * nv, *go = tab.go + (long long)t * no;
+  double *hv = tab.hv + (long long)t * nv, *ho = tab.ho + (long long)t * no;
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const bool occ = i < no;
-    const double v = exp(occ ? (e[i] - mu) * tt : -(e[i] - mu) * tt);
-    if (occ) go[(long long)t * no + i] = v;
-    else gv[(long long)t * nv + i - no] = v;
-    // exponent of v (zero: none)
+    const double x = occ ? (e[i] - mu) * tt : -(e[i] - mu) * tt;
+    const double v = exp(x), h = exp(0.5 * x);
+    (occ ? go[i] : gv[i - no]) = v;
+    (occ ? ho[i] : hv[i - no]) = h;
+    // largest exponents (zero and non-finite values: none)
     if (v > 0.0 && isfinite(v)) atomicMax(&mx[occ ? 1 : 0], ilogb(v));
+    if (h > 0.0 && isfinite(h)) atomicMax(&mx[occ ? 3 : 2], ilogb(h));
   }
-  if (!df) return;
   __syncthreads();
   const int ev = mx[0] > -100000 ? mx[0] : 0, eo = mx[1] > -100000 ? mx[1] : 0;
   if (threadIdx.x == 0) {
-    texp[t] = 2 * ev + eo;
-    eexp[t] = ev + eo;
+    tab.texp[t] = 2 * ev + eo;
+    tab.eexp[t] = ev + eo;
+    tab.hexp[t] = 2 * (mx[2] > -100000 ? mx[2] : 0) + (mx[3] > -100000 ? mx[3] : 0);
   }
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    if (i < no) gohl[(long long)t * no + i] = split_pair(scalbn(go[(long long)t * no + i], -eo));
-    else
-      gvhl[(long long)t * nv + i - no] = split_pair(scalbn(gv[(long long)t * nv + i - no], -ev));
+    if (i < no) tab.gohl[(long long)t * no + i] = split_pair(scalbn(go[i], -eo));
+    else tab.gvhl[(long long)t * nv + i - no] = split_pair(scalbn(gv[i - no], -ev));
   }
 }
 
@@ -388,9 +386,8 @@ cudaError_t mo_energy(const double *tr, const double *s2, int nt, int nkind, int
 }
 
 cudaError_t mo_tables(const double *orb_e, int n, int no, double mu, const double *tau, int nt,
-                      int df, double *gv, double *go, float2 *gvhl, float2 *gohl, int *texp,
-                      int *eexp, cudaStream_t s) {
-  mo_tables_kernel<<<nt, 256, 0, s>>>(orb_e, n, no, mu, tau, df, gv, go, gvhl, gohl, texp, eexp);
+                      const MoTab &t, cudaStream_t s) {
+  mo_tables_kernel<<<nt, 256, 0, s>>>(orb_e, n, no, mu, tau, t);
   ++launch_counter();
   return cudaGetLastError();
 }

@@ -71,6 +71,9 @@ __device__ __noinline__ void check_fail(int code, int line, long long idx) {
 #define OZ_IN(idx, cap, code) true
 #endif
 
+constexpr int GRAM_TILES = 8;  // row tiles of a Gram matrix at most (n <= 1024)
+constexpr int GRAM_TYPES = GRAM_TILES * (GRAM_TILES + 1) / 2;
+
 struct OzParams {
   CUtensorMap ta0, ta1, tb0, tb1;  // digits 0-3 and 4-5 of A and B
   int M, N;          // dense: C rows / columns per batch; exchange: n, n_aux
@@ -86,6 +89,12 @@ struct OzParams {
   long long ldc, sC;
   int bk, nl16, jtiles, lb0;  // exchange geometry
   int tiles, ntiles, mtiles;  // the output tiles the persistent CTAs share
+  // Gram matrices: tile types (row tile <= column tile) in the order of their first queue
+  // entry per batch entry, the K steps of a split of each, and the splits' stride in C
+  int ntypes, per_batch, smax;
+  unsigned char tm[GRAM_TYPES], tn[GRAM_TYPES];
+  short first[GRAM_TYPES + 1];
+  int tkst[GRAM_TYPES];
   int *err;
   long long ccap, efa_cap, efb_cap;  // bounds of C and the exponent arrays (checks)
   int wait_polls;  // 0: normal; > 0: test mode (see OzGemm)
@@ -163,9 +172,9 @@ __device__ __forceinline__ uint64_t digit_desc(uint32_t base, int p) {
   return p < 4 ? smem_desc_sw(base + 32 * p, 1024, 2)
                : smem_desc_sw(base + TILE0 + 32 * (p - 4), 512, 4);
 }
-// Instruction descriptor: D fp32, A and B bf16, both K-major, M = N = 128.
-__device__ __forceinline__ uint32_t instr_desc_bf16() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+// Instruction descriptor: D fp32, A and B bf16, both K-major, M = 128, N = nw.
+__device__ __forceinline__ uint32_t instr_desc_bf16(int nw) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nw >> 3) << 17) |
          ((uint32_t)(BM >> 4) << 24);
 }
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
@@ -276,14 +285,26 @@ __device__ __forceinline__ int row_scale(int ef) { return max(ef, 1) - 1022; }
 // ------------------------------------------------------------- the GEMM ----
 // One output tile of a persistent CTA's queue (tile q = n tile + ntiles * rest):
 // dense: rest = m tile + mtiles * (batch * ksplit + split); exchange: rest = row tile.
+// kst K steps from step k0; nw columns (a multiple of 16, at most BN) are computed.
 struct OzTile {
-  int n0, m0, zb, split, rt, mt, jt;
+  int n0, m0, zb, split, rt, mt, jt, k0, kst, nw;
 };
 // With mfast: q = m tile + mtiles * (n tile + ntiles * (batch * ksplit + split)).
 template <int MODE>
 __device__ __forceinline__ OzTile oz_tile(const OzParams &p, int q) {
   OzTile t;
-  if (MODE == 0) {
+  t.kst = p.kst;
+  if (MODE == 2) {
+    t.zb = q / p.per_batch;
+    const int idx = q - t.zb * p.per_batch;
+    int y = 0;
+    while (idx >= p.first[y + 1]) ++y;
+    t.split = idx - p.first[y];
+    t.m0 = p.tm[y] * BM;
+    t.n0 = p.tn[y] * BN;
+    t.kst = p.tkst[y];
+    t.rt = t.mt = t.jt = 0;
+  } else if (MODE == 0) {
     int z;
     if (p.mfast) {
       const int rest = q / p.mtiles;
@@ -307,6 +328,9 @@ __device__ __forceinline__ OzTile oz_tile(const OzParams &p, int q) {
     t.jt = rest - t.mt * p.jtiles;
     t.m0 = t.zb = t.split = 0;
   }
+  t.k0 = t.split * t.kst;
+  // a Gram matrix's last column tile: only its columns (rounded up to 16) are multiplied
+  t.nw = MODE == 2 ? min(BN, (p.N - t.n0 + 15) & ~15) : BN;
   return t;
 }
 
@@ -321,8 +345,6 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
   uint64_t *done = acce + 1;        // every product this CTA issued has completed
   uint32_t *tslot = (uint32_t *)(done + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kst = p.kst;
-  const int nchunks = (kst + CHUNK - 1) / CHUNK;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -352,20 +374,27 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
       int it = 0;  // K steps loaded so far (all tiles)
       for (int q = blockIdx.x; q < p.tiles && go; q += gridDim.x) {
         const OzTile t = oz_tile<MODE>(p, q);
-        for (int st = 0; st < kst; ++st, ++it) {
+        // a Gram tile on the diagonal multiplies its rows by themselves: one operand
+        const bool one = MODE == 2 && t.m0 == t.n0;
+        for (int st = 0; st < t.kst; ++st, ++it) {
           const int s = it % STAGES;
           if (it >= STAGES &&
               !bar_wait(&empty[s], ((it / STAGES) - 1) & 1, p.err, 1, p.wait_polls)) {
             go = false;
             break;
           }
-          bar_expect(&full[s], STAGE);
+          bar_expect(&full[s], one ? OPB : STAGE);
           uint8_t *sa = smem + s * STAGE, *sb = sa + OPB;
           // coordinates (inner, 16-column block, ...): dense (0, kb, row, batch);
-          // exchange A (0, st, 0, tile), B (0, l block, k, q)
+          // exchange A (0, st, 0, tile), B (0, l block, k, q); Gram (0, row, kb, tau)
           int ay, az, aw, by, bz, bw;
-          if (MODE == 0) {
-            ay = by = t.split * kst + st;
+          if (MODE == 2) {
+            az = bz = t.k0 + st;
+            ay = t.m0;
+            by = t.n0;
+            aw = bw = t.zb;
+          } else if (MODE == 0) {
+            ay = by = t.k0 + st;
             az = t.m0;
             aw = t.zb;
             bz = t.n0;
@@ -381,19 +410,23 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
           }
           tma_load4(sa, &p.ta0, &full[s], 0, ay, az, aw);
           tma_load4(sa + TILE0, &p.ta1, &full[s], 0, ay, az, aw);
-          tma_load4(sb, &p.tb0, &full[s], 0, by, bz, bw);
-          tma_load4(sb + TILE0, &p.tb1, &full[s], 0, by, bz, bw);
+          if (!one) {
+            tma_load4(sb, &p.tb0, &full[s], 0, by, bz, bw);
+            tma_load4(sb + TILE0, &p.tb1, &full[s], 0, by, bz, bw);
+          }
         }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
       // MMA issuer
-      const uint32_t idesc = instr_desc_bf16();
       bool ok = true;
       int it = 0, gc = 0;  // K steps and chunks issued so far (all tiles)
       for (int q = blockIdx.x; q < p.tiles && ok; q += gridDim.x) {
-        for (int st = 0; st < kst; ++st, ++it) {
+        const OzTile t = oz_tile<MODE>(p, q);
+        const uint32_t idesc = instr_desc_bf16(t.nw);
+        const uint32_t b_off = MODE == 2 && t.m0 == t.n0 ? 0u : (uint32_t)OPB;
+        for (int st = 0; st < t.kst; ++st, ++it) {
           const int s = it % STAGES, cs = st % CHUNK;
           if (cs == 0 && gc > 0) {
             // the previous chunk's accumulators have been read
@@ -408,7 +441,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t base_a = s_u32(smem + s * STAGE), base_b = base_a + OPB;
+          const uint32_t base_a = s_u32(smem + s * STAGE), base_b = base_a + b_off;
 #pragma unroll
           for (int pa = 0; pa < OZ_S; ++pa)
 #pragma unroll
@@ -420,7 +453,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
                        digit_desc(base_b, pb), idesc, en);
             }
           mma_commit(&empty[s]);
-          if (cs == CHUNK - 1 || st == kst - 1) {
+          if (cs == CHUNK - 1 || st == t.kst - 1) {
             mma_commit(accf);
             ++gc;
           }
@@ -447,6 +480,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
       float hi[DC], lo[DC];
 #pragma unroll
       for (int c = 0; c < DC; ++c) hi[c] = lo[c] = 0.f;
+      const int nchunks = (t.kst + CHUNK - 1) / CHUNK;
       for (int c = 0; c < nchunks; ++c, ++gc) {
         if (!bar_wait(accf, gc & 1, p.err, 4, p.wait_polls) ||
             (p.err && *(volatile int *)p.err)) {
@@ -454,6 +488,8 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
           break;
         }
         asm volatile("tcgen05.fence::after_thread_sync;");
+        // (columns past nw hold nothing that is stored)
+        if (MODE != 2 || cq * DC < t.nw)
 #pragma unroll
         for (int f = 0; f < 8; ++f) {
           const uint32_t tl = tmem + ((uint32_t)(lq * 32 + 16 * (f >> 2)) << 16) +
@@ -484,14 +520,17 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
       for (int hr = 0; hr < 4; ++hr) {
         const int row = lq * 32 + 16 * (hr >> 1) + fr + 8 * (hr & 1);
         bool v;
-        if (MODE == 0) {
+        if (MODE != 1) {
           const int i = t.m0 + row;
           v = i < p.M;
           if (v && !OZ_IN(t.zb * p.efa_bs + i, p.efa_cap, 10)) v = false;
           ea[hr] = v ? row_scale(p.efa[t.zb * p.efa_bs + i]) : 0;
-          dst[hr] = p.ksplit > 1 ? p.C + (long long)(t.zb * p.ksplit + t.split) * p.M * p.N +
-                                       (long long)i * p.N
-                                 : p.C + t.zb * p.sC + (long long)i * p.ldc;
+          if (MODE == 2)
+            dst[hr] = p.C + ((long long)t.zb * p.smax + t.split) * p.M * p.N + (long long)i * p.N;
+          else
+            dst[hr] = p.ksplit > 1 ? p.C + (long long)(t.zb * p.ksplit + t.split) * p.M * p.N +
+                                         (long long)i * p.N
+                                   : p.C + t.zb * p.sC + (long long)i * p.ldc;
         } else {
           const int m = t.mt * 8 + (row >> 4), j = t.jt * 16 + (row & 15);
           v = m < p.M && j < p.M;
@@ -504,7 +543,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
       const int ncol = p.N;
       // the sign of -1 products flips the sign bit only
       const unsigned long long sgn = p.neg ? (1ull << 63) : 0ull;
-      const long long eb_off = MODE == 0 && !p.bshared ? t.zb * p.efb_bs : 0;
+      const long long eb_off = MODE != 1 && !p.bshared ? t.zb * p.efb_bs : 0;
 #pragma unroll
       for (int f = 0; f < 8; ++f) {
         const int j = t.n0 + cq * DC + 8 * (f & 3) + fc;  // this thread's column pair j, j + 1
@@ -1003,6 +1042,212 @@ __global__ void __launch_bounds__(256) oz_slice_short_kernel(OzView v, int rows,
   }
 }
 
+// ------------------------------------------------- Gram matrices (S7) -----
+// m[t][i] = bits of max_k |U_ik| y_tk (fp32 of the pairs' high parts): a block
+// walks 64-column pieces of 32 rows for up to 32 tau points; lane = row, so
+// that the 32 maxima stay in registers and y is a broadcast.  Two fp32
+// operations per element and tau point: ~1% of the products' time at N = 200.
+constexpr int GR = 32, GK = 64, GT = 32;
+__global__ void __launch_bounds__(256) oz_gram_max_kernel(const float2 *__restrict__ U,
+                                                          const float2 *__restrict__ y, int n,
+                                                          long long K, long long ldy, int nt,
+                                                          int slices, int *__restrict__ m) {
+  __shared__ float us[GK][GR + 1];
+  __shared__ float ys[GK][GT];
+  __shared__ int sm[GR][GT + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t0 = blockIdx.x * GT, i0 = blockIdx.y * GR;
+  const long long pieces = (K + GK - 1) / GK;
+  float mx[GT];
+#pragma unroll
+  for (int t = 0; t < GT; ++t) mx[t] = 0.f;
+  for (int e = threadIdx.x; e < GR * GT; e += 256) sm[e / GT][e % GT] = 0;
+  for (long long pc = blockIdx.z; pc < pieces; pc += slices) {
+    const long long k0 = pc * GK;
+    __syncthreads();
+    for (int e = threadIdx.x; e < GR * GK; e += 256) {
+      // 16 columns of a row are one 128-byte piece of U
+      const int u = e % KS, r = (e / KS) % GR, k = e / (KS * GR) * KS + u;
+      us[k][r] = i0 + r < n && k0 + k < K
+                     ? fabsf(U[(((k0 + k) >> 4) * n + i0 + r) * KS + u].x)
+                     : 0.f;
+    }
+    for (int e = threadIdx.x; e < GT * GK; e += 256) {
+      const int t = e / GK, k = e % GK;
+      ys[k][t] = t0 + t < nt && k0 + k < K ? y[(long long)(t0 + t) * ldy + k0 + k].x : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < GK / 8; ++u) {
+      const int k = warp * (GK / 8) + u;
+      const float a = us[k][lane];
+      const float4 *yr = reinterpret_cast<const float4 *>(ys[k]);
+#pragma unroll
+      for (int t = 0; t < GT / 4; ++t) {
+        const float4 v = yr[t];
+        mx[4 * t] = fmaxf(mx[4 * t], a * v.x);
+        mx[4 * t + 1] = fmaxf(mx[4 * t + 1], a * v.y);
+        mx[4 * t + 2] = fmaxf(mx[4 * t + 2], a * v.z);
+        mx[4 * t + 3] = fmaxf(mx[4 * t + 3], a * v.w);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < GT; ++t) atomicMax(&sm[lane][t], __float_as_int(mx[t]));
+  __syncthreads();
+  for (int e = threadIdx.x; e < GR * GT; e += 256) {
+    const int r = e / GT, t = e % GT;
+    if (i0 + r < n && t0 + t < nt && sm[r][t] > 0)
+      atomicMax(&m[(long long)(t0 + t) * n + i0 + r], sm[r][t]);
+  }
+}
+
+// The balanced base-256 digits (pre-scaled, see OzDigits) of (p + q), |p + q| <=
+// 2^7 (1 + 2^-22), p and q a normalised pair: the nearest multiple of 2^(-8 d) is peeled off
+// for d = 0 ... 5 by adding and subtracting 1.5 2^(23 - 8 d), exact in fp32 as
+// the remainders stay below half a step; q joins once p's own bits (24 from
+// 2^6) are used up, and d_3 stays below 192 of its steps: 8 bits, as bf16 holds.
+__device__ __forceinline__ void pair_digits(float p, float q, float *d) {
+  const float M0 = 12582912.0f;
+  d[0] = __fsub_rn(__fadd_rn(p, M0), M0);
+  p = __fsub_rn(p, d[0]);
+  d[1] = __fsub_rn(__fadd_rn(p, M0 * 0x1p-8f), M0 * 0x1p-8f);
+  p = __fsub_rn(p, d[1]);
+  d[2] = __fsub_rn(__fadd_rn(p, M0 * 0x1p-16f), M0 * 0x1p-16f);
+  p = __fadd_rn(__fsub_rn(p, d[2]), q);
+  d[3] = __fsub_rn(__fadd_rn(p, M0 * 0x1p-24f), M0 * 0x1p-24f);
+  p = __fsub_rn(p, d[3]);
+  d[4] = __fsub_rn(__fadd_rn(p, M0 * 0x1p-32f), M0 * 0x1p-32f);
+  p = __fsub_rn(p, d[4]);
+  d[5] = __fsub_rn(__fadd_rn(p, M0 * 0x1p-40f), M0 * 0x1p-40f);
+}
+
+// Digits of U_ik y_tk for nt tau points (batch entries), 2^e > every magnitude of
+// a row, e from the maxima m (written to ef as a biased fp64 exponent).  A
+// block takes 32 rows x GKB blocks of 16 columns; a thread keeps its row and its
+// half of the 16 columns and walks the blocks four apart, so that reads and
+// writes run through whole 128-byte pieces of neighbouring rows.  fp32
+// operations only: the pass runs at the HBM rate, 8 bytes read (U) and 12
+// written per value.
+//
+// The products drop digit pairs p + q >= 6.  Their signs are random between
+// different rows, but in a row's product with itself d_3^2 is not: its sum
+// grows with K (2^-49.6 of the squared row maximum per term) where the few
+// largest terms make up the result.  So the slicer also sums
+// d_3^2 + 2 d_2 d_4 + 2 d_1 d_5 (the whole level 6) per row and block, and
+// oz_gram_diag_kernel adds the blocks in order for the diagonal.
+constexpr int GKB = 64;
+__global__ void __launch_bounds__(256) oz_gram_slice_kernel(
+    const float2 *__restrict__ U, const float2 *__restrict__ y, int n, long long K, long long ldy,
+    const int *__restrict__ m, int *__restrict__ ef, __nv_bfloat16 *__restrict__ out, long long g1,
+    float *__restrict__ lev6) {
+  __shared__ float l6[4][GR];
+  const int b = blockIdx.z;
+  const int half = threadIdx.x & 1, rl = (threadIdx.x >> 1) & 31, kq = threadIdx.x >> 6;
+  const int r = blockIdx.y * GR + rl;
+  const bool row = r < n;
+  const int bits = row ? m[(long long)b * n + r] : 0;
+  if (blockIdx.x == 0 && kq == 0 && half == 0 && row)
+    // magnitudes below 2^e (1 + 2^-22), e = the maximum's exponent + 1
+    ef[(long long)b * n + r] = bits > 0 ? ((bits >> 23) & 0xFF) - 127 + 1 + 1022 : 1;
+  // 2^(7 - e): magnitudes up to 2^7
+  const int se = 127 + 7 - (((bits >> 23) & 0xFF) - 127 + 1);
+  const float sc = bits > 0 && se > 0 && se < 255 ? __int_as_float(se << 23) : 0.f;
+  const long long KB = ldy / KS;
+  const long long kb1 = min(KB, ((long long)blockIdx.x + 1) * GKB);
+  float s6 = 0.f;
+  if (row)
+#pragma unroll 2
+    for (long long kb = (long long)blockIdx.x * GKB + kq; kb < kb1; kb += 4) {
+      const long long k0 = kb * KS + half * KC;
+      const float4 *src = reinterpret_cast<const float4 *>(U + (kb * n + r) * KS + half * KC);
+      const float4 *yw = reinterpret_cast<const float4 *>(y + (long long)b * ldy + k0);
+      uint32_t o[OZ_S][KC / 2];
+#pragma unroll
+      for (int u = 0; u < KC; u += 2) {
+        const float4 v = src[u / 2], w = yw[u / 2];
+        float d0[OZ_S], d1[OZ_S];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float xh = (h ? v.z : v.x) * sc, xl = (h ? v.w : v.y) * sc;
+          const float yh = h ? w.z : w.x, yl = h ? w.w : w.y;
+          const float p = __fmul_rn(xh, yh);
+          float q = __fmaf_rn(xh, yh, -p);
+          q = __fmaf_rn(xh, yl, q);
+          q = __fmaf_rn(xl, yh, q);
+          // normalised, so that |q| is at most half a unit of p's last place
+          const float pn = __fadd_rn(p, q);
+          q = __fsub_rn(q, __fsub_rn(pn, p));
+          // columns past K: U and y are not written there
+          const bool in = k0 + u + h < K;
+          pair_digits(in ? pn : 0.f, in ? q : 0.f, h ? d1 : d0);
+        }
+#pragma unroll
+        for (int dgt = 0; dgt < OZ_S; ++dgt)
+          o[dgt][u / 2] = __byte_perm(__float_as_uint(d0[dgt]), __float_as_uint(d1[dgt]), 0x7632);
+        s6 += fmaf(d0[3], d0[3], 2.f * fmaf(d0[2], d0[4], d0[1] * d0[5]));
+        s6 += fmaf(d1[3], d1[3], 2.f * fmaf(d1[2], d1[4], d1[1] * d1[5]));
+      }
+      const long long blk = ((long long)b * KB + kb) * n + r;
+      if (!OZ_IN(blk * 64 + 63, g1, 36)) continue;
+#pragma unroll
+      for (int dgt = 0; dgt < OZ_S; ++dgt)
+        *reinterpret_cast<uint4 *>(out + digit_off(blk, half * KC, dgt, g1)) =
+            make_uint4(o[dgt][0], o[dgt][1], o[dgt][2], o[dgt][3]);
+    }
+  s6 += __shfl_xor_sync(0xffffffffu, s6, 1);
+  if (half == 0) l6[kq][rl] = s6;
+  __syncthreads();
+  if (threadIdx.x < GR && blockIdx.y * GR + threadIdx.x < n)
+    lev6[((long long)b * n + blockIdx.y * GR + threadIdx.x) * gridDim.x + blockIdx.x] =
+        (l6[0][threadIdx.x] + l6[1][threadIdx.x]) + (l6[2][threadIdx.x] + l6[3][threadIdx.x]);
+}
+
+// diag[t][i] = 2^(2 e - 14) times the sum of row i's level-6 sums over the slicer's
+// blocks, one warp per row, in a fixed order.
+__global__ void oz_gram_diag_kernel(const float *__restrict__ lev6, const int *__restrict__ ef,
+                                    long long rows, int blocks, double *__restrict__ diag) {
+  const long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  double s = 0.0;
+  for (int q = lane; q < blocks; q += 32) s += (double)lev6[r * blocks + q];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) diag[r] = scalbn(s, 2 * row_scale(ef[r]) - 14);
+}
+
+// out[t][i][j] (+)= -scale 2^(2 e_t) sum_s work[t][s][i][j] over the splits of the tile
+// of (min, max) of i and j, in order.
+struct GramSplits {
+  int T, smax;
+  short ks[GRAM_TILES][GRAM_TILES];
+};
+__global__ void oz_gram_reduce_kernel(const double *__restrict__ work, const GramSplits sp, int n,
+                                      int nt, double scale, const int *__restrict__ yexp,
+                                      int accumulate, const double *__restrict__ diag,
+                                      double *__restrict__ out) {
+  const long long nn = (long long)n * n, tot = nn * nt;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
+       e += (long long)gridDim.x * blockDim.x) {
+    const long long t = e / nn, r = e - t * nn;
+    int i = (int)(r / n), j = (int)(r - (long long)i * n);
+    if (i > j) {
+      const int x = i;
+      i = j;
+      j = x;
+    }
+    const int ks = sp.ks[i / BM][j / BN];
+    const double *p = work + t * sp.smax * nn + (long long)i * n + j;
+    double s = 0.0;
+    for (int k = 0; k < ks; ++k) s += p[k * nn];
+    if (i == j) s += diag[t * n + i];
+    s = -scale * scalbn(s, 2 * yexp[t]);
+    out[e] = accumulate ? out[e] + s : s;
+  }
+}
+
 // ---------------------------------------------------- exchange operand -----
 __global__ void oz_exch_gather_kernel(int n, int bk, int nl16, int jtiles, long long kx,
                                       const double *__restrict__ D, int P,
@@ -1146,6 +1391,8 @@ cudaError_t prepare() {
     RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SMEM));
     RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)SMEM));
+    RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SMEM));
     // the launch needs THREADS threads at the kernel's register count
     cudaFuncAttributes fa;
@@ -1367,6 +1614,179 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
     RS_TRY(cudaGetLastError());
   }
   return cudaSuccess;
+}
+
+// Gram matrices at N = 200 (100 virtual orbitals, 64 tau points): 1.38 ms per tau
+// point for the products (1,125 TFLOP/s of issued tensor work; 72-row tiles read
+// as much shared memory as 128-row ones) and 0.72 ms for the digits (HBM); the
+// whole setup and sampling call takes 177 ms against 281 with the contraction
+// over the kept pairs (exchange 136, dense products 60, digits 48).  With rows of
+// digits K-contiguous over the whole contraction, 12 MB apart, the same products
+// took 2.2 ms: their 128-byte pieces came from 128 different DRAM pages.
+namespace {
+// Tile types of a Gram matrix and the K split of each.  The tiles on and above
+// the diagonal differ in cost (the last column is narrower), so each type's K
+// is split in proportion: the splits of all types take about L K steps of a
+// full tile, and L is the one for which the rounds of tiles over the SMs,
+// times L plus a tile's drain and stores (~9 steps), come out least.
+struct GramPlan {
+  int T = 0, types = 0, per_batch = 0, smax = 0;
+  int tm[GRAM_TYPES], tn[GRAM_TYPES], ks[GRAM_TYPES], kst[GRAM_TYPES];
+};
+bool gram_plan(const OzGram &g, GramPlan *pl) {
+  pl->T = ceil_div(g.n, BM);
+  if (pl->T > GRAM_TILES) return false;
+  const long long steps = (g.K + KS - 1) / KS;
+  double w[GRAM_TYPES];
+  pl->types = 0;
+  for (int i = 0; i < pl->T; ++i)
+    for (int j = i; j < pl->T; ++j) {
+      pl->tm[pl->types] = i;
+      pl->tn[pl->types] = j;
+      // A's rows are read from shared memory whatever the width
+      w[pl->types++] = 0.25 + 0.75 * std::min(BN, (g.n - j * BN + 15) / 16 * 16) / BN;
+    }
+  double wsum = 0;
+  for (int y = 0; y < pl->types; ++y) wsum += w[y];
+  double best = 0;
+  bool have = false;
+  for (int rounds = 1; rounds <= 24; ++rounds) {
+    // L such that about rounds * 152 tiles are made
+    const double L = std::max(8.0, (double)steps * wsum * g.nt / (rounds * 152.0 * 0.985));
+    long long items = 0;
+    int smax = 0;
+    GramPlan c = *pl;
+    double longest = 0;
+    for (int y = 0; y < pl->types; ++y) {
+      long long ks = std::max<long long>(1, (long long)(steps * w[y] / L + 0.5));
+      ks = std::min<long long>({ks, steps, 512});
+      c.kst[y] = (int)((steps + ks - 1) / ks);
+      c.ks[y] = (int)((steps + c.kst[y] - 1) / c.kst[y]);
+      items += c.ks[y];
+      smax = std::max(smax, c.ks[y]);
+      longest = std::max(longest, c.kst[y] * w[y]);
+    }
+    const double cost = (double)((items * g.nt + 151) / 152) * (longest + 9.0) +
+                        (double)items * g.nt * BM * BN * 16.0 / 5.3e6;
+    if (!have || cost < best) {
+      have = true;
+      best = cost;
+      c.per_batch = (int)items;
+      c.smax = smax;
+      c.T = pl->T;
+      c.types = pl->types;
+      *pl = c;
+    }
+  }
+  return pl->per_batch <= 32767 && pl->smax <= 32767;
+}
+}  // namespace
+
+size_t oz_gram_lev6_floats(const OzGram &g) {
+  return (size_t)g.nt * g.n * ceil_div(g.ldy, (long long)GKB * KS);
+}
+size_t oz_gram_work(const OzGram &g) {
+  GramPlan pl;
+  return gram_plan(g, &pl) ? (size_t)g.nt * pl.smax * g.n * g.n : 0;
+}
+double oz_gram_flops(const OzGram &g) {
+  GramPlan pl;
+  if (!gram_plan(g, &pl)) return 0.0;
+  double f = 0.0;
+  for (int y = 0; y < pl.types; ++y)
+    f += OZ_PRODUCTS * 2.0 * BM * std::min(BN, (g.n - pl.tn[y] * BN + 15) / 16 * 16) * (double)KS *
+         pl.kst[y] * pl.ks[y];
+  return f * g.nt;
+}
+
+cudaError_t oz_gram_max(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
+                        int *m, cudaStream_t s) {
+  if (n <= 0 || nt <= 0 || K <= 0) return cudaSuccess;
+  RS_TRY(cudaMemsetAsync(m, 0, (size_t)nt * n * sizeof(int), s));
+  const long long pieces = (K + GK - 1) / GK;
+  dim3 g(ceil_div(nt, GT), ceil_div(n, GR), 1);
+  const int slices = (int)std::max<long long>(
+      1, std::min<long long>({pieces, 152LL * 8 / (g.x * g.y) + 1, 65535}));
+  g.z = slices;
+  oz_gram_max_kernel<<<g, 256, 0, s>>>(U, y, n, K, ldy, nt, slices, m);
+  ++launch_counter();
+  return cudaGetLastError();
+}
+
+cudaError_t oz_gram_slice(const OzGram &g, cudaStream_t s) {
+  if (g.ldy % KS || ((uintptr_t)g.U % 16) || ((uintptr_t)g.y % 16) || g.nt > 65535)
+    return cudaErrorInvalidValue;
+  dim3 gr(ceil_div(g.ldy, (long long)GKB * KS), ceil_div(g.n, GR), g.nt);
+  oz_gram_slice_kernel<<<gr, 256, 0, s>>>(g.U, g.y, g.n, g.K, g.ldy, g.m, g.ef, g.d,
+                                          (long long)g.nt * g.n * g.ldy * 4, g.lev6);
+  ++launch_counter();
+  RS_TRY(cudaGetLastError());
+  const long long rows = (long long)g.nt * g.n;
+  oz_gram_diag_kernel<<<ceil_div(rows * 32, 256), 256, 0, s>>>(g.lev6, g.ef, rows, (int)gr.x, g.diag);
+  ++launch_counter();
+  return cudaGetLastError();
+}
+
+cudaError_t oz_gram(const OzGram &g, double *work, cudaStream_t s) {
+  if (!oz_available()) return cudaErrorNotSupported;
+  if (g.n <= 0 || g.nt <= 0 || g.K <= 0) return cudaSuccess;
+  GramPlan pl;
+  if (!gram_plan(g, &pl)) return cudaErrorInvalidValue;
+  OzParams p;
+  std::memset(&p, 0, sizeof(p));
+  {
+    // (slot, row, K block, tau): the 128 rows of a box are one contiguous piece
+    const cuuint64_t kb = (cuuint64_t)(g.ldy / KS), n = (cuuint64_t)g.n;
+    const cuuint64_t d0[4] = {64, n, kb, (cuuint64_t)g.nt};
+    const cuuint64_t s0[3] = {128, n * 128, kb * n * 128};
+    const cuuint32_t b0[4] = {64, BM, 1, 1};
+    RS_TRY(make_map4(&p.ta0, g.d, d0, s0, b0));
+    const cuuint64_t d1[4] = {32, n, kb, (cuuint64_t)g.nt};
+    const cuuint64_t s1[3] = {64, n * 64, kb * n * 64};
+    const cuuint32_t b1[4] = {32, BM, 1, 1};
+    RS_TRY(make_map4(&p.ta1, g.d + (long long)g.nt * g.n * g.ldy * 4, d1, s1, b1));
+  }
+  p.tb0 = p.ta0;
+  p.tb1 = p.ta1;
+  p.M = p.N = g.n;
+  p.ksplit = 2;
+  p.efa = p.efb = g.ef;
+  p.efa_bs = p.efb_bs = g.n;
+  p.C = work;
+  p.vec2 = (uintptr_t)work % 16 == 0 && g.n % 2 == 0;
+  p.err = g.err;
+  p.ccap = (long long)g.nt * pl.smax * g.n * g.n;
+  p.efa_cap = p.efb_cap = (long long)g.nt * g.n;
+  p.wait_polls = g.wait_polls;
+  p.ntypes = pl.types;
+  p.per_batch = pl.per_batch;
+  p.smax = pl.smax;
+  GramSplits sp;
+  std::memset(&sp, 0, sizeof(sp));
+  sp.T = pl.T;
+  sp.smax = pl.smax;
+  int at = 0;
+  for (int y = 0; y < pl.types; ++y) {
+    p.tm[y] = (unsigned char)pl.tm[y];
+    p.tn[y] = (unsigned char)pl.tn[y];
+    p.first[y] = (short)at;
+    p.tkst[y] = pl.kst[y];
+    at += pl.ks[y];
+    sp.ks[pl.tm[y]][pl.tn[y]] = (short)pl.ks[y];
+  }
+  p.first[pl.types] = (short)at;
+  const long long tiles = (long long)pl.per_batch * g.nt;
+  if (tiles > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
+  p.tiles = (int)tiles;
+  RS_TRY(prepare());
+  oz_gemm_kernel<2><<<(unsigned)std::min<long long>(tiles, sm_count()), THREADS, SMEM, s>>>(p);
+  ++launch_counter();
+  RS_TRY(cudaGetLastError());
+  const long long tot = (long long)g.nt * g.n * g.n;
+  oz_gram_reduce_kernel<<<(int)std::min<long long>((tot + 255) / 256, 152 * 8), 256, 0, s>>>(
+      work, sp, g.n, g.nt, g.scale, g.yexp, g.accumulate, g.diag, g.out);
+  ++launch_counter();
+  return cudaGetLastError();
 }
 
 cudaError_t oz_rows_kp(const double *KP, const int *rowptr, int n, int na, int W, double *out,

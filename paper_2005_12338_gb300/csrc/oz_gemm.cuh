@@ -115,6 +115,41 @@ cudaError_t oz_exch(const OzExch &x, const OzDigits &X, const OzDigits &At, doub
                     long long tcap, double alpha, int *err, cudaStream_t s, int wait_polls = 0);
 double oz_exch_flops(const OzExch &x);
 
+// Gram matrices of the block on the orbitals (mo.cuh): out[t] (+)= -scale 2^(2 e_t)
+// Y_t Y_t^T with Y_t,ik = U_ik y_tk, y [nt][K] pairs (rows of stride ldy, a multiple
+// of 16), e_t = yexp[t], and U [n x K] pairs in blocks of 16 columns, column
+// 16 kb + u of row i at U[(kb n + i) 16 + u], so that U and the digits (in the same
+// order, 128 + 64 bytes per row and block) are streamed in whole pieces.  oz_gram_max finds
+// each row's largest magnitude per tau point (m[t][i], fp32 bits), oz_gram_slice
+// writes the digits of nt tau points (d: OZ_S nt n ldy values, ef[t][i]) and the
+// digit products of the diagonal that the tensor cores leave out (lev6, diag),
+// and oz_gram multiplies them on the tensor cores: the tiles on and above the
+// diagonal, each tile's K split over CTAs, the partial sums in `work`
+// (oz_gram_work() doubles) added in a fixed order; n <= 1024.
+struct OzGram {
+  int n = 0, nt = 1;
+  long long K = 0, ldy = 0;
+  const float2 *U = nullptr, *y = nullptr;
+  const int *m = nullptr;
+  __nv_bfloat16 *d = nullptr;
+  int *ef = nullptr;
+  double scale = 1.0;
+  float *lev6 = nullptr;   // the slicer's level-6 sums (oz_gram_lev6_floats())
+  double *diag = nullptr;  // [nt][n], what they add to the diagonal
+  const int *yexp = nullptr;
+  double *out = nullptr;
+  int accumulate = 0;
+  int *err = nullptr;
+  int wait_polls = 0;
+};
+size_t oz_gram_lev6_floats(const OzGram &g);
+size_t oz_gram_work(const OzGram &g);
+double oz_gram_flops(const OzGram &g);
+cudaError_t oz_gram_max(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
+                        int *m, cudaStream_t s);
+cudaError_t oz_gram_slice(const OzGram &g, cudaStream_t s);
+cudaError_t oz_gram(const OzGram &g, double *work, cudaStream_t s);
+
 // Row-batched operands of K^Q G, the block's first product (PG[i][m][Q] =
 // sum over the kept pairs a = (i, k) of row i of K_P[a][Q] G[k][m]), padded to
 // W columns per row i of the pair list (CSR rowptr, pair columns pcol):
