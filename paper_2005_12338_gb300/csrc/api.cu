@@ -1963,12 +1963,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
 // Coefficients c(tau, i, j) of the trained network for the current G and Sigma_DD.
 constexpr int CV_CHUNK = 65536;
 
-size_t cv_work_floats(int batch) {
-  const int m = std::max(batch, 2048);
-  return cv_tc_work_floats() + std::max({sgemm_work_floats(CV_HIDDEN, CV_HIDDEN, m),
-                   sgemm_work_floats(CV_HIDDEN, CV_NFEAT, m), sgemm_work_floats(1, CV_HIDDEN, m),
-                   (size_t)1024});
-}
+size_t cv_work_floats(int batch) { return cv_tc_work_floats() + cv_sum_floats(batch); }
 
 cudaError_t cv_compute_c(rssri_handle *h, const double *G, const double *Gb) {
   cudaStream_t s = h->stream;
@@ -2637,7 +2632,7 @@ int rssri_cv_train(rssri_handle *h, const rssri_options *o, const float *init_pa
   // fixed evaluation set: the first E elements
   auto eval = [&](double *out) {
     ck(cv_forward(P, X, E, act, work, s));
-    ck(cv_backward(P, X, E, T, Wt, act, grad, loss, work, s));
+    ck(cv_loss(E, T, Wt, act, loss, work, s));
     float l = 0;
     ck(cudaMemcpyAsync(&l, loss, sizeof(float), cudaMemcpyDeviceToHost, s));
     ck(cudaStreamSynchronize(s));
@@ -2658,9 +2653,7 @@ int rssri_cv_train(rssri_handle *h, const rssri_options *o, const float *init_pa
   while (gcd(stride, total) != 1) ++stride;
   for (int step = 1; step <= steps && e == cudaSuccess; ++step) {
     const long long start = ((long long)(step - 1) * batch) % total;
-    ck(cv_gather(X, CV_NFEAT, total, start, stride, batch, bx, s));
-    ck(cv_gather(T, 1, total, start, stride, batch, bt, s));
-    ck(cv_gather(Wt, 1, total, start, stride, batch, bw, s));
+    ck(cv_gather(X, T, Wt, total, start, stride, batch, bx, bt, bw, s));
     ck(cv_forward(P, bx, batch, act, work, s));
     ck(cv_backward(P, bx, batch, bt, bw, act, grad, nullptr, work, s));
     ck(cv_adam(P, grad, h->cv_m.as<float>(), h->cv_v.as<float>(), (int)CV_NPARAM, lr, step, s));

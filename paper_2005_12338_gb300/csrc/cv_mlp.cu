@@ -12,6 +12,13 @@
 // operands and fp32 accumulation (tcgen05); the 10-wide input layer, the
 // 1-wide output layer, activations, loss and Adam are fp32.  Fixed-order
 // reductions throughout.
+//
+// A training step of 2,048 rows is small work in a long chain of launches: 17
+// launches, each as wide as the shape allows, where element-wise passes join
+// the product or the transposes next to them and the sums over rows (biases,
+// input and output layer) run side by side in one launch.  100 steps with the
+// statistics run at N = 64 take 21 ms; one launch per operation with the sums
+// over rows on one or two blocks took 92 ms (the column sums ~150 us each).
 #include <cuda_bf16.h>
 
 #include "cv_mlp.cuh"
@@ -23,69 +30,6 @@ namespace {
 int grid_cap(long long work, int threads) {
   long long b = (work + threads - 1) / threads;
   return (int)(b < 1 ? 1 : (b > 152 * 32 ? 152 * 32 : b));
-}
-
-// ------------------------------------------------------------- sgemm -----
-// C = alpha * op(A) op(B) + beta * C (row-major fp32); partial = 1 writes the
-// raw sum of this block's K chunk to C + z * M * N.
-template <int TA, int TB>
-__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, int kchunk,
-                                                    const float *__restrict__ A, long long lda,
-                                                    const float *__restrict__ B, long long ldb,
-                                                    float *__restrict__ C, long long ldc,
-                                                    float alpha, float beta, int partial) {
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ float As[BK][BM + 1];
-  __shared__ float Bs[BK][BN + 1];
-  const int z = blockIdx.z;
-  const int kbeg = z * kchunk, kend = min(K, kbeg + kchunk);
-  const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float acc[4][4] = {};
-  for (int kt = kbeg; kt < kend; kt += BK) {
-    for (int e = tid; e < BM * BK; e += 256) {
-      const int i = TA ? e % BM : e / BK, k = TA ? e / BM : e % BK;
-      const int gi = row0 + i, gk = kt + k;
-      float v = 0.f;
-      if (gi < M && gk < kend) v = TA ? A[(long long)gk * lda + gi] : A[(long long)gi * lda + gk];
-      As[k][i] = v;
-    }
-    for (int e = tid; e < BN * BK; e += 256) {
-      const int j = TB ? e / BK : e % BN, k = TB ? e % BK : e / BN;
-      const int gj = col0 + j, gk = kt + k;
-      float v = 0.f;
-      if (gj < N && gk < kend) v = TB ? B[(long long)gj * ldb + gk] : B[(long long)gk * ldb + gj];
-      Bs[k][j] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-  for (int i = 0; i < 4; ++i) {
-    const int gi = row0 + ty * 4 + i;
-    if (gi >= M) continue;
-    for (int j = 0; j < 4; ++j) {
-      const int gj = col0 + tx * 4 + j;
-      if (gj >= N) continue;
-      if (partial) {
-        C[(long long)z * M * N + (long long)gi * N + gj] = acc[i][j];
-      } else {
-        float *p = C + (long long)gi * ldc + gj;
-        *p = (beta != 0.f) ? alpha * acc[i][j] + beta * *p : alpha * acc[i][j];
-      }
-    }
-  }
 }
 
 __global__ void sreduce_kernel(const float *__restrict__ part, int ks, int M, int N,
@@ -100,75 +44,157 @@ __global__ void sreduce_kernel(const float *__restrict__ part, int ks, int M, in
   }
 }
 
-// Z += b (per column), A = silu(Z) (A may be null)
-__global__ void bias_silu_kernel(float *__restrict__ Z, const float *__restrict__ b, long long M,
-                                 int N, float *__restrict__ A) {
-  const long long total = M * N;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const float z = Z[e] + b[e % N];
+__device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
+
+// Layer 0 (10 inputs, fp32): Z = X W0^T + b, h = bf16(silu(Z)), A = silu(Z).  One
+// thread per output; the ten products are added in ascending order.
+__global__ void __launch_bounds__(256) layer0_kernel(const float *__restrict__ X,
+                                                     const float *__restrict__ W,
+                                                     const float *__restrict__ b, int m,
+                                                     float *__restrict__ Z, float *__restrict__ A,
+                                                     __nv_bfloat16 *__restrict__ h) {
+  // block: 256 outputs of a row group; this thread's weights stay in registers
+  const int j = threadIdx.x;
+  float w[CV_NFEAT];
+#pragma unroll
+  for (int k = 0; k < CV_NFEAT; ++k) w[k] = W[j * CV_NFEAT + k];
+  const float bj = b[j];
+  for (long long r = blockIdx.x; r < m; r += gridDim.x) {
+    float acc = 0.f;
+#pragma unroll
+    for (int k = 0; k < CV_NFEAT; ++k) acc = fmaf(X[r * CV_NFEAT + k], w[k], acc);
+    const float z = acc + bj, av = silu(z);
+    const long long e = r * CV_HIDDEN + j;
     Z[e] = z;
-    if (A) A[e] = z / (1.f + __expf(-z));
+    A[e] = av;
+    h[e] = __float2bfloat16_rn(av);
   }
 }
 
-// dZ = dA * silu'(Z)
-__global__ void silu_back_kernel(const float *__restrict__ dA, const float *__restrict__ Z,
-                                 long long total, float *__restrict__ dZ) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const float z = Z[e];
-    const float s = 1.f / (1.f + __expf(-z));
-    dZ[e] = dA[e] * s * (1.f + z * (1.f - s));
+// Z += b, A = silu(Z), h = bf16(A), four elements per thread (256 columns).
+__global__ void __launch_bounds__(256) bias_silu_kernel(float *__restrict__ Z,
+                                                        const float *__restrict__ b, long long total,
+                                                        float *__restrict__ A,
+                                                        __nv_bfloat16 *__restrict__ h) {
+  for (long long e = 4 * (blockIdx.x * (long long)blockDim.x + threadIdx.x); e < total;
+       e += 4LL * gridDim.x * blockDim.x) {
+    float4 z = *reinterpret_cast<float4 *>(Z + e);
+    const float4 bv = *reinterpret_cast<const float4 *>(b + (e & (CV_HIDDEN - 1)));
+    z.x += bv.x;
+    z.y += bv.y;
+    z.z += bv.z;
+    z.w += bv.w;
+    const float4 a = make_float4(silu(z.x), silu(z.y), silu(z.z), silu(z.w));
+    *reinterpret_cast<float4 *>(Z + e) = z;
+    *reinterpret_cast<float4 *>(A + e) = a;
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a.x, a.y), hi = __floats2bfloat162_rn(a.z, a.w);
+    *reinterpret_cast<uint2 *>(h + e) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo),
+                                                   *reinterpret_cast<const uint32_t *>(&hi));
   }
 }
 
-// dst = bf16(src), elementwise
-__global__ void to_bf16_kernel(const float *__restrict__ src, long long n,
-                               __nv_bfloat16 *__restrict__ dst) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x)
-    dst[e] = __float2bfloat16_rn(src[e]);
-}
-
-// dst[c][r] = bf16(src[r][c]) for r < rows, c < cols (dst row stride ldd,
-// columns rows..ldd-1 set to zero), through 32 x 32 shared-memory tiles
-__global__ void transpose_bf16_kernel(const float *__restrict__ src, int rows, int cols,
-                                      long long lds, __nv_bfloat16 *__restrict__ dst,
-                                      long long ldd) {
-  __shared__ float t[32][33];
+// The last hidden layer's bias and silu, and the output layer: Z += b, A = silu(Z),
+// y = sum_k A_k w_k + b3, k ascending.  32 rows per block through shared memory; a
+// lane owns a row, so that the sum runs in order at register speed.
+__global__ void __launch_bounds__(256) output_kernel(float *__restrict__ Z, const float *__restrict__ b,
+                                                     const float *__restrict__ w3,
+                                                     const float *__restrict__ b3, int m,
+                                                     float *__restrict__ A, float *__restrict__ y) {
+  __shared__ float s[32][CV_HIDDEN + 1];
+  __shared__ float w[CV_HIDDEN];
   const long long r0 = (long long)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int k = ty; k < 32; k += blockDim.x >> 5) {
-    const long long r = r0 + k;
-    const int c = c0 + tx;
-    t[k][tx] = (r < rows && c < cols) ? src[r * lds + c] : 0.f;
+  const int c = threadIdx.x;
+  w[c] = w3[c];
+  const float bc = b[c];
+#pragma unroll 8
+  for (int r = 0; r < 32; ++r) {
+    if (r0 + r >= m) break;
+    const long long e = (r0 + r) * CV_HIDDEN + c;
+    const float z = Z[e] + bc, a = silu(z);
+    Z[e] = z;
+    A[e] = a;
+    s[r][c] = a;
   }
   __syncthreads();
-  for (int k = ty; k < 32; k += blockDim.x >> 5) {
-    const int c = c0 + k;
-    const long long r = r0 + tx;
-    if (c < cols && r < ldd) dst[(long long)c * ldd + r] = __float2bfloat16_rn(t[tx][k]);
+  if (threadIdx.x < 32 && r0 + threadIdx.x < m) {
+    float acc = 0.f;
+#pragma unroll 16
+    for (int k = 0; k < CV_HIDDEN; ++k) acc = fmaf(s[threadIdx.x][k], w[k], acc);
+    y[r0 + threadIdx.x] = acc + b3[0];
   }
 }
 
-// out[j] = sum_i X[i][j], i in order (one thread per column)
-__global__ void colsum_kernel(const float *__restrict__ X, int M, int N, float *__restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N) return;
-  float s = 0.f;
-  for (int i = 0; i < M; ++i) s += X[(long long)i * N + j];
-  out[j] = s;
+// d = dA silu'(Z) for one element.
+__device__ __forceinline__ float silu_back(float dA, float z) {
+  const float s = 1.f / (1.f + __expf(-z));
+  return dA * s * (1.f + z * (1.f - s));
 }
 
-// dy = 2 w (1 + y - t) / sum w ; loss = sum w (1 + y - t)^2 / sum w
-__global__ void loss_kernel(const float *__restrict__ y, const float *__restrict__ t,
-                            const float *__restrict__ w, int M, float *__restrict__ dy,
-                            float *__restrict__ loss) {
-  __shared__ double sh[2][32];
+// Z <- dA silu'(Z) with dA given, or dA = dy w3^T (w3 non-null); h = bf16(Z) (may be
+// null); and with t0: bf16 transposes t0 of the new Z and t1 of A, [256][ldt] with
+// columns m..ldt-1 zero.  32 x 32 tiles through shared memory.
+__global__ void __launch_bounds__(256) back_kernel(const float *__restrict__ dA,
+                                                   const float *__restrict__ dy,
+                                                   const float *__restrict__ w3, float *__restrict__ Z,
+                                                   const float *__restrict__ A, int m,
+                                                   __nv_bfloat16 *__restrict__ h,
+                                                   __nv_bfloat16 *__restrict__ t0,
+                                                   __nv_bfloat16 *__restrict__ t1, long long ldt) {
+  __shared__ float sz[32][33], sa[32][33];
+  const long long r0 = (long long)blockIdx.x * 32;
+  const int c0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = ty; k < 32; k += 8) {
+    const long long r = r0 + k;
+    float d = 0.f, a = 0.f;
+    if (r < m) {
+      const long long e = r * CV_HIDDEN + c0 + tx;
+      // dy w3 as a product of one term: fma(dy, w3, 0)
+      d = silu_back(w3 ? fmaf(dy[r], w3[c0 + tx], 0.f) : dA[e], Z[e]);
+      Z[e] = d;
+      if (h) h[e] = __float2bfloat16_rn(d);
+      if (t0) a = A[e];
+    }
+    sz[k][tx] = d;
+    sa[k][tx] = a;
+  }
+  if (!t0) return;
+  __syncthreads();
+#pragma unroll
+  for (int k = ty; k < 32; k += 8) {
+    const long long r = r0 + tx;
+    if (r < ldt) {
+      t0[(long long)(c0 + k) * ldt + r] = __float2bfloat16_rn(sz[tx][k]);
+      t1[(long long)(c0 + k) * ldt + r] = __float2bfloat16_rn(sa[tx][k]);
+    }
+  }
+}
+
+// bf16 copies of W1, W2 and their transposes (32 x 32 tiles; blockIdx.z: which).
+__global__ void __launch_bounds__(256) weights_kernel(const float *__restrict__ W1,
+                                                      const float *__restrict__ W2,
+                                                      __nv_bfloat16 *__restrict__ w) {
+  constexpr int H = CV_HIDDEN;
+  __shared__ float t[32][33];
+  const float *W = blockIdx.z ? W2 : W1;
+  __nv_bfloat16 *o = w + (long long)blockIdx.z * H * H, *ot = w + (2LL + blockIdx.z) * H * H;
+  const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int k = ty; k < 32; k += 8) {
+    const float v = W[(r0 + k) * H + c0 + tx];
+    o[(r0 + k) * H + c0 + tx] = __float2bfloat16_rn(v);
+    t[k][tx] = v;
+  }
+  __syncthreads();
+  for (int k = ty; k < 32; k += 8) ot[(c0 + k) * H + r0 + tx] = __float2bfloat16_rn(t[tx][k]);
+}
+
+// Per warp of the loss sum: thread t of 1024 adds the elements t, t + 1024, ... in
+// order, then the warp its 32 sums; block b is warp b.  sums [2][32].
+constexpr int LOSS_T = 1024;
+__global__ void loss_sums_kernel(const float *__restrict__ y, const float *__restrict__ t,
+                                 const float *__restrict__ w, int M, double *__restrict__ sums) {
   double sw = 0, sl = 0;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
+  for (int i = blockIdx.x * 32 + threadIdx.x; i < M; i += LOSS_T) {
     sw += w[i];
     const double r = 1.0 + y[i] - t[i];
     sl += w[i] * r * r;
@@ -177,26 +203,144 @@ __global__ void loss_kernel(const float *__restrict__ y, const float *__restrict
     sw += __shfl_down_sync(0xffffffffu, sw, o);
     sl += __shfl_down_sync(0xffffffffu, sl, o);
   }
-  const int wi = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (l == 0) {
-    sh[0][wi] = sw;
-    sh[1][wi] = sl;
-  }
-  __syncthreads();
   if (threadIdx.x == 0) {
-    double a = 0, b = 0;
-    for (int k = 0; k < nw; ++k) {
-      a += sh[0][k];
-      b += sh[1][k];
-    }
-    sh[0][0] = a;
-    sh[1][0] = b;
+    sums[blockIdx.x] = sw;
+    sums[32 + blockIdx.x] = sl;
   }
-  __syncthreads();
-  const double swt = sh[0][0];
-  if (threadIdx.x == 0 && loss) loss[0] = (float)(sh[1][0] / swt);
-  for (int i = threadIdx.x; i < M; i += blockDim.x)
+}
+// dy = 2 w (1 + y - t) / sum w (dy may be null); loss = sum w (1 + y - t)^2 / sum w
+__global__ void loss_kernel(const float *__restrict__ y, const float *__restrict__ t,
+                            const float *__restrict__ w, int M, const double *__restrict__ sums,
+                            float *__restrict__ dy, float *__restrict__ loss) {
+  double swt = 0, slt = 0;
+  for (int k = 0; k < 32; ++k) {
+    swt += sums[k];
+    slt += sums[32 + k];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0 && loss) loss[0] = (float)(slt / swt);
+  if (!dy) return;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x)
     dy[i] = (float)(2.0 * w[i] * (1.0 + y[i] - t[i]) / swt);
+}
+
+// The sums over the m rows that the parameter gradients need, one launch, each in
+// ascending row order within its chunk of kc rows (ks chunks; the biases in one):
+//   block roles  [0, 24)              db of layer 2, 1, 0: column sums of dZ2, dZ1, dZ0
+//                [24, 24 + 8 ks)      dW3 = dy^T A2 (32 columns, one chunk)
+//                [.., + 8 ks)         dW0 = dZ0^T X (32 rows, one chunk)
+//                last                 db3 = sum dy
+// Rows are staged through shared memory in double-buffered pieces, so that the
+// chain of dependent adds (4 cycles each) is what a block waits for, not memory:
+// one thread per column straight from memory took ~150 us for 2,048 rows.
+struct SumArgs {
+  const float *dz[3], *dy, *a2, *x;
+  float *db[3], *db3, *w3, *w0;  // w3, w0: results (ks = 1) or [ks] partials
+  int m, ks, kc;
+};
+constexpr int SROWS = 128;
+__global__ void __launch_bounds__(320) sums_kernel(const SumArgs g) {
+  __shared__ float buf[2][SROWS][33];
+  __shared__ float aux[2][SROWS][CV_NFEAT];
+  const int role = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float *src;
+  int c0, kbeg = 0, kend = g.m, kind, z = 0;  // kind: 0 column sum, 1 dW3, 2 dW0, 3 sum of dy
+  if (role < 24) {
+    kind = 0;
+    src = g.dz[role >> 3];
+    c0 = (role & 7) * 32;
+  } else if (role < 24 + 16 * g.ks) {
+    const int q = role - 24;
+    kind = q < 8 * g.ks ? 1 : 2;
+    const int u = kind == 1 ? q : q - 8 * g.ks;
+    src = kind == 1 ? g.a2 : g.dz[2];
+    c0 = (u & 7) * 32;
+    z = u >> 3;
+    kbeg = z * g.kc;
+    kend = min(g.m, kbeg + g.kc);
+  } else {
+    kind = 3;
+    src = g.dy;
+    c0 = 0;
+  }
+  // a piece: 128 rows x 32 columns (kind 3: 128 values of dy in column 0)
+  constexpr int PER = (SROWS * 32 + 319) / 320;
+  constexpr int PAX = (SROWS * CV_NFEAT + 319) / 320;
+  float v[PER], ax[PAX];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = tid + p * 320, r = e >> 5, c = e & 31;
+      v[p] = 0.f;
+      if (e < SROWS * 32 && k0 + r < kend) {
+        if (kind != 3) v[p] = src[(long long)(k0 + r) * CV_HIDDEN + c0 + c];
+        else if (c == 0) v[p] = src[k0 + r];
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < PAX; ++p) {
+      const int e = tid + p * 320;
+      ax[p] = 0.f;
+      if (kind == 2 && e < SROWS * CV_NFEAT && k0 + e / CV_NFEAT < kend)
+        ax[p] = g.x[(long long)k0 * CV_NFEAT + e];
+      if (kind == 1 && e < SROWS && k0 + e < kend) ax[p] = g.dy[k0 + e];
+    }
+  };
+  auto store = [&](int bsel) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int e = tid + p * 320;
+      if (e < SROWS * 32) buf[bsel][e >> 5][e & 31] = v[p];
+    }
+#pragma unroll
+    for (int p = 0; p < PAX; ++p) {
+      const int e = tid + p * 320;
+      if (kind == 2 && e < SROWS * CV_NFEAT) aux[bsel][e / CV_NFEAT][e % CV_NFEAT] = ax[p];
+      if (kind == 1 && e < SROWS) aux[bsel][e][0] = ax[p];
+    }
+  };
+  float acc = 0.f;
+  int bsel = 0;
+  load(kbeg);
+  store(0);
+  __syncthreads();
+  for (int k0 = kbeg; k0 < kend; k0 += SROWS) {
+    const bool more = k0 + SROWS < kend;
+    if (more) load(k0 + SROWS);
+    const int cnt = min(SROWS, kend - k0);
+    if (kind == 2) {
+#pragma unroll 16
+      for (int r = 0; r < cnt; ++r) acc = fmaf(buf[bsel][r][lane], aux[bsel][r][warp], acc);
+    } else if (warp == 0 && kind == 1) {
+#pragma unroll 16
+      for (int r = 0; r < cnt; ++r) acc = fmaf(aux[bsel][r][0], buf[bsel][r][lane], acc);
+    } else if (warp == 0) {
+#pragma unroll 16
+      for (int r = 0; r < cnt; ++r) acc += buf[bsel][r][lane];
+    }
+    if (more) {
+      store(bsel ^ 1);
+      __syncthreads();
+      bsel ^= 1;
+    }
+  }
+  if (kind == 0 && warp == 0) g.db[role >> 3][c0 + lane] = acc;
+  if (kind == 1 && warp == 0) g.w3[(long long)z * CV_HIDDEN + c0 + lane] = acc;
+  if (kind == 2) g.w0[((long long)z * CV_HIDDEN + c0 + lane) * CV_NFEAT + warp] = acc;
+  if (kind == 3 && tid == 0) g.db3[0] = acc;
+}
+
+// The chunks' partial sums of dW3 and dW0, added in order.
+__global__ void sums_reduce_kernel(const float *__restrict__ p3, const float *__restrict__ p0, int ks,
+                                   float *__restrict__ w3, float *__restrict__ w0) {
+  const int n3 = CV_HIDDEN, n0 = CV_HIDDEN * CV_NFEAT;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n3 + n0; e += gridDim.x * blockDim.x) {
+    const bool a = e < n3;
+    const float *p = a ? p3 + e : p0 + (e - n3);
+    const int st = a ? n3 : n0;
+    float s = 0.f;
+    for (int k = 0; k < ks; ++k) s += p[(long long)k * st];
+    (a ? w3[e] : w0[e - n3]) = s;
+  }
 }
 
 __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g,
@@ -340,16 +484,21 @@ __global__ void cv_features_kernel(const double *__restrict__ sdd, const double 
   }
 }
 
-// rows of a [total][cols] array taken at (s * stride + k) mod total, k < m
-__global__ void gather_stride_kernel(const float *__restrict__ src, int cols, long long total,
-                                     long long start, long long stride, int m,
-                                     float *__restrict__ dst) {
-  const long long n = (long long)m * cols;
+// Rows (start + k stride) mod total, k < m, of the features, targets and weights.
+__global__ void gather_batch_kernel(const float *__restrict__ X, const float *__restrict__ T,
+                                    const float *__restrict__ W, long long total, long long start,
+                                    long long stride, int m, float *__restrict__ bx,
+                                    float *__restrict__ bt, float *__restrict__ bw) {
+  constexpr int C = CV_NFEAT + 2;
+  const long long n = (long long)m * C;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
-    const long long k = e / cols, c = e - k * cols;
+    const long long k = e / C;
+    const int c = (int)(e - k * C);
     const long long row = (start + k * stride) % total;
-    dst[e] = src[row * cols + c];
+    if (c < CV_NFEAT) bx[k * CV_NFEAT + c] = X[row * CV_NFEAT + c];
+    else if (c == CV_NFEAT) bt[k] = T[row];
+    else bw[k] = W[row];
   }
 }
 
@@ -430,39 +579,19 @@ __global__ void trace_prod_w_kernel(const double *__restrict__ X, const double *
     RS_TRY(cudaGetLastError()); \
   } while (0)
 
-size_t sgemm_work_floats(int M, int N, int K) {
-  const long long tiles = (long long)ceil_div(M, 64) * ceil_div(N, 64);
-  if (tiles >= 152 || K < 2048) return 0;
-  const int ks = (int)std::min<long long>(ceil_div(2 * 152, tiles), K / 512);
-  return ks > 1 ? (size_t)ks * M * N : 0;
+// Chunks of the m rows that dW3 and dW0 are summed in.
+namespace {
+void row_chunks(int m, int *ks, int *kc) {
+  const int k = m < 2048 ? 1 : std::min(76, m / 512);
+  *kc = k > 1 ? (ceil_div(m, k) + 15) / 16 * 16 : m;
+  *ks = ceil_div(m, *kc);
 }
+}  // namespace
 
-cudaError_t sgemm(int M, int N, int K, const float *A, long long lda, int ta, const float *B,
-                  long long ldb, int tb, float *C, long long ldc, float alpha, float beta,
-                  float *work, cudaStream_t s) {
-  if (M <= 0 || N <= 0) return cudaSuccess;
-  const size_t wn = sgemm_work_floats(M, N, K);
-  int ks = 1, kc = K;
-  if (wn && work && beta == 0.f) {
-    ks = (int)(wn / ((size_t)M * N));
-    kc = ((ceil_div(K, ks) + 15) / 16) * 16;
-    ks = ceil_div(K, kc);
-  }
-  dim3 grid(ceil_div(N, 64), ceil_div(M, 64), ks);
-  const int part = ks > 1;
-  float *out = part ? work : C;
-#define RS_SG(a, b) sgemm_kernel<a, b><<<grid, 256, 0, s>>>(M, N, K, kc, A, lda, B, ldb, out, ldc, alpha, beta, part)
-  if (!ta && !tb) RS_SG(0, 0);
-  else if (!ta && tb) RS_SG(0, 1);
-  else if (ta && !tb) RS_SG(1, 0);
-  else RS_SG(1, 1);
-#undef RS_SG
-  RS_L();
-  if (part) {
-    sreduce_kernel<<<grid_cap((long long)M * N, 256), 256, 0, s>>>(work, ks, M, N, C, ldc, alpha);
-    RS_L();
-  }
-  return cudaSuccess;
+size_t cv_sum_floats(int m) {
+  int ks, kc;
+  row_chunks(std::max(m, 1), &ks, &kc);
+  return (size_t)ks * (CV_HIDDEN + CV_HIDDEN * CV_NFEAT) + 128;  // and the loss sums (64 doubles)
 }
 
 // Parameter layout (floats): W0 [256][10], b0, W1 [256][256], b1, W2, b2, W3 [1][256], b3.
@@ -572,105 +701,103 @@ cudaError_t tc_wgrad(const __nv_bfloat16 *At, const __nv_bfloat16 *Bt, long long
   t.K[0] = kc;
   t.A[0] = tco(At, ldt, kc, H);
   t.B[0] = tco(Bt, ldt, kc, H);
-  t.c32 = part;
+  t.c32 = g == 1 ? out : part;
   RS_TRY(tc_gemm(t, s));
+  if (g == 1) return cudaSuccess;
   sreduce_kernel<<<grid_cap((long long)H * H, 256), 256, 0, s>>>(part, g, H, H, out, H, 1.f);
   ++launch_counter();
   return cudaGetLastError();
 }
 
-cudaError_t to_bf16(const float *src, long long n, __nv_bfloat16 *dst, cudaStream_t s) {
-  to_bf16_kernel<<<grid_cap(n, 256), 256, 0, s>>>(src, n, dst);
-  ++launch_counter();
-  return cudaGetLastError();
-}
-
-// dst [cols][ldd] = bf16 src[rows][cols]^T (zero beyond rows)
-cudaError_t transpose_bf16(const float *src, int rows, int cols, long long lds,
-                           __nv_bfloat16 *dst, long long ldd, cudaStream_t s) {
-  dim3 grid((unsigned)((ldd + 31) / 32), (unsigned)ceil_div(cols, 32));
-  transpose_bf16_kernel<<<grid, 256, 0, s>>>(src, rows, cols, lds, dst, ldd);
-  ++launch_counter();
-  return cudaGetLastError();
-}
 }  // namespace
 
 cudaError_t cv_forward(const float *params, const float *X, int m, float *act, float *work,
                        cudaStream_t s) {
   const int H = CV_HIDDEN;
-  float *Z0 = act, *A0 = Z0 + (long long)m * H, *Z1 = A0 + (long long)m * H,
-        *A1 = Z1 + (long long)m * H, *Z2 = A1 + (long long)m * H, *A2 = Z2 + (long long)m * H,
-        *y = A2 + (long long)m * H;
+  const long long mh = (long long)m * H;
+  float *Z0 = act, *A0 = Z0 + mh, *Z1 = A0 + mh, *A1 = Z1 + mh, *Z2 = A1 + mh, *A2 = Z2 + mh,
+        *y = A2 + mh;
   Bf16Bufs b = bf16_bufs(params, act, work, m);
-  // bf16 copies of the hidden weights W1, W2 (the B operands: rows = outputs)
-  RS_TRY(to_bf16(params + O_W1, (long long)H * H, b.w[0], s));
-  RS_TRY(to_bf16(params + O_W2, (long long)H * H, b.w[1], s));
+  // bf16 copies of the hidden weights W1, W2 (the B operands: rows = outputs) and
+  // of their transposes (the backward pass: rows = inputs)
+  weights_kernel<<<dim3(H / 32, H / 32, 2), 256, 0, s>>>(params + O_W1, params + O_W2, b.w[0]);
+  RS_L();
   // layer 0 (10 inputs): fp32
-  RS_TRY(sgemm(m, H, CV_NFEAT, X, CV_NFEAT, 0, params + O_W0, CV_NFEAT, 1, Z0, H, 1.f, 0.f,
-               b.work, s));
-  bias_silu_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(Z0, params + O_B0, m, H, A0);
+  layer0_kernel<<<std::min(m, 152 * 8), H, 0, s>>>(X, params + O_W0, params + O_B0, m, Z0, A0, b.h0);
   RS_L();
   // layers 1, 2: tensor cores on bf16 activations
-  RS_TRY(to_bf16(A0, (long long)m * H, b.h0, s));
   RS_TRY(tc_mm(b.h0, H, b.w[0], H, m, H, H, Z1, s));
-  bias_silu_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(Z1, params + O_B1, m, H, A1);
+  bias_silu_kernel<<<grid_cap(mh / 4, 256), 256, 0, s>>>(Z1, params + O_B1, mh, A1, b.h1);
   RS_L();
-  RS_TRY(to_bf16(A1, (long long)m * H, b.h1, s));
   RS_TRY(tc_mm(b.h1, H, b.w[1], H, m, H, H, Z2, s));
-  bias_silu_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(Z2, params + O_B2, m, H, A2);
-  RS_L();
-  // output layer (1 output): fp32
-  RS_TRY(sgemm(m, 1, H, A2, H, 0, params + O_W3, H, 1, y, 1, 1.f, 0.f, b.work, s));
-  bias_silu_kernel<<<grid_cap(m, 256), 256, 0, s>>>(y, params + O_B3, m, 1, nullptr);
+  // the last bias and the output layer (1 output): fp32
+  output_kernel<<<ceil_div(m, 32), 256, 0, s>>>(Z2, params + O_B2, params + O_W3, params + O_B3, m,
+                                                A2, y);
   RS_L();
   return cudaSuccess;
+}
+
+namespace {
+// The loss after cv_forward, and with dy its derivative.
+cudaError_t loss_pass(const float *y, int m, const float *target, const float *weight, double *sums,
+                      float *dy, float *loss, cudaStream_t s) {
+  loss_sums_kernel<<<32, 32, 0, s>>>(y, target, weight, m, sums);
+  RS_L();
+  loss_kernel<<<dy ? std::min(152, ceil_div(m, 32)) : 1, 32, 0, s>>>(y, target, weight, m, sums, dy,
+                                                                     loss);
+  RS_L();
+  return cudaSuccess;
+}
+}  // namespace
+
+cudaError_t cv_loss(int m, const float *target, const float *weight, float *act, float *loss,
+                    float *work, cudaStream_t s) {
+  Bf16Bufs b = bf16_bufs(nullptr, act, work, m);
+  return loss_pass(act + 6LL * m * CV_HIDDEN, m, target, weight, reinterpret_cast<double *>(b.work),
+                   nullptr, loss, s);
 }
 
 cudaError_t cv_backward(const float *params, const float *X, int m, const float *target,
                         const float *weight, float *act, float *grad, float *loss, float *work,
                         cudaStream_t s) {
   const int H = CV_HIDDEN;
-  float *Z0 = act, *A0 = Z0 + (long long)m * H, *Z1 = A0 + (long long)m * H,
-        *A1 = Z1 + (long long)m * H, *Z2 = A1 + (long long)m * H, *A2 = Z2 + (long long)m * H,
-        *y = A2 + (long long)m * H, *dy = y + m;
+  const long long mh = (long long)m * H;
+  float *Z0 = act, *A0 = Z0 + mh, *Z1 = A0 + mh, *A1 = Z1 + mh, *Z2 = A1 + mh, *A2 = Z2 + mh,
+        *y = A2 + mh, *dy = y + m;
   Bf16Bufs b = bf16_bufs(params, act, work, m);
-  // bf16 W1^T, W2^T (the B operands of dA = dZ W: rows = inputs)
-  RS_TRY(transpose_bf16(params + O_W1, H, H, H, b.wt[0], H, s));
-  RS_TRY(transpose_bf16(params + O_W2, H, H, H, b.wt[1], H, s));
-  loss_kernel<<<1, 1024, 0, s>>>(y, target, weight, m, dy, loss);
+  double *sums = reinterpret_cast<double *>(b.work);
+  RS_TRY(loss_pass(y, m, target, weight, sums, dy, loss, s));
+  const dim3 gt((unsigned)((b.ldt + 31) / 32), H / 32), gm((unsigned)ceil_div(m, 32), H / 32);
+  // layer 3: dA2 = dy W3, dZ2 = dA2 silu'(Z2) (in Z2's place)
+  back_kernel<<<gt, 256, 0, s>>>(nullptr, dy, params + O_W3, Z2, A1, m, b.h1, b.t0, b.t1, b.ldt);
   RS_L();
-  // layer 3: dW3 = dy^T A2, db3 = sum dy, dA2 = dy W3 (fp32)
-  RS_TRY(sgemm(1, H, m, dy, 1, 1, A2, H, 0, grad + O_W3, H, 1.f, 0.f, b.work, s));
-  colsum_kernel<<<1, 32, 0, s>>>(dy, m, 1, grad + O_B3);
-  RS_L();
-  RS_TRY(sgemm(m, H, 1, dy, 1, 0, params + O_W3, H, 0, A2, H, 1.f, 0.f, b.work, s));
-  silu_back_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(A2, Z2, (long long)m * H, Z2);
-  RS_L();  // Z2 now holds dZ2
-  // layer 2: dW2 = dZ2^T A1, db2; dA1 = dZ2 W2; dZ1 = dA1 silu'(Z1)
-  RS_TRY(transpose_bf16(Z2, m, H, H, b.t0, b.ldt, s));
-  RS_TRY(transpose_bf16(A1, m, H, H, b.t1, b.ldt, s));
+  // layer 2: dW2 = dZ2^T A1; dA1 = dZ2 W2 (in A1's place); dZ1 = dA1 silu'(Z1)
   RS_TRY(tc_wgrad(b.t0, b.t1, b.ldt, m, b.part, grad + O_W2, s));
-  colsum_kernel<<<ceil_div(H, 128), 128, 0, s>>>(Z2, m, H, grad + O_B2);
-  RS_L();
-  RS_TRY(to_bf16(Z2, (long long)m * H, b.h1, s));
   RS_TRY(tc_mm(b.h1, H, b.wt[1], H, m, H, H, A1, s));
-  silu_back_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(A1, Z1, (long long)m * H, Z1);
-  RS_L();  // Z1 now holds dZ1
-  // layer 1: dW1 = dZ1^T A0, db1; dA0 = dZ1 W1; dZ0 = dA0 silu'(Z0)
-  RS_TRY(transpose_bf16(Z1, m, H, H, b.t0, b.ldt, s));
-  RS_TRY(transpose_bf16(A0, m, H, H, b.t1, b.ldt, s));
+  back_kernel<<<gt, 256, 0, s>>>(A1, nullptr, nullptr, Z1, A0, m, b.h0, b.t0, b.t1, b.ldt);
+  RS_L();
+  // layer 1: dW1 = dZ1^T A0; dA0 = dZ1 W1; dZ0 = dA0 silu'(Z0)
   RS_TRY(tc_wgrad(b.t0, b.t1, b.ldt, m, b.part, grad + O_W1, s));
-  colsum_kernel<<<ceil_div(H, 128), 128, 0, s>>>(Z1, m, H, grad + O_B1);
-  RS_L();
-  RS_TRY(to_bf16(Z1, (long long)m * H, b.h0, s));
   RS_TRY(tc_mm(b.h0, H, b.wt[0], H, m, H, H, A0, s));
-  silu_back_kernel<<<grid_cap((long long)m * H, 256), 256, 0, s>>>(A0, Z0, (long long)m * H, Z0);
-  RS_L();  // Z0 now holds dZ0
-  // layer 0 (10 inputs): dW0 = dZ0^T X, db0 (fp32)
-  RS_TRY(sgemm(H, CV_NFEAT, m, Z0, H, 1, X, CV_NFEAT, 0, grad + O_W0, CV_NFEAT, 1.f, 0.f, b.work,
-               s));
-  colsum_kernel<<<ceil_div(H, 128), 128, 0, s>>>(Z0, m, H, grad + O_B0);
+  back_kernel<<<gm, 256, 0, s>>>(A0, nullptr, nullptr, Z0, nullptr, m, nullptr, nullptr, nullptr, 0);
   RS_L();
+  // the sums over the rows: db2, db1, db0, dW3 = dy^T A2, db3, dW0 = dZ0^T X (fp32)
+  SumArgs g;
+  row_chunks(m, &g.ks, &g.kc);
+  float *p3 = b.work + 128, *p0 = p3 + (long long)g.ks * H;
+  g.dz[0] = Z2; g.dz[1] = Z1; g.dz[2] = Z0;
+  g.dy = dy; g.a2 = A2; g.x = X;
+  g.db[0] = grad + O_B2; g.db[1] = grad + O_B1; g.db[2] = grad + O_B0;
+  g.db3 = grad + O_B3;
+  g.w3 = g.ks > 1 ? p3 : grad + O_W3;
+  g.w0 = g.ks > 1 ? p0 : grad + O_W0;
+  g.m = m;
+  sums_kernel<<<24 + 16 * g.ks + 1, 320, 0, s>>>(g);
+  RS_L();
+  if (g.ks > 1) {
+    sums_reduce_kernel<<<11, 256, 0, s>>>(p3, p0, g.ks, grad + O_W3, grad + O_W0);
+    RS_L();
+  }
   return cudaSuccess;
 }
 
@@ -714,10 +841,11 @@ cudaError_t cv_features(const double *sdd, const double *G, const double *Gb, co
   return cudaSuccess;
 }
 
-cudaError_t cv_gather(const float *src, int cols, long long total, long long start,
-                      long long stride, int m, float *dst, cudaStream_t s) {
-  gather_stride_kernel<<<grid_cap((long long)m * cols, 256), 256, 0, s>>>(src, cols, total, start,
-                                                                          stride, m, dst);
+cudaError_t cv_gather(const float *X, const float *T, const float *W, long long total,
+                      long long start, long long stride, int m, float *bx, float *bt, float *bw,
+                      cudaStream_t s) {
+  gather_batch_kernel<<<grid_cap((long long)m * (CV_NFEAT + 2), 256), 256, 0, s>>>(
+      X, T, W, total, start, stride, m, bx, bt, bw);
   RS_L();
   return cudaSuccess;
 }

@@ -12,22 +12,19 @@ constexpr long long CV_NPARAM =
     (long long)CV_HIDDEN * CV_NFEAT + CV_HIDDEN + 2LL * (CV_HIDDEN * CV_HIDDEN + CV_HIDDEN) +
     CV_HIDDEN + 1;
 
-// fp32 C = alpha op(A) op(B) + beta C; work (may be null) of sgemm_work_floats
-// floats enables a split over K with a fixed-order reduction.
-size_t sgemm_work_floats(int M, int N, int K);
-cudaError_t sgemm(int M, int N, int K, const float *A, long long lda, int ta, const float *B,
-                  long long ldb, int tb, float *C, long long ldc, float alpha, float beta,
-                  float *work, cudaStream_t s);
-
 // Activations of m rows: [Z0 A0 Z1 A1 Z2 A2] (m x 256 each), y (m), dy (m),
 // then the bf16 operands of the tensor-core hidden layers.
 size_t cv_act_floats(int m);
 // Floats of `work` that the tensor-core hidden layers use (bf16 weights and
-// weight-gradient partials); the fp32 products' split-K scratch follows them.
+// weight-gradient partials); the row sums' partials (cv_sum_floats(m)) follow them.
 size_t cv_tc_work_floats();
+size_t cv_sum_floats(int m);
 // Forward: y = MLP(X) - 1 in act (see cv_act_floats), X [m][10].
 cudaError_t cv_forward(const float *params, const float *X, int m, float *act, float *work,
                        cudaStream_t s);
+// After cv_forward: loss = sum w (1 + y - t)^2 / sum w alone.
+cudaError_t cv_loss(int m, const float *target, const float *weight, float *act, float *loss,
+                    float *work, cudaStream_t s);
 // After cv_forward: loss = sum w (1 + y - t)^2 / sum w and its gradient.
 cudaError_t cv_backward(const float *params, const float *X, int m, const float *target,
                         const float *weight, float *act, float *grad, float *loss, float *work,
@@ -43,9 +40,10 @@ cudaError_t cv_targets(const double *stats, int n, int nt, int ns, float *target
 cudaError_t cv_features(const double *sdd, const double *G, const double *Gb, const double *tau,
                         double beta, const double *KP, const int *rowptr, int naux, int n, int nt,
                         double *scratch, float *X, cudaStream_t s);
-// dst[k] = src[(start + k stride) mod total] (rows of `cols` floats), k < m.
-cudaError_t cv_gather(const float *src, int cols, long long total, long long start,
-                      long long stride, int m, float *dst, cudaStream_t s);
+// Rows (start + k stride) mod total, k < m, of X [total][10], T and W [total].
+cudaError_t cv_gather(const float *X, const float *T, const float *W, long long total,
+                      long long start, long long stride, int m, float *bx, float *bt, float *bw,
+                      cudaStream_t s);
 // sig = (init ? c o base : sig) + sum_x (BC[x] + c o BC[nh+x]) / ns.
 cudaError_t cv_accumulate(const double *BC, int nh, int n, double ns, const double *base,
                           const double *c, int init, double *sig, cudaStream_t s);

@@ -308,7 +308,11 @@ cudaError_t tc_gemm(const TcGemm &g, cudaStream_t s) {
   std::memset(&p, 0, sizeof(p));
   // N tile: <= 256, a multiple of 16, with the least padding
   const int ntiles = (g.N + 255) / 256;
-  const int BN = std::min(256, ((ceil_div(g.N, ntiles) + 15) / 16) * 16);
+  int BN = std::min(256, ((ceil_div(g.N, ntiles) + 15) / 16) * 16);
+  // few tiles (the network's layers: 16 of 128 x 256 for 2,048 rows): narrower
+  // ones fill more SMs; each output's sum over K is the same
+  const long long mtg = (long long)ceil_div(g.M, TBM) * ceil_div(g.batch, g.bpc);
+  while (BN % 32 == 0 && BN >= 64 && mtg * ceil_div(g.N, BN) * 2 <= 152) BN /= 2;
   long long iters = 0;
   for (int s2 = 0; s2 < g.nseg; ++s2) {
     if (g.K[s2] <= 0) return cudaErrorInvalidValue;
