@@ -441,7 +441,7 @@ RSSRI_API int rssri_cv_loss_grad(rssri_handle *h, const float *x, const float *t
  *   e_corr device, [1]            output, written on `stream`
  *   stream cudaStream_t as void* (NULL = legacy default stream)
  * Its scratch is a static device array of RSSRI_STATIC_MAX_TAU doubles
- * (32 KiB), present on every GPU that loads the library until the process
+ * (32 KiB) and a counter, present on every GPU that loads the library until the process
  * exits.  The first call on each device looks up that array's device address
  * (cudaGetSymbolAddress) with the device current; make that first call before
  * any stream capture.  All calls share the array: calls whose work overlaps on

@@ -15,6 +15,7 @@
 #include "oz_gemm.cuh"
 #include "tc_gemm.cuh"
 #include "tc_group.cuh"
+#include "trace.cuh"
 
 using namespace rssri;
 
@@ -2151,8 +2152,8 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
   // ---- buffers
   RS_CK(ensure(h->sig_raw, (size_t)nt * nn * sizeof(double)));
   RS_CK(ensure(h->sig_out, (size_t)nt * nn * sizeof(double)));
-  RS_CK(ensure(h->trdd, nt * sizeof(double)));
-  RS_CK(ensure(h->tr, nt * sizeof(double)));
+  RS_CK(ensure(h->trdd, std::max(nt, TRACE_SLOTS) * sizeof(double)));
+  RS_CK(ensure(h->tr, std::max(nt, TRACE_SLOTS) * sizeof(double)));
   RS_CK(ensure(h->res, 8 * sizeof(double)));
   RS_CK(ensure(h->theta, (size_t)2 * ns * na * sizeof(double)));
   RS_CK(ensure(h->Ut, (size_t)2 * ns * na * sizeof(double)));
@@ -2449,7 +2450,8 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
     RS_CK(trace_prod(sdd, Gb, n, nt, h->trdd.as<double>(), s));
   }
   { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(trace_prod(h->sig_out.as<double>(), Gb, n, nt, h->tr.as<double>(), s)); }
-  { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(energy_finalize(h->tau_w, h->trdd.as<double>(), h->tr.as<double>(), nt, ne,
+  { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(energy_finalize(h->tau_w, h->trdd.as<double>(), use_cv ? 1 : trace_parts(n, nt),
+                        h->tr.as<double>(), trace_parts(n, nt), nt, ne,
                         h->e_st.as<double>(), ns, h->e_pair.as<double>(), h->res.as<double>(), s)); }
   const cudaMemcpyKind dk = h->ptr_kind == RSSRI_PTR_HOST ? cudaMemcpyDeviceToHost
                                                           : cudaMemcpyDeviceToDevice;

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "kernels.cuh"
+#include "trace.cuh"
 
 namespace rssri {
 namespace {
@@ -607,31 +608,22 @@ __global__ void lit_add_kernel(const double *__restrict__ Z, int cnt, int n,
 }
 
 // ------------------------------------------------------------------ S9 ----
-__global__ void trace_prod_kernel(const double *__restrict__ X, const double *__restrict__ Y, int n,
-                                  double *__restrict__ out) {
-  const int ti = blockIdx.x;
+__global__ void __launch_bounds__(256) trace_prod_kernel(const double *__restrict__ X,
+                                                         const double *__restrict__ Y, int n,
+                                                         int parts, double *__restrict__ out) {
   const long long nn = (long long)n * n;
-  const double *x = X + ti * nn, *y = Y + ti * nn;
-  double s = 0.0;
-  for (long long e = threadIdx.x; e < nn; e += blockDim.x) {
-    const long long i = e / n, j = e - i * n;
-    s += x[e] * y[j * n + i];
-  }
-  s = block_sum(s);
-  if (threadIdx.x == 0) out[ti] = s;
+  const int t = blockIdx.x / parts, p = blockIdx.x - t * parts;
+  const double s = trace_part(X + t * nn, Y + t * nn, n, p, parts);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
-__global__ void energy_finalize_kernel(const double *__restrict__ w, const double *__restrict__ trdd,
-                                       const double *__restrict__ tr, int ntau, double ne,
-                                       const double *__restrict__ e_st, int ns,
-                                       double *__restrict__ e_pair, double *__restrict__ res) {
+__global__ void __launch_bounds__(256) energy_finalize_kernel(
+    const double *__restrict__ w, const double *__restrict__ trdd, int pdd,
+    const double *__restrict__ tr, int ptr, int ntau, double ne, const double *__restrict__ e_st,
+    int ns, double *__restrict__ e_pair, double *__restrict__ res) {
   __shared__ double sh_edd, sh_e;
+  const double a = trace_weighted(w, trdd, pdd, ntau), b = trace_weighted(w, tr, ptr, ntau);
   if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < ntau; ++k) {
-      a += w[k] * trdd[k];
-      b += w[k] * tr[k];
-    }
     sh_edd = -a / ne;
     sh_e = -b / ne;
   }
@@ -925,15 +917,17 @@ cudaError_t lit_add(const double *Z, int cnt, int n, const double *Gb, double w,
 
 cudaError_t trace_prod(const double *X, const double *Y, int n, int ntau, double *out,
                        cudaStream_t s) {
-  trace_prod_kernel<<<ntau, 256, 0, s>>>(X, Y, n, out);
+  const int parts = trace_parts(n, ntau);
+  trace_prod_kernel<<<(unsigned)parts * ntau, 256, 0, s>>>(X, Y, n, parts, out);
   RS_LAUNCHED();
   return cudaSuccess;
 }
 
-cudaError_t energy_finalize(const double *tau_w, const double *trdd, const double *tr, int ntau,
-                            double ne, const double *e_st, int ns, double *e_pair, double *res,
-                            cudaStream_t s) {
-  energy_finalize_kernel<<<1, 256, 0, s>>>(tau_w, trdd, tr, ntau, ne, e_st, ns, e_pair, res);
+cudaError_t energy_finalize(const double *tau_w, const double *trdd, int pdd, const double *tr,
+                            int ptr, int ntau, double ne, const double *e_st, int ns,
+                            double *e_pair, double *res, cudaStream_t s) {
+  energy_finalize_kernel<<<1, 256, 0, s>>>(tau_w, trdd, pdd, tr, ptr, ntau, ne, e_st, ns, e_pair,
+                                           res);
   RS_LAUNCHED();
   return cudaSuccess;
 }

@@ -95,14 +95,15 @@ cudaError_t lit_add(const double *Z, int cnt, int n, const double *Gb, double w,
                     double *F0, double *e_st, cudaStream_t s);
 
 // ---------------------------------------------------------------- S9 ------
-// out[t] = sum_ij X[t][i][j] Y[t][j][i]
+// out[t][p] = part p of sum_ij X[t][i][j] Y[t][j][i], trace_parts(n, ntau) parts (trace.cuh)
 cudaError_t trace_prod(const double *X, const double *Y, int n, int ntau, double *out,
                        cudaStream_t s);
+// trdd, tr: pdd and ptr partial traces per tau point; with their sums,
 // e_dd = -sum_t w_t trdd[t] / ne, e = -sum_t w_t tr[t] / ne, e_pair[x] = e_dd + e_st[x],
 // res = {e_dd, e, mean(e_pair), std(e_pair)/sqrt(ns)}.
-cudaError_t energy_finalize(const double *tau_w, const double *trdd, const double *tr, int ntau,
-                            double ne, const double *e_st, int ns, double *e_pair, double *res,
-                            cudaStream_t s);
+cudaError_t energy_finalize(const double *tau_w, const double *trdd, int pdd, const double *tr,
+                            int ptr, int ntau, double ne, const double *e_st, int ns,
+                            double *e_pair, double *res, cudaStream_t s);
 
 // --------------------------------------------------------------- S10 ------
 cudaError_t symmetrize(const double *in, int n, int ntau, double *out, cudaStream_t s);

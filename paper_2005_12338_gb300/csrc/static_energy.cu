@@ -6,17 +6,21 @@
 // that hand every byte of device memory to their own pool allocator and forbid
 // libraries from allocating behind their back, and real-time loops that must
 // not hit the allocator's synchronisation.  This entry point creates no handle
-// and allocates nothing: its only scratch (one partial trace per tau point) is
-// a file-scope __device__ array of fixed size, loaded with the library and
-// held by every GPU that loads it until the process exits.
+// and allocates nothing: its only scratch (partial traces and a counter of
+// finished blocks) is file-scope __device__ memory of fixed size, loaded with
+// the library and held by every GPU that loads it until the process exits.
+//
+// One launch: the block that finishes last adds the partial traces (a second
+// launch for that cost as much as the traces of small problems).
 #include <mutex>
 
-#include "kernels.cuh"
+#include "trace.cuh"
 
 namespace {
 
-// One fp64 slot per tau point; RSSRI_STATIC_MAX_TAU slots (32 KiB).
-static __device__ __align__(256) double g_energy_scratch[RSSRI_STATIC_MAX_TAU];
+// RSSRI_STATIC_MAX_TAU partial traces (32 KiB), then the counter, zero between calls.
+static __device__ __align__(256) double g_energy_scratch[RSSRI_STATIC_MAX_TAU + 1];
+static_assert(RSSRI_STATIC_MAX_TAU >= rssri::TRACE_SLOTS, "slots of trace_parts");
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
@@ -41,15 +45,32 @@ cudaError_t scratch_on_current_device(double **out) {
   return cudaSuccess;
 }
 
+// Partial traces by block (p, t); the last block to finish forms
 // e_corr = -(sum_t w_t tr[t]) / ne, summed in tau order (the same order as
-// the energy of rssri_sigma).
-__global__ void static_energy_finalize_kernel(const double *__restrict__ tau_w,
-                                              const double *__restrict__ tr, int ntau, double ne,
-                                              double *__restrict__ e_corr) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  double b = 0.0;
-  for (int k = 0; k < ntau; ++k) b += tau_w[k] * tr[k];
-  e_corr[0] = -b / ne;
+// the energy of rssri_sigma), and clears the counter.
+__global__ void __launch_bounds__(256) static_energy_kernel(const double *__restrict__ sigma,
+                                                            const double *__restrict__ gb,
+                                                            const double *__restrict__ tau_w, int n,
+                                                            double ne, double *scratch,
+                                                            double *__restrict__ e_corr) {
+  __shared__ bool last;
+  const long long nn = (long long)n * n;
+  const int t = blockIdx.y, parts = gridDim.x, nt = gridDim.y;
+  unsigned *count = reinterpret_cast<unsigned *>(scratch + RSSRI_STATIC_MAX_TAU);
+  const double s = rssri::trace_part(sigma + t * nn, gb + t * nn, n, blockIdx.x, parts);
+  if (threadIdx.x == 0) {
+    scratch[(long long)t * parts + blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(count, 1u) == (unsigned)(parts * nt) - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const double b = rssri::trace_weighted(tau_w, scratch, parts, nt);
+  if (threadIdx.x == 0) {
+    e_corr[0] = -b / ne;
+    *count = 0u;
+  }
 }
 
 }  // namespace
@@ -63,10 +84,8 @@ extern "C" int rssri_energy_static(const double *sigma, const double *gb, const 
   cudaError_t e = scratch_on_current_device(&scratch);
   if (e != cudaSuccess) return RSSRI_ERR_CUDA;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // every slot read below is written first by this call, so nothing needs clearing
-  e = rssri::trace_prod(sigma, gb, n, n_tau, scratch, s);
-  if (e != cudaSuccess) return RSSRI_ERR_CUDA;
-  static_energy_finalize_kernel<<<1, 32, 0, s>>>(tau_w, scratch, n_tau, 2.0 * n_occ, e_corr);
+  static_energy_kernel<<<dim3(rssri::trace_parts(n, n_tau), n_tau), 256, 0, s>>>(
+      sigma, gb, tau_w, n, 2.0 * n_occ, scratch, e_corr);
   e = cudaGetLastError();
   return e == cudaSuccess ? RSSRI_OK : RSSRI_ERR_CUDA;
 }
