@@ -13,6 +13,7 @@
 #include "kernels.cuh"
 #include "mo.cuh"
 #include "oz_gemm.cuh"
+#include "tc_dual.cuh"
 #include "tc_gemm.cuh"
 #include "tc_group.cuh"
 #include "trace.cuh"
@@ -150,7 +151,7 @@ struct rssri_handle {
   bool mo_tab_ready = false;  // moTab, moChl made for this setup
   bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
   // bf16 chain buffers
-  DevBuf hxsl, hy3, hg, hgb, hP, hdc32, hcl32, hdcl16, hxy32, ha6, hct, hdct, hpart, hfold;
+  DevBuf hxsl, hy3, hg, hgb, hP, hdcl16, hxy32, ha6, hct, hdct, hpart, hfold;
   DevBuf hclt, hfl;  // learned control variate on the tensor-core chain: (C^L)^T, F^L per pair
   // the bf16 chain captured as a CUDA graph, valid for the key it was built for
   cudaGraphExec_t chain_graph = nullptr;
@@ -507,8 +508,7 @@ void rssri_destroy(rssri_handle *h) {
                     &h->G, &h->Gb, &h->cs, &h->XG, &h->Cc, &h->Bm, &h->BC, &h->tarr, &h->sarr,
                     &h->e_st, &h->sig_raw, &h->sdd, &h->PG, &h->At, &h->T, &h->AP, &h->Gam, &h->L,
                     &h->trdd, &h->tr, &h->res, &h->sig_out, &h->e_pair, &h->gwork, &h->outbuf,
-                    &h->hxsl, &h->hy3, &h->hg, &h->hgb, &h->hP, &h->hdc32, &h->hcl32,
-                    &h->hdcl16, &h->hxy32, &h->ha6, &h->hct, &h->hdct, &h->hpart, &h->hfold, &h->hclt, &h->hfl, &h->Dhl,
+                    &h->hxsl, &h->hy3, &h->hg, &h->hgb, &h->hP, &h->hdcl16, &h->hxy32, &h->ha6, &h->hct, &h->hdct, &h->hpart, &h->hfold, &h->hclt, &h->hfl, &h->Dhl,
                     &h->Ahl, &h->KPhl, &h->PGhl, &h->APhl, &h->Gamhl, &h->GGhl, &h->litMP, &h->litT, &h->litMhl, &h->eri_hl, &h->ut_hl, &h->nsA2, &h->nsB2, &h->elHl, &h->facHl, &h->xgHl, &h->cHl, &h->bHl, &h->cv_params, &h->cv_m, &h->cv_v, &h->cv_grad, &h->cv_ptmp,
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
                     &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
@@ -1621,7 +1621,7 @@ struct ChainBufs {
   int tc;     // tau points per chunk
   // per chunk slot j < tc (buffers hold tc slots):
   void *xsl, *y3, *gh, *gbh, *P, *dcl, *a6, *ct, *dct;
-  float *dc32, *cl32, *xy32, *part;
+  float *xy32, *part;
   double *fold;
   int bpc, groups;
 };
@@ -1648,29 +1648,14 @@ void chain_stage_probs(rssri_handle *h, const ChainBufs &b, int ns, int t0, int 
     g.A[0] = op(b.xsl, 0, 2 * ns * n); g.B[0] = op(at(b.gh, (long long)t0 * mat), mat, n);
     g.cop = b.P; g.ldcop = ldp;
     out.push_back(g);
-  } else if (stage == 1) {  // dC = P_S R' + P_L R'^S and C^L = P_L R'^L per tau
-    for (int j = 0; j < c; ++j) {
-      void *Pj = at(b.P, (long long)j * 2 * ns * mat);
-      TcProb g;
-      g.M = n; g.N = n; g.batch = ns; g.nseg = 2; g.K[0] = g.K[1] = n;
-      g.A[0] = op(Pj, mat, n); g.B[0] = op(b.y3, mat, n);
-      g.A[1] = op(at(Pj, ns * mat), mat, n); g.B[1] = op(at(b.y3, ns * mat), mat, n);
-      g.c32 = b.dc32 + (long long)j * ns * nn;
-      g.cop = at(b.dcl, (long long)j * 2 * ns * mat); g.ldcop = ldp;
-      out.push_back(g);
-      TcProb l;
-      l.M = n; l.N = n; l.batch = ns; l.K[0] = n;
-      l.A[0] = op(at(Pj, ns * mat), mat, n); l.B[0] = op(at(b.y3, 2 * ns * mat), mat, n);
-      l.c32 = b.cl32 + (long long)j * ns * nn;
-      l.cop = at(b.dcl, ((long long)j * 2 * ns + ns) * mat); l.ldcop = ldp;
-      out.push_back(l);
-    }
   } else if (stage == 2) {  // [X; Y] = [dC; C^L] Gb for every tau: batch over tau
     TcProb g;
     g.M = 2 * ns * n; g.N = n; g.K[0] = n; g.batch = c;
     g.A[0] = op(b.dcl, 2 * ns * mat, 2 * ns * n);
     g.B[0] = op(at(b.gbh, (long long)t0 * mat), mat, n);
     g.c32 = b.xy32;
+    // -X and -Y as the next product's left operands (fold_tc sets their diagonals)
+    g.cop = b.a6; g.ldcop = ldp; g.copneg = 1;
     out.push_back(g);
   } else if (stage == 3) {  // sum over pairs of (2 dt I - X) C + (2 t^L I - Y) dC per tau
     for (int j = 0; j < c; ++j) {
@@ -1708,22 +1693,21 @@ cudaError_t issue_chain_tc(rssri_handle *h, cudaStream_t s, int ns, const double
   std::vector<TcProb> probs;
   for (int t0 = 0; t0 < nt; t0 += b.tc) {
     const int c = std::min(b.tc, nt - t0);
-    for (int stage = 0; stage < 3; ++stage) {
-      chain_stage_probs(h, b, ns, t0, c, stage, probs);
-      RS_TRY(tc_group(b.kind, probs.data(), (int)probs.size(), err, s, b.wait_polls));
-    }
-    for (int j = 0; j < c; ++j)
-      RS_TRY(fold_tc(b.kind, b.xy32 + (long long)j * 2 * ns * nn, b.dc32 + (long long)j * ns * nn,
-                     b.cl32 + (long long)j * ns * nn, ns, n, ldp, h->h_tau_w[t0 + j], ne,
-                     at(b.a6, (long long)j * 2 * ns * mat), at(b.ct, (long long)j * ns * mat),
-                     at(b.dct, (long long)j * ns * mat),
-                     b.cvc ? at(b.clt, (long long)j * ns * mat) : nullptr, h->e_st.as<double>(),
-                     b.fold + (long long)j * ns * ceil_div(n, 32) * 4, s));
+    chain_stage_probs(h, b, ns, t0, c, 0, probs);
+    RS_TRY(tc_group(b.kind, probs.data(), (int)probs.size(), err, s, b.wait_polls));
+    TcDual d;
+    d.n = n; d.ns = ns; d.c = c; d.ld = ldp;
+    d.P = b.P; d.y3 = b.y3;
+    d.dcl = b.dcl; d.ct = b.ct; d.dct = b.dct; d.clt = b.cvc ? b.clt : nullptr;
+    d.err = err; d.wait_polls = b.wait_polls;
+    RS_TRY(tc_dual(b.kind, d, s));
+    chain_stage_probs(h, b, ns, t0, c, 2, probs);
+    RS_TRY(tc_group(b.kind, probs.data(), (int)probs.size(), err, s, b.wait_polls));
+    RS_TRY(fold_tc(b.kind, b.xy32, ns, n, ldp, c, h->h_tau_w.data() + t0, ne, b.a6,
+                   h->e_st.as<double>(), b.fold, s));
     chain_stage_probs(h, b, ns, t0, c, 3, probs);
     RS_TRY(tc_group(b.kind, probs.data(), (int)probs.size(), err, s, b.wait_polls));
-    for (int j = 0; j < c; ++j)
-      RS_TRY(reduce_tc(b.part + (long long)j * b.groups * nn, b.groups, n, sdd + (t0 + j) * nn,
-                       (double)ns, sig + (t0 + j) * nn, s));
+    RS_TRY(reduce_tc(b.part, b.groups, n, c, sdd + t0 * nn, (double)ns, sig + t0 * nn, s));
     if (b.cvc) {
       chain_stage_probs(h, b, ns, t0, c, 4, probs);
       RS_TRY(tc_group(b.kind, probs.data(), (int)probs.size(), err, s, b.wait_polls));
@@ -1753,12 +1737,11 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
   b.bpc = std::max(1, ceil_div(ns, 152));
   b.groups = ceil_div(ns, b.bpc);
   // tau points per chunk: as many as fit a scratch budget of 8 GB (at least 1)
-  const size_t per_tau = 2 * ns * mat * b16 /*P*/ + 2 * ns * nn * 4 /*dC, C^L fp32*/ +
-                         2 * ns * mat * b16 /*dcl*/ + 2 * ns * nn * 4 /*X, Y*/ +
+  const size_t per_tau = 2 * ns * mat * b16 /*P*/ + 2 * ns * mat * b16 /*dcl*/ + 2 * ns * nn * 4 /*X, Y*/ +
                          2 * ns * mat * b16 /*a6*/ + 2 * ns * mat * b16 /*ct, dct*/ +
                          (size_t)b.groups * nn * 4 /*part*/ +
                          (cvc ? ns * mat * b16 + ns * nn * 4 : 0);
-  b.tc = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::min(nt, 12),
+  b.tc = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::min(nt, TC_CHUNK),
                                                    ((size_t)8 << 30) / per_tau));
   const int tc = b.tc;
   RS_TRY(ensure(h->hxsl, 2 * ns * mat * b16));
@@ -1766,8 +1749,6 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
   RS_TRY(ensure(h->hg, nt * mat * b16));
   RS_TRY(ensure(h->hgb, nt * mat * b16));
   RS_TRY(ensure(h->hP, (size_t)tc * 2 * ns * mat * b16));
-  RS_TRY(ensure(h->hdc32, (size_t)tc * ns * nn * sizeof(float)));
-  RS_TRY(ensure(h->hcl32, (size_t)tc * ns * nn * sizeof(float)));
   RS_TRY(ensure(h->hdcl16, (size_t)tc * 2 * ns * mat * b16));
   RS_TRY(ensure(h->hxy32, (size_t)tc * 2 * ns * nn * sizeof(float)));
   RS_TRY(ensure(h->ha6, (size_t)tc * 2 * ns * mat * b16));
@@ -1783,17 +1764,18 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
   }
   b.xsl = h->hxsl.p; b.y3 = h->hy3.p; b.gh = h->hg.p; b.gbh = h->hgb.p; b.P = h->hP.p;
   b.dcl = h->hdcl16.p; b.a6 = h->ha6.p; b.ct = h->hct.p; b.dct = h->hdct.p;
-  b.dc32 = h->hdc32.as<float>(); b.cl32 = h->hcl32.as<float>(); b.xy32 = h->hxy32.as<float>();
+  b.xy32 = h->hxy32.as<float>();
   b.part = h->hpart.as<float>();
   b.fold = h->hfold.as<double>();
   RS_TRY(tc_prepare());
+  RS_TRY(tc_dual_prepare());
   // the graph is keyed on every pointer and value baked into its launches
   std::vector<uintptr_t> key = {(uintptr_t)kind, (uintptr_t)b.wait_polls, (uintptr_t)ns, (uintptr_t)n,
                                 (uintptr_t)nt, (uintptr_t)h->n_occ, (uintptr_t)tc,
                                 (uintptr_t)G, (uintptr_t)Gb, (uintptr_t)sig, (uintptr_t)err,
                                 (uintptr_t)cvc, (uintptr_t)b.clt, (uintptr_t)b.fl,
                                 (uintptr_t)h->fac.p, (uintptr_t)h->e_st.p, (uintptr_t)sdd};
-  for (DevBuf *d : {&h->hxsl, &h->hy3, &h->hg, &h->hgb, &h->hP, &h->hdc32, &h->hcl32, &h->hdcl16,
+  for (DevBuf *d : {&h->hxsl, &h->hy3, &h->hg, &h->hgb, &h->hP, &h->hdcl16,
                     &h->hxy32, &h->ha6, &h->hct, &h->hdct, &h->hpart, &h->hfold})
     key.push_back((uintptr_t)d->p);
   if (!h->chain_graph || key != h->chain_key_ptr || h->h_tau_w != h->chain_key_w) {
@@ -1804,6 +1786,7 @@ cudaError_t chain_tc(rssri_handle *h, int kind, int ns, const double *G, const d
     if (!b.wait_polls) {
       std::vector<TcProb> probs;
       for (int stage = 0; stage < (cvc ? 5 : 4); ++stage) {
+        if (stage == 1) continue;  // tc_dual: one tile shape
         chain_stage_probs(h, b, ns, 0, std::min(tc, nt), stage, probs);
         tc_group_tune(kind, probs[0], err, s);
       }

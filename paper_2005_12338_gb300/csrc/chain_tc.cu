@@ -98,20 +98,16 @@ __global__ void matrices_kernel(const double *__restrict__ src, int cnt, int n, 
   }
 }
 
-// The fold works on 32 x 32 tiles staged in shared memory, so that every
-// global read and write is coalesced (including the transposes), in two
-// passes over a grid of (tile row, sample pair) blocks of 256 threads:
-//  1. partial sums of Tr X, Tr Y, Tr(X X) = sum X_ij X_ji, Tr(X Y) = sum Y_ij X_ji
-//     per tile row;
-//  2. the operands 2 dt I - X, 2 t^L I - Y, (C^L + dC)^T and dC^T of that tile
-//     row, after summing the partials of pass 1 in a fixed order; the block of
-//     tile row 0 adds the pair energy.
+// Partial sums of Tr X, Tr Y, Tr(X X) = sum X_ij X_ji and Tr(X Y) = sum Y_ij X_ji per
+// tile row of 32, for every (tile row, sample pair, tau point of the chunk): 32 x
+// 32 tiles staged in shared memory, so that the transposed reads are coalesced,
+// the next tile's loads in flight while one is summed.
 __global__ void __launch_bounds__(256) fold_traces_kernel(const float *__restrict__ xy, int ns,
                                                           int n, double *__restrict__ part) {
   __shared__ float ta[32][33], tb[32][33], tc[32][33];
   const int bi = blockIdx.x, x = blockIdx.y, nt = gridDim.x;
   const long long nn = (long long)n * n;
-  const float *X = xy + x * nn, *Y = xy + (ns + x) * nn;
+  const float *X = xy + ((long long)blockIdx.z * 2 * ns + x) * nn, *Y = X + ns * nn;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   double dx = 0, dy = 0;
   float sxx = 0.f, sxy = 0.f;  // per thread: 4 rows x the tile columns (fp32)
@@ -122,18 +118,34 @@ __global__ void __launch_bounds__(256) fold_traces_kernel(const float *__restric
       dy = Y[(long long)i * n + i];
     }
   }
+  float xa[4], ya[4], xb[4];
+  auto load = [&](int bj) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = ty + 8 * u;
+      const int i = bi * 32 + r, j = bj * 32 + tx;
+      const int i2 = bj * 32 + r, j2 = bi * 32 + tx;  // block (bj, bi) of X
+      const bool in1 = i < n && j < n, in2 = i2 < n && j2 < n;
+      xa[u] = in1 ? X[(long long)i * n + j] : 0.f;
+      ya[u] = in1 ? Y[(long long)i * n + j] : 0.f;
+      xb[u] = in2 ? X[(long long)i2 * n + j2] : 0.f;
+    }
+  };
+  load(0);
   for (int bj = 0; bj < nt; ++bj) {
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-      const int i = bi * 32 + r, j = bj * 32 + tx;
-      const int i2 = bj * 32 + r, j2 = bi * 32 + tx;
-      const bool in1 = i < n && j < n, in2 = i2 < n && j2 < n;
-      ta[r][tx] = in1 ? X[(long long)i * n + j] : 0.f;
-      tc[r][tx] = in1 ? Y[(long long)i * n + j] : 0.f;
-      tb[r][tx] = in2 ? X[(long long)i2 * n + j2] : 0.f;  // block (bj, bi) of X
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = ty + 8 * u;
+      ta[r][tx] = xa[u];
+      tc[r][tx] = ya[u];
+      tb[r][tx] = xb[u];
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
+    if (bj + 1 < nt) load(bj + 1);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = ty + 8 * u;
       const float xt = tb[tx][r];  // X_ji, i = bi*32 + r, j = bj*32 + tx
       sxx = fmaf(ta[r][tx], xt, sxx);
       sxy = fmaf(tc[r][tx], xt, sxy);
@@ -142,7 +154,7 @@ __global__ void __launch_bounds__(256) fold_traces_kernel(const float *__restric
   const double v0 = block_sum_d(dx), v1 = block_sum_d(dy), v2 = block_sum_d((double)sxx),
                v3 = block_sum_d((double)sxy);
   if (threadIdx.x == 0) {
-    double *o = part + ((long long)x * nt + bi) * 4;
+    double *o = part + (((long long)blockIdx.z * ns + x) * nt + bi) * 4;
     o[0] = v0;
     o[1] = v1;
     o[2] = v2;
@@ -150,66 +162,46 @@ __global__ void __launch_bounds__(256) fold_traces_kernel(const float *__restric
   }
 }
 
-// One 32 x 32 tile (bi, bj) of pair x per block: every load of the tile is
-// issued before the first store; the transposes go through shared memory.
+struct TauWeights {
+  double w[TC_CHUNK];
+};
+
+// What needs the traces: the diagonals 2 dt - X_ii and 2 t^L - Y_ii of the
+// operands a6 = [-X; -Y] that the product before wrote, and the pair energies
+// (tau points of the chunk in order).  One block per sample pair.
 template <class T>
-__global__ void __launch_bounds__(256) fold_operands_kernel(
-    const float *__restrict__ xy, const float *__restrict__ dc, const float *__restrict__ cl, int ns,
-    int n, int ldp, int nt, const double *__restrict__ part, double w, double ne,
-    T *__restrict__ a6, T *__restrict__ ct, T *__restrict__ dct, T *__restrict__ clt,
-    double *__restrict__ e_st) {
-  __shared__ float ta[32][33], tb[32][33], tl32[32][33];
-  __shared__ double sums[4];
-  const int bj = blockIdx.x, bi = blockIdx.y, x = blockIdx.z;
+__global__ void __launch_bounds__(128) fold_diag_kernel(const float *__restrict__ xy, int ns, int n,
+                                                        int ldp, int nt, int c,
+                                                        const double *__restrict__ part,
+                                                        const TauWeights w, double ne,
+                                                        T *__restrict__ a6,
+                                                        double *__restrict__ e_st) {
+  __shared__ double sums[TC_CHUNK][4];
+  const int x = blockIdx.x;
   const long long nn = (long long)n * n, mat = (long long)n * ldp;
-  if (threadIdx.x < 4) {
+  if (threadIdx.x < 4 * c) {
+    const int j = threadIdx.x >> 2, q = threadIdx.x & 3;
     double v = 0;
-    for (int t = 0; t < nt; ++t) v += part[((long long)x * nt + t) * 4 + threadIdx.x];
-    sums[threadIdx.x] = v;
-  }
-  const float *X = xy + x * nn, *Y = xy + (ns + x) * nn;
-  const float *DC = dc + x * nn, *CL = cl + x * nn;
-  T *A = a6 + x * mat, *Ab = a6 + (ns + x) * mat;
-  T *Ct = ct + x * mat, *Dt = dct + x * mat;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  // loads: rows ty, ty + 8, ... of the tile of X and Y, and of the
-  // transposed-source tile (bj, bi) of C^L and dC
-  float xv[4], yv[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = ty + 8 * u;
-    const int i = bi * 32 + r, j = bj * 32 + tx;
-    const bool in = i < n && j < n;
-    xv[u] = in ? X[(long long)i * n + j] : 0.f;
-    yv[u] = in ? Y[(long long)i * n + j] : 0.f;
-    const int i2 = bj * 32 + r, j2 = bi * 32 + tx;  // source (i2, j2) of C and dC
-    const bool in2 = i2 < n && j2 < n;
-    const float c = in2 ? CL[(long long)i2 * n + j2] : 0.f;
-    const float d = in2 ? DC[(long long)i2 * n + j2] : 0.f;
-    ta[r][tx] = c + d;
-    tb[r][tx] = d;
-    tl32[r][tx] = c;
+    for (int t = 0; t < nt; ++t) v += part[(((long long)j * ns + x) * nt + t) * 4 + q];
+    sums[j][q] = v;
   }
   __syncthreads();
-  const double dt = sums[0], tl = sums[1];
-  const float dt2 = (float)(2.0 * dt), tl2 = (float)(2.0 * tl);
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = ty + 8 * u;
-    const int i = bi * 32 + r, j = bj * 32 + tx;  // destination (i, j) = source (j, i)
-    if (i < n && j < ldp) {
-      const long long o = (long long)i * ldp + j;
-      const bool in = j < n;
-      putf(&A[o], in ? (i == j ? dt2 : 0.f) - xv[u] : 0.f);
-      putf(&Ab[o], in ? (i == j ? tl2 : 0.f) - yv[u] : 0.f);
-      putf(&Ct[o], in ? ta[tx][r] : 0.f);
-      putf(&Dt[o], in ? tb[tx][r] : 0.f);
-      if (clt) putf(&clt[x * mat + o], in ? tl32[tx][r] : 0.f);
-    }
+  for (int e = threadIdx.x; e < c * n; e += blockDim.x) {
+    const int j = e / n, i = e - j * n;
+    const long long z = (long long)j * 2 * ns + x;
+    const float dt2 = (float)(2.0 * sums[j][0]), tl2 = (float)(2.0 * sums[j][1]);
+    putf(&a6[z * mat + (long long)i * ldp + i], dt2 - xy[z * nn + (long long)i * n + i]);
+    putf(&a6[(z + ns) * mat + (long long)i * ldp + i],
+         tl2 - xy[(z + ns) * nn + (long long)i * n + i]);
   }
-  if (bi == 0 && bj == 0 && threadIdx.x == 0) {
-    const double de = 2.0 * dt * (2.0 * tl + dt) - sums[2] - 2.0 * sums[3];
-    e_st[x] += -w * de / ne;
+  if (threadIdx.x == 0) {
+    double e = e_st[x];
+    for (int j = 0; j < c; ++j) {
+      const double dt = sums[j][0], tl = sums[j][1];
+      const double de = 2.0 * dt * (2.0 * tl + dt) - sums[j][2] - 2.0 * sums[j][3];
+      e += -w.w[j] * de / ne;
+    }
+    e_st[x] = e;
   }
 }
 
@@ -243,14 +235,30 @@ __global__ void __launch_bounds__(256) cv_tc_energy_kernel(const float *__restri
   if (threadIdx.x == 0) e_st[x] += -w * q / ne;
 }
 
-__global__ void reduce_tc_kernel(const float *__restrict__ part, int groups, long long nn,
-                                   const double *__restrict__ base, double ns,
-                                   double *__restrict__ sig) {
+// One tau point of the chunk per blockIdx.y; the loads of 16 groups in flight.
+__global__ void __launch_bounds__(128) reduce_tc_kernel(const float *__restrict__ part, int groups,
+                                                        long long nn,
+                                                        const double *__restrict__ base, double ns,
+                                                        double *__restrict__ sig) {
+  const long long t = blockIdx.y;
+  part += t * groups * nn;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nn;
        e += (long long)gridDim.x * blockDim.x) {
-    // four independent partial sums (loads in flight), added in a fixed order
+    // four independent partial sums, added in a fixed order
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
     int g = 0;
+    for (; g + 16 <= groups; g += 16) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = part[(long long)(g + u) * nn + e];
+#pragma unroll
+      for (int u = 0; u < 16; u += 4) {
+        a0 += v[u];
+        a1 += v[u + 1];
+        a2 += v[u + 2];
+        a3 += v[u + 3];
+      }
+    }
     for (; g + 4 <= groups; g += 4) {
       a0 += part[(long long)g * nn + e];
       a1 += part[(long long)(g + 1) * nn + e];
@@ -259,7 +267,7 @@ __global__ void reduce_tc_kernel(const float *__restrict__ part, int groups, lon
     }
     for (; g < groups; ++g) a0 += part[(long long)g * nn + e];
     const double acc = ((double)a0 + (double)a1) + ((double)a2 + (double)a3);
-    sig[e] = base[e] + acc / ns;
+    sig[t * nn + e] = base[t * nn + e] + acc / ns;
   }
 }
 
@@ -289,27 +297,21 @@ cudaError_t chain_matrices(int kind, const double *src, int cnt, int n, int ldp,
   return cudaGetLastError();
 }
 
-cudaError_t fold_tc(int kind, const float *xy, const float *dc, const float *cl, int ns, int n,
-                    int ldp, double w, double ne, void *a6, void *ct, void *dct, void *clt,
-                    double *e_st, double *part, cudaStream_t s) {
+cudaError_t fold_tc(int kind, const float *xy, int ns, int n, int ldp, int c, const double *w,
+                    double ne, void *a6, double *e_st, double *part, cudaStream_t s) {
   const int nt = (n + 31) / 32;
-  dim3 grid(nt, ns);
-  fold_traces_kernel<<<grid, 256, 0, s>>>(xy, ns, n, part);
+  if (ns > 65535 || c > TC_CHUNK) return cudaErrorInvalidValue;
+  fold_traces_kernel<<<dim3(nt, ns, c), 256, 0, s>>>(xy, ns, n, part);
   ++launch_counter();
   RS_TRY(cudaGetLastError());
-  if (ns > 65535) return cudaErrorInvalidValue;
-  dim3 go((ldp + 31) / 32, nt, ns);
+  TauWeights tw;
+  for (int j = 0; j < TC_CHUNK; ++j) tw.w[j] = j < c ? w[j] : 0.0;
   if (kind == TC_BF16)
-    fold_operands_kernel<<<go, 256, 0, s>>>(xy, dc, cl, ns, n, ldp, nt, part, w, ne,
-                                              static_cast<__nv_bfloat16 *>(a6),
-                                              static_cast<__nv_bfloat16 *>(ct),
-                                              static_cast<__nv_bfloat16 *>(dct),
-                                              static_cast<__nv_bfloat16 *>(clt), e_st);
+    fold_diag_kernel<<<ns, 128, 0, s>>>(xy, ns, n, ldp, nt, c, part, tw, ne,
+                                        static_cast<__nv_bfloat16 *>(a6), e_st);
   else
-    fold_operands_kernel<<<go, 256, 0, s>>>(xy, dc, cl, ns, n, ldp, nt, part, w, ne,
-                                              static_cast<float *>(a6), static_cast<float *>(ct),
-                                              static_cast<float *>(dct),
-                                              static_cast<float *>(clt), e_st);
+    fold_diag_kernel<<<ns, 128, 0, s>>>(xy, ns, n, ldp, nt, c, part, tw, ne,
+                                        static_cast<float *>(a6), e_st);
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -326,10 +328,10 @@ cudaError_t cv_tc_apply(const float *fl, int ns, int n, const double *c, const d
   return cudaGetLastError();
 }
 
-cudaError_t reduce_tc(const float *part, int groups, int n, const double *base, double ns,
+cudaError_t reduce_tc(const float *part, int groups, int n, int c, const double *base, double ns,
                       double *sig, cudaStream_t s) {
   const long long nn = (long long)n * n;
-  reduce_tc_kernel<<<grid_cap(nn, 256), 256, 0, s>>>(part, groups, nn, base, ns, sig);
+  reduce_tc_kernel<<<dim3(grid_cap(nn, 128), c), 128, 0, s>>>(part, groups, nn, base, ns, sig);
   ++launch_counter();
   return cudaGetLastError();
 }

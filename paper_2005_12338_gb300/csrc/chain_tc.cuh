@@ -13,15 +13,13 @@ cudaError_t chain_factors(int kind, const double *fac, int ns, int n, int ldp, v
 // dst[c][i][j] = src[c][i][j] in the operand type with row stride ldp (zero padding).
 cudaError_t chain_matrices(int kind, const double *src, int cnt, int n, int ldp, void *dst,
                            cudaStream_t s);
-// Per sample pair: traces, the energy increment (weight w, N_e = ne), and the
-// operands of the final contraction: a6 = [2 dt I - X; 2 t^L I - Y],
-// ct = (C^L + dC)^T, dct = dC^T, all [.][n][ldp].  part: scratch of
-// ns * ceil(n/32) * 4 doubles.
-// clt (may be null): (C^L)^T as well, the right operand of F^L = (2 t^L I - Y) C^L
-// used by the learned control variate.
-cudaError_t fold_tc(int kind, const float *xy, const float *dc, const float *cl, int ns, int n,
-                    int ldp, double w, double ne, void *a6, void *ct, void *dct, void *clt,
-                    double *e_st, double *part, cudaStream_t s);
+// Per sample pair and tau point j of a chunk of c: from xy [c][X: ns, Y: ns] the
+// traces (part: scratch of c * ns * ceil(n/32) * 4 doubles), the energy increments
+// (weights w[j], host; N_e = ne), and the diagonals 2 dt - X_ii, 2 t^L - Y_ii of
+// a6 [c][2 ns][n][ldp], which holds -X and -Y.
+constexpr int TC_CHUNK = 12;  // tau points per chunk at most
+cudaError_t fold_tc(int kind, const float *xy, int ns, int n, int ldp, int c, const double *w,
+                    double ne, void *a6, double *e_st, double *part, cudaStream_t s);
 // The learned control variate on the tensor-core chain (Eq. 25 with the large
 // part weighted element-wise by c): with fl[x] = F(R^L, R'^L) of pair x (fp32),
 //   sig += (1 - c) o (mean_x fl[x] - sdd)           (fixed order over x),
@@ -29,8 +27,9 @@ cudaError_t fold_tc(int kind, const float *xy, const float *dc, const float *cl,
 cudaError_t cv_tc_apply(const float *fl, int ns, int n, const double *c, const double *sdd,
                         const double *gb, double w, double ne, double *sig, double *e_st,
                         cudaStream_t s);
-// sig = base + (sum over groups of part) / ns, groups summed in order in fp64.
-cudaError_t reduce_tc(const float *part, int groups, int n, const double *base, double ns,
+// sig[j] = base[j] + (sum over groups of part[j]) / ns for c tau points, groups summed in
+// order.
+cudaError_t reduce_tc(const float *part, int groups, int n, int c, const double *base, double ns,
                       double *sig, cudaStream_t s);
 
 }  // namespace rssri

@@ -273,6 +273,27 @@ cudaError_t tc_make_out_map(CUtensorMap *m, void *base, int elem_bytes, long lon
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+cudaError_t tc_make_box_map(CUtensorMap *m, void *base, int elem_bytes, long long cols,
+                            long long rows, long long batch, long long ld, int box_cols,
+                            int box_rows) {
+  if (!g_encode) return cudaErrorNotSupported;
+  const int inner = box_cols * elem_bytes;
+  if ((elem_bytes != 4 && elem_bytes != 2) || (inner != 64 && inner != 128) ||
+      (uintptr_t)base % 16 || (ld * elem_bytes) % 16 || cols <= 0 || rows <= 0 || batch <= 0 ||
+      cols > ld)
+    return cudaErrorInvalidValue;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch};
+  cuuint64_t strides[2] = {(cuuint64_t)(ld * elem_bytes), (cuuint64_t)(ld * rows * elem_bytes)};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1};
+  cuuint32_t es[3] = {1, 1, 1};
+  const CUresult r = g_encode(m, elem_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
+                                                 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
+                              3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              inner == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                              CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 bool tc_available() {
   std::call_once(g_encode_once, load_encode);
   return g_encode != nullptr;

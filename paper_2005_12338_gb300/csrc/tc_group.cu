@@ -50,6 +50,7 @@ struct GProb {
   float *c32;
   void *cop;
   long long ldcop;
+  uint32_t copsign;       // XORed into the operand-type output's sign
   CUtensorMap t32, top;  // output maps (valid where tma bit 0 / bit 1 is set)
   int tma;
 };
@@ -106,8 +107,9 @@ __device__ void epilogue_store(const GProb &P, int z, int row, int col0, const u
         uint32_t *w = reinterpret_cast<uint32_t *>(&q);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * u]),
-                                                          __uint_as_float(r[8 * v + 2 * u + 1]));
+          const __nv_bfloat162 h2 =
+              __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * u] ^ P.copsign),
+                                    __uint_as_float(r[8 * v + 2 * u + 1] ^ P.copsign));
           w[u] = *reinterpret_cast<const uint32_t *>(&h2);
         }
         reinterpret_cast<uint4 *>(dst)[v] = q;
@@ -115,7 +117,7 @@ __device__ void epilogue_store(const GProb &P, int z, int row, int col0, const u
     } else {
 #pragma unroll
       for (int j = 0; j < 16; ++j)
-        if (col0 + j < P.N) dst[j] = __float2bfloat16_rn(__uint_as_float(r[j]));
+        if (col0 + j < P.N) dst[j] = __float2bfloat16_rn(__uint_as_float(r[j] ^ P.copsign));
     }
   }
   if (P.cop && !(P.tma & 2) && KIND == TC_TF32) {
@@ -123,7 +125,7 @@ __device__ void epilogue_store(const GProb &P, int z, int row, int col0, const u
                  (long long)row * P.ldcop + col0;
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-      if (col0 + j < P.N) dst[j] = round_tf32(__uint_as_float(r[j]));
+      if (col0 + j < P.N) dst[j] = round_tf32(__uint_as_float(r[j] ^ P.copsign));
   }
 }
 
@@ -294,6 +296,7 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
               d[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
           }
           if (P.tma & 2) {
+            const uint32_t sx = P.copsign;
             if (KIND == TC_BF16) {
               uint4 *d = reinterpret_cast<uint4 *>(sbuf + STG_HALF + lane * 32);
 #pragma unroll
@@ -301,8 +304,9 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
                 uint32_t w[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                  const __nv_bfloat162 h2 = __floats2bfloat162_rn(
-                      __uint_as_float(r[8 * v + 2 * u]), __uint_as_float(r[8 * v + 2 * u + 1]));
+                  const __nv_bfloat162 h2 =
+                      __floats2bfloat162_rn(__uint_as_float(r[8 * v + 2 * u] ^ sx),
+                                            __uint_as_float(r[8 * v + 2 * u + 1] ^ sx));
                   w[u] = *reinterpret_cast<const uint32_t *>(&h2);
                 }
                 d[v] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -311,10 +315,10 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
               float4 *d = reinterpret_cast<float4 *>(sbuf + STG_HALF + lane * 64);
 #pragma unroll
               for (int v = 0; v < 4; ++v)
-                d[v] = make_float4(round_tf32(__uint_as_float(r[4 * v])),
-                                   round_tf32(__uint_as_float(r[4 * v + 1])),
-                                   round_tf32(__uint_as_float(r[4 * v + 2])),
-                                   round_tf32(__uint_as_float(r[4 * v + 3])));
+                d[v] = make_float4(round_tf32(__uint_as_float(r[4 * v] ^ sx)),
+                                   round_tf32(__uint_as_float(r[4 * v + 1] ^ sx)),
+                                   round_tf32(__uint_as_float(r[4 * v + 2] ^ sx)),
+                                   round_tf32(__uint_as_float(r[4 * v + 3] ^ sx)));
             }
           }
           fence_async_smem();
@@ -437,6 +441,7 @@ cudaError_t launch_group(int kind, const TcProb *probs, int np, int *err, cudaSt
     P.c32 = t.c32;
     P.cop = t.cop;
     P.ldcop = t.ldcop ? t.ldcop : t.N;
+    P.copsign = t.copneg ? 0x80000000u : 0u;
     // outputs whose rows are 16-byte aligned are written by TMA stores
     P.tma = 0;
     const long long zc = ceil_div(t.batch, t.bpc);

@@ -24,6 +24,7 @@ struct TcProb {
   float *c32 = nullptr;
   void *cop = nullptr;
   long long ldcop = 0;
+  int copneg = 0;  // cop holds minus the product
   int bn = 0;
 };
 

@@ -135,5 +135,10 @@ cudaError_t tc_make_map(CUtensorMap *m, int kind, const TcOperand &op, int K, in
 // boxes, no swizzle.  ld * elem_bytes and the base must be 16-byte aligned.
 cudaError_t tc_make_out_map(CUtensorMap *m, void *base, int elem_bytes, long long cols,
                             long long rows, long long batch, long long ld);
+// The same with boxes of box_rows rows x box_cols columns of 64 or 128 bytes per row,
+// swizzled accordingly (64-byte or 128-byte swizzle) in shared memory.
+cudaError_t tc_make_box_map(CUtensorMap *m, void *base, int elem_bytes, long long cols,
+                            long long rows, long long batch, long long ld, int box_cols,
+                            int box_rows);
 
 }  // namespace rssri
