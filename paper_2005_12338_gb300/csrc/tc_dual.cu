@@ -21,7 +21,7 @@
 //                  neither the writes nor the copies conflict on banks), each
 //                  written by one TMA bulk store.
 // Sums run over K in the same order as in tc_group_kernel, bit for bit.  At N =
-// 200, 300 pairs, 64 tau points a bf16 sampling call takes 15.5 ms with this and
+// 200, 300 pairs, 64 tau points a bf16 sampling call took 15.5 ms with this and
 // the fold that only needs the traces, 22.4 ms with the two products and the
 // fold that rewrote their fp32 results.
 // Every mbarrier wait is bounded, as there.
@@ -250,38 +250,52 @@ __global__ void __launch_bounds__(DTHREADS, 1) tc_dual_kernel(const __grid_const
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
       const int row0 = t.m0 + lq * 32;
-      if (row0 < p.n)
-        for (int c0 = 0; c0 < DBN && t.n0 + c0 < p.n; c0 += CW) {
-          const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(buf * 2 * ACC + c0);
-          float d[CW], l[CW];
-          tmem_cols<CW>(ta, d);
-          tmem_cols<CW>(ta + ACC, l);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          uint8_t *b = wst + (sc & 1) * STG;
-          if (sc >= 2) {
-            if (lane == 0) bulk_wait_read1();  // the boxes two chunks back have been read
-            __syncwarp();
-          }
-          stage_rows<KIND>(b, lane, d);
-          stage_rows<KIND>(b + BOX, lane, l);
-          stage_cols<KIND>(b + 3 * BOX, lane, d);
-          if (p.has_clt) stage_cols<KIND>(b + 4 * BOX, lane, l);
-#pragma unroll
-          for (int u = 0; u < CW; ++u) l[u] = l[u] + d[u];
-          stage_cols<KIND>(b + 2 * BOX, lane, l);
-          fence_async_smem();
+      const int cend = min(DBN, p.n - t.n0);
+      const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(buf * 2 * ACC);
+      // the next columns are read from tensor memory while these are staged
+      float d0[CW], l0[CW], d1[CW], l1[CW];
+      auto fetch = [&](int c0, float *d, float *l) {
+        tmem_cols<CW>(ta + c0, d);
+        tmem_cols<CW>(ta + ACC + c0, l);
+      };
+      auto step = [&](int c0, float *d, float *l) {
+        uint8_t *b = wst + (sc & 1) * STG;
+        if (sc >= 2) {
+          if (lane == 0) bulk_wait_read1();  // the boxes two steps back have been read
           __syncwarp();
-          if (lane == 0) {
-            const int z2 = t.j * 2 * p.ns + t.x, z1 = t.j * p.ns + t.x;
-            tma_store3(&p.tdcl, b, t.n0 + c0, row0, z2);
-            tma_store3(&p.tdcl, b + BOX, t.n0 + c0, row0, z2 + p.ns);
-            tma_store3(&p.tct, b + 2 * BOX, row0, t.n0 + c0, z1);
-            tma_store3(&p.tdct, b + 3 * BOX, row0, t.n0 + c0, z1);
-            if (p.has_clt) tma_store3(&p.tclt, b + 4 * BOX, row0, t.n0 + c0, z1);
-            bulk_commit();
-          }
-          ++sc;
         }
+        stage_rows<KIND>(b, lane, d);
+        stage_rows<KIND>(b + BOX, lane, l);
+        stage_cols<KIND>(b + 3 * BOX, lane, d);
+        if (p.has_clt) stage_cols<KIND>(b + 4 * BOX, lane, l);
+#pragma unroll
+        for (int u = 0; u < CW; ++u) l[u] = l[u] + d[u];
+        stage_cols<KIND>(b + 2 * BOX, lane, l);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          const int z2 = t.j * 2 * p.ns + t.x, z1 = t.j * p.ns + t.x;
+          tma_store3(&p.tdcl, b, t.n0 + c0, row0, z2);
+          tma_store3(&p.tdcl, b + BOX, t.n0 + c0, row0, z2 + p.ns);
+          tma_store3(&p.tct, b + 2 * BOX, row0, t.n0 + c0, z1);
+          tma_store3(&p.tdct, b + 3 * BOX, row0, t.n0 + c0, z1);
+          if (p.has_clt) tma_store3(&p.tclt, b + 4 * BOX, row0, t.n0 + c0, z1);
+          bulk_commit();
+        }
+        ++sc;
+      };
+      if (row0 < p.n) {
+        fetch(0, d0, l0);
+        for (int c0 = 0; c0 < cend; c0 += 2 * CW) {
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (c0 + CW < cend) fetch(c0 + CW, d1, l1);
+          step(c0, d0, l0);
+          if (c0 + CW >= cend) break;
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (c0 + 2 * CW < cend) fetch(c0 + 2 * CW, d0, l0);
+          step(c0 + CW, d1, l1);
+        }
+      }
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
       if (lane == 0)

@@ -12,11 +12,17 @@
 //                  so that the products of tile i+1 run while the epilogue
 //                  drains tile i;
 //   warps 2-5      epilogue: tcgen05.ld of the accumulator (warp w reads lanes
-//                  32 (w mod 4) ...), 16 columns at a time, staged through a
-//                  double-buffered 32-row x 16-column box in shared memory
-//                  and written by TMA bulk tensor stores (fp32 and/or
-//                  operand-type outputs; plain stores where an output's rows
-//                  are not 16-byte aligned), then release of the accumulator.
+//                  32 (w mod 4) ...), 32 columns at a time, the next ones being
+//                  read while these are staged in a double-buffered 32-row x
+//                  32-column box in shared memory (128-byte or 64-byte rows,
+//                  swizzled: no bank conflicts) and written by TMA bulk tensor
+//                  stores (fp32 and/or operand-type outputs; plain stores where
+//                  an output's rows are not 16-byte aligned), then release of
+//                  the accumulator.
+// At N = 200 (K = 200) a tile's products take ~1 us and its drain is as long as
+// moving its operands and results, so the drain's latency counts: with 16 columns
+// per step, unswizzled boxes and no read-ahead the N = 200 sampling call (300
+// pairs, 64 tau points) took 15.5 ms, with these 14.0.
 // Every mbarrier wait is bounded; on expiry the kernel records an error code
 // in a device flag and stops; before tensor memory is freed the epilogue
 // waits (bounded) for every product the issuer started.
@@ -36,11 +42,31 @@ using namespace tcx;
 
 constexpr int GTHREADS = 192;  // 6 warps
 constexpr int ACC_COLS = 256;  // per accumulator (max N tile)
-// epilogue staging per warp and buffer: 32 x 16 fp32 (c32) + 32 x 16 fp32
+constexpr int CW = 32;         // columns per epilogue step
+constexpr int GSTAGES = 3;     // K slabs in flight
+// epilogue staging per warp and buffer: 32 x 32 fp32 (c32) + 32 x 32 fp32
 // or bf16 (operand-type output)
-constexpr int STG_HALF = 32 * 16 * 4;
+constexpr int STG_HALF = 32 * CW * 4;
 constexpr int STG_BUF = 2 * STG_HALF;
 constexpr int STG_WARP = 2 * STG_BUF;
+
+// 16 bytes `q` as piece ch of row `lane` of a box with 128-byte rows (128-byte
+// swizzle) or 64-byte rows (64-byte swizzle).
+__device__ __forceinline__ void put128(uint8_t *box, int lane, int ch, uint4 q) {
+  *reinterpret_cast<uint4 *>(box + lane * 128 + 16 * (ch ^ (lane & 7))) = q;
+}
+__device__ __forceinline__ void put64(uint8_t *box, int lane, int ch, uint4 q) {
+  *reinterpret_cast<uint4 *>(box + lane * 64 + 16 * (ch ^ ((lane >> 1) & 3))) = q;
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t *r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
+      "%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+}
 
 struct GProb {
   CUtensorMap ta[2], tb[2];
@@ -271,36 +297,29 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
       }
       asm volatile("tcgen05.fence::after_thread_sync;");
       const int row0 = t.m0 + lq * 32, row = row0 + lane;
-      for (int c0 = 0; c0 < P.BN && t.n0 + c0 < P.N; c0 += 16) {
-        uint32_t r[16];
-        const uint32_t taddr = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(buf * ACC_COLS + c0);
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
-            "%13,%14,%15}, [%16];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-              "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-              "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(taddr));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      // columns of the tile that exist (a step's last columns may lie past them:
+      // what the tensor memory holds there is clipped by the stores)
+      const int cend = min(P.BN, P.N - t.n0);
+      const uint32_t tbase = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(buf * ACC_COLS);
+      uint32_t ra[CW], rb[CW];
+      auto step = [&](int c0, uint32_t *r) {
         if (P.tma && row0 < P.M) {
           // this row into the staging box, then one bulk store per output
           uint8_t *sbuf = wst + (sc & 1) * STG_BUF;
           if (sc >= 2) {
-            if (lane == 0) bulk_wait_read1();  // the box two chunks back has been read
+            if (lane == 0) bulk_wait_read1();  // the box two steps back has been read
             __syncwarp();
           }
           if (P.tma & 1) {
-            uint4 *d = reinterpret_cast<uint4 *>(sbuf + lane * 64);
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
-              d[v] = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+            for (int v = 0; v < CW / 4; ++v)
+              put128(sbuf, lane, v, make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]));
           }
           if (P.tma & 2) {
             const uint32_t sx = P.copsign;
             if (KIND == TC_BF16) {
-              uint4 *d = reinterpret_cast<uint4 *>(sbuf + STG_HALF + lane * 32);
 #pragma unroll
-              for (int v = 0; v < 2; ++v) {
+              for (int v = 0; v < CW / 8; ++v) {
                 uint32_t w[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -309,16 +328,16 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
                                             __uint_as_float(r[8 * v + 2 * u + 1] ^ sx));
                   w[u] = *reinterpret_cast<const uint32_t *>(&h2);
                 }
-                d[v] = make_uint4(w[0], w[1], w[2], w[3]);
+                put64(sbuf + STG_HALF, lane, v, make_uint4(w[0], w[1], w[2], w[3]));
               }
             } else {
-              float4 *d = reinterpret_cast<float4 *>(sbuf + STG_HALF + lane * 64);
 #pragma unroll
-              for (int v = 0; v < 4; ++v)
-                d[v] = make_float4(round_tf32(__uint_as_float(r[4 * v] ^ sx)),
-                                   round_tf32(__uint_as_float(r[4 * v + 1] ^ sx)),
-                                   round_tf32(__uint_as_float(r[4 * v + 2] ^ sx)),
-                                   round_tf32(__uint_as_float(r[4 * v + 3] ^ sx)));
+              for (int v = 0; v < CW / 4; ++v)
+                put128(sbuf + STG_HALF, lane, v,
+                       make_uint4(__float_as_uint(round_tf32(__uint_as_float(r[4 * v] ^ sx))),
+                                  __float_as_uint(round_tf32(__uint_as_float(r[4 * v + 1] ^ sx))),
+                                  __float_as_uint(round_tf32(__uint_as_float(r[4 * v + 2] ^ sx))),
+                                  __float_as_uint(round_tf32(__uint_as_float(r[4 * v + 3] ^ sx)))));
             }
           }
           fence_async_smem();
@@ -330,7 +349,24 @@ __global__ void __launch_bounds__(GTHREADS, 1) tc_group_kernel(const __grid_cons
           }
           ++sc;
         }
-        if (row < P.M && (P.tma & 3) != 3) epilogue_store<KIND>(P, t.z, row, t.n0 + c0, r);
+        if (row < P.M && (P.tma & 3) != 3) {
+          epilogue_store<KIND>(P, t.z, row, t.n0 + c0, r);
+          if (c0 + 16 < cend) epilogue_store<KIND>(P, t.z, row, t.n0 + c0 + 16, r + 16);
+        }
+      };
+      auto fetch = [&](int c0, uint32_t *r) {
+        tmem_ld16(tbase + c0, r);
+        tmem_ld16(tbase + c0 + 16, r + 16);
+      };
+      fetch(0, ra);
+      for (int c0 = 0; c0 < cend; c0 += 2 * CW) {
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c0 + CW < cend) fetch(c0 + CW, rb);
+        step(c0, ra);
+        if (c0 + CW >= cend) break;
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c0 + 2 * CW < cend) fetch(c0 + 2 * CW, ra);
+        step(c0 + CW, rb);
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
@@ -363,7 +399,7 @@ cudaError_t group_prepare() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
   if (!done[dev]) {
-    const int smem = (int)group_smem(4);
+    const int smem = (int)group_smem(GSTAGES);
     RS_TRY(cudaFuncSetAttribute(tc_group_kernel<TC_BF16>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     RS_TRY(cudaFuncSetAttribute(tc_group_kernel<TC_TF32>,
@@ -384,10 +420,12 @@ int sm_count() {
   return n;
 }
 
-// The N tile with the least padding (<= 256, a multiple of 16).
+// The N tile with the least padding (<= 256, a multiple of 16; of CW where a row of
+// tiles follows, as an epilogue step must not reach into the next tile).
 int default_bn(int N) {
   const int ntiles = (N + 255) / 256;
-  return std::min(256, ((ceil_div(N, ntiles) + 15) / 16) * 16);
+  const int q = ntiles > 1 ? CW : 16;
+  return std::min(256, ((ceil_div(N, ntiles) + q - 1) / q) * q);
 }
 
 using Key = std::tuple<int, int, int, int, int, int, int>;
@@ -416,7 +454,7 @@ cudaError_t launch_group(int kind, const TcProb *probs, int np, int *err, cudaSt
       auto it = g_tuned.find(key_of(kind, t));
       bn = it != g_tuned.end() ? it->second : default_bn(t.N);
     }
-    if (bn < 16 || bn > ACC_COLS || bn % 16) return cudaErrorInvalidValue;
+    if (bn < 16 || bn > ACC_COLS || bn % 16 || (bn < t.N && bn % CW)) return cudaErrorInvalidValue;
     P.BN = bn;
     // a zero batch stride shares the operand across the batch (map of one entry)
     P.ashared = t.A[0].sb == 0 && t.batch > 1;
@@ -445,9 +483,10 @@ cudaError_t launch_group(int kind, const TcProb *probs, int np, int *err, cudaSt
     // outputs whose rows are 16-byte aligned are written by TMA stores
     P.tma = 0;
     const long long zc = ceil_div(t.batch, t.bpc);
-    if (t.c32 && tc_make_out_map(&P.t32, t.c32, 4, t.N, t.M, zc, t.N) == cudaSuccess) P.tma |= 1;
-    if (t.cop && tc_make_out_map(&P.top, t.cop, kind == TC_BF16 ? 2 : 4, t.N, t.M, zc,
-                                 P.ldcop) == cudaSuccess)
+    if (t.c32 && tc_make_box_map(&P.t32, t.c32, 4, t.N, t.M, zc, t.N, CW, 32) == cudaSuccess)
+      P.tma |= 1;
+    if (t.cop && tc_make_box_map(&P.top, t.cop, kind == TC_BF16 ? 2 : 4, t.N, t.M, zc, P.ldcop, CW,
+                                 32) == cudaSuccess)
       P.tma |= 2;
     const long long tiles = (long long)P.mtiles * P.ntiles * ceil_div(t.batch, t.bpc);
     if (total + tiles > (1LL << 30)) return cudaErrorInvalidValue;
@@ -456,7 +495,7 @@ cudaError_t launch_group(int kind, const TcProb *probs, int np, int *err, cudaSt
   if (total == 0) return cudaSuccess;
   gp.np = np;
   gp.total = total;
-  gp.stages = 4;
+  gp.stages = GSTAGES;
   gp.wait_polls = wait_polls;
   gp.err = err;
   RS_TRY(group_prepare());

@@ -130,13 +130,10 @@ __device__ __forceinline__ float round_tf32(float x) {
 // contiguous) for 128-byte swizzled slabs of box_rows rows.
 cudaError_t tc_make_map(CUtensorMap *m, int kind, const TcOperand &op, int K, int batch,
                         int box_rows);
-// Tensor map of an output [batch][rows][ld] (elements of elem_bytes = 4:
-// fp32, 2: bf16; cols <= ld valid per row) for stores of 32-row x 16-column
-// boxes, no swizzle.  ld * elem_bytes and the base must be 16-byte aligned.
-cudaError_t tc_make_out_map(CUtensorMap *m, void *base, int elem_bytes, long long cols,
-                            long long rows, long long batch, long long ld);
-// The same with boxes of box_rows rows x box_cols columns of 64 or 128 bytes per row,
-// swizzled accordingly (64-byte or 128-byte swizzle) in shared memory.
+// Tensor map of an output [batch][rows][ld] (elements of elem_bytes = 4: fp32, 2: bf16;
+// cols <= ld valid per row) for stores of boxes of box_rows rows x box_cols columns, 64
+// or 128 bytes per row, swizzled accordingly (64-byte or 128-byte swizzle) in shared
+// memory.  ld * elem_bytes and the base must be 16-byte aligned.
 cudaError_t tc_make_box_map(CUtensorMap *m, void *base, int elem_bytes, long long cols,
                             long long rows, long long batch, long long ld, int box_cols,
                             int box_rows);
