@@ -2,10 +2,11 @@
 // weights of its contraction index per tau point, and the Gram matrices.
 //
 // Bound by the fp64 (or fp32) pipe.  Whole calls, the contraction over the kept
-// pairs before and this after: N = 20, 32 tau points, fp64 19.7 -> 2.8 ms (32
+// pairs before and this after: N = 20, 32 tau points, fp64 19.7 -> 2.7 ms (32
 // tau points in one launch instead of nine launches each); N = 100, 32 tau
-// points, fp64 350.5 -> 93.6 ms; N = 150, 24 tau points, double-float 293.8 ->
-// 138.5 ms.
+// points, fp64 350.5 -> 85.2 ms; N = 150, 24 tau points, double-float 293.8 ->
+// 128.0 ms (93.6 and 138.5 before 16-wide tiles, which waste the least on the
+// diagonal).
 #include "mo_tile.cuh"
 
 namespace rssri {

@@ -339,18 +339,20 @@ cudaError_t mo_sum(const MoSum &g, double *work, cudaStream_t s) {
   cudaError_t e;
   if (g.df) {
     switch (k) {
-      case 0: e = launch_sum<DF, S24>(a, g.nt, s); break;
-      case 1: e = launch_sum<DF, S32>(a, g.nt, s); break;
-      case 2: e = launch_sum<DF, S40>(a, g.nt, s); break;
+      case 0: e = launch_sum<DF, S16>(a, g.nt, s); break;
+      case 1: e = launch_sum<DF, S24>(a, g.nt, s); break;
+      case 2: e = launch_sum<DF, S32>(a, g.nt, s); break;
+      case 3: e = launch_sum<DF, S40>(a, g.nt, s); break;
       default: e = launch_sum<DF, S64>(a, g.nt, s);
     }
   } else {
     switch (k) {
-      case 0: e = launch_sum<F64, D24>(a, g.nt, s); break;
-      case 1: e = launch_sum<F64, D32>(a, g.nt, s); break;
-      case 2: e = launch_sum<F64, D40>(a, g.nt, s); break;
-      case 3: e = launch_sum<F64, D48>(a, g.nt, s); break;
-      case 4: e = launch_sum<F64, D64>(a, g.nt, s); break;
+      case 0: e = launch_sum<F64, D16>(a, g.nt, s); break;
+      case 1: e = launch_sum<F64, D24>(a, g.nt, s); break;
+      case 2: e = launch_sum<F64, D32>(a, g.nt, s); break;
+      case 3: e = launch_sum<F64, D40>(a, g.nt, s); break;
+      case 4: e = launch_sum<F64, D48>(a, g.nt, s); break;
+      case 5: e = launch_sum<F64, D64>(a, g.nt, s); break;
       default: e = launch_sum<F64, D100>(a, g.nt, s);
     }
   }

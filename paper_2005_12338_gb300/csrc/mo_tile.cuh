@@ -242,16 +242,18 @@ __global__ void mo_reduce_kernel(const double *__restrict__ part, int ns, int n,
 }
 
 // ------------------------------------------------------------ tile choice --
-// fp64: 64-thread tiles of edge 24, 32, 40, 48 (3 to 6 outputs per thread and
+// fp64: 64-thread tiles of edge 16, 24, 32, 40, 48 (2 to 6 outputs per thread and
 // side), 256 threads for 64 and 400 (of 416 lanes) for 100.  Every tile sums k
 // in ascending order, so the choice does not change a result.
+using D16 = Geo<8, 8, 2, 2, 16, 12, 8>;
 using D24 = Geo<8, 8, 3, 3, 16, 8, 8>;
 using D32 = Geo<8, 8, 4, 4, 16, 8, 8>;
 using D40 = Geo<8, 8, 5, 5, 8, 8, 8>;
 using D48 = Geo<8, 8, 6, 6, 8, 6, 8>;
 using D64 = Geo<16, 16, 4, 4, 16, 2, 8>;
 using D100 = Geo<20, 20, 5, 5, 8, 1, 8>;
-// double-float: 64-thread tiles of 24, 32, 40, 256-thread tile of 64
+// double-float: 64-thread tiles of 16, 24, 32, 40, 256-thread tile of 64
+using S16 = Geo<8, 8, 2, 2, 16, 12, 4>;
 using S24 = Geo<8, 8, 3, 3, 16, 8, 2>;
 using S32 = Geo<8, 8, 4, 4, 16, 6, 2>;
 using S40 = Geo<8, 8, 5, 5, 8, 6, 1>;
@@ -259,10 +261,14 @@ using S64 = Geo<16, 16, 4, 4, 16, 2, 4>;
 
 struct TileInfo {
   int edge;
-  double cost;  // relative time per padded output and k step (lane use, overlap)
+  double cost;  // relative time per padded output and k step
 };
-constexpr TileInfo kD[] = {{24, 1.0}, {32, 1.0}, {40, 1.0}, {48, 1.0}, {64, 1.0}, {100, 1.04}};
-constexpr TileInfo kS[] = {{24, 1.35}, {32, 1.15}, {40, 1.25}, {64, 1.0}};
+// Measured on Gram matrices of n = 64 to 200 (padded multiply-adds, TFLOP/s): fp64
+// 1.14-1.18 for edges 24 to 48, 1.20 for 64, 1.03 for 100; double-float 4.15, 3.75,
+// 3.8, 4.67 for 24, 32, 40, 64.
+constexpr TileInfo kD[] = {{16, 1.06}, {24, 1.03}, {32, 1.03}, {40, 1.04}, {48, 1.03}, {64, 1.0}, {100, 1.14}};
+constexpr TileInfo kS[] = {{16, 1.25}, {24, 1.13}, {32, 1.24}, {40, 1.22}, {64, 1.0}};
+constexpr int kND = sizeof(kD) / sizeof(kD[0]), kNS = sizeof(kS) / sizeof(kS[0]);
 
 // The tile of least padded work (sym: tiles on and above the diagonal).
 int pick(const TileInfo *t, int cnt, int M, int N, int sym) {
@@ -279,7 +285,7 @@ int pick(const TileInfo *t, int cnt, int M, int N, int sym) {
   return best;
 }
 int pick_tile(int df, int M, int N, int sym) {
-  return df ? pick(kS, 4, M, N, sym) : pick(kD, 6, M, N, sym);
+  return df ? pick(kS, kNS, M, N, sym) : pick(kD, kND, M, N, sym);
 }
 int tile_edge(int df, int k) { return df ? kS[k].edge : kD[k].edge; }
 long long tile_count(int edge, int M, int N, int sym) {
@@ -301,18 +307,20 @@ template <int RAW> cudaError_t nt_dispatch(int df, const NtArgs &a, long long z,
   const int k = pick_tile(df, a.M, a.N, a.sym);
   if (df) {
     switch (k) {
-      case 0: return launch_nt<DF, S24, RAW>(a, z, s);
-      case 1: return launch_nt<DF, S32, RAW>(a, z, s);
-      case 2: return launch_nt<DF, S40, RAW>(a, z, s);
+      case 0: return launch_nt<DF, S16, RAW>(a, z, s);
+      case 1: return launch_nt<DF, S24, RAW>(a, z, s);
+      case 2: return launch_nt<DF, S32, RAW>(a, z, s);
+      case 3: return launch_nt<DF, S40, RAW>(a, z, s);
       default: return launch_nt<DF, S64, RAW>(a, z, s);
     }
   }
   switch (k) {
-    case 0: return launch_nt<F64, D24, RAW>(a, z, s);
-    case 1: return launch_nt<F64, D32, RAW>(a, z, s);
-    case 2: return launch_nt<F64, D40, RAW>(a, z, s);
-    case 3: return launch_nt<F64, D48, RAW>(a, z, s);
-    case 4: return launch_nt<F64, D64, RAW>(a, z, s);
+    case 0: return launch_nt<F64, D16, RAW>(a, z, s);
+    case 1: return launch_nt<F64, D24, RAW>(a, z, s);
+    case 2: return launch_nt<F64, D32, RAW>(a, z, s);
+    case 3: return launch_nt<F64, D40, RAW>(a, z, s);
+    case 4: return launch_nt<F64, D48, RAW>(a, z, s);
+    case 5: return launch_nt<F64, D64, RAW>(a, z, s);
     default: return launch_nt<F64, D100, RAW>(a, z, s);
   }
 }
