@@ -391,12 +391,14 @@ int metric_inv_sqrt(rssri_handle *h, int *rc, bool df64) {
       RS_TRY(to_df64(A, (long long)na * na, h->nsA2.as<float2>(), s, range_flag(h)));
       RS_TRY(to_df64(B, (long long)na * na, h->nsB2.as<float2>(), s, range_flag(h)));
     }
-    SPAN(RSSRI_PROF_SETUP_GEMM, 2.0 * na * (double)na * na * 1e-9);
+    SPAN(RSSRI_PROF_SETUP_GEMM, 1.0 * na * (double)na * na * 1e-9);
     DfGemm g;
     g.M = g.N = g.K = na;
     g.A = h->nsA2.as<float2>(); g.lda = na;
     g.B = h->nsB2.as<float2>(); g.ldb = na;
     g.C64 = C; g.ldc = na;
+    // polynomials of one symmetric matrix: their products are symmetric
+    g.sym = 1;
     return df_gemm_w(h, g);
   };
   const int max_it = 100;
@@ -404,16 +406,20 @@ int metric_inv_sqrt(rssri_handle *h, int *rc, bool df64) {
   bool final_step = false;
   int it = 0;
   for (; it < max_it; ++it) {
-    RS_CK(mm(Z, Y, Pm));
-    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(ns_tbuild(Pm, na, Tm, scal, part, s)); }
+    if (it > 0) RS_CK(mm(Z, Y, Pm));  // Z_0 = I: Z_0 Y_0 = Y_0
+    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(ns_tbuild(it > 0 ? Pm : Y, na, Tm, scal, part, s)); }
     RS_CK(fetch(&resid, scal + 1, s));
     if (!std::isfinite(resid) || resid > 1e6) break;
     if (final_step) break;
     if (resid < 1e-8) final_step = true;
     RS_CK(mm(Y, Tm, Y2));
-    RS_CK(mm(Tm, Z, Z2));
+    if (it > 0) {
+      RS_CK(mm(Tm, Z, Z2));
+      std::swap(Z, Z2);
+    } else {
+      std::swap(Z, Tm);  // T_0 Z_0 = T_0
+    }
     std::swap(Y, Y2);
-    std::swap(Z, Z2);
   }
   h->ns_iters = it;
   h->ns_resid = resid;
