@@ -147,7 +147,7 @@ struct rssri_handle {
   // weights of a chunk of tau points, row norms of K_P
   DevBuf moB1, moB2, moV, moU, moW, moRow;
   OzBuf ozY;    // its digits on the tensor cores (RSSRI_DD_OZ)
-  DevBuf ozYm, ozY6;  // row maxima per tau point, the slicer's level-6 sums
+  DevBuf ozYm, ozY6, ozYsel;  // row maxima per tau point, the slicer's level-6 sums, block levels
   bool mo_tab_ready = false;  // moTab, moChl made for this setup
   bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
   // bf16 chain buffers
@@ -203,7 +203,11 @@ struct rssri_handle {
 namespace {
 
 // Device flags (ints): [4] tensor-core chain timeout, [5] sliced-block timeout,
-// [8..10] the double-float range check (flag, running maximum, block count).
+// [8..10] the double-float range check (flag, running maximum, block count),
+// [12..13] digit products of the block's Gram matrices (one 64-bit count).
+unsigned long long *gram_steps(rssri_handle *h) {
+  return reinterpret_cast<unsigned long long *>(h->flags.as<int>() + 12);
+}
 int *range_flag(rssri_handle *h) { return h->flags.as<int>() + 8; }
 
 // ------------------------------------------------------------ profiling ----
@@ -519,7 +523,7 @@ void rssri_destroy(rssri_handle *h) {
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
                     &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
                     &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork,
-                    &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow, &h->ozYm, &h->ozY6};
+                    &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow, &h->ozYm, &h->ozY6, &h->ozYsel};
   for (DevBuf *b : bufs) release(*b);
   release(h->oz_pidx);
   release(h->oz_tmp);
@@ -1375,6 +1379,8 @@ cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
     RS_TRY(ensure(h->ozY6, (size_t)tcw * n * sizeof(double) + oz_gram_lev6_floats(z) * sizeof(float)));
     z.diag = h->ozY6.as<double>();
     z.lev6 = reinterpret_cast<float *>(z.diag + (long long)tcw * n);
+    RS_TRY(ensure(h->ozYsel, oz_gram_sel_bytes(n, ldc, nt)));
+    RS_TRY(cudaMemsetAsync(gram_steps(h), 0, sizeof(unsigned long long), s));
   }
   // U's pairs are scaled into the middle of fp32's range by [K]^L's largest
   // magnitude, 2^-2e each, an exact power of two (the sliced form takes [K]^L up
@@ -1456,19 +1462,23 @@ cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
       {
         SPAN(RSSRI_PROF_SLICE, 0.0);
         RS_TRY(mo_weights(1, tab.hv, tab.ho, nv, no, c0, c, nt, tab.hexp, z.ldy, h->moW.p, s));
-        RS_TRY(oz_gram_max(h->moU.as<float2>(), h->moW.as<float2>(), n, z.K, z.ldy, nt,
-                           h->ozYm.as<int>(), s));
+        RS_TRY(oz_gram_select(h->moU.as<float2>(), h->moW.as<float2>(), n, z.K, z.ldy, nt,
+                              h->ozYm.as<int>(), oz_gram_sel(h->ozYsel.p, n, z.ldy, nt),
+                              gram_steps(h), s));
       }
+      const OzGramSel sel = oz_gram_sel(h->ozYsel.p, n, z.ldy, nt);
+      const long long kb = z.ldy / 16;
       for (int t0 = 0; t0 < nt; t0 += tcw) {
         z.nt = std::min(tcw, nt - t0);
         z.U = h->moU.as<float2>(); z.y = h->moW.as<float2>() + t0 * z.ldy;
         z.m = h->ozYm.as<int>() + (long long)t0 * n;
+        z.lev = sel.lev + t0 * kb; z.list = sel.list + t0 * kb; z.cnt = sel.cnt + 4 * t0;
         z.d = h->ozY.d.as<__nv_bfloat16>(); z.ef = h->ozY.e.as<int>();
         z.scale = std::ldexp(1.0, 2 * e2); z.yexp = tab.hexp + t0;
         z.out = out + (long long)t0 * n * n; z.accumulate = c0 > 0;
         z.err = err; z.wait_polls = h->test_wait_polls;
         { SPAN(RSSRI_PROF_SLICE, 0.0); RS_TRY(oz_gram_slice(z, s)); }
-        SPAN_T(RSSRI_PROF_DD_SPMM, (double)n * n * z.K * z.nt * 1e-9, oz_gram_flops(z) * 1e-9);
+        SPAN(RSSRI_PROF_DD_SPMM, (double)n * n * z.K * z.nt * 1e-9);
         RS_TRY(oz_gram(z, h->moWork.as<double>(), s));
       }
       continue;
@@ -1591,6 +1601,12 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   if (dd_arith == RSSRI_DD_OZ || h->setup_arith == RSSRI_DD_OZ) {
     const int rc = oz_waits(h);
     if (rc) return rc;
+    if (mo && dd_arith == RSSRI_DD_OZ) {  // the tensor flops that the digits' levels left to do
+      unsigned long long steps = 0;
+      RS_CK(fetch(&steps, gram_steps(h), s));
+      h->recs.push_back({RSSRI_PROF_DD_SPMM, 0.0, steps * oz_gram_step_flops(n) * 1e-9, 0, nullptr,
+                         nullptr});
+    }
 #ifdef RSSRI_CHECKS
     int chk[4];
     RS_CK(oz_check_fetch(chk));

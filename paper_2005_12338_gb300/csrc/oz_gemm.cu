@@ -9,20 +9,30 @@
 //                  digits 4-5 as one 128 x 64-byte tile (64-byte swizzle):
 //                  the digit layout interleaves the digits of each block of
 //                  16 columns, so every TMA row is 128 or 64 bytes wide;
-//   warp 1 lane 0  MMA issuer: per K step, the 21 digit products p + q <= 5
+//   warp 1         MMA issuer: per K step, the 21 digit products p + q <= 5
 //                  (tcgen05.mma kind::f16, M = N = 128, K = 16) into four fp32
 //                  accumulators in tensor memory, one per level p + q = 0, 1,
 //                  2 and one for p + q >= 3 (4 x 128 of the 512 columns);
-//   warps 2-17     drain: after every 256 terms of K (16 steps) they read the
-//                  four accumulators (tcgen05.ld, 16 x 8 fragments) and add them
-//                  exactly into double-float running totals held in registers
-//                  (each thread: 32 outputs, column pairs of four rows), then
-//                  release the accumulators; at the end they assemble fp64 from
-//                  the running totals with integer exponent arithmetic and
-//                  store column pairs as 16-byte stores.
-// Levels 0-2 are exact over 256 terms (< 2^24 grid units), so a chunk's sum
-// a0 + a1 + a2 is exact in two TwoSums; level >= 3 (~2^-24 of the result)
-// and the running sum round at ~2^-48 relative.
+//   warps 2-17     drain: they read one accumulator at a time (tcgen05.ld,
+//                  16 x 8 fragments) and add it into double-float running totals
+//                  held in registers (each thread: 32 outputs, column pairs of
+//                  four rows); at the end of a tile they assemble fp64 from the
+//                  running totals with integer exponent arithmetic and store
+//                  column pairs as 16-byte stores.
+// Levels 0, 1, 2 are exact over 768, 384 and 256 terms of K (0.75 2^24 grid
+// units), so they are drained after every 48, 24 and 16 steps and added by
+// TwoSum; level >= 3 (~2^-24 of the result, drained after 16 steps) and the
+// running totals round at ~2^-48 relative.
+//
+// What bounds it: a product takes the tensor cores 64 cycles (66 measured alone, 1,384
+// per K step).  The drains are staggered so that the products into the other three
+// accumulators go on during each, with two fp32 values per add instruction; and the
+// issuer is a whole warp of warp-uniform values with few instructions between the
+// products.  At n = 500, K^Q (m x l) summed over 193 steps per tile, a step takes 1,660
+// cycles against 2,130 with one-lane issue (72 cycles per product) and a joint drain of
+// all four accumulators after every 16 steps (5,200 cycles without products): exchange
+// 122.6 -> 105 ms per call; Gram products at n = 200: 71.6 -> 53.2 ms.  The TMA loads
+// (32 KB per step at most from HBM, the rest L2) are hidden: without them nothing changes.
 //
 // Every mbarrier wait is bounded; on expiry the kernel records an error code
 // in a device flag and stops waiting; tensor memory is freed on every path.
@@ -33,6 +43,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "oz_gemm.cuh"
 
@@ -45,7 +56,7 @@ constexpr int TILE1 = BM * 32 * 2;           // digits 4-5: 128 rows x 64 bytes
 constexpr int OPB = TILE0 + TILE1;           // one operand's digits of one K step
 constexpr int STAGE = 2 * OPB;               // A and B digits of one K step
 constexpr int STAGES = 4;
-constexpr int CHUNK = 16;                    // K steps between drains (256 terms)
+constexpr int CHUNK = 16;                    // a Gram split starts on a multiple of this many K steps
 constexpr int EPI = 16;                      // drain warps (4 per tensor-memory lane quarter)
 constexpr int DC = BN / 4;                   // accumulator columns per drain thread
 constexpr int THREADS = (2 + EPI) * 32;
@@ -89,12 +100,13 @@ struct OzParams {
   long long ldc, sC;
   int bk, nl16, jtiles, lb0;  // exchange geometry
   int tiles, ntiles, mtiles;  // the output tiles the persistent CTAs share
-  // Gram matrices: tile types (row tile <= column tile) in the order of their first queue
-  // entry per batch entry, the K steps of a split of each, and the splits' stride in C
-  int ntypes, per_batch, smax;
+  // Gram matrices: the tiles (row tile <= column tile) of a batch entry, each split over
+  // ksplit CTAs (q = (batch entry * ntypes + type) * ksplit + split), and the lists of
+  // 16-column blocks to multiply per batch entry with how many there are of each level
+  int ntypes;
   unsigned char tm[GRAM_TYPES], tn[GRAM_TYPES];
-  short first[GRAM_TYPES + 1];
-  int tkst[GRAM_TYPES];
+  const int *list, *cnt;
+  long long lstride;
   int *err;
   long long ccap, efa_cap, efb_cap;  // bounds of C and the exponent arrays (checks)
   int wait_polls;  // 0: normal; > 0: test mode (see OzGemm)
@@ -155,27 +167,27 @@ __device__ __forceinline__ void tma_load4(void *dst, const CUtensorMap *m, uint6
       "l"(m), "r"(s_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w)
       : "memory");
 }
-// Shared-memory matrix descriptor of a K-major operand in rows of 128 bytes
-// (128-byte swizzle, layout code 2, 1024 bytes between groups of 8 rows) or
-// of 64 bytes (64-byte swizzle, code 4, 512 bytes between groups).
-__device__ __forceinline__ uint64_t smem_desc_sw(uint32_t saddr, uint32_t sbo, uint32_t layout) {
-  uint64_t d = (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(sbo >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)layout << 61;
-  return d;
-}
-// Digit p of an operand's stage slot at `base`: its 16 columns start 32 p
-// bytes into the 128-byte rows (p < 4) or 32 (p - 4) into the 64-byte rows.
+// Shared-memory matrix descriptor of digit p of a K-major operand whose stage slot starts at
+// `base` (in units of 16 bytes): its 16 columns start 32 p bytes into rows of 128 bytes
+// (p < 4: 128-byte swizzle, layout code 2, 1024 bytes between groups of 8 rows) or
+// 32 (p - 4) bytes into the rows of 64 bytes after them (64-byte swizzle, code 4, 512 bytes).
+// Only the low word depends on the stage, so that a product costs the issuer two additions.
 __device__ __forceinline__ uint64_t digit_desc(uint32_t base, int p) {
-  return p < 4 ? smem_desc_sw(base + 32 * p, 1024, 2)
-               : smem_desc_sw(base + TILE0 + 32 * (p - 4), 512, 4);
+  const uint32_t hi = p < 4 ? (1024u >> 4) | (1u << 14) | (2u << 29)
+                            : (512u >> 4) | (1u << 14) | (4u << 29);
+  return (uint64_t)hi << 32 | (base + (1u << 16) + (p < 4 ? 2 * p : TILE0 / 16 + 2 * (p - 4)));
 }
-// Instruction descriptor: D fp32, A and B bf16, both K-major, M = 128, N = nw.
-__device__ __forceinline__ uint32_t instr_desc_bf16(int nw) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nw >> 3) << 17) |
+// Instruction descriptor: D fp32, A and B bf16, both K-major, M = N = 128.
+__device__ __forceinline__ uint32_t instr_desc_bf16() {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
          ((uint32_t)(BM >> 4) << 24);
+}
+// True in one lane of a whole warp, the same one each time.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n}"
+               : "=r"(e));
+  return e != 0;
 }
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc,
                                          uint32_t acc) {
@@ -200,24 +212,63 @@ __device__ __forceinline__ void tmem_ld16x256(uint32_t taddr, uint32_t *r) {
 }
 
 // ----------------------------------------------------- exact float sums ----
-// Knuth's TwoSum: s + e == a + b exactly.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
+// Two fp32 values in one 64-bit register, added by one instruction.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(uint32_t x, uint32_t y) { return (f2)y << 32 | x; }
+__device__ __forceinline__ float f2_lo(f2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float f2_hi(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+  f2 c;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
+  return c;
 }
-// (hi, lo) += a0 + a1 + a2 + a3, where a0, a1, a2 are exact chunk sums and a3
-// the small rounded level.
-__device__ __forceinline__ void fold(float &hi, float &lo, float a0, float a1, float a2,
-                                     float a3) {
-  float s, e, s2, e2;
-  two_sum(a0, a1, s, e);
-  two_sum(s, a2, s2, e2);
-  e = (e + e2) + a3;
-  float t, f;
-  two_sum(hi, s2, t, f);
-  f = f + (lo + e);
-  two_sum(t, f, hi, lo);
+__device__ __forceinline__ f2 f2_sub(f2 a, f2 b) {
+  f2 c;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(c) : "l"(a), "l"(b));
+  return c;
+}
+// (hi, lo) += a, an exact sum of one level: Knuth's TwoSum, and with `norm` Fast2Sum to
+// renormalise (where hi has cancelled below lo it rounds at 2^-24 of lo, ~2^-48 of the terms).
+__device__ __forceinline__ void fold(f2 &hi, f2 &lo, f2 a, bool norm) {
+  const f2 s = f2_add(hi, a), bb = f2_sub(s, hi);
+  const f2 f = f2_add(lo, f2_add(f2_sub(hi, f2_sub(s, bb)), f2_sub(a, bb)));
+  hi = norm ? f2_add(s, f) : s;
+  lo = norm ? f2_sub(f, f2_sub(hi, s)) : f;
+}
+
+// Accumulator k (level 0, 1, 2, or 3 and more) is drained after the K steps st of a
+// tile with st % period == phase, and after the last one that it takes products of.
+// The periods keep a level's sum below 0.75 2^24 grid units; the phases spread the
+// drains, so that the products into the other accumulators go on during each, and leave
+// the first 7 steps of a tile to the stores of the tile before.
+__host__ __device__ constexpr int acc_period(int k) { return k == 0 ? 48 : (k == 1 ? 24 : 16); }
+__host__ __device__ constexpr int acc_phase(int k) {
+  return k == 0 ? 35 : (k == 1 ? 19 : (k == 2 ? 7 : 15));
+}
+// The accumulators drained after step 4 i + 3, in bits 4 i .. 4 i + 3 (i < 12).
+constexpr unsigned long long drain_table() {
+  unsigned long long m = 0;
+  for (int i = 0; i < 12; ++i)
+    for (int k = 0; k < 4; ++k)
+      if ((4 * i + 3) % acc_period(k) == acc_phase(k)) m |= 1ull << (4 * i + k);
+  return m;
+}
+constexpr unsigned long long DRAINS = drain_table();
+// A run of K steps of one level within a tile: up to step `end`, after which the
+// accumulators of `last` are drained for the tile; those of `live` take products.
+struct OzRun {
+  int end;
+  uint32_t live, last;
+};
+// The accumulators (bits) drained after step st; called for every st % 4 == 3 in turn and
+// for the last step of a run, tab = DRAINS at step 0 of a tile.
+__device__ __forceinline__ uint32_t drains_after(unsigned long long &tab, int st, const OzRun &r) {
+  uint32_t m = 0;
+  if ((st & 3) == 3) {
+    m = (uint32_t)tab & r.live;
+    tab = tab >> 4 | (tab & 15) << 44;
+  }
+  return st + 1 == r.end ? m | r.last : m;
 }
 
 // f * 2^E as an fp64 value, built from the float's bits (no fp64 arithmetic).
@@ -285,25 +336,62 @@ __device__ __forceinline__ int row_scale(int ef) { return max(ef, 1) - 1022; }
 // ------------------------------------------------------------- the GEMM ----
 // One output tile of a persistent CTA's queue (tile q = n tile + ntiles * rest):
 // dense: rest = m tile + mtiles * (batch * ksplit + split); exchange: rest = row tile.
-// kst K steps from step k0; nw columns (a multiple of 16, at most BN) are computed.
+// kst K steps from step k0.
+// Accumulators 0 and 1 take products of the steps before end01, 2 of those before end2,
+// 3 of all (Gram: steps end01.. are of level 1 or more, end2.. of level 2; else all 0).
 struct OzTile {
-  int n0, m0, zb, split, rt, mt, jt, k0, kst, nw;
+  int n0, m0, zb, split, rt, mt, jt, k0, kst, end01, end2;
 };
+// Cost of a K step of level 0, 1, 2 (21, 10 and 3 digit products; loads of 192, 128
+// and 128 bytes per row), for dealing a tile's steps out to its splits.
+constexpr int LC0 = 20, LC1 = 11, LC2 = 7;
+// The run of level lev (empty when its end is not past the one before).
+__device__ __forceinline__ OzRun oz_run(const OzTile &t, int lev) {
+  OzRun r;
+  r.end = lev == 0 ? t.end01 : (lev == 1 ? t.end2 : t.kst);
+  r.live = lev == 0 ? 15u : (lev == 1 ? 12u : 8u);
+  r.last = (lev == 0 ? 3u : 0u) | (r.end == t.end2 && lev < 2 ? 4u : 0u) | (r.end == t.kst ? 8u : 0u);
+  return r;
+}
+// The next step from st on that an accumulator may be drained after, and which (bits); the
+// same sequence as drains_after()'s, from the step alone: the drain warps' registers are
+// taken by the running totals.
+__device__ __forceinline__ uint32_t next_drains(const OzTile &t, int &st) {
+  const OzRun r = oz_run(t, st < t.end01 ? 0 : (st < t.end2 ? 1 : 2));
+  st = min(st | 3, r.end - 1);
+  unsigned long long tab = DRAINS >> (4 * ((st >> 2) % 12));
+  return drains_after(tab, st, r);
+}
+// First step of split s of ks: the splits cost about the same and start on a drain's
+// boundary (a multiple of CHUNK).
+__device__ __forceinline__ int gram_start(int n0, int n1, int n2, int s, int ks) {
+  const int total = n0 + n1 + n2;
+  if (s >= ks) return total;
+  const long long w0 = (long long)LC0 * n0, w1 = (long long)LC1 * n1;
+  const long long at = (w0 + w1 + (long long)LC2 * n2) * s / ks;
+  const long long pos = at < w0 ? at / LC0
+                                : (at < w0 + w1 ? n0 + (at - w0) / LC1
+                                                : n0 + n1 + (at - w0 - w1) / LC2);
+  return (int)pos / CHUNK * CHUNK;
+}
 // With mfast: q = m tile + mtiles * (n tile + ntiles * (batch * ksplit + split)).
 template <int MODE>
 __device__ __forceinline__ OzTile oz_tile(const OzParams &p, int q) {
   OzTile t;
   t.kst = p.kst;
   if (MODE == 2) {
-    t.zb = q / p.per_batch;
-    const int idx = q - t.zb * p.per_batch;
-    int y = 0;
-    while (idx >= p.first[y + 1]) ++y;
-    t.split = idx - p.first[y];
+    const int yz = q / p.ksplit;
+    t.split = q - yz * p.ksplit;
+    t.zb = yz / p.ntypes;
+    const int y = yz - t.zb * p.ntypes;
     t.m0 = p.tm[y] * BM;
     t.n0 = p.tn[y] * BN;
-    t.kst = p.tkst[y];
     t.rt = t.mt = t.jt = 0;
+    const int4 c = *reinterpret_cast<const int4 *>(p.cnt + 4 * t.zb);
+    t.k0 = gram_start(c.x, c.y, c.z, t.split, p.ksplit);
+    t.kst = gram_start(c.x, c.y, c.z, t.split + 1, p.ksplit) - t.k0;
+    t.end01 = min(max(c.x - t.k0, 0), t.kst);
+    t.end2 = min(max(c.x + c.y - t.k0, 0), t.kst);
   } else if (MODE == 0) {
     int z;
     if (p.mfast) {
@@ -328,9 +416,10 @@ __device__ __forceinline__ OzTile oz_tile(const OzParams &p, int q) {
     t.jt = rest - t.mt * p.jtiles;
     t.m0 = t.zb = t.split = 0;
   }
-  t.k0 = t.split * t.kst;
-  // a Gram matrix's last column tile: only its columns (rounded up to 16) are multiplied
-  t.nw = MODE == 2 ? min(BN, (p.N - t.n0 + 15) & ~15) : BN;
+  if (MODE != 2) {
+    t.k0 = t.split * t.kst;
+    t.end01 = t.end2 = t.kst;
+  }
   return t;
 }
 
@@ -340,19 +429,21 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t *full = (uint64_t *)(smem + STAGES * STAGE);
   uint64_t *empty = full + STAGES;
-  uint64_t *accf = empty + STAGES;  // a chunk's accumulators are complete
-  uint64_t *acce = accf + 1;        // the drain warps have read them
-  uint64_t *done = acce + 1;        // every product this CTA issued has completed
+  uint64_t *accf = empty + STAGES;  // accumulator k's sums are complete
+  uint64_t *acce = accf + 4;        // the drain warps have read accumulator k
+  uint64_t *done = acce + 4;        // every product this CTA issued has completed
   uint32_t *tslot = (uint32_t *)(done + 1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       bar_init(&full[s], 1);
       bar_init(&empty[s], 1);
     }
-    bar_init(accf, 1);
-    bar_init(acce, EPI);
+    for (int k = 0; k < 4; ++k) {
+      bar_init(&accf[k], 1);
+      bar_init(&acce[k], EPI);
+    }
     bar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -365,7 +456,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tslot, 0);
 
   if (warp == 0) {
     if (lane == 0) {
@@ -376,20 +467,25 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
         const OzTile t = oz_tile<MODE>(p, q);
         // a Gram tile on the diagonal multiplies its rows by themselves: one operand
         const bool one = MODE == 2 && t.m0 == t.n0;
+        const int *list = MODE == 2 ? p.list + t.zb * p.lstride + t.k0 : nullptr;
+        int kb = MODE == 2 && t.kst > 0 ? list[0] : 0;  // read one step ahead
         for (int st = 0; st < t.kst; ++st, ++it) {
+          const int kb_next = MODE == 2 && st + 1 < t.kst ? list[st + 1] : 0;
           const int s = it % STAGES;
           if (it >= STAGES &&
               !bar_wait(&empty[s], ((it / STAGES) - 1) & 1, p.err, 1, p.wait_polls)) {
             go = false;
             break;
           }
-          bar_expect(&full[s], one ? OPB : STAGE);
+          // level 1 and 2 steps: the 128-byte slots only
+          const bool deep = MODE == 2 && st >= t.end01;
+          bar_expect(&full[s], (deep ? TILE0 : OPB) * (one ? 1 : 2));
           uint8_t *sa = smem + s * STAGE, *sb = sa + OPB;
           // coordinates (inner, 16-column block, ...): dense (0, kb, row, batch);
           // exchange A (0, st, 0, tile), B (0, l block, k, q); Gram (0, row, kb, tau)
           int ay, az, aw, by, bz, bw;
           if (MODE == 2) {
-            az = bz = t.k0 + st;
+            az = bz = kb;
             ay = t.m0;
             by = t.n0;
             aw = bw = t.zb;
@@ -409,61 +505,147 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
             bw = t.n0;                      // q
           }
           tma_load4(sa, &p.ta0, &full[s], 0, ay, az, aw);
-          tma_load4(sa + TILE0, &p.ta1, &full[s], 0, ay, az, aw);
+          if (!deep) tma_load4(sa + TILE0, &p.ta1, &full[s], 0, ay, az, aw);
           if (!one) {
             tma_load4(sb, &p.tb0, &full[s], 0, by, bz, bw);
-            tma_load4(sb + TILE0, &p.tb1, &full[s], 0, by, bz, bw);
+            if (!deep) tma_load4(sb + TILE0, &p.tb1, &full[s], 0, by, bz, bw);
           }
+          kb = kb_next;
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // MMA issuer
-      bool ok = true;
-      int it = 0, gc = 0;  // K steps and chunks issued so far (all tiles)
-      for (int q = blockIdx.x; q < p.tiles && ok; q += gridDim.x) {
-        const OzTile t = oz_tile<MODE>(p, q);
-        const uint32_t idesc = instr_desc_bf16(t.nw);
-        const uint32_t b_off = MODE == 2 && t.m0 == t.n0 ? 0u : (uint32_t)OPB;
-        for (int st = 0; st < t.kst; ++st, ++it) {
-          const int s = it % STAGES, cs = st % CHUNK;
-          if (cs == 0 && gc > 0) {
-            // the previous chunk's accumulators have been read
-            if (!bar_wait(acce, (gc - 1) & 1, p.err, 2, p.wait_polls)) {
-              ok = false;
-              break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;");
-          }
-          if (!bar_wait(&full[s], (it / STAGES) & 1, p.err, 3, p.wait_polls)) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t base_a = s_u32(smem + s * STAGE), base_b = base_a + b_off;
-#pragma unroll
-          for (int pa = 0; pa < OZ_S; ++pa)
-#pragma unroll
-            for (int pb = 0; pb < OZ_S - pa; ++pb) {
-              const int acc = min(pa + pb, 3);
-              // the first product into each accumulator in a chunk overwrites it
-              const uint32_t en = (cs > 0 || !(pa == 0 && pb <= 3)) ? 1u : 0u;
-              mma_bf16(tmem + (uint32_t)(acc * 128), digit_desc(base_a, pa),
-                       digit_desc(base_b, pb), idesc, en);
-            }
-          mma_commit(&empty[s]);
-          if (cs == CHUNK - 1 || st == t.kst - 1) {
-            mma_commit(accf);
-            ++gc;
-          }
-        }
+    // MMA issuer.  The whole warp runs the loop, so that descriptors and addresses are
+    // warp-uniform values, and one lane issues.  With the loop inside a one-lane branch the
+    // issue of a product took 72 cycles, more than the product itself (64).
+    constexpr uint32_t ALL = 0xffffffffu;
+    bool ok = true;
+    int s = 0;                        // stage of the next K step,
+    uint32_t ph = 0;                  // parity of its phase,
+    uint32_t drained = 0, ever = 0;   // parity of each accumulator's drains, and any yet
+    const uint32_t idesc = instr_desc_bf16();
+    const uint32_t base0 = s_u32(smem) >> 4;
+    for (int q = blockIdx.x; q < p.tiles && ok; q += gridDim.x) {
+      OzTile t = oz_tile<MODE>(p, q);
+      uint32_t b_off = MODE == 2 && t.m0 == t.n0 ? 0u : (uint32_t)OPB >> 4;
+      if (MODE == 2) {
+        // (values read from memory: made warp-uniform for the compiler too)
+        t.kst = __shfl_sync(ALL, t.kst, 0);
+        t.end01 = __shfl_sync(ALL, t.end01, 0);
+        t.end2 = __shfl_sync(ALL, t.end2, 0);
+        b_off = __shfl_sync(ALL, b_off, 0);
       }
-      // a drain that is still waiting sees its phase complete once the MMAs
-      // issued so far are done (and then stops on the error flag)
-      if (!ok) mma_commit(accf);
+      uint32_t fresh = 15;  // bit k: accumulator k starts again, its first product overwrites
+      unsigned long long tab = DRAINS;
+      int st = 0;
+      auto run = [&](auto level) {
+        constexpr int lev = decltype(level)::value;
+        const OzRun r = oz_run(t, lev);
+        for (; st < r.end; ++st) {
+          ok = __all_sync(ALL, bar_wait(&full[s], ph, p.err, 3, p.wait_polls));
+          if (!ok) return;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t a0 = base0 + s * (STAGE >> 4), b0 = a0 + b_off;
+          // accumulator k's last sums have been read
+          auto freed = [&](int k) {
+            if ((fresh & ever) >> k & 1) {
+              ok = ok && __all_sync(ALL, bar_wait(&acce[k], (drained >> k & 1) ^ 1, p.err, 2,
+                                                  p.wait_polls));
+              asm volatile("tcgen05.fence::after_thread_sync;");
+            }
+            return ok;
+          };
+          // level 0: the products of digits into accumulator k
+          auto level0 = [&](int k, uint32_t over) {
+#pragma unroll
+            for (int pa = 0; pa < OZ_S; ++pa)
+#pragma unroll
+              for (int pb = 0; pb < OZ_S - pa; ++pb) {
+                if (min(pa + pb, 3) != k) continue;
+                mma_bf16(tmem + (uint32_t)(k * 128), digit_desc(a0, pa), digit_desc(b0, pb), idesc,
+                         pa == 0 && pb == k ? over ^ 1u : 1u);
+              }
+          };
+          if (lev == 0) {
+            if (fresh == 0) {
+              if (elect_one()) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) level0(k, 0);
+                mma_commit(&empty[s]);
+              }
+            } else {
+              // an accumulator that is being read comes last
+              const bool late3 = fresh == 8;
+              if (!late3) {
+                if (freed(3) && elect_one()) level0(3, fresh >> 3);
+                __syncwarp();
+              }
+#pragma unroll
+              for (int k = 0; k < 3; ++k) {
+                if (freed(k) && elect_one()) level0(k, fresh >> k & 1);
+                __syncwarp();
+              }
+              if (late3) {
+                if (freed(3) && elect_one()) level0(3, 1);
+                __syncwarp();
+              }
+              if (elect_one()) mma_commit(&empty[s]);
+            }
+          } else if (lev == 1) {
+            // digits 1 to 4 in slots 0 to 3: (1, 1) into accumulator 2, the others into 3
+            if (freed(2) && freed(3) && elect_one()) {
+#pragma unroll
+              for (int pa = 1; pa < 5; ++pa)
+#pragma unroll
+                for (int pb = 1; pb < OZ_S - pa; ++pb) {
+                  const int k = pa + pb == 2 ? 2 : 3;
+                  mma_bf16(tmem + (uint32_t)(k * 128), digit_desc(a0, pa - 1),
+                           digit_desc(b0, pb - 1), idesc,
+                           pa == 1 && pb <= 2 ? (fresh >> k & 1) ^ 1u : 1u);
+                }
+              mma_commit(&empty[s]);
+            }
+          } else {
+            // digits 2 and 3 in slots 0 and 1, accumulator 3
+            if (freed(3) && elect_one()) {
+#pragma unroll
+              for (int q3 = 0; q3 < 3; ++q3)
+                mma_bf16(tmem + 3u * 128, digit_desc(a0, q3 == 2), digit_desc(b0, q3 == 1), idesc,
+                         q3 == 0 ? (fresh >> 3) ^ 1u : 1u);
+              mma_commit(&empty[s]);
+            }
+          }
+          __syncwarp();
+          if (!ok) return;
+          if (++s == STAGES) {
+            s = 0;
+            ph ^= 1;
+          }
+          fresh = 0;
+          if ((st & 3) != 3 && st + 1 != r.end) continue;
+          fresh = drains_after(tab, st, r);
+          if (elect_one()) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (fresh >> ((i + 3) & 3) & 1) mma_commit(&accf[(i + 3) & 3]);
+          }
+          __syncwarp();
+          drained ^= fresh;
+          ever |= fresh;
+        }
+      };
+      run(std::integral_constant<int, 0>{});
+      if (MODE == 2 && ok) run(std::integral_constant<int, 1>{});
+      if (MODE == 2 && ok) run(std::integral_constant<int, 2>{});
+    }
+    // a drain that is still waiting sees its phase complete once the MMAs
+    // issued so far are done (and then stops on the error flag)
+    if (elect_one()) {
+      if (!ok)
+        for (int k = 0; k < 4; ++k) mma_commit(&accf[k]);
       mma_commit(done);
     }
+    __syncwarp();
   } else {
     // drain warps: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (the
     // rows of its lane quarter) and columns 32 cq .. + 31 of each accumulator,
@@ -474,43 +656,53 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
     const int cq = (warp - 2) >> 2;
     const int fr = lane >> 2, fc = 2 * (lane & 3);
     bool ok = true;
-    int gc = 0;  // chunks drained so far (all tiles)
+    uint32_t drained = 0;  // parity bits of each accumulator's drains so far (all tiles)
     for (int q = blockIdx.x; q < p.tiles && ok; q += gridDim.x) {
-      const OzTile t = oz_tile<MODE>(p, q);
-      float hi[DC], lo[DC];
+      OzTile t = oz_tile<MODE>(p, q);
+      f2 hi[DC / 2], lo[DC / 2];  // pairs of neighbouring columns: values 2 c and 2 c + 1
 #pragma unroll
-      for (int c = 0; c < DC; ++c) hi[c] = lo[c] = 0.f;
-      const int nchunks = (t.kst + CHUNK - 1) / CHUNK;
-      for (int c = 0; c < nchunks; ++c, ++gc) {
-        if (!bar_wait(accf, gc & 1, p.err, 4, p.wait_polls) ||
-            (p.err && *(volatile int *)p.err)) {
-          ok = false;
-          break;
+      for (int c = 0; c < DC / 2; ++c) hi[c] = lo[c] = 0;
+      for (int st = 0; st < t.kst && ok; ++st) {
+        const uint32_t now = next_drains(t, st);
+        if (now == 0) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int k = (i + 3) & 3;
+          if (!ok || !(now >> k & 1)) continue;
+          ok = __all_sync(0xffffffffu,
+                          bar_wait(&accf[k], drained >> k & 1, p.err, 4, p.wait_polls) &&
+                              !(p.err && *(volatile int *)p.err));
+          if (!ok) continue;
+          drained ^= 1u << k;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t tl = tmem + ((uint32_t)(lq * 32 + 16 * h) << 16) +
+                                (uint32_t)(k * 128 + cq * DC);
+            uint32_t r[16];
+#pragma unroll
+            for (int g = 0; g < 4; ++g) tmem_ld16x256(tl + 8 * g, r + 4 * g);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (h == 1) {
+              // the accumulator is free for the next products (of this tile or the next)
+              asm volatile("tcgen05.fence::before_thread_sync;");
+              __syncwarp();
+              if (lane == 0) bar_arrive(&acce[k]);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const int c = 8 * h + u;
+              const f2 v = f2_pack(r[2 * u], r[2 * u + 1]);
+              if (k == 3)
+                lo[c] = f2_add(lo[c], v);
+              else
+                fold(hi[c], lo[c], v, k == 2);
+            }
+          }
         }
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        // (columns past nw hold nothing that is stored)
-        if (MODE != 2 || cq * DC < t.nw)
-#pragma unroll
-        for (int f = 0; f < 8; ++f) {
-          const uint32_t tl = tmem + ((uint32_t)(lq * 32 + 16 * (f >> 2)) << 16) +
-                              (uint32_t)(cq * DC + 8 * (f & 3));
-          uint32_t r0[4], r1[4], r2[4], r3[4];
-          tmem_ld16x256(tl, r0);
-          tmem_ld16x256(tl + 128, r1);
-          tmem_ld16x256(tl + 256, r2);
-          tmem_ld16x256(tl + 384, r3);
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            fold(hi[4 * f + u], lo[4 * f + u], __uint_as_float(r0[u]), __uint_as_float(r1[u]),
-                 __uint_as_float(r2[u]), __uint_as_float(r3[u]));
-        }
-        // the accumulators are free for the next chunk (of this tile or the next)
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncwarp();
-        if (lane == 0) bar_arrive(acce);
       }
       if (!ok) break;
+      t = oz_tile<MODE>(p, q);  // (again, so that the drains need not keep it)
       // assemble fp64 (while the issuer runs the next tile): C = +-2^(eA + eB - 14) (hi + lo).
       // A thread's four rows: hr = 2 h + (u >> 1), tile row 32 lq + 16 h + fr + 8 (u >> 1).
       double *dst[4];
@@ -525,12 +717,10 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
           v = i < p.M;
           if (v && !OZ_IN(t.zb * p.efa_bs + i, p.efa_cap, 10)) v = false;
           ea[hr] = v ? row_scale(p.efa[t.zb * p.efa_bs + i]) : 0;
-          if (MODE == 2)
-            dst[hr] = p.C + ((long long)t.zb * p.smax + t.split) * p.M * p.N + (long long)i * p.N;
-          else
-            dst[hr] = p.ksplit > 1 ? p.C + (long long)(t.zb * p.ksplit + t.split) * p.M * p.N +
-                                         (long long)i * p.N
-                                   : p.C + t.zb * p.sC + (long long)i * p.ldc;
+          dst[hr] = MODE == 2 || p.ksplit > 1
+                        ? p.C + (long long)(t.zb * p.ksplit + t.split) * p.M * p.N +
+                              (long long)i * p.N
+                        : p.C + t.zb * p.sC + (long long)i * p.ldc;
         } else {
           const int m = t.mt * 8 + (row >> 4), j = t.jt * 16 + (row & 15);
           v = m < p.M && j < p.M;
@@ -554,18 +744,18 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
         const int eb1 = two ? row_scale(p.efb[eb_off + j + 1]) - 14 : 0;
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
-          const int hr = 2 * (f >> 2) + rr, c = 4 * f + 2 * rr;
+          const int hr = 2 * (f >> 2) + rr, c = 2 * f + rr;
           if (!valid[hr]) continue;
           double *d = dst[hr] + j;
           if (!OZ_IN((long long)(d - p.C) + (two ? 1 : 0), p.ccap, 13)) continue;
           const double v0 = __longlong_as_double(
               (long long)((unsigned long long)__double_as_longlong(
-                              df_to_f64(hi[c], lo[c], ea[hr] + eb0)) ^
+                              df_to_f64(f2_lo(hi[c]), f2_lo(lo[c]), ea[hr] + eb0)) ^
                           sgn));
           if (two) {
             const double v1 = __longlong_as_double(
                 (long long)((unsigned long long)__double_as_longlong(
-                                df_to_f64(hi[c + 1], lo[c + 1], ea[hr] + eb1)) ^
+                                df_to_f64(f2_hi(hi[c]), f2_hi(lo[c]), ea[hr] + eb1)) ^
                             sgn));
             if (p.vec2) {
               *reinterpret_cast<double2 *>(d) = make_double2(v0, v1);
@@ -1051,7 +1241,8 @@ constexpr int GR = 32, GK = 64, GT = 32;
 __global__ void __launch_bounds__(256) oz_gram_max_kernel(const float2 *__restrict__ U,
                                                           const float2 *__restrict__ y, int n,
                                                           long long K, long long ldy, int nt,
-                                                          int slices, int *__restrict__ m) {
+                                                          int slices, int *__restrict__ m,
+                                                          float *__restrict__ bm) {
   __shared__ float us[GK][GR + 1];
   __shared__ float ys[GK][GT];
   __shared__ int sm[GR][GT + 1];
@@ -1077,6 +1268,16 @@ __global__ void __launch_bounds__(256) oz_gram_max_kernel(const float2 *__restri
       ys[k][t] = t0 + t < nt && k0 + k < K ? y[(long long)(t0 + t) * ldy + k0 + k].x : 0.f;
     }
     __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x < GK / KS * GR) {  // maxima of blocks of 16 columns
+      const int r = threadIdx.x % GR, q = threadIdx.x / GR;
+      const long long kb = (k0 >> 4) + q;
+      if (i0 + r < n && kb * KS < K) {
+        float v = 0.f;
+#pragma unroll
+        for (int u = 0; u < KS; ++u) v = fmaxf(v, us[q * KS + u][r]);
+        bm[kb * n + i0 + r] = v;
+      }
+    }
 #pragma unroll
     for (int u = 0; u < GK / 8; ++u) {
       const int k = warp * (GK / 8) + u;
@@ -1100,6 +1301,88 @@ __global__ void __launch_bounds__(256) oz_gram_max_kernel(const float2 *__restri
     const int r = e / GT, t = e % GT;
     if (i0 + r < n && t0 + t < nt && sm[r][t] > 0)
       atomicMax(&m[(long long)(t0 + t) * n + i0 + r], sm[r][t]);
+  }
+}
+
+// Level of a 16-column block at a tau point: how many leading digits are zero in
+// every row, from r = the largest |U_ik| y_tk 2^-e_i bounded by the block's maxima
+// (with 2^-20 to spare for the pairs' low parts): digits 0 .. L-1 vanish for r <= 2^-8L.
+//   0: all 21 digit products; 1: the 10 of digits 1-4; 2: the 3 of digits 2, 3;
+//   3: none (p + q >= 6), only the diagonal's level-6 sum; 4: nothing at all.
+// Leaving out products of digits that are zero changes no bit of the result; at
+// large tau the weights leave most blocks at the deeper levels.
+// One warp per block of columns: its row maxima stay in registers for all tau.
+constexpr int GRR = 1024 / 32;  // rows per lane at most (n <= 1024)
+__global__ void __launch_bounds__(256) oz_gram_level_kernel(
+    const float *__restrict__ bm, const float2 *__restrict__ y, const int *__restrict__ m, int n,
+    long long K, long long KB, int nt, unsigned char *__restrict__ lev) {
+  const long long kb = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (kb >= KB) return;
+  float b[GRR];
+  const int per = (n + 31) / 32;
+#pragma unroll
+  for (int q = 0; q < GRR; ++q) {
+    const int i = q * 32 + lane;
+    b[q] = q < per && i < n ? bm[kb * n + i] : 0.f;
+  }
+  const bool in = lane < KS && kb * KS + lane < K;
+  for (int t = 0; t < nt; ++t) {
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < GRR; ++q) {
+      if (q >= per) break;
+      const int i = q * 32 + lane;
+      // 2^-(E + 1), E the exponent of the row's maximum
+      const int se = i < n ? 127 - (((m[(long long)t * n + i] >> 23) & 0xFF) - 127 + 1) : 0;
+      v = fmaxf(v, b[q] * (se > 0 && se < 255 ? __int_as_float(se << 23) : 0.f));
+    }
+    const float yk = in ? y[(long long)t * KB * KS + kb * KS + lane].x : 0.f;
+    const float vm = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(v)));
+    const float ym = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(yk)));
+    const float r = vm * ym * (1.f + 0x1p-20f);
+    if (lane == 0)
+      lev[(long long)t * KB + kb] =
+          r > 0x1p-8f ? 0 : (r > 0x1p-16f ? 1 : (r > 0x1p-24f ? 2 : (r > 0x1p-32f ? 3 : 4)));
+  }
+}
+
+// Blocks of level 0, then 1, then 2 of tau point blockIdx.x, each in ascending order;
+// cnt[t] = how many of each; steps += 21, 10, 3 per block (the products' count).
+__global__ void __launch_bounds__(1024) oz_gram_list_kernel(const unsigned char *__restrict__ lev,
+                                                            long long KB, int *__restrict__ list,
+                                                            int *__restrict__ cnt,
+                                                            unsigned long long *__restrict__ steps) {
+  __shared__ int wsum[32];
+  const long long t = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  lev += t * KB;
+  list += t * KB;
+  int at = 0, c[3];
+  for (int L = 0; L < 3; ++L) {
+    const int at0 = at;
+    for (long long k0 = 0; k0 < KB; k0 += 1024) {
+      const long long kb = k0 + threadIdx.x;
+      const bool on = kb < KB && lev[kb] == L;
+      const unsigned b = __ballot_sync(0xffffffffu, on);
+      if (lane == 0) wsum[warp] = __popc(b);
+      __syncthreads();
+      const int w = wsum[lane];
+      int before = lane < warp ? w : 0, all = w;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        all += __shfl_xor_sync(0xffffffffu, all, o);
+      }
+      if (on) list[at + before + __popc(b & ((1u << lane) - 1))] = (int)kb;
+      at += all;
+      __syncthreads();
+    }
+    c[L] = at - at0;
+  }
+  if (threadIdx.x == 0) {
+    *reinterpret_cast<int4 *>(cnt + 4 * t) = make_int4(c[0], c[1], c[2], 0);
+    atomicAdd(steps, 21ull * c[0] + 10ull * c[1] + 3ull * c[2]);
   }
 }
 
@@ -1140,8 +1423,8 @@ __device__ __forceinline__ void pair_digits(float p, float q, float *d) {
 constexpr int GKB = 64;
 __global__ void __launch_bounds__(256) oz_gram_slice_kernel(
     const float2 *__restrict__ U, const float2 *__restrict__ y, int n, long long K, long long ldy,
-    const int *__restrict__ m, int *__restrict__ ef, __nv_bfloat16 *__restrict__ out, long long g1,
-    float *__restrict__ lev6) {
+    const int *__restrict__ m, const unsigned char *__restrict__ lev, int *__restrict__ ef,
+    __nv_bfloat16 *__restrict__ out, long long g1, float *__restrict__ lev6) {
   __shared__ float l6[4][GR];
   const int b = blockIdx.z;
   const int half = threadIdx.x & 1, rl = (threadIdx.x >> 1) & 31, kq = threadIdx.x >> 6;
@@ -1160,6 +1443,8 @@ __global__ void __launch_bounds__(256) oz_gram_slice_kernel(
   if (row)
 #pragma unroll 2
     for (long long kb = (long long)blockIdx.x * GKB + kq; kb < kb1; kb += 4) {
+      const int L = lev[b * KB + kb];
+      if (L > 3) continue;
       const long long k0 = kb * KS + half * KC;
       const float4 *src = reinterpret_cast<const float4 *>(U + (kb * n + r) * KS + half * KC);
       const float4 *yw = reinterpret_cast<const float4 *>(y + (long long)b * ldy + k0);
@@ -1191,10 +1476,21 @@ __global__ void __launch_bounds__(256) oz_gram_slice_kernel(
       }
       const long long blk = ((long long)b * KB + kb) * n + r;
       if (!OZ_IN(blk * 64 + 63, g1, 36)) continue;
-#pragma unroll
-      for (int dgt = 0; dgt < OZ_S; ++dgt)
-        *reinterpret_cast<uint4 *>(out + digit_off(blk, half * KC, dgt, g1)) =
+      // the digits the block's level multiplies, from slot 0 on
+      auto put = [&](int slot, int dgt) {
+        *reinterpret_cast<uint4 *>(out + digit_off(blk, half * KC, slot, g1)) =
             make_uint4(o[dgt][0], o[dgt][1], o[dgt][2], o[dgt][3]);
+      };
+      if (L == 0) {
+#pragma unroll
+        for (int dgt = 0; dgt < OZ_S; ++dgt) put(dgt, dgt);
+      } else if (L == 1) {
+#pragma unroll
+        for (int dgt = 1; dgt < 5; ++dgt) put(dgt - 1, dgt);
+      } else if (L == 2) {
+        put(0, 2);
+        put(1, 3);
+      }
     }
   s6 += __shfl_xor_sync(0xffffffffu, s6, 1);
   if (half == 0) l6[kq][rl] = s6;
@@ -1218,29 +1514,18 @@ __global__ void oz_gram_diag_kernel(const float *__restrict__ lev6, const int *_
   if (lane == 0) diag[r] = scalbn(s, 2 * row_scale(ef[r]) - 14);
 }
 
-// out[t][i][j] (+)= -scale 2^(2 e_t) sum_s work[t][s][i][j] over the splits of the tile
-// of (min, max) of i and j, in order.
-struct GramSplits {
-  int T, smax;
-  short ks[GRAM_TILES][GRAM_TILES];
-};
-__global__ void oz_gram_reduce_kernel(const double *__restrict__ work, const GramSplits sp, int n,
-                                      int nt, double scale, const int *__restrict__ yexp,
-                                      int accumulate, const double *__restrict__ diag,
-                                      double *__restrict__ out) {
+// out[t][i][j] (+)= -scale 2^(2 e_t) sum_s work[t][s][min][max of i and j], in order of s.
+__global__ void oz_gram_reduce_kernel(const double *__restrict__ work, int ks, int n, int nt,
+                                      double scale, const int *__restrict__ yexp, int accumulate,
+                                      const double *__restrict__ diag, double *__restrict__ out) {
   const long long nn = (long long)n * n, tot = nn * nt;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
        e += (long long)gridDim.x * blockDim.x) {
     const long long t = e / nn, r = e - t * nn;
-    int i = (int)(r / n), j = (int)(r - (long long)i * n);
-    if (i > j) {
-      const int x = i;
-      i = j;
-      j = x;
-    }
-    const int ks = sp.ks[i / BM][j / BN];
-    const double *p = work + t * sp.smax * nn + (long long)i * n + j;
+    const int i = (int)(r / n), j = (int)(r - (long long)i * n);
+    const double *p = work + t * ks * nn + (long long)min(i, j) * n + max(i, j);
     double s = 0.0;
+#pragma unroll 8
     for (int k = 0; k < ks; ++k) s += p[k * nn];
     if (i == j) s += diag[t * n + i];
     s = -scale * scalbn(s, 2 * yexp[t]);
@@ -1616,69 +1901,48 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
   return cudaSuccess;
 }
 
-// Gram matrices at N = 200 (100 virtual orbitals, 64 tau points): 1.38 ms per tau
-// point for the products (1,125 TFLOP/s of issued tensor work; 72-row tiles read
-// as much shared memory as 128-row ones) and 0.72 ms for the digits (HBM); the
-// whole setup and sampling call takes 177 ms against 281 with the contraction
-// over the kept pairs (exchange 136, dense products 60, digits 48).  With rows of
-// digits K-contiguous over the whole contraction, 12 MB apart, the same products
-// took 2.2 ms: their 128-byte pieces came from 128 different DRAM pages.
+// Gram matrices at n = 200 (100 virtual orbitals, 64 tau points): 0.83 ms for the
+// products of a tau point with all digits (1,600 TFLOP/s) and 53 ms for all 64 (blocks of
+// columns that are small at a tau point have only their leading digits multiplied),
+// against 88 ms with all 21 products of every block; the digits take 32 ms (HBM).  The
+// whole setup and sampling call takes 124 ms against 281 with the contraction over the
+// kept pairs (exchange 136, dense products 60, digits 48).  With rows of digits
+// K-contiguous over the whole contraction, 12 MB apart, the products took 1.6 times as
+// long: their 128-byte pieces came from 128 different DRAM pages.  A narrower last column
+// tile (80 of 128 columns) does not help: the products are not faster below 128 columns
+// (A's rows are read from shared memory whatever the width), and 1,139 us became 1,003.
 namespace {
-// Tile types of a Gram matrix and the K split of each.  The tiles on and above
-// the diagonal differ in cost (the last column is narrower), so each type's K
-// is split in proportion: the splits of all types take about L K steps of a
-// full tile, and L is the one for which the rounds of tiles over the SMs,
-// times L plus a tile's drain and stores (~9 steps), come out least.
+// The tiles on and above the diagonal, and the K splits of each: as many as make the
+// rounds of tiles over the SMs, times a split's K steps plus a tile's drain and stores
+// (~9 steps), and the partial sums' traffic, come out least.
 struct GramPlan {
-  int T = 0, types = 0, per_batch = 0, smax = 0;
-  int tm[GRAM_TYPES], tn[GRAM_TYPES], ks[GRAM_TYPES], kst[GRAM_TYPES];
+  int types = 0, ks = 0;
+  int tm[GRAM_TYPES], tn[GRAM_TYPES];
 };
 bool gram_plan(const OzGram &g, GramPlan *pl) {
-  pl->T = ceil_div(g.n, BM);
-  if (pl->T > GRAM_TILES) return false;
+  const int T = ceil_div(g.n, BM);
+  if (T > GRAM_TILES) return false;
   const long long steps = (g.K + KS - 1) / KS;
-  double w[GRAM_TYPES];
   pl->types = 0;
-  for (int i = 0; i < pl->T; ++i)
-    for (int j = i; j < pl->T; ++j) {
+  for (int i = 0; i < T; ++i)
+    for (int j = i; j < T; ++j) {
       pl->tm[pl->types] = i;
-      pl->tn[pl->types] = j;
-      // A's rows are read from shared memory whatever the width
-      w[pl->types++] = 0.25 + 0.75 * std::min(BN, (g.n - j * BN + 15) / 16 * 16) / BN;
+      pl->tn[pl->types++] = j;
     }
-  double wsum = 0;
-  for (int y = 0; y < pl->types; ++y) wsum += w[y];
+  const long long tiles = (long long)pl->types * g.nt;
   double best = 0;
-  bool have = false;
+  pl->ks = 0;
   for (int rounds = 1; rounds <= 24; ++rounds) {
-    // L such that about rounds * 152 tiles are made
-    const double L = std::max(8.0, (double)steps * wsum * g.nt / (rounds * 152.0 * 0.985));
-    long long items = 0;
-    int smax = 0;
-    GramPlan c = *pl;
-    double longest = 0;
-    for (int y = 0; y < pl->types; ++y) {
-      long long ks = std::max<long long>(1, (long long)(steps * w[y] / L + 0.5));
-      ks = std::min<long long>({ks, steps, 512});
-      c.kst[y] = (int)((steps + ks - 1) / ks);
-      c.ks[y] = (int)((steps + c.kst[y] - 1) / c.kst[y]);
-      items += c.ks[y];
-      smax = std::max(smax, c.ks[y]);
-      longest = std::max(longest, c.kst[y] * w[y]);
-    }
-    const double cost = (double)((items * g.nt + 151) / 152) * (longest + 9.0) +
-                        (double)items * g.nt * BM * BN * 16.0 / 5.3e6;
-    if (!have || cost < best) {
-      have = true;
+    const long long ks =
+        std::min<long long>({std::max<long long>(1, rounds * 152LL / tiles), steps, 512});
+    const double cost = (double)((ks * tiles + 151) / 152) * ((double)((steps + ks - 1) / ks) + 9.0) +
+                        (double)ks * tiles * BM * BN * 16.0 / 5.3e6;
+    if (pl->ks == 0 || cost < best) {
       best = cost;
-      c.per_batch = (int)items;
-      c.smax = smax;
-      c.T = pl->T;
-      c.types = pl->types;
-      *pl = c;
+      pl->ks = (int)ks;
     }
   }
-  return pl->per_batch <= 32767 && pl->smax <= 32767;
+  return true;
 }
 }  // namespace
 
@@ -1687,28 +1951,46 @@ size_t oz_gram_lev6_floats(const OzGram &g) {
 }
 size_t oz_gram_work(const OzGram &g) {
   GramPlan pl;
-  return gram_plan(g, &pl) ? (size_t)g.nt * pl.smax * g.n * g.n : 0;
+  return gram_plan(g, &pl) ? (size_t)g.nt * pl.ks * g.n * g.n : 0;
 }
-double oz_gram_flops(const OzGram &g) {
-  GramPlan pl;
-  if (!gram_plan(g, &pl)) return 0.0;
+double oz_gram_step_flops(int n) {
   double f = 0.0;
-  for (int y = 0; y < pl.types; ++y)
-    f += OZ_PRODUCTS * 2.0 * BM * std::min(BN, (g.n - pl.tn[y] * BN + 15) / 16 * 16) * (double)KS *
-         pl.kst[y] * pl.ks[y];
-  return f * g.nt;
+  for (int i = 0; i < n; i += BM)
+    for (int j = i; j < n; j += BN) f += 2.0 * BM * BN * (double)KS;
+  return f;
 }
 
-cudaError_t oz_gram_max(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
-                        int *m, cudaStream_t s) {
+size_t oz_gram_sel_bytes(int n, long long ldy, int nt) {
+  const size_t kb = ldy / KS;
+  return kb * n * sizeof(float) + (size_t)nt * kb * (sizeof(int) + 1) + (size_t)nt * 16 + 64;
+}
+OzGramSel oz_gram_sel(void *buf, int n, long long ldy, int nt) {
+  const size_t kb = ldy / KS;
+  OzGramSel v;
+  v.cnt = static_cast<int *>(buf);
+  v.bm = reinterpret_cast<float *>(v.cnt + 4 * (size_t)nt);
+  v.list = reinterpret_cast<int *>(v.bm + kb * n);
+  v.lev = reinterpret_cast<unsigned char *>(v.list + (size_t)nt * kb);
+  return v;
+}
+
+cudaError_t oz_gram_select(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
+                           int *m, const OzGramSel &v, unsigned long long *steps, cudaStream_t s) {
   if (n <= 0 || nt <= 0 || K <= 0) return cudaSuccess;
+  if (n > GRR * 32) return cudaErrorInvalidValue;
   RS_TRY(cudaMemsetAsync(m, 0, (size_t)nt * n * sizeof(int), s));
-  const long long pieces = (K + GK - 1) / GK;
+  const long long pieces = (K + GK - 1) / GK, KB = ldy / KS;
   dim3 g(ceil_div(nt, GT), ceil_div(n, GR), 1);
   const int slices = (int)std::max<long long>(
       1, std::min<long long>({pieces, 152LL * 8 / (g.x * g.y) + 1, 65535}));
   g.z = slices;
-  oz_gram_max_kernel<<<g, 256, 0, s>>>(U, y, n, K, ldy, nt, slices, m);
+  oz_gram_max_kernel<<<g, 256, 0, s>>>(U, y, n, K, ldy, nt, slices, m, v.bm);
+  ++launch_counter();
+  RS_TRY(cudaGetLastError());
+  oz_gram_level_kernel<<<ceil_div(KB * 32, 256), 256, 0, s>>>(v.bm, y, m, n, K, KB, nt, v.lev);
+  ++launch_counter();
+  RS_TRY(cudaGetLastError());
+  oz_gram_list_kernel<<<nt, 1024, 0, s>>>(v.lev, KB, v.list, v.cnt, steps);
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -1717,7 +1999,7 @@ cudaError_t oz_gram_slice(const OzGram &g, cudaStream_t s) {
   if (g.ldy % KS || ((uintptr_t)g.U % 16) || ((uintptr_t)g.y % 16) || g.nt > 65535)
     return cudaErrorInvalidValue;
   dim3 gr(ceil_div(g.ldy, (long long)GKB * KS), ceil_div(g.n, GR), g.nt);
-  oz_gram_slice_kernel<<<gr, 256, 0, s>>>(g.U, g.y, g.n, g.K, g.ldy, g.m, g.ef, g.d,
+  oz_gram_slice_kernel<<<gr, 256, 0, s>>>(g.U, g.y, g.n, g.K, g.ldy, g.m, g.lev, g.ef, g.d,
                                           (long long)g.nt * g.n * g.ldy * 4, g.lev6);
   ++launch_counter();
   RS_TRY(cudaGetLastError());
@@ -1749,33 +2031,24 @@ cudaError_t oz_gram(const OzGram &g, double *work, cudaStream_t s) {
   p.tb0 = p.ta0;
   p.tb1 = p.ta1;
   p.M = p.N = g.n;
-  p.ksplit = 2;
+  p.ksplit = pl.ks;
   p.efa = p.efb = g.ef;
   p.efa_bs = p.efb_bs = g.n;
   p.C = work;
   p.vec2 = (uintptr_t)work % 16 == 0 && g.n % 2 == 0;
   p.err = g.err;
-  p.ccap = (long long)g.nt * pl.smax * g.n * g.n;
+  p.ccap = (long long)g.nt * pl.ks * g.n * g.n;
   p.efa_cap = p.efb_cap = (long long)g.nt * g.n;
   p.wait_polls = g.wait_polls;
+  p.list = g.list;
+  p.cnt = g.cnt;
+  p.lstride = g.ldy / KS;
   p.ntypes = pl.types;
-  p.per_batch = pl.per_batch;
-  p.smax = pl.smax;
-  GramSplits sp;
-  std::memset(&sp, 0, sizeof(sp));
-  sp.T = pl.T;
-  sp.smax = pl.smax;
-  int at = 0;
   for (int y = 0; y < pl.types; ++y) {
     p.tm[y] = (unsigned char)pl.tm[y];
     p.tn[y] = (unsigned char)pl.tn[y];
-    p.first[y] = (short)at;
-    p.tkst[y] = pl.kst[y];
-    at += pl.ks[y];
-    sp.ks[pl.tm[y]][pl.tn[y]] = (short)pl.ks[y];
   }
-  p.first[pl.types] = (short)at;
-  const long long tiles = (long long)pl.per_batch * g.nt;
+  const long long tiles = (long long)pl.types * pl.ks * g.nt;
   if (tiles > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
   p.tiles = (int)tiles;
   RS_TRY(prepare());
@@ -1784,7 +2057,7 @@ cudaError_t oz_gram(const OzGram &g, double *work, cudaStream_t s) {
   RS_TRY(cudaGetLastError());
   const long long tot = (long long)g.nt * g.n * g.n;
   oz_gram_reduce_kernel<<<(int)std::min<long long>((tot + 255) / 256, 152 * 8), 256, 0, s>>>(
-      work, sp, g.n, g.nt, g.scale, g.yexp, g.accumulate, g.diag, g.out);
+      work, pl.ks, g.n, g.nt, g.scale, g.yexp, g.accumulate, g.diag, g.out);
   ++launch_counter();
   return cudaGetLastError();
 }

@@ -12,14 +12,13 @@
 // A product sum_k a_k b_k is then 2^(eA+eB-14) sum_{p,q} sum_k D^A_p D^B_q.
 // Every bf16 x bf16 product of digits is exact in fp32, and a level
 // p + q = L sums terms on the common grid 2^(-8L) with at most
-// (L+1) 2^14 grid units each; over 256 terms of K the levels L = 0, 1, 2
-// stay below 2^24 grid units, so the tensor core's fp32 accumulation of them
-// is exact.  Levels 3 to 5 (p + q <= 5 are kept: 21 digit products; the
+// (L+1) 2^14 grid units each; over 768, 384 and 256 terms of K the levels L = 0,
+// 1, 2 stay below 0.75 2^24 grid units, so the tensor core's fp32 accumulation
+// of them is exact.  Levels 3 to 5 (p + q <= 5 are kept: 21 digit products; the
 // dropped ones are below 2^-46 of the row maxima's product) share a fourth
 // accumulator, which is ~2^-24 of the result and rounds at ~2^-48 of it.
-// After every 256 terms of K the four accumulators are added into
-// double-float (fp32 pair) running totals; the fp64 result is assembled once
-// per output.
+// After that many terms of K an accumulator is added into double-float (fp32
+// pair) running totals; the fp64 result is assembled once per output.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -119,18 +118,32 @@ double oz_exch_flops(const OzExch &x);
 // Y_t Y_t^T with Y_t,ik = U_ik y_tk, y [nt][K] pairs (rows of stride ldy, a multiple
 // of 16), e_t = yexp[t], and U [n x K] pairs in blocks of 16 columns, column
 // 16 kb + u of row i at U[(kb n + i) 16 + u], so that U and the digits (in the same
-// order, 128 + 64 bytes per row and block) are streamed in whole pieces.  oz_gram_max finds
-// each row's largest magnitude per tau point (m[t][i], fp32 bits), oz_gram_slice
-// writes the digits of nt tau points (d: OZ_S nt n ldy values, ef[t][i]) and the
-// digit products of the diagonal that the tensor cores leave out (lev6, diag),
-// and oz_gram multiplies them on the tensor cores: the tiles on and above the
-// diagonal, each tile's K split over CTAs, the partial sums in `work`
-// (oz_gram_work() doubles) added in a fixed order; n <= 1024.
+// order, 128 + 64 bytes per row and block) are streamed in whole pieces.
+// oz_gram_select finds each row's largest magnitude per tau point (m[t][i], fp32
+// bits) and, per tau point, which blocks of columns have which digits to multiply
+// (OzGramSel); oz_gram_slice writes those digits for nt tau points (d: OZ_S nt n ldy
+// values, ef[t][i]) and the digit products of the diagonal that the tensor cores
+// leave out (lev6, diag), and oz_gram multiplies them on the tensor cores: the
+// tiles on and above the diagonal, each tile's K split over CTAs, the partial sums
+// in `work` (oz_gram_work() doubles) added in a fixed order; n <= 1024.
+struct OzGramSel {
+  float *bm = nullptr;           // [ldy / 16][n] block maxima of |U|
+  unsigned char *lev = nullptr;  // [nt][ldy / 16] levels
+  int *list = nullptr;           // [nt][ldy / 16] the blocks of level 0, 1, 2
+  int *cnt = nullptr;            // [nt][4] how many of each
+};
+size_t oz_gram_sel_bytes(int n, long long ldy, int nt);
+OzGramSel oz_gram_sel(void *buf, int n, long long ldy, int nt);
+// steps: += the digit products of all listed blocks (per tile)
+cudaError_t oz_gram_select(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
+                           int *m, const OzGramSel &v, unsigned long long *steps, cudaStream_t s);
 struct OzGram {
   int n = 0, nt = 1;
   long long K = 0, ldy = 0;
   const float2 *U = nullptr, *y = nullptr;
   const int *m = nullptr;
+  const unsigned char *lev = nullptr;
+  const int *list = nullptr, *cnt = nullptr;  // from the first of the nt tau points
   __nv_bfloat16 *d = nullptr;
   int *ef = nullptr;
   double scale = 1.0;
@@ -144,9 +157,8 @@ struct OzGram {
 };
 size_t oz_gram_lev6_floats(const OzGram &g);
 size_t oz_gram_work(const OzGram &g);
-double oz_gram_flops(const OzGram &g);
-cudaError_t oz_gram_max(const float2 *U, const float2 *y, int n, long long K, long long ldy, int nt,
-                        int *m, cudaStream_t s);
+// Tensor flops of one digit product of one block, all tiles.
+double oz_gram_step_flops(int n);
 cudaError_t oz_gram_slice(const OzGram &g, cudaStream_t s);
 cudaError_t oz_gram(const OzGram &g, double *work, cudaStream_t s);
 

@@ -113,3 +113,27 @@ def test_orbitals_that_are_not_orthonormal_keep_the_general_form(B):
     o = B.Handle.options(0.02, 1e-2, 7, 5)
     a, b = both(B, s, o)
     close(a, b, 1e-12)
+
+
+# Blocks of 16 columns that are small at a tau point have only their leading digits
+# multiplied on the tensor cores: at large tau most triples are, so that all levels occur,
+# in runs of whatever length, with n below and above one 128-row tile.  A digit product
+# that is left out (p + q >= 6) is at most 2^-46 of the product of its rows' maxima, of
+# either sign, a handful per term: over the K = n_occ n_virt^2 terms they add up like
+# sqrt(K) 2^-46 of the largest element, taken 8 times.
+@pytest.mark.parametrize("n,n_occ", [(37, 11), (130, 40)])
+def test_gram_levels(B, n, n_occ):
+    s = synth.make_system(n, n_occ, 3 * n, 24, input_seed=n)
+    tol = 8.0 * n_occ ** 0.5 * (n - n_occ) * 2.0 ** -46
+    sig = {}
+    for dd in (0, 2):
+        h = B.Handle(0)
+        o = B.Handle.options(0.0, 0.0, 2, 1, dd_arith=dd)
+        h.setup(*[torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in
+                  (s.eri3, s.metric, s.orb_e, s.orb_c, s.tau, s.tau_w)],
+                n_occ=s.n_occ, mu=s.mu, beta=s.beta, opts=o)
+        h.sigma(o, torch.empty((s.n_tau, n, n), dtype=torch.float64, device="cuda"))
+        sig[dd] = h.export("SIGMA_DD").reshape(s.n_tau, n, n)
+        h.close()
+    for x, y in zip(sig[2], sig[0]):
+        assert np.abs(x - y).max() <= tol * np.abs(y).max()
