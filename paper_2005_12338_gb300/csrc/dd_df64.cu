@@ -5,6 +5,7 @@
 // a dozen fp32 operations replace one DFMA, at ~1e-13 relative error.
 #include <climits>
 #include <algorithm>
+#include <cmath>
 
 #include "dd_arith.cuh"
 #include "dd_df64.cuh"
@@ -114,6 +115,13 @@ struct DfGeo {
 };
 using G64 = DfGeo<16, 16, 4, 4, 16, 2, 4>;
 using G40 = DfGeo<8, 8, 5, 5, 8, 6, 1>;
+// 24- and 16-wide tiles of 64 threads for products that would be a few 64-wide
+// tiles only (the metric root of a small N_aux: a lone 64-wide tile keeps one SM busy
+// for tens of microseconds and the others idle).  Slabs of 8 like G40's: the running
+// pair is renormalised after every slab, and with slabs of 16 V^{-1/2} at N_aux = 80 to
+// 270 was 1.3 times further from its value than with G40.
+using G24 = DfGeo<8, 8, 3, 3, 8, 8, 2>;
+using G16 = DfGeo<8, 8, 2, 2, 8, 12, 4>;
 
 template <class GEO, int MODE, int TA, int TB, int OUT>
 __global__ void __launch_bounds__(GEO::NT, GEO::MINB) df_gemm_kernel(
@@ -354,6 +362,31 @@ void df_plan(const DfGemm &g, int *ks_out, int *kc_out) {
   *ks_out = std::max(1, ceil_div(g.K, kc));
 }
 
+// The geometry of a product: for one product with an fp64 result (the setup's) by
+// a time model (the metric root at N_aux = 60 to 600: 2.6-8.3 -> 1.3-5.4 ms, the setup
+// with it), the padded work per SM over how well the resident warps fill it;
+// else (batches, pair results: chain and block) by the padding alone, so that
+// the number of pairs in a batch never changes a pair's result.
+enum { DF_G64 = 0, DF_G40, DF_G24, DF_G16 };
+template <class GEO> double df_time(const DfGemm &g, double cost) {
+  int ks, kc;
+  df_plan<GEO>(g, &ks, &kc);
+  const double tm = ceil_div(g.M, GEO::BM), tn = ceil_div(g.N, GEO::BN);
+  const double ctas = std::ceil((g.sym ? tm * (tm + 1) / 2 : tm * tn) * ks / 152.0);
+  const double warps = std::min(ctas, (double)GEO::MINB) * GEO::NT / 32;
+  return ctas * GEO::BM * GEO::BN * kc * cost / std::min(1.0, warps / 12.0);
+}
+int df_pick(const DfGemm &g) {
+  if (g.batch != 1 || !g.C64) return use_g40(g.M, g.N) ? DF_G40 : DF_G64;
+  // costs: measured rates per padded output (4.67, 3.8, 4.15, 3.85 TFLOP/s)
+  const double t[4] = {df_time<G64>(g, 1.0), df_time<G40>(g, 1.23), df_time<G24>(g, 1.13),
+                       df_time<G16>(g, 1.21)};
+  int best = 0;
+  for (int k = 1; k < 4; ++k)
+    if (t[k] < 0.95 * t[best]) best = k;
+  return best;
+}
+
 template <class GEO>
 cudaError_t df_gemm_geo(const DfGemm &g, double *work, size_t work_elems, cudaStream_t s) {
   int ks, kc;
@@ -396,14 +429,19 @@ cudaError_t df_gemm(const DfGemm &g, double *work, size_t work_elems, cudaStream
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if ((g.C64 == nullptr) == (g.C2 == nullptr)) return cudaErrorInvalidValue;
   if (g.sym && (g.M != g.N || !g.C64 || g.batch != 1)) return cudaErrorInvalidValue;
-  return use_g40(g.M, g.N) ? df_gemm_geo<G40>(g, work, work_elems, s)
-                           : df_gemm_geo<G64>(g, work, work_elems, s);
+  switch (df_pick(g)) {
+    case DF_G40: return df_gemm_geo<G40>(g, work, work_elems, s);
+    case DF_G24: return df_gemm_geo<G24>(g, work, work_elems, s);
+    case DF_G16: return df_gemm_geo<G16>(g, work, work_elems, s);
+    default: return df_gemm_geo<G64>(g, work, work_elems, s);
+  }
 }
 
 double df_gemm_flops(const DfGemm &g) {
   if (!g.sym) return 2.0 * g.M * (double)g.N * g.K * g.batch;
   // symmetric: only the tiles on and above the diagonal are computed
-  const int bm = use_g40(g.M, g.N) ? G40::BM : G64::BM;
+  const int edges[4] = {G64::BM, G40::BM, G24::BM, G16::BM};
+  const int bm = edges[df_pick(g)];
   const int t = ceil_div(g.M, bm);
   double f = 0.0;
   for (int i = 0; i < t; ++i)
@@ -414,8 +452,12 @@ double df_gemm_flops(const DfGemm &g) {
 
 size_t df_gemm_work(const DfGemm &g) {
   int ks, kc;
-  if (use_g40(g.M, g.N)) df_plan<G40>(g, &ks, &kc);
-  else df_plan<G64>(g, &ks, &kc);
+  switch (df_pick(g)) {
+    case DF_G40: df_plan<G40>(g, &ks, &kc); break;
+    case DF_G24: df_plan<G24>(g, &ks, &kc); break;
+    case DF_G16: df_plan<G16>(g, &ks, &kc); break;
+    default: df_plan<G64>(g, &ks, &kc);
+  }
   return ks > 1 ? (size_t)ks * g.M * g.N : 0;
 }
 

@@ -3,7 +3,7 @@
 // On GB300 the fp64 ceiling is the scalar DFMA pipe (two fp64 FMAs per clock
 // per SM, about 1.2 TFLOP/s for the GPU; the fp64 mma.sync path is slower),
 // so these are register-tiled SIMT kernels: an output tile per block (64, 40,
-// 48 or 100 wide, 4x4 or 5x5 outputs per thread), K slabs double-buffered
+// 48, 100, 24 or 16 wide, 2x2 to 5x5 outputs per thread), K slabs double-buffered
 // through shared memory with coalesced global loads for either operand
 // layout.  Since the DFMA pipe is the bound, the work that matters is the
 // zero-padded part of the edge tiles; the tile is chosen per problem shape.
@@ -31,9 +31,14 @@ using T64 = Tile<64, 64, 16, 4, 4>;
 using T40 = Tile<40, 40, 8, 4, 4>;
 using T48 = Tile<48, 48, 16, 4, 4>;
 using T100 = Tile<100, 100, 8, 5, 5>;
-constexpr int kNumTiles = 4;
-constexpr int kTileEdge[kNumTiles] = {64, 40, 48, 100};
-constexpr int kTileDepth[kNumTiles] = {16, 8, 16, 8};
+// small products (the metric root of a small N_aux, a few hundred outputs): one
+// 64-wide tile would keep the fp64 pipe of one SM busy for tens of microseconds
+// (N = 20, N_aux = 60: setup and sampling 2.67 -> 1.47 ms; N = 100: 85.2 -> 80.7)
+using T24 = Tile<24, 24, 16, 3, 3>;
+using T16 = Tile<16, 16, 16, 2, 2>;
+constexpr int kNumTiles = 6;
+constexpr int kTileEdge[kNumTiles] = {64, 40, 48, 100, 24, 16};
+constexpr int kTileDepth[kNumTiles] = {16, 8, 16, 8, 16, 16};
 // split-K planning always uses the 64-wide reference tile, so the chunking of
 // K (and therefore the result) does not depend on the tile shape chosen.
 constexpr int RBM = 64, RBN = 64, RBK = 16;
@@ -232,6 +237,8 @@ cudaError_t launch_tile(int tile, const GemmArgs &g, int ks, int kc, int b0, int
     case 1: return launch_strided<T40>(g, ks, kc, b0, nb, work, s);
     case 2: return launch_strided<T48>(g, ks, kc, b0, nb, work, s);
     case 3: return launch_strided<T100>(g, ks, kc, b0, nb, work, s);
+    case 4: return launch_strided<T24>(g, ks, kc, b0, nb, work, s);
+    case 5: return launch_strided<T16>(g, ks, kc, b0, nb, work, s);
     default: return launch_strided<T64>(g, ks, kc, b0, nb, work, s);
   }
 }
@@ -383,6 +390,8 @@ cudaError_t dgemm_segmented(int batch, int M, int N, const int *seg, const int *
       case 1: e = launch_segmented<T40>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s); break;
       case 2: e = launch_segmented<T48>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s); break;
       case 3: e = launch_segmented<T100>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s); break;
+      case 4: e = launch_segmented<T24>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s); break;
+      case 5: e = launch_segmented<T16>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s); break;
       default: e = launch_segmented<T64>(nb, M, N, sg, col, A, lda, B, ldb, Cb, ldc, sC, s);
     }
     RS_TRY(e);
