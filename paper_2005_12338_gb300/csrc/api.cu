@@ -1522,6 +1522,12 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   RS_CK(ensure(h->Gb, (size_t)nt * nn * sizeof(double)));
   RS_CK(ensure(h->sdd, (size_t)nt * nn * sizeof(double)));
   const bool mo = P > 0 && !g_in && use_mo_block(h, dd_arith);
+  // The sliced Gram matrix of a small system takes IEEE fp64 instead: the digits'
+  // truncation of 5e-13 is nowhere less than the pair contraction's up to n = 32 (3e-13 to
+  // 7e-13; 4e-13 against 3e-12 at n = 90), and fp64 is as fast there (n = 27: a few tens of
+  // microseconds).  (Test mode keeps the kernels whose waits it tests.)
+  const int mo_arith =
+      dd_arith == RSSRI_DD_OZ && n <= 32 && !h->test_wait_polls ? RSSRI_DD_FP64 : dd_arith;
   const bool dd_df64 = P > 0 && !mo && dd_arith == RSSRI_DD_DF64;
   const bool dd_oz = P > 0 && !mo && dd_arith == RSSRI_DD_OZ;
   if (P > 0 && !mo) RS_CK(ensure_d(h));
@@ -1587,7 +1593,7 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
     RS_CK(mo_range_check(G, nt, nn, range_flag(h), s));
     RS_CK(mo_range_check(Gb, nt, nn, range_flag(h), s));
   }
-  if (mo) RS_CK(block_mo(h, dd_arith, h->sdd.as<double>()));
+  if (mo) RS_CK(block_mo(h, mo_arith, h->sdd.as<double>()));
   for (int t = 0; t < nt && !mo; ++t) {
     double *out = h->sdd.as<double>() + t * nn;
     if (dd_oz) {
@@ -1601,7 +1607,7 @@ int build_block(rssri_handle *h, int dd_arith, const double *g_in, const double 
   if (dd_arith == RSSRI_DD_OZ || h->setup_arith == RSSRI_DD_OZ) {
     const int rc = oz_waits(h);
     if (rc) return rc;
-    if (mo && dd_arith == RSSRI_DD_OZ) {  // the tensor flops that the digits' levels left to do
+    if (mo && mo_arith == RSSRI_DD_OZ) {  // the tensor flops that the digits' levels left to do
       unsigned long long steps = 0;
       RS_CK(fetch(&steps, gram_steps(h), s));
       h->recs.push_back({RSSRI_PROF_DD_SPMM, 0.0, steps * oz_gram_step_flops(n) * 1e-9, 0, nullptr,

@@ -84,9 +84,10 @@ def test_orbital_and_general_form_agree(B, n, n_occ, n_aux, n_tau, prec):
 # triples against the contraction over the kept pairs: nothing cut (eps = eps' =
 # 0, P = n^2) and n_tau = 8, so that the orbital form is the cheaper one; numbers of
 # virtual orbitals around the packing tiles' 32, one occupied orbital, one virtual, and
-# n just above the tensor cores' 128-row tile (a last column tile of 16).
+# n just above the tensor cores' 128-row tile (a last column tile of 16).  n = 32 and 33: the sliced
+# form takes fp64 up to 32.
 BLOCKS = [(20, 4, 24), (21, 20, 24), (40, 7, 42), (70, 38, 40), (66, 1, 40), (45, 13, 60),
-          (130, 62, 33), (129, 100, 48)]
+          (130, 62, 33), (129, 100, 48), (32, 15, 64), (33, 16, 66)]
 
 
 @pytest.mark.parametrize("n,n_occ,n_aux", BLOCKS)
