@@ -1343,7 +1343,7 @@ cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
   const long long nva = (long long)nv * na, row = (long long)n * nv;
   RS_TRY(ensure_mo_tab(h));
   const MoTab tab = mo_tab(h);
-  const size_t budget = (size_t)(oz ? 1024 : 256) << 20;
+  const size_t budget = (size_t)256 << 20;  // of U
   const long long per_c = row * nv;
   const int cc = (int)std::max<long long>(1, std::min<long long>(no, (long long)(budget / 8) / per_c));
   // V of as many c at a time as fit 256 MB

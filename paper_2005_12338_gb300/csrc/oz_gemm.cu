@@ -1411,7 +1411,7 @@ __device__ __forceinline__ void pair_digits(float p, float q, float *d) {
 // block takes 32 rows x GKB blocks of 16 columns; a thread keeps its row and its
 // half of the 16 columns and walks the blocks four apart, so that reads and
 // writes run through whole 128-byte pieces of neighbouring rows.  fp32
-// operations only: the pass runs at the HBM rate, 8 bytes read (U) and 12
+// operations only, 8 bytes read (U, per SLT tau points) and 12
 // written per value.
 //
 // The products drop digit pairs p + q >= 6.  Their signs are random between
@@ -1420,84 +1420,121 @@ __device__ __forceinline__ void pair_digits(float p, float q, float *d) {
 // largest terms make up the result.  So the slicer also sums
 // d_3^2 + 2 d_2 d_4 + 2 d_1 d_5 (the whole level 6) per row and block, and
 // oz_gram_diag_kernel adds the blocks in order for the diagonal.
-constexpr int GKB = 64;
-__global__ void __launch_bounds__(256) oz_gram_slice_kernel(
+//
+// A block writes the digits of SLT tau points, U read once for them: read again for every
+// tau point it was two fifths of the traffic.  At n = 200, all digits: 3.2 us per 10^6
+// values at 6.3 TB/s before, 2.8 us at 5.1 TB/s now (the conversion's ~60 fp32
+// instructions per value take 60% of that; 3 blocks per SM, with 2 it is 7% slower).
+constexpr int GKB = 64, SLT = 4;
+__global__ void __launch_bounds__(256, 3) oz_gram_slice_kernel(
     const float2 *__restrict__ U, const float2 *__restrict__ y, int n, long long K, long long ldy,
-    const int *__restrict__ m, const unsigned char *__restrict__ lev, int *__restrict__ ef,
-    __nv_bfloat16 *__restrict__ out, long long g1, float *__restrict__ lev6) {
-  __shared__ float l6[4][GR];
-  const int b = blockIdx.z;
+    int nt, const int *__restrict__ m, const unsigned char *__restrict__ lev,
+    int *__restrict__ ef, __nv_bfloat16 *__restrict__ out, long long g1,
+    float *__restrict__ lev6) {
+  __shared__ float l6[SLT][256], scale[SLT][GR];
+  const int t0 = blockIdx.z * SLT, tn = min(SLT, nt - t0);
   const int half = threadIdx.x & 1, rl = (threadIdx.x >> 1) & 31, kq = threadIdx.x >> 6;
   const int r = blockIdx.y * GR + rl;
-  const bool row = r < n;
-  const int bits = row ? m[(long long)b * n + r] : 0;
-  if (blockIdx.x == 0 && kq == 0 && half == 0 && row)
-    // magnitudes below 2^e (1 + 2^-22), e = the maximum's exponent + 1
-    ef[(long long)b * n + r] = bits > 0 ? ((bits >> 23) & 0xFF) - 127 + 1 + 1022 : 1;
-  // 2^(7 - e): magnitudes up to 2^7
-  const int se = 127 + 7 - (((bits >> 23) & 0xFF) - 127 + 1);
-  const float sc = bits > 0 && se > 0 && se < 255 ? __int_as_float(se << 23) : 0.f;
+  if (threadIdx.x < SLT * GR) {
+    const int t = threadIdx.x / GR, rr = blockIdx.y * GR + threadIdx.x % GR;
+    float sc = 0.f;
+    if (t < tn && rr < n) {
+      const int bits = m[(long long)(t0 + t) * n + rr];
+      if (blockIdx.x == 0)
+        // magnitudes below 2^e (1 + 2^-22), e = the maximum's exponent + 1
+        ef[(long long)(t0 + t) * n + rr] = bits > 0 ? ((bits >> 23) & 0xFF) - 127 + 1 + 1022 : 1;
+      // 2^(7 - e): magnitudes up to 2^7
+      const int se = 127 + 7 - (((bits >> 23) & 0xFF) - 127 + 1);
+      if (bits > 0 && se > 0 && se < 255) sc = __int_as_float(se << 23);
+    }
+    scale[t][threadIdx.x % GR] = sc;
+  }
+#pragma unroll
+  for (int t = 0; t < SLT; ++t) l6[t][threadIdx.x] = 0.f;
+  __syncthreads();
   const long long KB = ldy / KS;
   const long long kb1 = min(KB, ((long long)blockIdx.x + 1) * GKB);
-  float s6 = 0.f;
-  if (row)
-#pragma unroll 2
+  if (r < n)
     for (long long kb = (long long)blockIdx.x * GKB + kq; kb < kb1; kb += 4) {
-      const int L = lev[b * KB + kb];
-      if (L > 3) continue;
+      int L[SLT], least = 4;
+#pragma unroll
+      for (int t = 0; t < SLT; ++t) {
+        L[t] = t < tn ? lev[(t0 + t) * KB + kb] : 4;
+        least = min(least, L[t]);
+      }
+      if (least > 3) continue;
       const long long k0 = kb * KS + half * KC;
       const float4 *src = reinterpret_cast<const float4 *>(U + (kb * n + r) * KS + half * KC);
-      const float4 *yw = reinterpret_cast<const float4 *>(y + (long long)b * ldy + k0);
-      uint32_t o[OZ_S][KC / 2];
+      float4 uv[KC / 2];
 #pragma unroll
-      for (int u = 0; u < KC; u += 2) {
-        const float4 v = src[u / 2], w = yw[u / 2];
-        float d0[OZ_S], d1[OZ_S];
+      for (int u = 0; u < KC / 2; ++u) uv[u] = src[u];
+      uint32_t lv = 0;  // the levels, a byte each
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float xh = (h ? v.z : v.x) * sc, xl = (h ? v.w : v.y) * sc;
-          const float yh = h ? w.z : w.x, yl = h ? w.w : w.y;
-          const float p = __fmul_rn(xh, yh);
-          float q = __fmaf_rn(xh, yh, -p);
-          q = __fmaf_rn(xh, yl, q);
-          q = __fmaf_rn(xl, yh, q);
-          // normalised, so that |q| is at most half a unit of p's last place
-          const float pn = __fadd_rn(p, q);
-          q = __fsub_rn(q, __fsub_rn(pn, p));
-          // columns past K: U and y are not written there
-          const bool in = k0 + u + h < K;
-          pair_digits(in ? pn : 0.f, in ? q : 0.f, h ? d1 : d0);
+      for (int t = 0; t < SLT; ++t) lv |= (uint32_t)L[t] << (8 * t);
+#pragma unroll 1
+      for (int t = 0; t < tn; ++t, lv >>= 8) {
+        const int Lt = lv & 255;
+        if (Lt > 3) continue;
+        const float4 *yw = reinterpret_cast<const float4 *>(y + (t0 + t) * ldy + k0);
+        const float sc = scale[t][rl];
+        float s6 = l6[t][threadIdx.x];
+        uint32_t o[OZ_S][KC / 2];
+#pragma unroll
+        for (int u = 0; u < KC; u += 2) {
+          const float4 v = uv[u / 2], w = yw[u / 2];
+          float d0[OZ_S], d1[OZ_S];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float xh = (h ? v.z : v.x) * sc, xl = (h ? v.w : v.y) * sc;
+            const float yh = h ? w.z : w.x, yl = h ? w.w : w.y;
+            const float p = __fmul_rn(xh, yh);
+            float q = __fmaf_rn(xh, yh, -p);
+            q = __fmaf_rn(xh, yl, q);
+            q = __fmaf_rn(xl, yh, q);
+            // normalised, so that |q| is at most half a unit of p's last place
+            const float pn = __fadd_rn(p, q);
+            q = __fsub_rn(q, __fsub_rn(pn, p));
+            // columns past K: U and y are not written there
+            const bool in = k0 + u + h < K;
+            pair_digits(in ? pn : 0.f, in ? q : 0.f, h ? d1 : d0);
+          }
+#pragma unroll
+          for (int dgt = 0; dgt < OZ_S; ++dgt)
+            o[dgt][u / 2] = __byte_perm(__float_as_uint(d0[dgt]), __float_as_uint(d1[dgt]), 0x7632);
+          s6 += fmaf(d0[3], d0[3], 2.f * fmaf(d0[2], d0[4], d0[1] * d0[5]));
+          s6 += fmaf(d1[3], d1[3], 2.f * fmaf(d1[2], d1[4], d1[1] * d1[5]));
         }
+        l6[t][threadIdx.x] = s6;
+        const long long blk = ((t0 + t) * KB + kb) * n + r;
+        if (!OZ_IN(blk * 64 + 63, g1, 36)) continue;
+        // the digits the block's level multiplies, from slot 0 on
+        auto put = [&](int slot, int dgt) {
+          *reinterpret_cast<uint4 *>(out + digit_off(blk, half * KC, slot, g1)) =
+              make_uint4(o[dgt][0], o[dgt][1], o[dgt][2], o[dgt][3]);
+        };
+        if (Lt == 0) {
 #pragma unroll
-        for (int dgt = 0; dgt < OZ_S; ++dgt)
-          o[dgt][u / 2] = __byte_perm(__float_as_uint(d0[dgt]), __float_as_uint(d1[dgt]), 0x7632);
-        s6 += fmaf(d0[3], d0[3], 2.f * fmaf(d0[2], d0[4], d0[1] * d0[5]));
-        s6 += fmaf(d1[3], d1[3], 2.f * fmaf(d1[2], d1[4], d1[1] * d1[5]));
-      }
-      const long long blk = ((long long)b * KB + kb) * n + r;
-      if (!OZ_IN(blk * 64 + 63, g1, 36)) continue;
-      // the digits the block's level multiplies, from slot 0 on
-      auto put = [&](int slot, int dgt) {
-        *reinterpret_cast<uint4 *>(out + digit_off(blk, half * KC, slot, g1)) =
-            make_uint4(o[dgt][0], o[dgt][1], o[dgt][2], o[dgt][3]);
-      };
-      if (L == 0) {
+          for (int dgt = 0; dgt < OZ_S; ++dgt) put(dgt, dgt);
+        } else if (Lt == 1) {
 #pragma unroll
-        for (int dgt = 0; dgt < OZ_S; ++dgt) put(dgt, dgt);
-      } else if (L == 1) {
-#pragma unroll
-        for (int dgt = 1; dgt < 5; ++dgt) put(dgt - 1, dgt);
-      } else if (L == 2) {
-        put(0, 2);
-        put(1, 3);
+          for (int dgt = 1; dgt < 5; ++dgt) put(dgt - 1, dgt);
+        } else if (Lt == 2) {
+          put(0, 2);
+          put(1, 3);
+        }
       }
     }
-  s6 += __shfl_xor_sync(0xffffffffu, s6, 1);
-  if (half == 0) l6[kq][rl] = s6;
   __syncthreads();
-  if (threadIdx.x < GR && blockIdx.y * GR + threadIdx.x < n)
-    lev6[((long long)b * n + blockIdx.y * GR + threadIdx.x) * gridDim.x + blockIdx.x] =
-        (l6[0][threadIdx.x] + l6[1][threadIdx.x]) + (l6[2][threadIdx.x] + l6[3][threadIdx.x]);
+  if (threadIdx.x < SLT * GR) {
+    const int t = threadIdx.x / GR, q = threadIdx.x % GR;
+    if (t < tn && blockIdx.y * GR + q < n) {
+      float s[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) s[k] = l6[t][64 * k + 2 * q] + l6[t][64 * k + 2 * q + 1];
+      lev6[((long long)(t0 + t) * n + blockIdx.y * GR + q) * gridDim.x + blockIdx.x] =
+          (s[0] + s[1]) + (s[2] + s[3]);
+    }
+  }
 }
 
 // diag[t][i] = 2^(2 e - 14) times the sum of row i's level-6 sums over the slicer's
@@ -1904,8 +1941,8 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
 // Gram matrices at n = 200 (100 virtual orbitals, 64 tau points): 0.83 ms for the
 // products of a tau point with all digits (1,600 TFLOP/s) and 53 ms for all 64 (blocks of
 // columns that are small at a tau point have only their leading digits multiplied),
-// against 88 ms with all 21 products of every block; the digits take 32 ms (HBM).  The
-// whole setup and sampling call takes 124 ms against 281 with the contraction over the
+// against 88 ms with all 21 products of every block; the digits take 28 ms.  The
+// whole setup and sampling call takes 123 ms against 281 with the contraction over the
 // kept pairs (exchange 136, dense products 60, digits 48).  With rows of digits
 // K-contiguous over the whole contraction, 12 MB apart, the products took 1.6 times as
 // long: their 128-byte pieces came from 128 different DRAM pages.  A narrower last column
@@ -1998,8 +2035,8 @@ cudaError_t oz_gram_select(const float2 *U, const float2 *y, int n, long long K,
 cudaError_t oz_gram_slice(const OzGram &g, cudaStream_t s) {
   if (g.ldy % KS || ((uintptr_t)g.U % 16) || ((uintptr_t)g.y % 16) || g.nt > 65535)
     return cudaErrorInvalidValue;
-  dim3 gr(ceil_div(g.ldy, (long long)GKB * KS), ceil_div(g.n, GR), g.nt);
-  oz_gram_slice_kernel<<<gr, 256, 0, s>>>(g.U, g.y, g.n, g.K, g.ldy, g.m, g.lev, g.ef, g.d,
+  dim3 gr(ceil_div(g.ldy, (long long)GKB * KS), ceil_div(g.n, GR), ceil_div(g.nt, SLT));
+  oz_gram_slice_kernel<<<gr, 256, 0, s>>>(g.U, g.y, g.n, g.K, g.ldy, g.nt, g.m, g.lev, g.ef, g.d,
                                           (long long)g.nt * g.n * g.ldy * 4, g.lev6);
   ++launch_counter();
   RS_TRY(cudaGetLastError());
