@@ -395,35 +395,40 @@ int metric_inv_sqrt(rssri_handle *h, int *rc, bool df64) {
       RS_TRY(to_df64(A, (long long)na * na, h->nsA2.as<float2>(), s, range_flag(h)));
       RS_TRY(to_df64(B, (long long)na * na, h->nsB2.as<float2>(), s, range_flag(h)));
     }
-    SPAN(RSSRI_PROF_SETUP_GEMM, 1.0 * na * (double)na * na * 1e-9);
+    SPAN(RSSRI_PROF_SETUP_GEMM, 2.0 * na * (double)na * na * 1e-9);
     DfGemm g;
     g.M = g.N = g.K = na;
     g.A = h->nsA2.as<float2>(); g.lda = na;
     g.B = h->nsB2.as<float2>(); g.ldb = na;
     g.C64 = C; g.ldc = na;
-    // polynomials of one symmetric matrix: their products are symmetric
-    g.sym = 1;
     return df_gemm_w(h, g);
+  };
+  // C = A I: A itself, or in double-float A rounded to pairs.  (The other products are
+  // polynomials of one symmetric matrix, but their upper and lower halves round
+  // differently, and the reduced-precision chains round W's products again: half of each
+  // would do, at the price of other bits in a rounded operand now and then.)
+  auto identity = [&](const double *A, double *C) -> cudaError_t {
+    if (!df64)
+      return cudaMemcpyAsync(C, A, bytes, cudaMemcpyDeviceToDevice, s);
+    SPAN(RSSRI_PROF_OTHER, 0.0);
+    RS_TRY(to_df64(A, (long long)na * na, h->nsA2.as<float2>(), s, range_flag(h)));
+    return from_df64(h->nsA2.as<float2>(), (long long)na * na, C, s);
   };
   const int max_it = 100;
   double resid = 0;
   bool final_step = false;
   int it = 0;
   for (; it < max_it; ++it) {
-    if (it > 0) RS_CK(mm(Z, Y, Pm));  // Z_0 = I: Z_0 Y_0 = Y_0
-    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(ns_tbuild(it > 0 ? Pm : Y, na, Tm, scal, part, s)); }
+    RS_CK(it > 0 ? mm(Z, Y, Pm) : identity(Y, Pm));  // Z_0 = I
+    { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(ns_tbuild(Pm, na, Tm, scal, part, s)); }
     RS_CK(fetch(&resid, scal + 1, s));
     if (!std::isfinite(resid) || resid > 1e6) break;
     if (final_step) break;
     if (resid < 1e-8) final_step = true;
     RS_CK(mm(Y, Tm, Y2));
-    if (it > 0) {
-      RS_CK(mm(Tm, Z, Z2));
-      std::swap(Z, Z2);
-    } else {
-      std::swap(Z, Tm);  // T_0 Z_0 = T_0
-    }
+    RS_CK(it > 0 ? mm(Tm, Z, Z2) : identity(Tm, Z2));
     std::swap(Y, Y2);
+    std::swap(Z, Z2);
   }
   h->ns_iters = it;
   h->ns_resid = resid;
@@ -955,6 +960,7 @@ cudaError_t oz_slice_p(rssri_handle *h, const OzView &v, const OzDigits &o) {
 cudaError_t oz_gemm_p(rssri_handle *h, int cls, const OzGemm &g_in) {
   OzGemm g = g_in;
   g.wait_polls = h->test_wait_polls;
+  g.joint = cls == RSSRI_PROF_FACTOR_GEMM;
   const double alg = 2.0 * g.M * (double)g.N * g.A.K * g.batch;
   SPAN_T(cls, alg * 1e-9, oz_gemm_flops(g) * 1e-9);
   const size_t need = oz_gemm_work(g) * sizeof(double);

@@ -18,6 +18,13 @@ int grid_cap(long long work, int threads) {
   return (int)(b < 1 ? 1 : (b > 152 * 32 ? 152 * 32 : b));
 }
 
+__global__ void from_df64_kernel(const float2 *__restrict__ x, long long len,
+                                 double *__restrict__ y) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len;
+       i += (long long)gridDim.x * blockDim.x)
+    y[i] = (double)x[i].x + (double)x[i].y;
+}
+
 // range[0] |= 1 when the largest magnitude of x lies outside [2^-40, 2^40]
 // (zero arrays pass): the block maxima of the exponent field go to range[1],
 // and the last block to finish (range[2] counts them) checks and resets both.
@@ -117,11 +124,10 @@ using G64 = DfGeo<16, 16, 4, 4, 16, 2, 4>;
 using G40 = DfGeo<8, 8, 5, 5, 8, 6, 1>;
 // 24- and 16-wide tiles of 64 threads for products that would be a few 64-wide
 // tiles only (the metric root of a small N_aux: a lone 64-wide tile keeps one SM busy
-// for tens of microseconds and the others idle).  Slabs of 8 like G40's: the running
-// pair is renormalised after every slab, and with slabs of 16 V^{-1/2} at N_aux = 80 to
-// 270 was 1.3 times further from its value than with G40.
-using G24 = DfGeo<8, 8, 3, 3, 8, 8, 2>;
-using G16 = DfGeo<8, 8, 2, 2, 8, 12, 4>;
+// for tens of microseconds and the others idle), in slabs of 8 like G40's or 16 like
+// G64's: the running pair is renormalised after every slab.
+template <int BK> using G24 = DfGeo<8, 8, 3, 3, BK, 8, 2>;
+template <int BK> using G16 = DfGeo<8, 8, 2, 2, BK, 12, 4>;
 
 template <class GEO, int MODE, int TA, int TB, int OUT>
 __global__ void __launch_bounds__(GEO::NT, GEO::MINB) df_gemm_kernel(
@@ -329,6 +335,13 @@ cudaError_t scale_pow2(double *x, long long len, const int *e, int mult, cudaStr
   return cudaGetLastError();
 }
 
+cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s) {
+  if (len <= 0) return cudaSuccess;
+  from_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y);
+  ++launch_counter();
+  return cudaGetLastError();
+}
+
 cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s, int *range) {
   if (len <= 0) return cudaSuccess;
   to_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y, range);
@@ -347,9 +360,11 @@ bool use_g40(int M, int N) {
   return 10 * a64 > 13 * a40;
 }
 
-// Split of K (fp64 output, batch 1, few tiles, long K) into ks chunks of kc.
+// Split of K (fp64 output, batch 1, few tiles, long K) into ks chunks of kc, and the slab
+// between renormalisations: of the 40- or 64-wide geometry whichever is run, so that the
+// geometry never changes a result (R and [K]^L are rounded again by the bf16 chain).
 template <class GEO>
-void df_plan(const DfGemm &g, int *ks_out, int *kc_out) {
+void df_plan_as(const DfGemm &g, int *ks_out, int *kc_out) {
   const long long tiles = (long long)ceil_div(g.M, GEO::BM) * ceil_div(g.N, GEO::BN) * g.batch;
   const long long target = 2LL * GEO::MINB * 152;  // resident CTAs x 2 waves
   int ks = 1;
@@ -361,36 +376,50 @@ void df_plan(const DfGemm &g, int *ks_out, int *kc_out) {
   *kc_out = kc;
   *ks_out = std::max(1, ceil_div(g.K, kc));
 }
+void df_plan(const DfGemm &g, int *ks, int *kc) {
+  if (use_g40(g.M, g.N)) df_plan_as<G40>(g, ks, kc);
+  else df_plan_as<G64>(g, ks, kc);
+}
 
-// The geometry of a product: for one product with an fp64 result (the setup's) by
-// a time model (the metric root at N_aux = 60 to 600: 2.6-8.3 -> 1.3-5.4 ms, the setup
-// with it), the padded work per SM over how well the resident warps fill it;
-// else (batches, pair results: chain and block) by the padding alone, so that
-// the number of pairs in a batch never changes a pair's result.
+// The geometry of a product: the 40- or 64-wide one by the padding, and for one product
+// with an fp64 result (the setup's) a narrower one where the padded work per SM, over how
+// well the resident warps fill it, is less (the metric root at N_aux = 60 to 270: 2.6-4.9
+// -> 1.3-2.0 ms, the whole setup with it).
 enum { DF_G64 = 0, DF_G40, DF_G24, DF_G16 };
 template <class GEO> double df_time(const DfGemm &g, double cost) {
   int ks, kc;
-  df_plan<GEO>(g, &ks, &kc);
+  df_plan(g, &ks, &kc);
   const double tm = ceil_div(g.M, GEO::BM), tn = ceil_div(g.N, GEO::BN);
   const double ctas = std::ceil((g.sym ? tm * (tm + 1) / 2 : tm * tn) * ks / 152.0);
   const double warps = std::min(ctas, (double)GEO::MINB) * GEO::NT / 32;
   return ctas * GEO::BM * GEO::BN * kc * cost / std::min(1.0, warps / 12.0);
 }
 int df_pick(const DfGemm &g) {
-  if (g.batch != 1 || !g.C64) return use_g40(g.M, g.N) ? DF_G40 : DF_G64;
+  const bool g40 = use_g40(g.M, g.N);
+  if (g.batch != 1 || !g.C64) return g40 ? DF_G40 : DF_G64;
   // costs: measured rates per padded output (4.67, 3.8, 4.15, 3.85 TFLOP/s)
-  const double t[4] = {df_time<G64>(g, 1.0), df_time<G40>(g, 1.23), df_time<G24>(g, 1.13),
-                       df_time<G16>(g, 1.21)};
-  int best = 0;
-  for (int k = 1; k < 4; ++k)
+  const double t[4] = {df_time<G64>(g, 1.0), df_time<G40>(g, 1.23), df_time<G24<8>>(g, 1.13),
+                       df_time<G16<8>>(g, 1.21)};
+  int best = g40 ? DF_G40 : DF_G64;  // (the other one of these two has other slabs)
+  for (int k = 2; k < 4; ++k)
     if (t[k] < 0.95 * t[best]) best = k;
   return best;
+}
+// f(geometry) for the geometry of a product.
+template <class F> auto with_geo(const DfGemm &g, F f) {
+  const bool g40 = use_g40(g.M, g.N);
+  switch (df_pick(g)) {
+    case DF_G40: return f(G40{});
+    case DF_G24: return g40 ? f(G24<8>{}) : f(G24<16>{});
+    case DF_G16: return g40 ? f(G16<8>{}) : f(G16<16>{});
+    default: return f(G64{});
+  }
 }
 
 template <class GEO>
 cudaError_t df_gemm_geo(const DfGemm &g, double *work, size_t work_elems, cudaStream_t s) {
   int ks, kc;
-  df_plan<GEO>(g, &ks, &kc);
+  df_plan(g, &ks, &kc);
   if (ks > 1 && work_elems < (size_t)ks * g.M * g.N) return cudaErrorInvalidValue;
   if (g.batch * ks > 65535) return cudaErrorInvalidValue;
   dim3 grid(ceil_div(g.N, GEO::BN), ceil_div(g.M, GEO::BM), g.batch * ks);
@@ -429,19 +458,13 @@ cudaError_t df_gemm(const DfGemm &g, double *work, size_t work_elems, cudaStream
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if ((g.C64 == nullptr) == (g.C2 == nullptr)) return cudaErrorInvalidValue;
   if (g.sym && (g.M != g.N || !g.C64 || g.batch != 1)) return cudaErrorInvalidValue;
-  switch (df_pick(g)) {
-    case DF_G40: return df_gemm_geo<G40>(g, work, work_elems, s);
-    case DF_G24: return df_gemm_geo<G24>(g, work, work_elems, s);
-    case DF_G16: return df_gemm_geo<G16>(g, work, work_elems, s);
-    default: return df_gemm_geo<G64>(g, work, work_elems, s);
-  }
+  return with_geo(g, [&](auto geo) { return df_gemm_geo<decltype(geo)>(g, work, work_elems, s); });
 }
 
 double df_gemm_flops(const DfGemm &g) {
   if (!g.sym) return 2.0 * g.M * (double)g.N * g.K * g.batch;
   // symmetric: only the tiles on and above the diagonal are computed
-  const int edges[4] = {G64::BM, G40::BM, G24::BM, G16::BM};
-  const int bm = edges[df_pick(g)];
+  const int bm = with_geo(g, [](auto geo) { return decltype(geo)::BM; });
   const int t = ceil_div(g.M, bm);
   double f = 0.0;
   for (int i = 0; i < t; ++i)
@@ -452,12 +475,7 @@ double df_gemm_flops(const DfGemm &g) {
 
 size_t df_gemm_work(const DfGemm &g) {
   int ks, kc;
-  switch (df_pick(g)) {
-    case DF_G40: df_plan<G40>(g, &ks, &kc); break;
-    case DF_G24: df_plan<G24>(g, &ks, &kc); break;
-    case DF_G16: df_plan<G16>(g, &ks, &kc); break;
-    default: df_plan<G64>(g, &ks, &kc);
-  }
+  df_plan(g, &ks, &kc);
   return ks > 1 ? (size_t)ks * g.M * g.N : 0;
 }
 

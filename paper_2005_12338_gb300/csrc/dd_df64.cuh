@@ -12,6 +12,8 @@ namespace rssri {
 // magnitude of x lies outside [2^-40, 2^40].
 cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s,
                     int *range = nullptr);
+// y = hi + lo of every pair.
+cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s);
 // Per segment c of len values: e[c] such that the largest magnitude lies in
 // [2^e, 2^(e+1)), and y = pairs of x 2^-e (exact scaling, so that the pairs
 // sit in the middle of fp32's exponent range whatever x's magnitude).

@@ -236,6 +236,23 @@ __device__ __forceinline__ void fold(f2 &hi, f2 &lo, f2 a, bool norm) {
   lo = norm ? f2_sub(f, f2_sub(hi, s)) : f;
 }
 
+// The same of a chunk's four accumulators at once, in the order of roundings that the
+// factors' products keep (see oz_gemm.cuh): a0, a1, a2 exact, a3 the small rounded level.
+__device__ __forceinline__ void two_sum(f2 a, f2 b, f2 &s, f2 &e) {
+  s = f2_add(a, b);
+  const f2 bb = f2_sub(s, a);
+  e = f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb));
+}
+__device__ __forceinline__ void fold_joint(f2 &hi, f2 &lo, f2 a0, f2 a1, f2 a2, f2 a3) {
+  f2 s, e, s2, e2, t, f;
+  two_sum(a0, a1, s, e);
+  two_sum(s, a2, s2, e2);
+  e = f2_add(f2_add(e, e2), a3);
+  two_sum(hi, s2, t, f);
+  f = f2_add(f, f2_add(lo, e));
+  two_sum(t, f, hi, lo);
+}
+
 // Accumulator k (level 0, 1, 2, or 3 and more) is drained after the K steps st of a
 // tile with st % period == phase, and after the last one that it takes products of.
 // The periods keep a level's sum below 0.75 2^24 grid units; the phases spread the
@@ -254,6 +271,7 @@ constexpr unsigned long long drain_table() {
   return m;
 }
 constexpr unsigned long long DRAINS = drain_table();
+constexpr unsigned long long DRAINS_JOINT = 0xF000F000F000ull;  // all four, every 16 steps
 // A run of K steps of one level within a tile: up to step `end`, after which the
 // accumulators of `last` are drained for the tile; those of `live` take products.
 struct OzRun {
@@ -261,7 +279,7 @@ struct OzRun {
   uint32_t live, last;
 };
 // The accumulators (bits) drained after step st; called for every st % 4 == 3 in turn and
-// for the last step of a run, tab = DRAINS at step 0 of a tile.
+// for the last step of a run, tab = DRAINS (or DRAINS_JOINT) at step 0 of a tile.
 __device__ __forceinline__ uint32_t drains_after(unsigned long long &tab, int st, const OzRun &r) {
   uint32_t m = 0;
   if ((st & 3) == 3) {
@@ -356,10 +374,11 @@ __device__ __forceinline__ OzRun oz_run(const OzTile &t, int lev) {
 // The next step from st on that an accumulator may be drained after, and which (bits); the
 // same sequence as drains_after()'s, from the step alone: the drain warps' registers are
 // taken by the running totals.
+template <bool JOINT>
 __device__ __forceinline__ uint32_t next_drains(const OzTile &t, int &st) {
   const OzRun r = oz_run(t, st < t.end01 ? 0 : (st < t.end2 ? 1 : 2));
   st = min(st | 3, r.end - 1);
-  unsigned long long tab = DRAINS >> (4 * ((st >> 2) % 12));
+  unsigned long long tab = (JOINT ? DRAINS_JOINT : DRAINS) >> (4 * ((st >> 2) % 12));
   return drains_after(tab, st, r);
 }
 // First step of split s of ks: the splits cost about the same and start on a drain's
@@ -423,7 +442,7 @@ __device__ __forceinline__ OzTile oz_tile(const OzParams &p, int q) {
   return t;
 }
 
-template <int MODE>
+template <int MODE, bool JOINT = false>
 __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_constant__ OzParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -536,7 +555,7 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
         b_off = __shfl_sync(ALL, b_off, 0);
       }
       uint32_t fresh = 15;  // bit k: accumulator k starts again, its first product overwrites
-      unsigned long long tab = DRAINS;
+      unsigned long long tab = JOINT ? DRAINS_JOINT : DRAINS;
       int st = 0;
       auto run = [&](auto level) {
         constexpr int lev = decltype(level)::value;
@@ -663,8 +682,39 @@ __global__ void __launch_bounds__(THREADS, 1) oz_gemm_kernel(const __grid_consta
 #pragma unroll
       for (int c = 0; c < DC / 2; ++c) hi[c] = lo[c] = 0;
       for (int st = 0; st < t.kst && ok; ++st) {
-        const uint32_t now = next_drains(t, st);
+        const uint32_t now = next_drains<JOINT>(t, st);
         if (now == 0) continue;
+        if (JOINT) {  // all four, after every 16 steps
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            ok = ok && __all_sync(0xffffffffu,
+                                  bar_wait(&accf[k], drained & 1, p.err, 4, p.wait_polls) &&
+                                      !(p.err && *(volatile int *)p.err));
+          if (!ok) continue;
+          drained ^= 1;
+          asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+          for (int f = 0; f < 8; ++f) {
+            const uint32_t tl = tmem + ((uint32_t)(lq * 32 + 16 * (f >> 2)) << 16) +
+                                (uint32_t)(cq * DC + 8 * (f & 3));
+            uint32_t r[4][4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tmem_ld16x256(tl + 128 * k, r[k]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+              fold_joint(hi[2 * f + u], lo[2 * f + u], f2_pack(r[0][2 * u], r[0][2 * u + 1]),
+                         f2_pack(r[1][2 * u], r[1][2 * u + 1]),
+                         f2_pack(r[2][2 * u], r[2][2 * u + 1]),
+                         f2_pack(r[3][2 * u], r[3][2 * u + 1]));
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;");
+          __syncwarp();
+          if (lane == 0)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) bar_arrive(&acce[k]);
+          continue;
+        }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int k = (i + 3) & 3;
@@ -1712,6 +1762,8 @@ cudaError_t prepare() {
   if (!done[dev]) {
     RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SMEM));
+    RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<0, true>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
     RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SMEM));
     RS_TRY(cudaFuncSetAttribute(oz_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1925,7 +1977,11 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
   const long long tiles = (long long)p.ntiles * p.mtiles * g.batch * ks;
   if (tiles > 0x7FFFFFFFLL) return cudaErrorInvalidValue;
   p.tiles = (int)tiles;
-  oz_gemm_kernel<0><<<(unsigned)std::min<long long>(tiles, sm_count()), THREADS, SMEM, s>>>(p);
+  const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());
+  if (g.joint)
+    oz_gemm_kernel<0, true><<<grid, THREADS, SMEM, s>>>(p);
+  else
+    oz_gemm_kernel<0><<<grid, THREADS, SMEM, s>>>(p);
   ++launch_counter();
   RS_TRY(cudaGetLastError());
   if (ks > 1) {

@@ -77,6 +77,10 @@ struct OzGemm {
   long long ldc = 0, sC = 0;
   long long ccap = 0;  // elements of C (bounds checks of RSSRI_CHECKS builds)
   double alpha = 1.0;
+  // 1: the levels are added after every 16 K steps, all four together: the order of
+  // roundings of R and R^L.  They are rounded to bf16 or tf32 for the chain, where another
+  // last bit can turn into another rounded operand (2^-9 of it); 5 to 10% slower.
+  int joint = 0;
   int *err = nullptr;  // device flag, set non-zero if a bounded wait gives up
   // testing only: > 0 issues no copy or product and gives up every wait after
   // this many polls (the error path with nothing in flight); 0 = normal
