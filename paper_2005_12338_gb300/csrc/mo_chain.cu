@@ -2,7 +2,7 @@
 // and tau point, its traces, and the sum over pairs of M_(:,o) go M_(o,:) - 2 t M.
 //
 // Bound by the fp64 pipe (or the fp32 pipes, double-float): at N = 200, 64
-// pairs, 16 tau points the fp64 sampling call takes 42.6 ms with these
+// pairs, 16 tau points the fp64 sampling call takes 41.2 ms with these
 // products, 146 ms with the four general ones per factor pair (137 of them
 // in those products), the pipe busy all along either way.
 #include "mo_tile.cuh"

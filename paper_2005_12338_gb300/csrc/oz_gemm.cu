@@ -1998,7 +1998,7 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
 // products of a tau point with all digits (1,600 TFLOP/s) and 53 ms for all 64 (blocks of
 // columns that are small at a tau point have only their leading digits multiplied),
 // against 88 ms with all 21 products of every block; the digits take 28 ms.  The
-// whole setup and sampling call takes 123 ms against 281 with the contraction over the
+// whole setup and sampling call takes 122 ms against 281 with the contraction over the
 // kept pairs (exchange 136, dense products 60, digits 48).  With rows of digits
 // K-contiguous over the whole contraction, 12 MB apart, the products took 1.6 times as
 // long: their 128-byte pieces came from 128 different DRAM pages.  A narrower last column

@@ -4,7 +4,7 @@
 //
 // A tau point's matrix is dealt out as 32 x 32 tiles to `parts` blocks (Y's
 // tile transposed through shared memory, so that both are read along rows).
-// rssri_energy_static at n = 40, 32 tau points: 8.4 us a call, most of it the
+// rssri_energy_static at n = 40, 32 tau points: 8.2 us a call, most of it the
 // host's; 10.6 to 12.3 with one block per tau point, strided reads of Y and a
 // second launch for the sum over tau.
 #pragma once
