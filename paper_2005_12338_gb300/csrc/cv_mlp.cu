@@ -579,21 +579,6 @@ __global__ void trace_prod_w_kernel(const double *__restrict__ X, const double *
     RS_TRY(cudaGetLastError()); \
   } while (0)
 
-// Chunks of the m rows that dW3 and dW0 are summed in.
-namespace {
-void row_chunks(int m, int *ks, int *kc) {
-  const int k = m < 2048 ? 1 : std::min(76, m / 512);
-  *kc = k > 1 ? (ceil_div(m, k) + 15) / 16 * 16 : m;
-  *ks = ceil_div(m, *kc);
-}
-}  // namespace
-
-size_t cv_sum_floats(int m) {
-  int ks, kc;
-  row_chunks(std::max(m, 1), &ks, &kc);
-  return (size_t)ks * (CV_HIDDEN + CV_HIDDEN * CV_NFEAT) + 128;  // and the loss sums (64 doubles)
-}
-
 // Parameter layout (floats): W0 [256][10], b0, W1 [256][256], b1, W2, b2, W3 [1][256], b3.
 namespace {
 constexpr long long O_W0 = 0, O_B0 = O_W0 + CV_HIDDEN * CV_NFEAT, O_W1 = O_B0 + CV_HIDDEN,
@@ -783,7 +768,7 @@ cudaError_t cv_backward(const float *params, const float *X, int m, const float 
   RS_L();
   // the sums over the rows: db2, db1, db0, dW3 = dy^T A2, db3, dW0 = dZ0^T X (fp32)
   SumArgs g;
-  row_chunks(m, &g.ks, &g.kc);
+  cv_row_chunks(m, &g.ks, &g.kc);
   float *p3 = b.work + 128, *p0 = p3 + (long long)g.ks * H;
   g.dz[0] = Z2; g.dz[1] = Z1; g.dz[2] = Z0;
   g.dy = dy; g.a2 = A2; g.x = X;

@@ -18,7 +18,19 @@ size_t cv_act_floats(int m);
 // Floats of `work` that the tensor-core hidden layers use (bf16 weights and
 // weight-gradient partials); the row sums' partials (cv_sum_floats(m)) follow them.
 size_t cv_tc_work_floats();
-size_t cv_sum_floats(int m);
+// Chunks of the m rows that dW3 and dW0 are summed in: at most cv_max_chunks(m), *ks of
+// *kc rows.
+inline int cv_max_chunks(int m) { return m < 2048 ? 1 : std::min(76, m / 512); }
+inline void cv_row_chunks(int m, int *ks, int *kc) {
+  const int k = cv_max_chunks(m);
+  *kc = k > 1 ? (ceil_div(m, k) + 15) / 16 * 16 : m;
+  *ks = ceil_div(m, *kc);
+}
+// Their partials, and the loss sums (64 doubles), for any number of rows up to m: from the
+// most chunks, which grow with m (*ks does not: 34 at 17,408 rows, 33 at 17,409).
+inline size_t cv_sum_floats(int m) {
+  return (size_t)cv_max_chunks(m) * (CV_HIDDEN + CV_HIDDEN * CV_NFEAT) + 128;
+}
 // Forward: y = MLP(X) - 1 in act (see cv_act_floats), X [m][10].
 cudaError_t cv_forward(const float *params, const float *X, int m, float *act, float *work,
                        cudaStream_t s);
