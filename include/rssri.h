@@ -440,13 +440,15 @@ RSSRI_API int rssri_cv_loss_grad(rssri_handle *h, const float *x, const float *t
  *   tau_w  device, [n_tau]        quadrature weights
  *   e_corr device, [1]            output, written on `stream`
  *   stream cudaStream_t as void* (NULL = legacy default stream)
- * Its scratch is a static device array of RSSRI_STATIC_MAX_TAU doubles
- * (32 KiB) and a counter, present on every GPU that loads the library until the process
- * exits.  The first call on each device looks up that array's device address
+ * Its scratch is a static device array of RSSRI_STATIC_MAX_TAU doubles and as
+ * many counters (48 KiB), present on every GPU that loads the library until the
+ * process exits.  The first call on each device looks up that array's device address
  * (cudaGetSymbolAddress) with the device current; make that first call before
  * any stream capture.  All calls share the array: calls whose work overlaps on
- * the GPU (different streams, or concurrent host threads) race on it and must
- * be serialised by the caller.  Returns RSSRI_ERR_INVALID_ARG for null
+ * the GPU (different streams, or concurrent host threads) race on it, which
+ * makes the e_corr of each of them worthless (it may also stay unwritten), and must
+ * be serialised by the caller; calls after them are not affected.  Returns
+ * RSSRI_ERR_INVALID_ARG for null
  * pointers, n outside [1, 4096], n_occ < 1 or n_tau outside
  * [1, RSSRI_STATIC_MAX_TAU]; RSSRI_ERR_CUDA if a launch fails.  Does not
  * synchronise. */

@@ -6,20 +6,25 @@
 // that hand every byte of device memory to their own pool allocator and forbid
 // libraries from allocating behind their back, and real-time loops that must
 // not hit the allocator's synchronisation.  This entry point creates no handle
-// and allocates nothing: its only scratch (partial traces and a counter of
+// and allocates nothing: its only scratch (partial traces and counters of
 // finished blocks) is file-scope __device__ memory of fixed size, loaded with
 // the library and held by every GPU that loads it until the process exits.
 //
 // One launch: the block that finishes last adds the partial traces (a second
-// launch for that cost as much as the traces of small problems).
+// launch for that cost as much as the traces of small problems).  The blocks of
+// a launch count modulo their number, on a counter that only launches of as many
+// blocks use: whatever calls overlap, each leaves the counter where it was, so that
+// an overlap, which the interface forbids, spoils the overlapping calls alone.
 #include <mutex>
 
 #include "trace.cuh"
 
 namespace {
 
-// RSSRI_STATIC_MAX_TAU partial traces (32 KiB), then the counter, zero between calls.
-static __device__ __align__(256) double g_energy_scratch[RSSRI_STATIC_MAX_TAU + 1];
+// RSSRI_STATIC_MAX_TAU partial traces (32 KiB), then a counter for every number of
+// blocks up to that (16 KiB), zero between calls.
+static __device__ __align__(256) double
+    g_energy_scratch[RSSRI_STATIC_MAX_TAU + RSSRI_STATIC_MAX_TAU / 2];
 static_assert(RSSRI_STATIC_MAX_TAU >= rssri::TRACE_SLOTS, "slots of trace_parts");
 
 constexpr int kMaxDevices = 64;
@@ -47,7 +52,7 @@ cudaError_t scratch_on_current_device(double **out) {
 
 // Partial traces by block (p, t); the last block to finish forms
 // e_corr = -(sum_t w_t tr[t]) / ne, summed in tau order (the same order as
-// the energy of rssri_sigma), and clears the counter.
+// the energy of rssri_sigma).
 __global__ void __launch_bounds__(256) static_energy_kernel(const double *__restrict__ sigma,
                                                             const double *__restrict__ gb,
                                                             const double *__restrict__ tau_w, int n,
@@ -56,21 +61,19 @@ __global__ void __launch_bounds__(256) static_energy_kernel(const double *__rest
   __shared__ bool last;
   const long long nn = (long long)n * n;
   const int t = blockIdx.y, parts = gridDim.x, nt = gridDim.y;
-  unsigned *count = reinterpret_cast<unsigned *>(scratch + RSSRI_STATIC_MAX_TAU);
+  const unsigned blocks = parts * nt;  // <= RSSRI_STATIC_MAX_TAU
+  unsigned *count = reinterpret_cast<unsigned *>(scratch + RSSRI_STATIC_MAX_TAU) + blocks - 1;
   const double s = rssri::trace_part(sigma + t * nn, gb + t * nn, n, blockIdx.x, parts);
   if (threadIdx.x == 0) {
     scratch[(long long)t * parts + blockIdx.x] = s;
     __threadfence();
-    last = atomicAdd(count, 1u) == (unsigned)(parts * nt) - 1;
+    last = atomicInc(count, blocks - 1) == blocks - 1;  // the last one wraps it to 0
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
   const double b = rssri::trace_weighted(tau_w, scratch, parts, nt);
-  if (threadIdx.x == 0) {
-    e_corr[0] = -b / ne;
-    *count = 0u;
-  }
+  if (threadIdx.x == 0) e_corr[0] = -b / ne;
 }
 
 }  // namespace
