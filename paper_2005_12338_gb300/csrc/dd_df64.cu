@@ -422,21 +422,29 @@ cudaError_t df_gemm_geo(const DfGemm &g, double *work, size_t work_elems, cudaSt
   df_plan(g, &ks, &kc);
   if (ks > 1 && work_elems < (size_t)ks * g.M * g.N) return cudaErrorInvalidValue;
   if (g.batch * ks > 65535) return cudaErrorInvalidValue;
-  dim3 grid(ceil_div(g.N, GEO::BN), ceil_div(g.M, GEO::BM), g.batch * ks);
-  void *out = ks > 1 ? (void *)work : (g.C64 ? (void *)g.C64 : (void *)g.C2);
   const int part = ks > 1;
+  // a launch has 65,535 rows of tiles at most: taller products in several (those with
+  // split K and the symmetric ones have a few rows only)
+  constexpr int ROWS = 65535 * GEO::BM;
+  for (int m0 = 0; m0 < g.M; m0 += std::min(ROWS, g.M - m0)) {
+    const int m = std::min(ROWS, g.M - m0);
+    const float2 *A = g.A + (long long)m0 * (g.transA ? 1 : g.lda);
+    const long long c0 = (long long)m0 * g.ldc;
+    void *out = part ? (void *)work : (g.C64 ? (void *)(g.C64 + c0) : (void *)(g.C2 + c0));
+    dim3 grid(ceil_div(g.N, GEO::BN), ceil_div(m, GEO::BM), g.batch * ks);
 #define RS_DF(TA, TB, OUT)                                                                \
   df_gemm_kernel<GEO, 0, TA, TB, OUT><<<grid, GEO::NT, 0, s>>>(                           \
-      g.M, g.N, g.K, kc, ks, g.A, g.lda, g.sA, g.B, g.ldb, g.sB, out, g.ldc, g.sC, g.alpha, \
+      m, g.N, g.K, kc, ks, A, g.lda, g.sA, g.B, g.ldb, g.sB, out, g.ldc, g.sC, g.alpha,   \
       part, g.sym, nullptr, nullptr)
-  const int o = g.C2 ? 1 : 0;
-  if (!g.transA && !g.transB) { if (o) RS_DF(0, 0, 1); else RS_DF(0, 0, 0); }
-  else if (!g.transA && g.transB) { if (o) RS_DF(0, 1, 1); else RS_DF(0, 1, 0); }
-  else if (g.transA && !g.transB) { if (o) RS_DF(1, 0, 1); else RS_DF(1, 0, 0); }
-  else { if (o) RS_DF(1, 1, 1); else RS_DF(1, 1, 0); }
+    const int o = g.C2 ? 1 : 0;
+    if (!g.transA && !g.transB) { if (o) RS_DF(0, 0, 1); else RS_DF(0, 0, 0); }
+    else if (!g.transA && g.transB) { if (o) RS_DF(0, 1, 1); else RS_DF(0, 1, 0); }
+    else if (g.transA && !g.transB) { if (o) RS_DF(1, 0, 1); else RS_DF(1, 0, 0); }
+    else { if (o) RS_DF(1, 1, 1); else RS_DF(1, 1, 0); }
 #undef RS_DF
-  ++launch_counter();
-  RS_TRY(cudaGetLastError());
+    ++launch_counter();
+    RS_TRY(cudaGetLastError());
+  }
   if (part) {
     const long long mn = (long long)g.M * g.N;
     df_reduce_kernel<<<grid_cap(mn, 256), 256, 0, s>>>(work, ks, g.M, g.N, g.C64, g.ldc, g.alpha,

@@ -202,14 +202,21 @@ __global__ void splitk_reduce_kernel(int M, int N, int batch, int ksplit,
 template <class TL, int TA, int TB>
 cudaError_t launch_strided_t(const GemmArgs &g, int ksplit, int kchunk, int b0, int nb,
                              double *work, cudaStream_t s) {
-  dim3 grid(ceil_div(g.N, TL::BN), ceil_div(g.M, TL::BM), nb * ksplit);
   const bool part = ksplit > 1;
-  dgemm_kernel<TL, 0, TA, TB><<<grid, TL::NT, 0, s>>>(
-      g.M, g.N, g.K, kchunk, ksplit, g.A + (long long)b0 * g.sA, g.lda, g.sA,
-      g.B + (long long)b0 * g.sB, g.ldb, g.sB, part ? work : g.C + (long long)b0 * g.sC,
-      g.ldc, g.sC, g.alpha, g.beta, part ? 1 : 0, nullptr, nullptr);
-  ++launch_counter();
-  RS_TRY(cudaGetLastError());
+  // a launch has 65,535 rows of tiles at most: taller products ([K]^L of a million kept
+  // pairs under 16-wide tiles) in several; those with split K have a few rows only
+  constexpr int ROWS = 65535 * TL::BM;
+  for (int m0 = 0; m0 < g.M; m0 += std::min(ROWS, g.M - m0)) {
+    const int m = std::min(ROWS, g.M - m0);
+    dim3 grid(ceil_div(g.N, TL::BN), ceil_div(m, TL::BM), nb * ksplit);
+    dgemm_kernel<TL, 0, TA, TB><<<grid, TL::NT, 0, s>>>(
+        m, g.N, g.K, kchunk, ksplit, g.A + (long long)b0 * g.sA + (long long)m0 * (TA ? 1 : g.lda),
+        g.lda, g.sA, g.B + (long long)b0 * g.sB, g.ldb, g.sB,
+        part ? work : g.C + (long long)b0 * g.sC + (long long)m0 * g.ldc, g.ldc, g.sC, g.alpha,
+        g.beta, part ? 1 : 0, nullptr, nullptr);
+    ++launch_counter();
+    RS_TRY(cudaGetLastError());
+  }
   if (part) {
     const long long total = (long long)g.M * g.N * nb;
     const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 16);
