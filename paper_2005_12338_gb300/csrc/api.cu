@@ -150,6 +150,7 @@ struct rssri_handle {
   DevBuf ozYm, ozY6, ozYsel;  // row maxima per tau point, the slicer's level-6 sums, block levels
   bool mo_tab_ready = false;  // moTab, moChl made for this setup
   bool orth_ok = false;       // C^T C = I to rounding: the orbital-basis chain applies
+  bool c_near = false;        // C^T C = I roughly: the orbitals' values are of order 1 at most
   // bf16 chain buffers
   DevBuf hxsl, hy3, hg, hgb, hP, hdcl16, hxy32, ha6, hct, hdct, hpart, hfold;
   DevBuf hclt, hfl;  // learned control variate on the tensor-core chain: (C^L)^T, F^L per pair
@@ -635,6 +636,7 @@ int rssri_setup(rssri_handle *h, const rssri_problem *p, const rssri_options *o)
   int hflags[3];
   RS_CK(fetch(hflags, flags, s, 3));
   h->orth_ok = hflags[2] == 0;
+  h->c_near = !(hflags[2] & 2);
   if (hflags[1]) return RSSRI_ERR_NONFINITE;
   if (hflags[0]) return RSSRI_ERR_NONSYMMETRIC_ERI;
 
@@ -1314,8 +1316,12 @@ cudaError_t ensure_mo_tab(rssri_handle *h) {
 // those flops per second (45% of the exchange's tile rows are outside the band,
 // and its digits are written for every tau point); the Gram tiles at ~78e12
 // with 20 bytes of HBM traffic per value and tau point, V at ~60e12.
+// C enters the orbital form by itself, and where that keeps pairs of floats (U is of degree
+// 2 in C) it has to be of order 1 for them to stay in fp32's range; the contraction over the
+// kept pairs meets C in G only, whose range the double-float form checks.
 bool use_mo_block(const rssri_handle *h, int dd_arith) {
   if (h->P == 0) return false;
+  if (dd_arith != RSSRI_DD_FP64 && !h->c_near) return false;
   const double n = h->n, no = h->n_occ, nv = n - no, na = h->n_aux, P = h->P, nt = h->n_tau;
   if (dd_arith == RSSRI_DD_OZ) {
     if (h->n > 1024) return false;

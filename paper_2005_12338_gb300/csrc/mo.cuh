@@ -113,7 +113,7 @@ cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, double scale
 // out[a] = sum_q x[a][q]^2 (the diagonal of v^L on the kept pairs, where its largest magnitude is).
 cudaError_t mo_row_norm2(const double *x, int rows, int cols, double *out, cudaStream_t s);
 
-// flag |= 1 when some |CtC - I| element exceeds tol.
+// flag |= 1 when some |CtC - I| element exceeds tol, |= 2 when one exceeds 1/2.
 cudaError_t mo_orth_check(const double *CtC, int n, double tol, int *flag, cudaStream_t s);
 // The range rule of to_df64 (dd_df64.cuh) on each of `segments` matrices of len values, without
 // converting them.

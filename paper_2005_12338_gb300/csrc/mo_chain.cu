@@ -269,13 +269,13 @@ __global__ void __launch_bounds__(256) mo_tables_kernel(const double *__restrict
 
 __global__ void mo_orth_kernel(const double *__restrict__ m, int n, double tol, int *__restrict__ flag) {
   const long long nn = (long long)n * n;
-  bool bad = false;
+  int bad = 0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < nn;
        e += (long long)gridDim.x * blockDim.x) {
-    const double d = m[e] - (e / n == e % n ? 1.0 : 0.0);
-    bad |= !(fabs(d) <= tol);
+    const double d = fabs(m[e] - (e / n == e % n ? 1.0 : 0.0));
+    bad |= (d <= tol ? 0 : 1) | (d <= 0.5 ? 0 : 2);
   }
-  if (bad) atomicOr(flag, 1);
+  if (bad) atomicOr(flag, bad);
 }
 
 __global__ void __launch_bounds__(256) mo_range_kernel(const double *__restrict__ x, long long len,
