@@ -267,7 +267,11 @@ void split_plan(const GemmArgs &g, int *ksplit, int *kchunk) {
 // ------------------------------------------------------------ autotuner ----
 // The tile shape of each distinct problem shape is chosen once per process:
 // by timing every shape on the first call (when the product does not read C,
-// so repeating it is harmless), else by a model of the padded work.
+// so repeating it is harmless), else by a model of the padded work.  Large
+// products are timed on a part of the result that holds a dozen of the largest tiles
+// per SM, so that a first call does not run all of them six times more.  First calls of
+// a process, fp64: setup at N = 300, N_aux = 900: 1,955 -> 1,554 ms (532 again); sampling
+// with a caller's G at N = 200, which forms D: 1,013 -> 866 ms (391 again).
 struct ShapeKey {
   int M, N, K, batch, ta, tb, mode;
   bool operator<(const ShapeKey &o) const {
@@ -277,6 +281,23 @@ struct ShapeKey {
 };
 std::mutex g_tune_mutex;
 std::map<ShapeKey, int> g_tune;
+
+// The part of a product that its tiles are timed on: whole batch entries, then whole rows
+// or columns, the other dimension cut to a multiple of every tile's edge.
+GemmArgs tune_part(const GemmArgs &g, int ks) {
+  constexpr long long OUTPUTS = 152LL * 12 * 100 * 100;
+  constexpr long long EDGES = 4800;  // the tile edges' least common multiple
+  GemmArgs t = g;
+  if (ks > 1) return t;
+  const long long mn = (long long)g.M * g.N;
+  t.batch = (int)std::min<long long>(g.batch, (OUTPUTS + mn - 1) / mn);
+  if (mn > OUTPUTS) {
+    int &cut = g.N >= g.M ? t.N : t.M;
+    const long long other = std::min(g.M, g.N), want = (OUTPUTS + other - 1) / other;
+    cut = (int)std::min<long long>(cut, (want + EDGES - 1) / EDGES * EDGES);
+  }
+  return t;
+}
 
 int model_tile(int M, int N, int K, int batch) {
   int best = 0;
@@ -324,10 +345,10 @@ cudaError_t dgemm(const GemmArgs &g, double *work, size_t work_elems, cudaStream
     auto it = g_tune.find(key);
     if (it != g_tune.end()) tile = it->second;
   }
-  auto run = [&](int t) -> cudaError_t {
-    for (int b0 = 0; b0 < g.batch; b0 += per) {
-      const int nb = std::min(per, g.batch - b0);
-      RS_TRY(launch_tile(t, g, ks, kc, b0, nb, work, s));
+  auto run = [&](int t, const GemmArgs &a) -> cudaError_t {
+    for (int b0 = 0; b0 < a.batch; b0 += per) {
+      const int nb = std::min(per, a.batch - b0);
+      RS_TRY(launch_tile(t, a, ks, kc, b0, nb, work, s));
     }
     return cudaSuccess;
   };
@@ -340,11 +361,12 @@ cudaError_t dgemm(const GemmArgs &g, double *work, size_t work_elems, cudaStream
       RS_TRY(cudaEventCreate(&e0));
       RS_TRY(cudaEventCreate(&e1));
       float best_ms = 0;
+      const GemmArgs part = tune_part(g, ks);
       cudaError_t err = cudaSuccess;
       for (int t = 0; t < kNumTiles && err == cudaSuccess; ++t) {
         float ms = 0;
         err = cudaEventRecord(e0, s);
-        if (err == cudaSuccess) err = run(t);
+        if (err == cudaSuccess) err = run(t, part);
         if (err == cudaSuccess) err = cudaEventRecord(e1, s);
         if (err == cudaSuccess) err = cudaEventSynchronize(e1);
         if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, e0, e1);
@@ -360,7 +382,7 @@ cudaError_t dgemm(const GemmArgs &g, double *work, size_t work_elems, cudaStream
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     g_tune[key] = tile;
   }
-  return run(tile);
+  return run(tile, g);
 }
 
 int dgemm_tile_edge(const GemmArgs &g) {
