@@ -1306,42 +1306,16 @@ cudaError_t ensure_mo_tab(rssri_handle *h) {
   return cudaSuccess;
 }
 
-// Whether S7 for the orbitals' G is the Gram matrix of U (mo.cuh) or the
-// contraction over the P kept pairs: by flops, n^2 n_v^2 n_o (and a fifth for
-// the tiles on the diagonal) per tau point plus U once, against D once plus
-// 2 N_aux P^2 and the dense products per tau point.  Both run at the same
-// rate of the fp64 (or fp32) pipe.  At N = 100, N_aux = 300, eps = 1e-3 (P =
-// 3,560) a tau point is 1.5 against 9.5 GFLOP; the lines cross near N = 270.
-// The sliced block by time: the products of the kept pairs run at ~26e12 of
-// those flops per second (45% of the exchange's tile rows are outside the band,
-// and its digits are written for every tau point); the Gram tiles at ~78e12
-// with 20 bytes of HBM traffic per value and tau point, V at ~60e12.
-// C enters the orbital form by itself, and where that keeps pairs of floats (U is of degree
-// 2 in C) it has to be of order 1 for them to stay in fp32's range; the contraction over the
-// kept pairs meets C in G only, whose range the double-float form checks.
+// Whether S7 for the orbitals' G is the Gram matrix of U (mo.cuh) or the contraction over
+// the P kept pairs.  C enters the orbital form by itself, and where that keeps pairs of
+// floats (U is of degree 2 in C) it has to be of order 1 for them to stay in fp32's range; the
+// contraction over the kept pairs meets C in G only, whose range the double-float form checks.
 bool use_mo_block(const rssri_handle *h, int dd_arith) {
   if (h->P == 0) return false;
   if (dd_arith != RSSRI_DD_FP64 && !h->c_near) return false;
-  const double n = h->n, no = h->n_occ, nv = n - no, na = h->n_aux, P = h->P, nt = h->n_tau;
-  if (dd_arith == RSSRI_DD_OZ) {
-    if (h->n > 1024) return false;
-    const double K = nv * nv * no, tiles = std::ceil(n / 128.0);
-    const double width = std::ceil((n - 128.0 * (tiles - 1)) / 16.0) * 16.0;  // last column tile
-    const double area = 128.0 * (128.0 * tiles * (tiles - 1) / 2 + tiles * width);
-    const double pairs = 2.0 * P * P * na / 60e12 +
-                         nt * ((2.0 * na * P * P + 4.0 * na * n * n * n + 4.0 * P * na * na) / 26e12 +
-                               60e-6);
-    const double orbitals = (2.0 * P * nv * na + 2.0 * no * n * nv * na) / 4e12 +
-                            2.0 * n * nv * no * std::ceil(nv / 128.0) * 128.0 * na / 60e12 +
-                            40.0 * n * K / 5e12 + nt * (2.0 * area * K / 78e12 + 20.0 * n * K / 5e12);
-    return orbitals < pairs;
-  }
-  const double pairs = 2.0 * P * P * na +
-                       nt * (2.0 * na * P * P + 2.0 * P * n * na + 4.0 * na * n * n * n +
-                             4.0 * P * na * na);
-  const double orbitals = 2.0 * P * nv * na + 2.0 * no * n * nv * na + 2.0 * n * nv * nv * no * na +
-                          nt * 1.2 * n * n * nv * nv * no;
-  return orbitals < pairs;
+  if (dd_arith == RSSRI_DD_OZ)
+    return mo_block_pays_sliced(h->n, h->n_occ, h->n_aux, h->P, h->n_tau);
+  return mo_block_pays(h->n, h->n_occ, h->n_aux, h->P, h->n_tau);
 }
 
 // S7 for all tau points on the orbitals: out[t] = -U diag(w_t) U^T, in chunks of

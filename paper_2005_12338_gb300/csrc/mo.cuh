@@ -77,6 +77,42 @@ struct MoSum {
 size_t mo_sum_work(const MoSum &g);
 cudaError_t mo_sum(const MoSum &g, double *work, cudaStream_t s);
 
+// Whether the block on the orbitals is the cheaper one for P > 0 kept pairs.
+// fp64 and double-float, by flops: n^2 n_v^2 n_o (and a fifth for the tiles on the diagonal)
+// per tau point plus U once, against D once plus 2 N_aux P^2 and the dense products per tau
+// point.  Both run at the same rate of the fp64 (or fp32) pipe.  At N = 100, N_aux = 300,
+// eps = 1e-3 (P = 3,560) a tau point is 1.5 against 9.5 GFLOP; the lines cross near N = 270.
+inline bool mo_block_pays(int n_, int n_occ, int n_aux, int P_, int n_tau) {
+  const double n = n_, no = n_occ, nv = n - no, na = n_aux, P = P_, nt = n_tau;
+  const double pairs = 2.0 * P * P * na +
+                       nt * (2.0 * na * P * P + 2.0 * P * n * na + 4.0 * na * n * n * n +
+                             4.0 * P * na * na);
+  const double orbitals = 2.0 * P * nv * na + 2.0 * no * n * nv * na + 2.0 * n * nv * nv * no * na +
+                          nt * 1.2 * n * n * nv * nv * no;
+  return orbitals < pairs;
+}
+// Sliced (n <= 1024), by time, fitted to 122 sizes with both forms timed: N = 60 to 450, N_aux =
+// 3N, 0.3 to 0.55 of the orbitals occupied, eps = 1e-3 to 0.1, 2 to 64 tau points (setup in ms,
+// orbitals against pairs: N = 110, eps = 0.1, 8 tau points 4.3 : 7.0; N = 131, eps = 0.1, 64: 31 : 69;
+// N = 230, eps = 1e-2, 64: 204 : 261; N = 257, eps = 1e-3, 64: 420 : 576; N = 272, eps = 1e-2, 64:
+// 503 : 444; N = 400, eps = 1e-3, 16: 821 : 534).  The fit is within 21% of every time, and the
+// form it takes was the slower one at 3 sizes, by at most 6%.  Terms: V and U once, and per tau
+// point the Gram matrix's 128 x 128 tiles (with the digit products that its levels leave to do on
+// a gapped system's grid, about 0.6 of all) and the digits; the exchange, the dense products over
+// whole tiles, the passes over [n][n][N_aux], and the launches.
+inline bool mo_block_pays_sliced(int n, int n_occ, int n_aux, int P_, int n_tau) {
+  if (n > 1024) return false;
+  auto tiles = [](double x) { return (double)((long long)(x + 127) / 128 * 128); };
+  const double no = n_occ, nv = n - n_occ, na = n_aux, P = P_, nt = n_tau, K = nv * nv * no;
+  const double T = tiles(n) / 128.0, area = 128.0 * 128.0 * T * (T + 1.0) / 2.0;
+  const double orbitals = 2.0 * n * nv * no * tiles(nv) * na / 90e12 + 30e-12 * n * K +
+                          nt * (2.0 * area * K / 128e12 + 3e-12 * n * K);
+  const double pairs = nt * (2.0 * tiles(na) * P * P / 43e12 +
+                             2.0 * na * n * tiles(n) * (n + tiles(n)) / 40e12 +
+                             27e-12 * n * (double)n * na + 0.43e-3);
+  return orbitals < pairs;
+}
+
 // Per matrix z of M [nt][nb][n][n]: tr[z] = sum_o M_oo go_o and
 // s2[z] = sum_oo' M_oo' go_o' M_o'o go_o (fp64), go_t at go + t sgo.
 cudaError_t mo_traces(int df, const void *M, int nt, int nb, int n, int no, const void *go,
