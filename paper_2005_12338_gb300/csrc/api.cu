@@ -343,7 +343,7 @@ cudaError_t gemm_p(rssri_handle *h, int cls, const GemmArgs &g) {
 
 cudaError_t oz_product(rssri_handle *h, int cls, const OzView &va, int batch, int M,
                        const OzView *vb, int N, long long K, double *C, long long ldc,
-                       long long sC, int *err);
+                       long long sC, int *err, int joint = 0);
 OzView oz_rows(const double *x, long long ld, long long K, long long len);
 cudaError_t df_gemm_w(rssri_handle *h, const DfGemm &g);
 OzView oz_cols(const double *x, long long ld, long long K, long long len);
@@ -962,7 +962,6 @@ cudaError_t oz_slice_p(rssri_handle *h, const OzView &v, const OzDigits &o) {
 cudaError_t oz_gemm_p(rssri_handle *h, int cls, const OzGemm &g_in) {
   OzGemm g = g_in;
   g.wait_polls = h->test_wait_polls;
-  g.joint = cls == RSSRI_PROF_FACTOR_GEMM;
   const double alg = 2.0 * g.M * (double)g.N * g.A.K * g.batch;
   SPAN_T(cls, alg * 1e-9, oz_gemm_flops(g) * 1e-9);
   const size_t need = oz_gemm_work(g) * sizeof(double);
@@ -973,10 +972,10 @@ cudaError_t oz_gemm_p(rssri_handle *h, int cls, const OzGemm &g_in) {
 // C[b sC + i ldc + j] = sum_k A_b(i, k) B(j, k), fp64-accurate on the tensor
 // cores (digit slicing), for slicer views A (batch x M x K) and B (N x K,
 // shared by the batch; null: B is A with batch 1).  The digit buffers grow
-// as needed.  err: device flag of the bounded waits.
+// as needed.  err: device flag of the bounded waits; joint: see OzGemm.
 cudaError_t oz_product(rssri_handle *h, int cls, const OzView &va, int batch, int M,
                        const OzView *vb, int N, long long K, double *C, long long ldc,
-                       long long sC, int *err) {
+                       long long sC, int *err, int joint) {
   RS_TRY(oz_make(h->ozPA, batch, M, K));
   RS_TRY(oz_slice_p(h, va, h->ozPA.v));
   OzGemm g;
@@ -992,6 +991,7 @@ cudaError_t oz_product(rssri_handle *h, int cls, const OzView &va, int batch, in
   g.C = C; g.ldc = ldc; g.sC = sC;
   g.ccap = (long long)(batch - 1) * sC + (long long)(M - 1) * ldc + N;
   g.err = err;
+  g.joint = joint;
   return oz_gemm_p(h, cls, g);
 }
 
@@ -2233,7 +2233,7 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
     vt.bs = (long long)ns * na;
     const OzView vw = oz_cols(h->W.as<double>(), na, na, (long long)na * na);
     RS_CK(oz_product(h, RSSRI_PROF_FACTOR_GEMM, vt, 2, ns, &vw, na, na, Ut, na,
-                     (long long)ns * na, tc_err));
+                     (long long)ns * na, tc_err, 1));
   } else {
     GemmArgs g;
     g.M = ns; g.N = na; g.K = na; g.batch = 2;
@@ -2262,6 +2262,7 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
       g.C = fac + r0; g.ldc = nn; g.sC = 2LL * ns * nn;  // kind 0 of each set
       g.ccap = 4LL * ns * nn - r0;
       g.err = tc_err;
+      g.joint = 1;
       RS_CK(oz_gemm_p(h, RSSRI_PROF_FACTOR_GEMM, g));
     }
   } else if (fac_df64) {
@@ -2296,7 +2297,7 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
     vt.bs = (long long)ns * na;
     const OzView vk = oz_rows(h->KP.as<double>(), na, na, (long long)P * na);
     RS_CK(oz_product(h, RSSRI_PROF_FACTOR_GEMM, vt, 2, ns, &vk, P, na, h->RLp.as<double>(), P,
-                     (long long)ns * P, tc_err));
+                     (long long)ns * P, tc_err, 1));
   } else if (P > 0 && fac_df64) {
     // theta is +-1, exact as a pair; K_P was split at setup
     { SPAN(RSSRI_PROF_OTHER, 0.0); RS_CK(to_df64(theta, 2LL * ns * na, h->ut_hl.as<float2>(), s, range_flag(h))); }
