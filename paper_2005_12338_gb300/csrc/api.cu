@@ -1319,9 +1319,10 @@ bool use_mo_block(const rssri_handle *h, int dd_arith) {
 }
 
 // S7 for all tau points on the orbitals: out[t] = -U diag(w_t) U^T, in chunks of
-// occupied orbitals c (U and V of a chunk, 256 MB each at most; 1 GB of U for
-// the sliced form, whose launches per tau point want a long contraction) and of
-// tau points (their weights; the sliced form's digits, 1.6 GB).
+// occupied orbitals c, as many as keep U within 256 MB (V the same) but one at least, and of
+// tau points: their weights within 256 MB, or the sliced form's digits within 1.6 GB, one tau
+// point at least.  (One orbital of n = 1000 with 980 virtuals: U and V 7.7 GB each, the digits
+// of a tau point 11.5 GB.)
 cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
   const bool df = dd_arith != RSSRI_DD_FP64, oz = dd_arith == RSSRI_DD_OZ;
   cudaStream_t s = h->stream;
@@ -1329,17 +1330,15 @@ cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
   const long long nva = (long long)nv * na, row = (long long)n * nv;
   RS_TRY(ensure_mo_tab(h));
   const MoTab tab = mo_tab(h);
-  const size_t budget = (size_t)256 << 20;  // of U
+  const size_t budget = (size_t)256 << 20;
   const long long per_c = row * nv;
   const int cc = (int)std::max<long long>(1, std::min<long long>(no, (long long)(budget / 8) / per_c));
-  // V of as many c at a time as fit 256 MB
-  const int vc = (int)std::max<long long>(1, std::min<long long>(cc, (32LL << 20) / per_c));
   const long long kc = (long long)cc * nv * nv, ldc = oz ? (kc + 15) / 16 * 16 : kc;
   const int tcw = (int)std::max<long long>(
       1, std::min<long long>(nt, oz ? (1600LL << 20) / (12 * n * ldc) : (long long)(budget / 8) / kc));
   RS_TRY(ensure(h->moB1, (size_t)n * nva * 8));
   RS_TRY(ensure(h->moB2, (size_t)no * nva * 8));
-  RS_TRY(ensure(h->moV, (size_t)vc * per_c * 8));
+  RS_TRY(ensure(h->moV, (size_t)cc * per_c * 8));
   RS_TRY(ensure(h->moU, (size_t)n * ldc * 8));
   RS_TRY(ensure(h->moW, (size_t)(oz ? nt : tcw) * ldc * 8));
   MoGram q;
@@ -1437,12 +1436,11 @@ cudaError_t block_mo(rssri_handle *h, int dd_arith, double *out) {
     const int c = std::min(cc, no - c0);
     q.K = z.K = (long long)c * nv * nv;
     z.ldy = (z.K + 15) / 16 * 16;
-    for (int v0 = 0; v0 < c; v0 += vc) {
-      const int cv = std::min(vc, c - v0);
-      RS_TRY(form_v(c0 + v0, cv));
+    RS_TRY(form_v(c0, c));
+    {
       SPAN(RSSRI_PROF_OTHER, 0.0);
-      RS_TRY(mo_pack(df, h->moV.as<double>(), n, nv, cv, std::ldexp(1.0, -e2), oz ? 0 : q.K,
-                     (long long)v0 * nv * nv, h->moU.p, s));
+      RS_TRY(mo_pack(df, h->moV.as<double>(), n, nv, c, std::ldexp(1.0, -e2), oz ? 0 : q.K,
+                     h->moU.p, s));
     }
     if (oz) {
       {

@@ -140,11 +140,11 @@ cudaError_t mo_tables(const double *orb_e, int n, int no, double mu, const doubl
 // points, rows at stride ldw; df: pairs of the same times 2^-exps[t].
 cudaError_t mo_weights(int df, const double *gv, const double *go, int nv, int no, int c0, int nc,
                        int nt, const int *exps, long long ldw, void *w, cudaStream_t s);
-// U_ik, k = k0 + (c nv + a) nv + b, from V[c][b][i][a] (fp64, nc x nv x n x nv): slot a < b holds
+// U_ik, k = (c nv + a) nv + b, from V[c][b][i][a] (fp64, nc x nv x n x nv): slot a < b holds
 // (V_ab + V_ba) / sqrt 2, a = b holds V_aa, a > b holds (V_ba - V_ab) sqrt(3/2), all times
 // scale; df: pairs.  U_ik is at U[i ldu + k], or with ldu = 0 at U[((k / 16) n + i) 16 + k % 16].
 cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, double scale, long long ldu,
-                    long long k0, void *U, cudaStream_t s);
+                    void *U, cudaStream_t s);
 
 // out[a] = sum_q x[a][q]^2 (the diagonal of v^L on the kept pairs, where its largest magnitude is).
 cudaError_t mo_row_norm2(const double *x, int rows, int cols, double *out, cudaStream_t s);

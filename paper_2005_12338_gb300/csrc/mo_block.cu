@@ -34,7 +34,7 @@ __global__ void mo_weights_kernel(const double *__restrict__ gv, const double *_
 template <class P>
 __global__ void __launch_bounds__(256) mo_pack_kernel(const double *__restrict__ V, int n, int nv,
                                                       int nc, int T, double scale, long long ldu,
-                                                      long long koff, typename P::V *__restrict__ U) {
+                                                      typename P::V *__restrict__ U) {
   __shared__ double x[32][33], y[32][33];
   int ta, tb;
   tri_tile(blockIdx.x, T, ta, tb);
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) mo_pack_kernel(const double *__restrict__
     y[r][tx] = a2 < nv && b2 < nv ? Vc[((long long)b2 * n + i) * nv + a2] : 0.0;
   }
   __syncthreads();
-  const long long kc = koff + (long long)c * nv * nv;
+  const long long kc = (long long)c * nv * nv;
   auto at = [&](int a, int b) {
     const long long k = kc + (long long)a * nv + b;
     return ldu ? i * ldu + k : ((k >> 4) * n + i) * 16 + (k & 15);
@@ -149,13 +149,13 @@ cudaError_t mo_weights(int df, const double *gv, const double *go, int nv, int n
 }
 
 cudaError_t mo_pack(int df, const double *V, int n, int nv, int nc, double scale, long long ldu,
-                    long long k0, void *U, cudaStream_t s) {
+                    void *U, cudaStream_t s) {
   const int T = ceil_div(nv, 32);
   dim3 grid(T * (T + 1) / 2, n, nc);
   if (df)
-    mo_pack_kernel<DF><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, k0, static_cast<float2 *>(U));
+    mo_pack_kernel<DF><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, static_cast<float2 *>(U));
   else
-    mo_pack_kernel<F64><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, k0, static_cast<double *>(U));
+    mo_pack_kernel<F64><<<grid, 256, 0, s>>>(V, n, nv, nc, T, scale, ldu, static_cast<double *>(U));
   ++launch_counter();
   return cudaGetLastError();
 }
