@@ -122,7 +122,10 @@ typedef struct rssri_handle rssri_handle;
  *   eri3    [n][n][n_aux]  (ij|A) of Eq. 5; must satisfy (ij|A) == (ji|A) exactly
  *   metric  [n_aux][n_aux] V_AB of Eq. 6; symmetric positive definite
  *   orb_e   [n]            orbital energies, the first n_occ occupied
- *   orb_c   [n][n]         AO x MO coefficients, orthonormal (C^T C = I, S = I)
+ *   orb_c   [n][n]         AO x MO coefficients, orthonormal (C^T C = I, S = I).
+ *                          Where |C^T C - I| <= 5e-14 in every element, the fp64 and
+ *                          double-float chains run on the orbitals, about four times
+ *                          as fast as the products with G that other C keep
  *   tau     [n_tau]        grid nodes, each in (0, beta)
  *   tau_w   [n_tau]        quadrature weights of Eq. 26's tau integral
  *   mu      chemical potential; beta inverse temperature (finite, > 0)
@@ -181,13 +184,15 @@ typedef struct {
  *              cores: each row of an fp64 operand is scaled by a power of two
  *              and split into six 8-bit digits, every digit product and the
  *              accumulation of the leading levels are exact, ~1e-12 of
- *              sum |a||b| per dot product, with fp64's exponent range; the
- *              segmented product K^Q G runs in double-float on G(tau)
- *              normalised by a power of two per tau point and rescaled
- *              exactly, the block being homogeneous of degree 2 in G).  RSSRI_DD_OZ
- *              needs a GPU with tcgen05 (sm_100 family); its R, R^L and
- *              v^L are formed as for RSSRI_DD_DF64.
- *              The value given to rssri_setup sets how v^L and
+ *              sum |a||b| per dot product, with fp64's exponent range for
+ *              a caller's G; for the orbitals' G the block may be formed on
+ *              the orbitals, each tau point scaled by a power of two, where
+ *              rows of Sigma_DD below ~2^-200 of its largest element at that
+ *              tau point lose precision).  RSSRI_DD_OZ
+ *              needs a GPU with tcgen05 (sm_100 family); its metric root and
+ *              [K]^L are formed as for RSSRI_DD_DF64, and so are R and R^L except under
+ *              the tensor-core chains, where they are sliced products too.
+ *              The value given to rssri_setup sets how [K]^L, v^L and
  *              the cached block are formed; the value given to
  *              rssri_sigma_from_g sets the arithmetic of its rebuilt block,
  *              and that given to rssri_sigma the arithmetic of R, R^L and of
@@ -218,8 +223,10 @@ enum { RSSRI_DD_FP64 = 0, RSSRI_DD_DF64 = 1, RSSRI_DD_OZ = 2 };
 /* Kernel classes of the per-class profile (rssri_stats.prof_*). */
 enum {
   RSSRI_PROF_CHAIN_GEMM = 0,  /* S8 chain products X G, (X G) Y, C Gb, (2 t I - B) C */
-  RSSRI_PROF_DD_SPMM = 1,     /* S7 exchange term, pair-space contraction         */
-  RSSRI_PROF_DD_GEMM = 2,     /* S7 other products                                */
+  RSSRI_PROF_DD_SPMM = 1,     /* S7 exchange term, pair-space contraction; or the
+                                 sliced Gram matrices of the block on the orbitals */
+  RSSRI_PROF_DD_GEMM = 2,     /* S7 other products, and the Gram matrices in fp64
+                                 and double-float                                 */
   RSSRI_PROF_FACTOR_GEMM = 3, /* S4/S5 theta W, R, R^L                             */
   RSSRI_PROF_SETUP_GEMM = 4,  /* S1/S3 Newton-Schulz, [K]^L, D                     */
   RSSRI_PROF_GREEN = 5,       /* S6                                               */
@@ -250,7 +257,9 @@ typedef struct {
   double prof_ms[RSSRI_PROF_NCLASS];    /* device ms per class (profile = 1)     */
   double prof_gflop[RSSRI_PROF_NCLASS]; /* algorithmic fp64 GFLOP per class: 2mnk
                                            per product, 2 N_aux P^2 per S7 exchange
-                                           contraction (P kept pairs)            */
+                                           contraction (P kept pairs); a Gram matrix's
+                                           tiles on and above the diagonal (fp64,
+                                           double-float) or n^2 k (sliced)       */
   double prof_tensor_gflop[RSSRI_PROF_NCLASS]; /* GFLOP issued to the tensor cores
                                            per class (digit products of the sliced
                                            block and bf16/tf32 chain products, over
@@ -285,12 +294,14 @@ RSSRI_API const char *rssri_last_cuda_error(void);
 /* Steps that depend only on the system, the thresholds and G:
  *   S1  W = V^{-1/2} (Eq. 7) by the coupled Newton-Schulz iteration (fp64);
  *   S2  screen (ij|A) with eps' (Eq. 11) and compact the kept (i,j) pairs;
- *   S3  [K]^L = (ij|A)^L W on the kept pairs (Eq. 12), cut at eps (Eq. 13),
- *       and the pair-space product D = [K]^L [K]^L^T used by the exchange
- *       part of the deterministic block;
+ *   S3  [K]^L = (ij|A)^L W on the kept pairs (Eq. 12), cut at eps (Eq. 13);
  *   S6  G(tau), G(beta - tau) (Eq. 17) for every tau of the grid;
  *   S7  Sigma_DD(tau): Eq. 20 on v^L = sum_Q [K^Q]^L [K^Q]^L (the terms of
- *       Eq. 25 that hold no stochastic factor), in the arithmetic o->dd_arith.
+ *       Eq. 25 that hold no stochastic factor), in the arithmetic o->dd_arith:
+ *       on the orbitals, or as a contraction over the kept pairs with the
+ *       pair-space product D = [K]^L [K]^L^T, whichever is cheaper at the
+ *       problem's sizes.  D is formed where it is used, so after a setup on the
+ *       orbitals the first rssri_sigma_from_g (or RSSRI_EST_LITERAL) call forms it.
  * S6 and S7 do not depend on the draws: their results stay in the handle and
  * every rssri_sigma call on this setup reuses them (rssri_stats.t_green_dd_ms
  * is then 0).  Copies the problem into handle-owned device memory when it is
@@ -326,7 +337,10 @@ RSSRI_API int rssri_sigma(rssri_handle *h, const rssri_options *o, double *sigma
  * (the paper's general, e.g. self-consistent, G of Eq. 17) instead of being
  * built from the orbitals: g and gb are [n_tau][n][n], each matrix symmetric,
  * of the problem's ptr_kind.  The deterministic block (S7) is rebuilt for
- * this G in the arithmetic o->dd_arith on every call. */
+ * this G in the arithmetic o->dd_arith on every call, as a contraction over the
+ * kept pairs.  The first call after a setup whose own block was formed on the orbitals
+ * also forms that contraction's D (2 P^2 N_aux flops, P^2 doubles of device memory for
+ * P kept pairs) and, sliced, its digits, and may return RSSRI_ERR_OOM for them. */
 RSSRI_API int rssri_sigma_from_g(rssri_handle *h, const rssri_options *o,
                        const double *g, const double *gb, double *sigma,
                        double *e_pair, double *e_corr, double *e_stderr,

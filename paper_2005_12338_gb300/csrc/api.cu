@@ -176,7 +176,6 @@ struct rssri_handle {
   // left operand and the digits of K_P (setup); per-tau digit buffers
   bool oz_ready = false;
   OzExch oz_geo;
-  DevBuf oz_gs, oz_gexp;  // G(tau) 2^-e(tau) as pairs, and e(tau), for K^Q G
   DevBuf oz_pidx, oz_tmp;
   OzBuf ozX, ozKP, ozKPt, ozGb, ozBig0, ozBig1, ozAtP, ozGam;
   OzBuf ozPA, ozPB;  // operands of the setup and factor products (RSSRI_DD_OZ)
@@ -527,7 +526,7 @@ void rssri_destroy(rssri_handle *h) {
                     &h->hxsl, &h->hy3, &h->hg, &h->hgb, &h->hP, &h->hdcl16, &h->hxy32, &h->ha6, &h->hct, &h->hdct, &h->hpart, &h->hfold, &h->hclt, &h->hfl, &h->Dhl,
                     &h->Ahl, &h->KPhl, &h->PGhl, &h->APhl, &h->Gamhl, &h->GGhl, &h->litMP, &h->litT, &h->litMhl, &h->eri_hl, &h->ut_hl, &h->nsA2, &h->nsB2, &h->elHl, &h->facHl, &h->xgHl, &h->cHl, &h->bHl, &h->cv_params, &h->cv_m, &h->cv_v, &h->cv_grad, &h->cv_ptmp,
                     &h->cv_act, &h->cv_work, &h->cv_X, &h->cv_t, &h->cv_w, &h->cv_stats, &h->cv_c,
-                    &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0, &h->oz_gs, &h->oz_gexp,
+                    &h->cv_scr, &h->cv_bx, &h->cv_bt, &h->cv_bw, &h->cv_loss, &h->sdd0,
                     &h->moTab, &h->moChl, &h->moZ, &h->moM, &h->moTr, &h->moAcc, &h->moWork,
                     &h->moB1, &h->moB2, &h->moV, &h->moU, &h->moW, &h->moRow, &h->ozYm, &h->ozY6, &h->ozYsel};
   for (DevBuf *b : bufs) release(*b);

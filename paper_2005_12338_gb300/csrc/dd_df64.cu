@@ -62,42 +62,6 @@ __global__ void to_df64_kernel(const double *__restrict__ x, long long len, floa
   }
 }
 
-// One block per segment c of len values: e[c] = the exponent of the segment's
-// largest magnitude (2^e <= max < 2^(e+1); 0 for a zero segment) and
-// y = pairs of x 2^-e (an exact power-of-two scaling).
-__global__ void __launch_bounds__(1024) to_df64_scaled_kernel(const double *__restrict__ x,
-                                                              long long len,
-                                                              float2 *__restrict__ y,
-                                                              int *__restrict__ e_out) {
-  const long long base = (long long)blockIdx.x * len;
-  int mx = 0;
-  for (long long i = threadIdx.x; i < len; i += blockDim.x)
-    mx = max(mx, (int)((__double_as_longlong(x[base + i]) >> 52) & 0x7FF));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  __shared__ int smax;
-  if (threadIdx.x == 0) smax = 0;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) atomicMax(&smax, mx);
-  __syncthreads();
-  const int e = smax ? smax - 1023 : 0;
-  if (threadIdx.x == 0) e_out[blockIdx.x] = e;
-  for (long long i = threadIdx.x; i < len; i += blockDim.x) {
-    const double v = scalbn(x[base + i], -e);
-    const float hi = __double2float_rn(v);
-    y[base + i] = make_float2(hi, __double2float_rn(v - (double)hi));
-  }
-}
-
-// x *= 2^(mult e[0])
-__global__ void scale_pow2_kernel(double *__restrict__ x, long long len,
-                                  const int *__restrict__ e, int mult) {
-  const int k = mult * e[0];
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len;
-       i += (long long)gridDim.x * blockDim.x)
-    x[i] = scalbn(x[i], k);
-}
-
 // ------------------------------------------------- double-float products --
 // C = alpha op(A) op(B) with A, B already split into (hi, lo) float pairs.
 // MODE 0: strided operands; MODE 1: segmented (A(m,kk) = A[col[s0+kk]*lda + m],
@@ -319,21 +283,6 @@ __global__ void gather_rows_f2_kernel(const float2 *__restrict__ src, const int 
   for (int c = threadIdx.x; c < ncols; c += blockDim.x) d[c] = s[c];
 }
 }  // namespace
-
-cudaError_t to_df64_scaled(const double *x, int segments, long long len, float2 *y, int *e,
-                           cudaStream_t s) {
-  if (segments <= 0 || len <= 0) return cudaSuccess;
-  to_df64_scaled_kernel<<<segments, 1024, 0, s>>>(x, len, y, e);
-  ++launch_counter();
-  return cudaGetLastError();
-}
-
-cudaError_t scale_pow2(double *x, long long len, const int *e, int mult, cudaStream_t s) {
-  if (len <= 0) return cudaSuccess;
-  scale_pow2_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, e, mult);
-  ++launch_counter();
-  return cudaGetLastError();
-}
 
 cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s) {
   if (len <= 0) return cudaSuccess;

@@ -1994,16 +1994,14 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
   return cudaSuccess;
 }
 
-// Gram matrices at n = 200 (100 virtual orbitals, 64 tau points): 0.83 ms for the
-// products of a tau point with all digits (1,600 TFLOP/s) and 53 ms for all 64 (blocks of
-// columns that are small at a tau point have only their leading digits multiplied),
-// against 88 ms with all 21 products of every block; the digits take 28 ms.  The
+// Gram matrices at n = 200 (100 virtual orbitals, 64 tau points, K = 10^6): 53 ms for the
+// products of all tau points, 0.83 ms each (blocks of columns that are small at a tau point
+// have only their leading digits multiplied), against 88 ms, 1.38 ms each (1,500 TFLOP/s of
+// products issued), with all 21 products of every block; the digits take 37 ms.  The
 // whole setup and sampling call takes 122 ms against 281 with the contraction over the
 // kept pairs (exchange 136, dense products 60, digits 48).  With rows of digits
 // K-contiguous over the whole contraction, 12 MB apart, the products took 1.6 times as
-// long: their 128-byte pieces came from 128 different DRAM pages.  A narrower last column
-// tile (80 of 128 columns) does not help: the products are not faster below 128 columns
-// (A's rows are read from shared memory whatever the width), and 1,139 us became 1,003.
+// long: their 128-byte pieces came from 128 different DRAM pages.
 namespace {
 // The tiles on and above the diagonal, and the K splits of each: as many as make the
 // rounds of tiles over the SMs, times a split's K steps plus a tile's drain and stores
