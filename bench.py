@@ -735,7 +735,8 @@ def our_arm(args):
                     "(rssri_peak_measure) and the library DGEMM (torch float64 matmul, "
                     "4096^3)")
             bound, unit = "alu", "TFLOP/s"
-            work = "algorithmic fp64 flops (2 N_aux P^2 per exchange contraction, 2mnk per product)"
+            work = ("algorithmic fp64 flops (2mnk per product; of a Gram matrix the tiles on and "
+                    "above the diagonal; 2 N_aux P^2 per exchange contraction)")
         launches = int(pr["l"][dom])
         return {"bound": bound, "kernel": name, "achieved": achieved, "peak": peak,
                 "unit": unit, "frac": achieved / peak if peak else None,

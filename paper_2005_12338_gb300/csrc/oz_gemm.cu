@@ -1997,11 +1997,12 @@ cudaError_t oz_gemm(const OzGemm &g, double *work, size_t work_elems, cudaStream
 // Gram matrices at n = 200 (100 virtual orbitals, 64 tau points, K = 10^6): 53 ms for the
 // products of all tau points, 0.83 ms each (blocks of columns that are small at a tau point
 // have only their leading digits multiplied), against 88 ms, 1.38 ms each (1,500 TFLOP/s of
-// products issued), with all 21 products of every block; the digits take 37 ms.  The
-// whole setup and sampling call takes 122 ms against 281 with the contraction over the
-// kept pairs (exchange 136, dense products 60, digits 48).  With rows of digits
-// K-contiguous over the whole contraction, 12 MB apart, the products took 1.6 times as
-// long: their 128-byte pieces came from 128 different DRAM pages.
+// products issued), with all 21 products of every block; the digits take 28 ms (37 with the
+// row maxima, the levels and the digits of V's operands).  The whole setup and sampling call
+// takes 122 ms against 281 with the contraction over the kept pairs (exchange 136, dense
+// products 60, digits 48).  With rows of digits K-contiguous over the whole contraction, 12 MB
+// apart, the products took 1.6 times as long: their 128-byte pieces came from 128 different
+// DRAM pages.
 namespace {
 // The tiles on and above the diagonal, and the K splits of each: as many as make the
 // rounds of tiles over the SMs, times a split's K steps plus a tile's drain and stores
