@@ -1840,6 +1840,14 @@ bool use_mo_chain(const rssri_handle *h) {
   return h->orth_ok && 4LL * (h->n - h->n_occ) < 3LL * h->n_tau * h->n;
 }
 
+// The chain on the orbitals in pairs of floats keeps M, of degree 2 in the factors, and its
+// products, of degree 4, while G, normalised per tau point, no longer makes up for large or small
+// factors as it may in X G Y.  So the factors' pairs are scaled by 2^-e, exactly, e from the
+// setup's largest |[K]^L| (R of that element is a sum of N_aux terms +-K of its size at most).
+int mo_fac_exp(const rssri_handle *h) {
+  return h->k_l_max > 0 && std::isfinite(h->k_l_max) ? std::ilogb(h->k_l_max) : 0;
+}
+
 // S8 and the orbital-basis sum of S10 for all pairs, in batches of nb pairs and
 // chunks of tau points: sig[t] = sdd[t] + (C (sum over pairs of F) C^T) / ns, and
 // the pair energies are added to e_st.
@@ -1861,6 +1869,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
   RS_TRY(ensure(h->moAcc, (size_t)nt * nn * sizeof(double)));
   MoSum q;
   q.df = df; q.n = n; q.no = no; q.nkind = nkind;
+  q.fexp = df ? 4 * mo_fac_exp(h) : 0;
   size_t work = 0;
   for (int c : {std::min(nb, ns), ns % nb ? ns % nb : nb})
     for (int t : {tc, nt % tc ? nt % tc : tc}) {
@@ -1930,7 +1939,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
         SPAN(RSSRI_PROF_OTHER, 0.0);
         RS_TRY(mo_traces(df, h->moM.p, c, nkind * cnt, n, no, go, no, tr, s2, s));
         RS_TRY(mo_energy(tr, s2, c, nkind, cnt, h->tau_w + t0, df ? tab.eexp + t0 : nullptr,
-                         2.0 * no, h->e_st.as<double>() + x0, s));
+                         q.fexp, 2.0 * no, h->e_st.as<double>() + x0, s));
       }
       q.cnt = cnt; q.nt = c;
       q.M = h->moM.p; q.go = go; q.sgo = no; q.tr = tr;
@@ -2321,7 +2330,8 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
 
   if (chain_df64) {
     SPAN(RSSRI_PROF_OTHER, 0.0);
-    RS_CK(to_df64(fac, 4LL * ns * nn, h->facHl.as<float2>(), s, range_flag(h)));
+    RS_CK(to_df64(fac, 4LL * ns * nn, h->facHl.as<float2>(), s, range_flag(h),
+                  mo ? std::ldexp(1.0, -mo_fac_exp(h)) : 1.0));
   }
 
   // ---- learned control variate: coefficients, or statistics for training

@@ -29,13 +29,13 @@ __global__ void from_df64_kernel(const float2 *__restrict__ x, long long len,
 // (zero arrays pass): the block maxima of the exponent field go to range[1],
 // and the last block to finish (range[2] counts them) checks and resets both.
 __global__ void to_df64_kernel(const double *__restrict__ x, long long len, float2 *__restrict__ y,
-                               int *__restrict__ range) {
+                               double scale, int *__restrict__ range) {
   int mx = 0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < len;
        e += (long long)gridDim.x * blockDim.x) {
-    const double v = x[e];
-    const float hi = __double2float_rn(v);
-    y[e] = make_float2(hi, __double2float_rn(v - (double)hi));
+    const double v = x[e], u = v * scale;
+    const float hi = __double2float_rn(u);
+    y[e] = make_float2(hi, __double2float_rn(u - (double)hi));
     mx = max(mx, (int)((__double_as_longlong(v) >> 52) & 0x7FF));
   }
   if (!range) return;
@@ -291,9 +291,10 @@ cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s)
   return cudaGetLastError();
 }
 
-cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s, int *range) {
+cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s, int *range,
+                    double scale) {
   if (len <= 0) return cudaSuccess;
-  to_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y, range);
+  to_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y, scale, range);
   ++launch_counter();
   return cudaGetLastError();
 }

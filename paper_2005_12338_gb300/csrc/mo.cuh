@@ -62,7 +62,7 @@ double mo_gram_flops(const MoGram &g);
 // Sum over sample pairs x < cnt and kinds k < nkind (k = 0: sign +, else -) of
 // sgn (M_(:,o) go M_(o,:) - 2 t M) per tau: M [nt][nkind][cnt][n][n], go
 // [nt][no] at stride sgo, tr [nt][nkind][cnt] the traces t; acc[t] [n][n] (+)=
-// 2^e_t that sum (e_t = texp[t], null: 0).  The pairs are dealt to `groups`
+// 2^(e_t + fexp) that sum (e_t = texp[t]; texp null: neither).  The pairs are dealt to `groups`
 // partial sums, added in a fixed order; work: mo_sum_work() doubles.
 struct MoSum {
   int df = 0;
@@ -71,6 +71,7 @@ struct MoSum {
   long long sgo = 0;
   const double *tr = nullptr;
   const int *texp = nullptr;
+  int fexp = 0;
   double *acc = nullptr;  // [nt][n][n]
   int accumulate = 0;
 };
@@ -117,10 +118,10 @@ inline bool mo_block_pays_sliced(int n, int n_occ, int n_aux, int P_, int n_tau)
 // s2[z] = sum_oo' M_oo' go_o' M_o'o go_o (fp64), go_t at go + t sgo.
 cudaError_t mo_traces(int df, const void *M, int nt, int nb, int n, int no, const void *go,
                       long long sgo, double *tr, double *s2, cudaStream_t s);
-// e_st[x] += -(1 / ne) sum_t tau_w[t] 2^(2 e_t) sum_k (+-)(2 tr^2 - s2), tau in order; tau_w on the
-// device, e_t = texp[t] (null: 0).
+// e_st[x] += -(1 / ne) sum_t tau_w[t] 2^(2 e_t + fexp) sum_k (+-)(2 tr^2 - s2), tau in order; tau_w
+// on the device, e_t = texp[t] (texp null: neither).
 cudaError_t mo_energy(const double *tr, const double *s2, int nt, int nkind, int cnt,
-                      const double *tau_w, const int *texp, double ne, double *e_st,
+                      const double *tau_w, const int *texp, int fexp, double ne, double *e_st,
                       cudaStream_t s);
 
 // The diagonals gv[t][a] = exp(-(e_(no+a) - mu) tau_t), go[t][c] = exp((e_c - mu) tau_t) in fp64,

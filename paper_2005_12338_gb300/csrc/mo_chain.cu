@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(256) mo_traces_kernel(const typename P::V *__r
 
 __global__ void mo_energy_kernel(const double *__restrict__ tr, const double *__restrict__ s2, int nt,
                                  int nkind, int cnt, const double *__restrict__ tau_w,
-                                 const int *__restrict__ eexp, double ne,
+                                 const int *__restrict__ eexp, int fexp, double ne,
                                  double *__restrict__ e_st) {
   for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < cnt; x += gridDim.x * blockDim.x) {
     double e = e_st[x];
@@ -226,7 +226,7 @@ __global__ void mo_energy_kernel(const double *__restrict__ tr, const double *__
         const double v = 2.0 * tr[z] * tr[z] - s2[z];
         de += k == 0 ? v : -v;
       }
-      if (eexp) de = scalbn(de, 2 * eexp[t]);
+      if (eexp) de = scalbn(de, 2 * eexp[t] + fexp);
       e += -tau_w[t] * de / ne;
     }
     e_st[x] = e;
@@ -358,7 +358,7 @@ cudaError_t mo_sum(const MoSum &g, double *work, cudaStream_t s) {
   }
   RS_TRY(e);
   mo_reduce_kernel<<<grid_cap((long long)g.nt * g.n * g.n, 256), 256, 0, s>>>(
-      work, a.groups, g.n, g.nt, 1.0, g.texp, 0, g.accumulate, g.acc);
+      work, a.groups, g.n, g.nt, 1.0, g.texp, g.fexp, 0, g.accumulate, g.acc);
   ++launch_counter();
   return cudaGetLastError();
 }
@@ -380,9 +380,10 @@ cudaError_t mo_traces(int df, const void *M, int nt, int nb, int n, int no, cons
 }
 
 cudaError_t mo_energy(const double *tr, const double *s2, int nt, int nkind, int cnt,
-                      const double *tau_w, const int *texp, double ne, double *e_st,
+                      const double *tau_w, const int *texp, int fexp, double ne, double *e_st,
                       cudaStream_t s) {
-  mo_energy_kernel<<<grid_cap(cnt, 128), 128, 0, s>>>(tr, s2, nt, nkind, cnt, tau_w, texp, ne, e_st);
+  mo_energy_kernel<<<grid_cap(cnt, 128), 128, 0, s>>>(tr, s2, nt, nkind, cnt, tau_w, texp, fexp, ne,
+                                                      e_st);
   ++launch_counter();
   return cudaGetLastError();
 }
