@@ -1843,9 +1843,11 @@ bool use_mo_chain(const rssri_handle *h) {
 // The chain on the orbitals in pairs of floats keeps M, of degree 2 in the factors, and its
 // products, of degree 4, while G, normalised per tau point, no longer makes up for large or small
 // factors as it may in X G Y.  So the factors' pairs are scaled by 2^-e, exactly, e from the
-// setup's largest |[K]^L| (R of that element is a sum of N_aux terms +-K of its size at most).
+// setup's largest |[K]^L| (R of that element is a sum of N_aux terms +-K of its size at most);
+// beyond 2^+-100 the factors' own range check refuses the call.
 int mo_fac_exp(const rssri_handle *h) {
-  return h->k_l_max > 0 && std::isfinite(h->k_l_max) ? std::ilogb(h->k_l_max) : 0;
+  if (!(h->k_l_max > 0) || !std::isfinite(h->k_l_max)) return 0;
+  return std::max(-100, std::min(100, std::ilogb(h->k_l_max)));
 }
 
 // S8 and the orbital-basis sum of S10 for all pairs, in batches of nb pairs and
@@ -1869,7 +1871,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
   RS_TRY(ensure(h->moAcc, (size_t)nt * nn * sizeof(double)));
   MoSum q;
   q.df = df; q.n = n; q.no = no; q.nkind = nkind;
-  q.fexp = df ? 4 * mo_fac_exp(h) : 0;
+  const int fexp = df ? 4 * mo_fac_exp(h) : 0;
   size_t work = 0;
   for (int c : {std::min(nb, ns), ns % nb ? ns % nb : nb})
     for (int t : {tc, nt % tc ? nt % tc : tc}) {
@@ -1939,7 +1941,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
         SPAN(RSSRI_PROF_OTHER, 0.0);
         RS_TRY(mo_traces(df, h->moM.p, c, nkind * cnt, n, no, go, no, tr, s2, s));
         RS_TRY(mo_energy(tr, s2, c, nkind, cnt, h->tau_w + t0, df ? tab.eexp + t0 : nullptr,
-                         q.fexp, 2.0 * no, h->e_st.as<double>() + x0, s));
+                         fexp, 2.0 * no, h->e_st.as<double>() + x0, s));
       }
       q.cnt = cnt; q.nt = c;
       q.M = h->moM.p; q.go = go; q.sgo = no; q.tr = tr;
@@ -1950,7 +1952,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
       RS_TRY(mo_sum(q, h->moWork.as<double>(), s));
     }
   }
-  // sig = sdd + C acc C^T / ns
+  // sig = sdd + 2^fexp C acc C^T / ns
   RS_TRY(cudaMemcpyAsync(sig, sdd, nt * nn * sizeof(double), cudaMemcpyDeviceToDevice, s));
   GemmArgs g;
   g.M = g.N = g.K = n; g.batch = nt;
@@ -1960,7 +1962,7 @@ cudaError_t chain_mo(rssri_handle *h, int ns, int nb, int nkind, bool df, const 
   RS_TRY(gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g));
   g.A = h->moM.as<double>(); g.sA = nn;
   g.B = h->orb_c; g.sB = 0; g.transB = 1;
-  g.C = sig; g.alpha = 1.0 / ns; g.beta = 1.0;
+  g.C = sig; g.alpha = std::ldexp(1.0 / ns, fexp); g.beta = 1.0;
   return gemm_p(h, RSSRI_PROF_CHAIN_GEMM, g);
 }
 
@@ -2331,7 +2333,7 @@ int issue_sigma(rssri_handle *h, const rssri_options *o, const double *g_in, con
   if (chain_df64) {
     SPAN(RSSRI_PROF_OTHER, 0.0);
     RS_CK(to_df64(fac, 4LL * ns * nn, h->facHl.as<float2>(), s, range_flag(h),
-                  mo ? std::ldexp(1.0, -mo_fac_exp(h)) : 1.0));
+                  mo ? -mo_fac_exp(h) : 0));
   }
 
   // ---- learned control variate: coefficients, or statistics for training

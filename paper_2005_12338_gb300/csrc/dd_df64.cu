@@ -29,14 +29,19 @@ __global__ void from_df64_kernel(const float2 *__restrict__ x, long long len,
 // (zero arrays pass): the block maxima of the exponent field go to range[1],
 // and the last block to finish (range[2] counts them) checks and resets both.
 __global__ void to_df64_kernel(const double *__restrict__ x, long long len, float2 *__restrict__ y,
-                               double scale, int *__restrict__ range) {
+                               int k, int *__restrict__ range) {
   int mx = 0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < len;
        e += (long long)gridDim.x * blockDim.x) {
-    const double v = x[e], u = v * scale;
+    const double v = x[e];
+    // v 2^k by its exponent field (a multiplication on the fp64 pipe is a quarter of this
+    // kernel's work there); what is or becomes subnormal is zero as a pair of floats anyway
+    const int top = __double2hiint(v), ex = (top >> 20) & 0x7FF;
+    const double u = ex > max(0, -k) ? __hiloint2double(top + k * (1 << 20), __double2loint(v))
+                                      : __hiloint2double(top & (int)0x80000000u, 0);
     const float hi = __double2float_rn(u);
     y[e] = make_float2(hi, __double2float_rn(u - (double)hi));
-    mx = max(mx, (int)((__double_as_longlong(v) >> 52) & 0x7FF));
+    mx = max(mx, ex);
   }
   if (!range) return;
 #pragma unroll
@@ -292,9 +297,9 @@ cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s)
 }
 
 cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s, int *range,
-                    double scale) {
+                    int k) {
   if (len <= 0) return cudaSuccess;
-  to_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y, scale, range);
+  to_df64_kernel<<<grid_cap(len, 256), 256, 0, s>>>(x, len, y, k, range);
   ++launch_counter();
   return cudaGetLastError();
 }

@@ -5,13 +5,13 @@
 
 namespace rssri {
 
-// y[e] = (hi, lo) with hi = fl32(u), lo = fl32(u - hi), u = x[e] scale.  A pair keeps
+// y[e] = (hi, lo) with hi = fl32(u), lo = fl32(u - hi), u = x[e] 2^k, |k| <= 1000.  A pair keeps
 // ~48 bits only inside fp32's exponent range (normal numbers from 2^-126, and
 // products whose error terms stay normal), so when range is given (3 ints,
 // range[1..2] zero before the first call) range[0] |= 1 if the largest
 // magnitude of x lies outside [2^-40, 2^40].
 cudaError_t to_df64(const double *x, long long len, float2 *y, cudaStream_t s,
-                    int *range = nullptr, double scale = 1.0);
+                    int *range = nullptr, int k = 0);
 // y = hi + lo of every pair.
 cudaError_t from_df64(const float2 *x, long long len, double *y, cudaStream_t s);
 // T[m][q][j] = sum_{a in row m} sum_{b in row j} D[a*P+b] * At[(col[a]*n+col[b])*naux+q],

@@ -62,7 +62,7 @@ double mo_gram_flops(const MoGram &g);
 // Sum over sample pairs x < cnt and kinds k < nkind (k = 0: sign +, else -) of
 // sgn (M_(:,o) go M_(o,:) - 2 t M) per tau: M [nt][nkind][cnt][n][n], go
 // [nt][no] at stride sgo, tr [nt][nkind][cnt] the traces t; acc[t] [n][n] (+)=
-// 2^(e_t + fexp) that sum (e_t = texp[t]; texp null: neither).  The pairs are dealt to `groups`
+// 2^e_t that sum (e_t = texp[t], null: 0).  The pairs are dealt to `groups`
 // partial sums, added in a fixed order; work: mo_sum_work() doubles.
 struct MoSum {
   int df = 0;
@@ -71,7 +71,6 @@ struct MoSum {
   long long sgo = 0;
   const double *tr = nullptr;
   const int *texp = nullptr;
-  int fexp = 0;
   double *acc = nullptr;  // [nt][n][n]
   int accumulate = 0;
 };

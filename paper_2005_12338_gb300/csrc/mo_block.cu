@@ -130,7 +130,7 @@ cudaError_t mo_gram(const MoGram &g, double *work, cudaStream_t s) {
   a.out = work;
   RS_TRY(nt_dispatch<1>(g.df, a, (long long)g.nt * ks, s));
   mo_reduce_kernel<<<grid_cap((long long)g.nt * g.n * g.n, 256), 256, 0, s>>>(
-      work, ks, g.n, g.nt, -1.0, g.wexp, 0, 1, g.accumulate, g.out);
+      work, ks, g.n, g.nt, -1.0, g.wexp, 1, g.accumulate, g.out);
   ++launch_counter();
   return cudaGetLastError();
 }

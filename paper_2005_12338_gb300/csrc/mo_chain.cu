@@ -358,7 +358,7 @@ cudaError_t mo_sum(const MoSum &g, double *work, cudaStream_t s) {
   }
   RS_TRY(e);
   mo_reduce_kernel<<<grid_cap((long long)g.nt * g.n * g.n, 256), 256, 0, s>>>(
-      work, a.groups, g.n, g.nt, 1.0, g.texp, g.fexp, 0, g.accumulate, g.acc);
+      work, a.groups, g.n, g.nt, 1.0, g.texp, 0, g.accumulate, g.acc);
   ++launch_counter();
   return cudaGetLastError();
 }

@@ -219,10 +219,9 @@ __global__ void __launch_bounds__(G::NT, G::MINB) mo_nt_kernel(const NtArgs g) {
   }
 }
 
-// out[t][e] (+)= sign 2^(e_t + e0) sum_s part[t][s][src(e)] (texp null: neither), s in order;
-// sym: (i > j) reads (j, i).
+// out[t][e] (+)= sign 2^e_t sum_s part[t][s][src(e)], s in order; sym: (i > j) reads (j, i).
 __global__ void mo_reduce_kernel(const double *__restrict__ part, int ns, int n, int nt, double sign,
-                                 const int *__restrict__ texp, int e0, int sym, int accumulate,
+                                 const int *__restrict__ texp, int sym, int accumulate,
                                  double *__restrict__ out) {
   const long long nn = (long long)n * n, total = nn * nt;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -237,7 +236,7 @@ __global__ void mo_reduce_kernel(const double *__restrict__ part, int ns, int n,
     double s = 0.0;
     for (int k = 0; k < ns; ++k) s += p[k * nn];
     s *= sign;
-    if (texp) s = scalbn(s, texp[t] + e0);
+    if (texp) s = scalbn(s, texp[t]);
     out[e] = accumulate ? out[e] + s : s;
   }
 }
